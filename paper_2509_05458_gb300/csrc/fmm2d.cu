@@ -1313,10 +1313,10 @@ static void apply_t(cfmm_plan_s* P, Fmm2dState* S, const cd* sigma, const cd* ta
     if (T.nboxes <= 1) {
         for (int i = 2; i <= 6; ++i) rec(i);
         launch_p2p(2, KER, K, T.d_leaf_boxes.get(), T.nleaves, T.start.get(), T.end.get(), T.loff[0].get(),
-                   T.lent[0].get(), u, nrhs, false, st, P->precision == CFMM_MIXED);
+                   T.lent[0].get(), u, nrhs, false, st, P->precision == CFMM_MIXED, P->leaf_size);
         if (g)
             launch_p2p_grad(2, KER, K, T.d_leaf_boxes.get(), T.nleaves, T.start.get(), T.end.get(), T.loff[0].get(),
-                            T.lent[0].get(), g, nrhs, st);
+                            T.lent[0].get(), g, nrhs, st, P->leaf_size);
         rec(7);
         rec(8);
         return;
@@ -1334,10 +1334,10 @@ static void apply_t(cfmm_plan_s* P, Fmm2dState* S, const cd* sigma, const cd* ta
     {
         cudaStream_t ns = near_fork(P);
         launch_p2p(2, KER, K, S->d_leaves_l0.get(), (int)S->leaves_l0.size(), T.start.get(), T.end.get(),
-                   T.loff[0].get(), T.lent[0].get(), u, nrhs, false, ns, P->precision == CFMM_MIXED);
+                   T.loff[0].get(), T.lent[0].get(), u, nrhs, false, ns, P->precision == CFMM_MIXED, P->leaf_size);
         if (g)
             launch_p2p_grad(2, KER, K, S->d_leaves_l0.get(), (int)S->leaves_l0.size(), T.start.get(), T.end.get(),
-                            T.loff[0].get(), T.lent[0].get(), g, nrhs, ns);
+                            T.loff[0].get(), T.lent[0].get(), g, nrhs, ns, P->leaf_size);
     }
     near_launched(P);
     // (1) P2M (shared memory sized by the leaves' orders)

@@ -507,10 +507,10 @@ void fmm3d_apply(cfmm_plan_s* P, const cd* sigma, const cd* tau, int64_t dstride
     if (T.nboxes <= 1) {
         for (int i = 2; i <= 6; ++i) rec(i);
         launch_p2p(3, P->kernel, K, T.d_leaf_boxes.get(), T.nleaves, T.start.get(), T.end.get(), T.loff[0].get(),
-                   T.lent[0].get(), u, nrhs, false, st, mixed);
+                   T.lent[0].get(), u, nrhs, false, st, mixed, P->leaf_size);
         if (g)
             launch_p2p_grad(3, P->kernel, K, T.d_leaf_boxes.get(), T.nleaves, T.start.get(), T.end.get(),
-                            T.loff[0].get(), T.lent[0].get(), g, nrhs, st);
+                            T.loff[0].get(), T.lent[0].get(), g, nrhs, st, P->leaf_size);
         rec(7);
         rec(8);
         return;
@@ -533,10 +533,10 @@ void fmm3d_apply(cfmm_plan_s* P, const cd* sigma, const cd* tau, int64_t dstride
     {
         cudaStream_t ns = near_fork(P);
         launch_p2p(3, P->kernel, K, S->d_leaves_l0.get(), (int)S->leaves_l0.size(), T.start.get(), T.end.get(),
-                   T.loff[0].get(), T.lent[0].get(), u, nrhs, false, ns, mixed);
+                   T.loff[0].get(), T.lent[0].get(), u, nrhs, false, ns, mixed, P->leaf_size);
         if (g)
             launch_p2p_grad(3, P->kernel, K, S->d_leaves_l0.get(), (int)S->leaves_l0.size(), T.start.get(),
-                            T.end.get(), T.loff[0].get(), T.lent[0].get(), g, nrhs, ns);
+                            T.end.get(), T.loff[0].get(), T.lent[0].get(), g, nrhs, ns, P->leaf_size);
     }
     near_launched(P);
     // (1) P2M (single layer: one lane per harmonic column; complex64 products

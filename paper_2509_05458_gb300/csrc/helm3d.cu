@@ -2177,10 +2177,10 @@ void helm3d_apply(cfmm_plan_s* P, const cd* sigma, const cd* tau, int64_t dstrid
     if (T.nboxes <= 1) {
         for (int i = 2; i <= 6; ++i) rec(i);
         launch_p2p(3, P->kernel, K, T.d_leaf_boxes.get(), T.nleaves, T.start.get(), T.end.get(), T.loff[0].get(),
-                   T.lent[0].get(), u, nrhs, false, st, mixed);
+                   T.lent[0].get(), u, nrhs, false, st, mixed, P->leaf_size);
         if (g)
             launch_p2p_grad(3, P->kernel, K, T.d_leaf_boxes.get(), T.nleaves, T.start.get(), T.end.get(),
-                            T.loff[0].get(), T.lent[0].get(), g, nrhs, st);
+                            T.loff[0].get(), T.lent[0].get(), g, nrhs, st, P->leaf_size);
         rec(7);
         rec(8);
         return;
@@ -2201,10 +2201,11 @@ void helm3d_apply(cfmm_plan_s* P, const cd* sigma, const cd* tau, int64_t dstrid
     {
         cudaStream_t ns = near_fork(P);
         launch_p2p(3, P->kernel, K, S->d_leaves_l0.get(), (int)S->leaves_l0.size(), T.start.get(), T.end.get(),
-                   T.loff[0].get(), T.lent[0].get(), u, nrhs, false, ns, mixed, T.level.get(), P->W, P->sep);
+                   T.loff[0].get(), T.lent[0].get(), u, nrhs, false, ns, mixed, P->leaf_size, T.level.get(), P->W,
+                   P->sep);
         if (g)
             launch_p2p_grad(3, P->kernel, K, S->d_leaves_l0.get(), (int)S->leaves_l0.size(), T.start.get(),
-                            T.end.get(), T.loff[0].get(), T.lent[0].get(), g, nrhs, ns);
+                            T.end.get(), T.loff[0].get(), T.lent[0].get(), g, nrhs, ns, P->leaf_size);
     }
     near_launched(P);
     auto p2x_smem = [&](int PL, int& chunk) {

@@ -21,6 +21,8 @@ struct KParams {
     int64_t dens_stride;
     bool slp, dlp;
     double kappa;
+    // 1/kappa, its root, kappa 256/(2 pi), kappa 256/log 2 (set by the launches of p2p.cu)
+    double ikappa = 0.0, isqrt_kappa = 0.0, kappa_ang = 0.0, kappa_exp = 0.0;
 };
 
 // near field of an apply on the plan's side stream: near_fork() makes the
@@ -33,14 +35,16 @@ cudaStream_t near_fork(cfmm_plan_s* P);
 void near_launched(cfmm_plan_s* P);
 void near_join(cfmm_plan_s* P);
 // blevel/W/sep: the tree's box levels, root width and separation (the mixed
-// 3D Helmholtz near field sizes its coordinate grid from them; NULL = unknown)
+// 3D Helmholtz near field sizes its coordinate grid from them; NULL = unknown);
+// leaf_size bounds the points of a leaf
 void launch_p2p(int dim, int ker, const KParams& K, const int* leaf_boxes, int nleaves, const int* bst,
                 const int* ben, const int* l1off, const int* l1, cd* out, int nrhs, bool add, cudaStream_t st,
-                bool mixed = false, const int* blevel = nullptr, double W = 0.0, int sep = 1);
+                bool mixed, int leaf_size, const int* blevel = nullptr, double W = 0.0, int sep = 1);
 void launch_direct(int dim, int ker, const KParams& K, cd* out, int nrhs, cudaStream_t st, bool mixed = false);
 // near-field target gradient over List 1 in FP64: g = sorted [nrhs][dim][n], overwritten
 void launch_p2p_grad(int dim, int ker, const KParams& K, const int* leaf_boxes, int nleaves, const int* bst,
-                     const int* ben, const int* l1off, const int* l1, cd* g, int nrhs, cudaStream_t st);
+                     const int* ben, const int* l1off, const int* l1, cd* g, int nrhs, cudaStream_t st,
+                     int leaf_size);
 
 // tree construction (tree.cu)
 void build_tree(cfmm_plan_s* P, const double* re, const double* im, const double* nre, const double* nim,

@@ -3,12 +3,16 @@
 // layer, in float64 / complex128 or in mixed precision (complex64 kernel
 // arithmetic, FP32 hi/lo pair differences, compensated sums).
 //
-// Layout: one CTA per target leaf. 128 threads = 32 targets x 4 source
-// lanes; the sources of each List-1 leaf are staged through shared memory
-// in chunks; the 4 partial sums of a target are combined in a fixed order,
-// so results are bitwise reproducible.
-#include "cfmm_special.cuh"
+// Mixed precision: one CTA per target leaf, 128 threads = 32 targets x 4 source
+// lanes; the sources of each List-1 leaf are staged through shared memory in
+// chunks; the 4 partial sums of a target are combined in a fixed order, so
+// results are bitwise reproducible. FP64: see k_near.
+#include <algorithm>
+#include <cmath>
+#include <cstddef>
+
 #include "kernels.cuh"
+#include "pair64.cuh"
 
 namespace cfmm {
 
@@ -54,10 +58,46 @@ static SeriesTab make_series_tab() {
     return T;
 }
 
+static __device__ PairTab d_pair;
+
+void make_pair_tab(PairTab* T) {
+    const double kPi = 3.14159265358979323846;
+    for (int k = 0; k < kAngTab; ++k) {
+        // the first octant's values, so that the symmetric entries agree
+        int q = k / (kAngTab / 4), r = k % (kAngTab / 4);
+        double c = r > kAngTab / 8 ? std::sin(2 * kPi * (kAngTab / 4 - r) / kAngTab) : std::cos(2 * kPi * r / kAngTab);
+        double s = r > kAngTab / 8 ? std::cos(2 * kPi * (kAngTab / 4 - r) / kAngTab) : std::sin(2 * kPi * r / kAngTab);
+        T->ang[k] = q == 0 ? make_double2(c, s) : q == 1 ? make_double2(-s, c) : q == 2 ? make_double2(-c, -s)
+                                                                                       : make_double2(s, -c);
+    }
+    for (int k = 0; k < kExpTab; ++k) T->ex[k] = std::exp2((double)k / kExpTab);
+    for (int j = 0; j < kLogRad; ++j) {
+        double c = std::ldexp(std::rint(std::ldexp(1.0 / (1.0 + (j + 0.5) / kLogRad), 20)), -20);
+        T->lrad[j] = make_double2(c, -std::log(c));
+    }
+    for (int k = 0; k < kLogAng; ++k) {
+        double th = 2 * kPi * (k <= kLogAng / 2 ? k : k - kLogAng) / kLogAng;
+        double c = std::ldexp(std::rint(std::ldexp(std::cos(th), 27)), -27);
+        double s = std::ldexp(std::rint(std::ldexp(-std::sin(th), 27)), -27);
+        T->ldir[k] = make_double2(c, s);
+        // |dir|^2 - 1 is exact in FP64 (54 bits after the leading ones cancel)
+        T->llog[k] = make_double2(-0.5 * std::log1p(std::fma(c, c, std::fma(s, s, -1.0))),
+                                  k == kLogAng / 2 ? kPi : -std::atan2(s, c));
+    }
+}
+
 void upload_lag_rule_p2p() {
     upload_lag_rule_local();
     SeriesTab T = make_series_tab();
     CFMM_CUDA(cudaMemcpyToSymbol(c_ser, &T, sizeof(T)));
+    std::vector<char> buf(offsetof(PairTab, hk));
+    PairTab* d = nullptr;
+    CFMM_CUDA(cudaGetSymbolAddress((void**)&d, d_pair));
+    make_pair_tab(reinterpret_cast<PairTab*>(buf.data()));
+    CFMM_CUDA(cudaMemcpy(d, buf.data(), buf.size(), cudaMemcpyHostToDevice));
+    k_pair_hankel<<<(2 * kHkGrids * kHkNx * kHkNy + 127) / 128, 128>>>(d);
+    CFMM_LAUNCHED();
+    CFMM_CUDA(cudaDeviceSynchronize());
 }
 
 // number of series terms for |q|^2 = aq, FP64 (truncation below 1e-18)
@@ -69,8 +109,9 @@ __device__ __forceinline__ int series_terms32(float aq) {
     return aq <= 0.0625f ? 5 : aq <= 1.0f ? 7 : aq <= 5.0625f ? 9 : aq <= 16.0f ? 10 : 14;
 }
 
-// FP64 2D Helmholtz pair: returns SLP factor H0 and DLP factor kappa H1 / r
-__device__ __forceinline__ void helm2d_pair64(cd r2, double kappa, bool slp, bool dlp, cd& h0, cd& g1) {
+// The general FP64 2D Helmholtz pair: ascending series up to |z| = 6, the
+// quadrature of hankel01 beyond
+static __device__ __noinline__ void helm2d_pair64_general(cd r2, double kappa, bool dlp, cd& h0, cd& g1) {
     const double kPi = 3.14159265358979323846, kG = 0.57721566490153286061;
     double k2 = kappa * kappa;
     cd q = (0.25 * k2) * r2;
@@ -102,49 +143,131 @@ __device__ __forceinline__ void helm2d_pair64(cd r2, double kappa, bool slp, boo
     g1 = (kappa * h1) * cinv(r);
 }
 
+// sum of c[k] w^k, k <= N, real c, by the two-term recurrence in 2 Re w = s and
+// |w|^2 = v (two FP64 instructions a term instead of four)
+template <int N>
+__device__ __forceinline__ cd real_poly(const double* c, cd w, double s, double v) {
+    double b1 = fma(s, c[N], c[N - 1]), b2 = c[N];
+#pragma unroll
+    for (int k = N - 2; k >= 1; --k) {
+        double b = fma(-v, b2, fma(s, b1, c[k]));
+        b2 = b1;
+        b1 = b;
+    }
+    return cd{fma(-v, b2, fma(w.x, b1, c[0])), w.y * b1};
+}
+
+// H_0 and kappa H_1 / r by N terms of the series, q = (kappa r/2)^2
+template <int N>
+__device__ __forceinline__ void helm2d_series(cd r2, cd q, double aq, double k2, bool slp, bool dlp, cd& h0, cd& g1) {
+    const double kPi = 3.14159265358979323846, kG = 0.57721566490153286061;
+    cd w = -q;
+    double s = w.x + w.x;
+    cd L = 0.5 * clog64(&d_pair, q);
+    if (slp) {
+        cd A = real_poly<N>(c_ser.a, w, s, aq), Cs = real_poly<N>(c_ser.c, w, s, aq);
+        cd t = cmac(-Cs, cd{L.x + kG, L.y}, A);
+        h0 = cd{fma(-2.0 / kPi, t.y, A.x), fma(2.0 / kPi, t.x, A.y)};
+    }
+    if (dlp) {
+        cd Bs = real_poly<N>(c_ser.b, w, s, aq), Ds = real_poly<N>(c_ser.d, w, s, aq);
+        cd t = (k2 / kPi) * (L * Bs) - (2.0 / kPi) * crcp64(r2) - (k2 / (2.0 * kPi)) * Ds;
+        g1 = (0.5 * k2) * Bs + mul_i(t);
+    }
+}
+
+// FP64 2D Helmholtz pair: SLP factor H_0 and DLP factor kappa H_1 / r. The series
+// close to z = 0, the Taylor cells of hankel_factor beyond, outside the cells'
+// sector the general evaluation. The first two cost 140 (8 terms) to 190 FP64
+// instructions a combined-field pair, the general one about 670 at |z| = 3 and
+// 6000 beyond 6. A warp whose lanes fall on both sides of a limit pays for both,
+// and a leaf's near field spans |z| up to 2 or so in most plans; so a converged
+// warp (WARP) takes the series as a whole while every lane has |z| <= 2 (11
+// terms), and cells for |z| > 1/2 otherwise.
+template <bool WARP>
+__device__ __forceinline__ void helm2d_pair64(cd r2, const Wave& k, bool slp, bool dlp, cd& h0, cd& g1) {
+    double k2 = k.k * k.k;
+    cd q = (0.25 * k2) * r2;
+    double aq = cabs2(q);
+    if (WARP) {
+        // (comparisons on the high words: an FP64 compare costs an FP64 slot)
+        const int ha = __double2hiint(aq);
+        if (__all_sync(0xffffffffu, ha < 0x3fb00000)) {      // aq < 1/16
+            helm2d_series<8>(r2, q, aq, k2, slp, dlp, h0, g1);
+            return;
+        }
+        if (__all_sync(0xffffffffu, ha < 0x3ff00000)) {      // aq < 1
+            helm2d_series<11>(r2, q, aq, k2, slp, dlp, h0, g1);
+            return;
+        }
+    }
+    cd y = crsqrt64(r2), ds;
+    int cell = hankel_cell(k.ik * y, ds);
+    if (cell >= 0) {
+        cd r;
+        cd e = wave64(&d_pair, k, r2, y, r);
+        e = e * (k.isk * crsqrt64(r));
+        if (slp) h0 = e * hankel_factor(d_pair.hk[cell][0], ds);
+        if (dlp) g1 = (e * hankel_factor(d_pair.hk[cell][1], ds)) * (k.k * y);
+    } else if (aq <= 0.0625) {
+        helm2d_series<8>(r2, q, aq, k2, slp, dlp, h0, g1);
+    } else {
+        helm2d_pair64_general(r2, k.k, dlp, h0, g1);
+    }
+}
+
 constexpr int kP2PThreads = 128;
 constexpr int kP2PTargets = 32;
 constexpr int kP2PSplit = kP2PThreads / kP2PTargets;
 constexpr int kP2PChunk = 128;
 
+// r^2 = sum d_a^2 of the complex differences (3 DIM + 1 FP64 instructions)
+template <int DIM>
+__device__ __forceinline__ cd pair_r2(const double* dr, const double* di) {
+    double x = dr[0] * dr[0], y = dr[0] * di[0];
+    x = fma(-di[0], di[0], x);
+#pragma unroll
+    for (int a = 1; a < DIM; ++a) {
+        x = fma(-di[a], di[a], fma(dr[a], dr[a], x));
+        y = fma(dr[a], di[a], y);
+    }
+    return cd{x, y + y};
+}
+
 // K(x, y) sigma + (n . grad_y K)(x, y) tau for one pair (d = x - y != 0)
 template <int DIM, int KER>
 __device__ __forceinline__ void pair_kernel(const double* dr, const double* di, const double* nr,
                                             const double* ni, cd sg, cd ta, bool slp, bool dlp,
-                                            double kappa, cd& acc) {
+                                            const Wave& k, cd& acc) {
+    const double kappa = k.k;
     cd d[DIM];
-    cd r2 = {0.0, 0.0};
+    cd r2 = pair_r2<DIM>(dr, di);
 #pragma unroll
-    for (int a = 0; a < DIM; ++a) {
-        d[a] = cd{dr[a], di[a]};
-        r2 += d[a] * d[a];
-    }
+    for (int a = 0; a < DIM; ++a) d[a] = cd{dr[a], di[a]};
     cd nd = {0.0, 0.0};
     if (dlp) {
 #pragma unroll
-        for (int a = 0; a < DIM; ++a) nd += cd{nr[a], ni[a]} * d[a];
+        for (int a = 0; a < DIM; ++a) nd = cmac(nd, cd{nr[a], ni[a]}, d[a]);
     }
     if (DIM == 2 && KER == CFMM_LAPLACE) {
         // log r = Log(r^2)/2 ; grad_y log r = (y - x)/r^2
-        if (slp) acc += cd{0.25 * log(cabs2(r2)), 0.5 * atan2(r2.y, r2.x)} * sg;
-        if (dlp) acc -= (nd * cinv(r2)) * ta;
+        if (slp) acc = cmac(acc, 0.5 * clog64(&d_pair, r2), sg);
+        if (dlp) acc = cmac(acc, -nd * crcp64(r2), ta);
     } else if (DIM == 2) {
         cd h0, g1;
-        helm2d_pair64(r2, kappa, slp, dlp, h0, g1);
-        if (slp) acc += h0 * sg;
-        if (dlp) acc += (g1 * nd) * ta;
+        helm2d_pair64<true>(r2, k, slp, dlp, h0, g1);
+        if (slp) acc = cmac(acc, h0, sg);
+        if (dlp) acc = cmac(acc, g1 * nd, ta);
     } else if (KER == CFMM_LAPLACE) {
-        cd r = csqrt_p(r2);
-        cd ir = cinv(r);
-        if (slp) acc += ir * sg;
-        if (dlp) acc += (nd * (ir * ir * ir)) * ta;
+        cd ir = crsqrt64(r2);
+        if (slp) acc = cmac(acc, ir, sg);
+        if (dlp) acc = cmac(acc, nd * (ir * (ir * ir)), ta);
     } else {
-        cd r = csqrt_p(r2);
-        cd ir = cinv(r);
-        cd e = cexp_i(kappa * r);
-        cd g = e * ir;
-        if (slp) acc += g * sg;
-        if (dlp) acc += (nd * (cd{1.0, 0.0} - mul_i(kappa * r)) * g * (ir * ir)) * ta;
+        cd ir = crsqrt64(r2);
+        cd r;
+        cd g = wave64(&d_pair, k, r2, ir, r) * ir;
+        if (slp) acc = cmac(acc, g, sg);
+        if (dlp) acc = cmac(acc, (nd * cd{fma(kappa, r.y, 1.0), -kappa * r.x}) * (g * (ir * ir)), ta);
     }
 }
 
@@ -154,36 +277,31 @@ __device__ __forceinline__ void pair_kernel(const double* dr, const double* di, 
 // ((K'' - K'/r)/r^2) (n.d) d.
 template <int DIM, int KER>
 __device__ __forceinline__ void pair_grad(const double* dr, const double* di, const double* nr, const double* ni,
-                                          cd sg, cd ta, bool slp, bool dlp, double kappa, cd* g) {
+                                          cd sg, cd ta, bool slp, bool dlp, const Wave& k, cd* g) {
+    const double kappa = k.k;
     cd d[DIM];
-    cd r2 = {0.0, 0.0};
+    cd r2 = pair_r2<DIM>(dr, di);
 #pragma unroll
-    for (int a = 0; a < DIM; ++a) {
-        d[a] = cd{dr[a], di[a]};
-        r2 += d[a] * d[a];
-    }
+    for (int a = 0; a < DIM; ++a) d[a] = cd{dr[a], di[a]};
     cd a1, a2;   // K'/r and (K'' - K'/r)/r^2
     if (DIM == 2 && KER == CFMM_LAPLACE) {
-        cd ir2 = cinv(r2);
+        cd ir2 = crcp64(r2);
         a1 = ir2;
         a2 = -2.0 * (ir2 * ir2);
     } else if (DIM == 2) {
-        cd r = csqrt_p(r2);
-        cd h0, h1;
-        hankel01(kappa * r, &h0, &h1);
-        cd ir = cinv(r), ir2 = cinv(r2);
-        a1 = (-kappa) * (h1 * ir);
-        a2 = (-kappa * kappa * h0 + (2.0 * kappa) * (h1 * ir)) * ir2;
+        cd h0, g1;                      // H_0, kappa H_1 / r
+        helm2d_pair64<true>(r2, k, true, true, h0, g1);
+        a1 = -g1;
+        a2 = (2.0 * g1 - (kappa * kappa) * h0) * crcp64(r2);
     } else if (KER == CFMM_LAPLACE) {
-        cd r = csqrt_p(r2);
-        cd ir = cinv(r), ir2 = cinv(r2);
+        cd ir = crsqrt64(r2), ir2 = ir * ir;
         cd ir3 = ir * ir2;
         a1 = -ir3;
         a2 = 3.0 * (ir3 * ir2);
     } else {
-        cd r = csqrt_p(r2);
-        cd ir = cinv(r), ir2 = cinv(r2);
-        cd e = cexp_i(kappa * r);
+        cd ir = crsqrt64(r2), ir2 = ir * ir;
+        cd r;
+        cd e = wave64(&d_pair, k, r2, ir, r);
         cd ikr = mul_i(kappa * r);
         cd ir3 = ir * ir2;
         a1 = (e * (ikr - cd{1.0, 0.0})) * ir3;
@@ -206,53 +324,169 @@ __device__ __forceinline__ void pair_grad(const double* dr, const double* di, co
     }
 }
 
-struct SrcTile {
-    double re[kP2PChunk][3];
-    double im[kP2PChunk][3];
-    double nr[kP2PChunk][3];
-    double ni[kP2PChunk][3];
-    cd sg[kP2PChunk];
-    cd ta[kP2PChunk];
+// ---------------------------------------------------------------------------
+// FP64 near field, its gradient and the direct sum.
+//
+// The FP64 pipe bounds them (pair64.cuh), so what counts is that every lane of
+// an FP64 instruction holds a pair. Lanes therefore stand for sources, 32 of the
+// concatenated source leaves at a time, which leaves a partial warp only at the
+// end of a list; with lanes as targets of one leaf, 25 of 32 were in use (leaf
+// size 128). A lane keeps its source in registers and meets the block's nt
+// targets in turn, target (lane + k) mod nt at step k, so the lanes of a step add
+// to different entries of the warp's accumulator row in shared memory (for nt <
+// 32 the lanes beyond nt use further copies of the row). Each warp takes every
+// fourth 32-source group; rows and copies are added in a fixed order at the end,
+// so results are bitwise reproducible.
+//
+// A block takes at most kNearTargets targets of a leaf; the launch lowers that
+// until the grid covers the chip, which a few dozen leaves with all their targets
+// in one block each do not.
+// ---------------------------------------------------------------------------
+constexpr int kNearThreads = 128;
+constexpr int kNearWarps = kNearThreads / 32;
+constexpr int kNearTargets = 128;     // targets of a block at most
+constexpr int kNearSeg = kNearThreads;   // source leaves whose ranges are staged at once
+
+// targets and sources of a launch: index ranges per box into the sorted points,
+// or a single range each (direct sum: boxes == nullptr)
+struct NearLists {
+    const int* boxes;
+    const int* bst;
+    const int* ben;
+    const int* l1off;
+    const int* l1;
 };
 
-template <int DIM, int KER>
-__device__ void accumulate_sources(SrcTile& S, const KParams& K, int rhs, int s, int e, int ti, bool tvalid,
-                                   const double* xr, const double* xim, cd& acc, int split) {
-    const int64_t n = K.n_src;
-    for (int c0 = s; c0 < e; c0 += kP2PChunk) {
-        int cn = min(kP2PChunk, e - c0);
-        __syncthreads();
-        for (int j = threadIdx.x; j < cn; j += blockDim.x) {
-            int g = c0 + j;
+template <int DIM, int KER, bool GRAD>
+__global__ void __launch_bounds__(kNearThreads) k_near(KParams K, NearLists L, int tb, cd* __restrict__ out) {
+    constexpr int NA = GRAD ? DIM : 1;                  // complex accumulators of a target
+    constexpr int kRow = kNearTargets + 32;             // nt, or copies * nt < nt + 32
+    extern __shared__ double near_sm[];
+    double* tx = near_sm;                               // [2 DIM][kNearTargets]
+    cd* acc = reinterpret_cast<cd*>(tx + 2 * DIM * kNearTargets);   // [warps][NA][kRow]
+    __shared__ int seg_pos[kNearSeg], seg_end[kNearSeg], warp_sum[kNearWarps];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const int rhs = blockIdx.y;
+    const int b = L.boxes ? L.boxes[blockIdx.x] : 0;
+    const Wave wave{K.kappa, K.ikappa, K.isqrt_kappa, K.kappa_ang, K.kappa_exp};
+    const int qa = L.boxes ? L.l1off[b] : 0, qb = L.boxes ? L.l1off[b + 1] : 1;
+    // groups of targets blockIdx.z, + gridDim.z, ..: the grid covers leaf_size
+    // points a leaf; leaves at the deepest level may hold more
+    const int64_t tstep = (int64_t)(L.boxes ? gridDim.z : gridDim.x) * tb, tend = L.boxes ? L.ben[b] : K.n_trg;
+    for (int64_t t0 = L.boxes ? L.bst[b] + (int64_t)blockIdx.z * tb : (int64_t)blockIdx.x * tb; t0 < tend; t0 += tstep) {
+    const int nt = (int)min((int64_t)tb, tend - t0);
+    __syncthreads();
+    for (int i = threadIdx.x; i < nt; i += kNearThreads) {
 #pragma unroll
-            for (int a = 0; a < DIM; ++a) {
-                S.re[j][a] = K.src_re[a * n + g];
-                S.im[j][a] = K.src_im[a * n + g];
-                if (K.dlp) {
-                    S.nr[j][a] = K.nrm_re[a * n + g];
-                    S.ni[j][a] = K.nrm_im[a * n + g];
-                }
-            }
-            if (K.slp) S.sg[j] = K.sigma[(int64_t)rhs * K.dens_stride + g];
-            if (K.dlp) S.ta[j] = K.tau[(int64_t)rhs * K.dens_stride + g];
-        }
-        __syncthreads();
-        if (tvalid) {
-            for (int j = split; j < cn; j += kP2PSplit) {
-                double dr[DIM], di[DIM];
-                bool zero = true;
-#pragma unroll
-                for (int a = 0; a < DIM; ++a) {
-                    dr[a] = xr[a] - S.re[j][a];
-                    di[a] = xim[a] - S.im[j][a];
-                    zero = zero && dr[a] == 0.0 && di[a] == 0.0;
-                }
-                if (zero) continue;   // x == y: self pair / coincident point
-                pair_kernel<DIM, KER>(dr, di, S.nr[j], S.ni[j], K.slp ? S.sg[j] : cd{0, 0},
-                                      K.dlp ? S.ta[j] : cd{0, 0}, K.slp, K.dlp, K.kappa, acc);
-            }
+        for (int a = 0; a < DIM; ++a) {
+            tx[a * kNearTargets + i] = K.trg_re[a * K.n_trg + t0 + i];
+            tx[(DIM + a) * kNearTargets + i] = K.trg_im[a * K.n_trg + t0 + i];
         }
     }
+    const int copies = nt >= 32 ? 1 : (31 + nt) / nt;
+    cd* row = acc + wid * NA * kRow;
+    for (int i = lane; i < NA * kRow; i += 32) row[i] = cd{0.0, 0.0};
+    row += (lane / nt) * (nt >= 32 ? 0 : nt);
+    const int first = lane % nt;
+    for (int q0 = qa; q0 < qb; q0 += kNearSeg) {
+        // ranges of the next source leaves and the running total of their sizes
+        int q = q0 + threadIdx.x, s0 = 0, cnt = 0;
+        if (q < qb) {
+            int src = L.boxes ? L.l1[q] : 0;
+            s0 = L.boxes ? L.bst[src] : 0;
+            cnt = L.boxes ? L.ben[src] - s0 : (int)K.n_src;
+        }
+        int sum = cnt;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            int v = __shfl_up_sync(0xffffffffu, sum, o);
+            if (lane >= o) sum += v;
+        }
+        __syncthreads();                                // the last round's ranges have been read
+        if (lane == 31) warp_sum[wid] = sum;
+        __syncthreads();
+        for (int w = 0; w < wid; ++w) sum += warp_sum[w];
+        seg_pos[threadIdx.x] = s0;
+        seg_end[threadIdx.x] = sum;
+        __syncthreads();
+        const unsigned total = (unsigned)seg_end[kNearSeg - 1];
+        for (unsigned c0 = wid * 32; c0 < total; c0 += kNearThreads) {
+            const unsigned f = c0 + lane;
+            const bool valid = f < total;
+            double yr[DIM], yi[DIM], nr[DIM], ni[DIM];
+            cd sg = {0.0, 0.0}, ta = {0.0, 0.0};
+            if (valid) {
+                int lo = 0, hi = kNearSeg - 1;          // first range that ends beyond f
+                while (lo < hi) {
+                    int m = (lo + hi) >> 1;
+                    if ((unsigned)seg_end[m] > f) hi = m;
+                    else lo = m + 1;
+                }
+                const int64_t j = seg_pos[lo] + (int)(f - (lo ? seg_end[lo - 1] : 0)), n = K.n_src;
+#pragma unroll
+                for (int a = 0; a < DIM; ++a) {
+                    yr[a] = K.src_re[a * n + j];
+                    yi[a] = K.src_im[a * n + j];
+                    nr[a] = K.dlp ? K.nrm_re[a * n + j] : 0.0;
+                    ni[a] = K.dlp ? K.nrm_im[a * n + j] : 0.0;
+                }
+                if (K.slp) sg = K.sigma[(int64_t)rhs * K.dens_stride + j];
+                if (K.dlp) ta = K.tau[(int64_t)rhs * K.dens_stride + j];
+            }
+            int t = first;
+            for (int k = 0; k < nt; ++k) {
+                __syncwarp();                           // the neighbour lane's sum of the last step
+                // lanes without a source and pairs with x == y (self pair, coincident
+                // point) take a harmless distance and store nothing: the warp stays whole
+                double dr[DIM], di[DIM];
+                int bits = 0;                           // 0 when every difference is (FP64 compares cost an FP64 slot)
+#pragma unroll
+                for (int a = 0; a < DIM; ++a) {
+                    dr[a] = tx[a * kNearTargets + t] - yr[a];
+                    di[a] = tx[(DIM + a) * kNearTargets + t] - yi[a];
+                    bits |= __double2hiint(dr[a]) | __double2loint(dr[a]) | __double2hiint(di[a]) | __double2loint(di[a]);
+                }
+                // (x - x is +0 in every rounding but one, which is not in use)
+                const bool skip = !valid || bits == 0;
+                if (skip) {
+                    dr[0] = wave.k > 0.0 ? wave.ik : 1.0;
+                    di[0] = 0.0;
+#pragma unroll
+                    for (int a = 1; a < DIM; ++a) dr[a] = di[a] = 0.0;
+                }
+                if (GRAD) {
+                    cd g[DIM];
+#pragma unroll
+                    for (int a = 0; a < DIM; ++a) g[a] = row[a * kRow + t];
+                    pair_grad<DIM, KER>(dr, di, nr, ni, sg, ta, K.slp, K.dlp, wave, g);
+#pragma unroll
+                    for (int a = 0; a < DIM; ++a)
+                        if (!skip) row[a * kRow + t] = g[a];
+                } else {
+                    cd u = row[t];
+                    pair_kernel<DIM, KER>(dr, di, nr, ni, sg, ta, K.slp, K.dlp, wave, u);
+                    if (!skip) row[t] = u;
+                }
+                if (++t == nt) t = 0;
+            }
+            __syncwarp();
+        }
+    }
+    __syncthreads();
+    for (int i = threadIdx.x; i < nt * NA; i += kNearThreads) {
+        int a = i / nt, t = i - a * nt;
+        cd s = {0.0, 0.0};
+        for (int w = 0; w < kNearWarps; ++w)
+            for (int c = 0; c < copies; ++c) s += acc[(w * NA + a) * kRow + c * nt + t];
+        out[((int64_t)rhs * NA + a) * K.n_trg + t0 + t] = s;
+    }
+    }
+}
+
+template <int DIM, bool GRAD>
+constexpr size_t near_smem() {
+    return sizeof(double) * 2 * DIM * kNearTargets +
+           sizeof(cd) * kNearWarps * (GRAD ? DIM : 1) * (kNearTargets + 32);
 }
 
 template <int DIM, int KER>
@@ -266,126 +500,6 @@ __device__ void finish_target(cd acc, cd* red, int tl, int split, bool tvalid, c
         else *out = s;
     }
     __syncthreads();
-}
-
-// near field over List 1; out = sorted potential [rhs][n] (overwritten)
-template <int DIM, int KER>
-__global__ void __launch_bounds__(kP2PThreads) k_p2p(KParams K, const int* __restrict__ leaf_boxes,
-                                                     const int* __restrict__ bst, const int* __restrict__ ben,
-                                                     const int* __restrict__ l1off, const int* __restrict__ l1,
-                                                     cd* __restrict__ out, int add) {
-    __shared__ SrcTile S;
-    __shared__ cd red[kP2PThreads];
-    int b = leaf_boxes[blockIdx.x];
-    int rhs = blockIdx.y;
-    int tl = threadIdx.x % kP2PTargets, split = threadIdx.x / kP2PTargets;
-    int ts = bst[b], te = ben[b];
-    for (int t0 = ts; t0 < te; t0 += kP2PTargets) {
-        int ti = t0 + tl;
-        bool tvalid = ti < te;
-        double xr[DIM], xim[DIM];
-#pragma unroll
-        for (int a = 0; a < DIM; ++a) {
-            xr[a] = tvalid ? K.trg_re[a * K.n_trg + ti] : 0.0;
-            xim[a] = tvalid ? K.trg_im[a * K.n_trg + ti] : 0.0;
-        }
-        cd acc = {0.0, 0.0};
-        for (int q = l1off[b]; q < l1off[b + 1]; ++q) {
-            int a = l1[q];
-            accumulate_sources<DIM, KER>(S, K, rhs, bst[a], ben[a], ti, tvalid, xr, xim, acc, split);
-        }
-        finish_target<DIM, KER>(acc, red, tl, split, tvalid, out + (int64_t)rhs * K.n_trg + ti, add != 0);
-    }
-}
-
-// near-field gradient over List 1 (FP64); g = sorted gradient [rhs][DIM][n]
-// (overwritten). Same staging and fixed-order combination as k_p2p.
-template <int DIM, int KER>
-__global__ void __launch_bounds__(kP2PThreads) k_p2p_grad(KParams K, const int* __restrict__ leaf_boxes,
-                                                          const int* __restrict__ bst, const int* __restrict__ ben,
-                                                          const int* __restrict__ l1off, const int* __restrict__ l1,
-                                                          cd* __restrict__ g) {
-    __shared__ SrcTile S;
-    __shared__ cd red[kP2PThreads];
-    const int64_t n = K.n_src;
-    int b = leaf_boxes[blockIdx.x];
-    int rhs = blockIdx.y;
-    int tl = threadIdx.x % kP2PTargets, split = threadIdx.x / kP2PTargets;
-    int ts = bst[b], te = ben[b];
-    for (int t0 = ts; t0 < te; t0 += kP2PTargets) {
-        int ti = t0 + tl;
-        bool tvalid = ti < te;
-        double xr[DIM], xim[DIM];
-#pragma unroll
-        for (int a = 0; a < DIM; ++a) {
-            xr[a] = tvalid ? K.trg_re[a * K.n_trg + ti] : 0.0;
-            xim[a] = tvalid ? K.trg_im[a * K.n_trg + ti] : 0.0;
-        }
-        cd acc[DIM];
-#pragma unroll
-        for (int a = 0; a < DIM; ++a) acc[a] = cd{0.0, 0.0};
-        for (int q = l1off[b]; q < l1off[b + 1]; ++q) {
-            int src = l1[q];
-            int s0 = bst[src], s1 = ben[src];
-            for (int c0 = s0; c0 < s1; c0 += kP2PChunk) {
-                int cn = min(kP2PChunk, s1 - c0);
-                __syncthreads();
-                for (int j = threadIdx.x; j < cn; j += blockDim.x) {
-                    int gi = c0 + j;
-#pragma unroll
-                    for (int a = 0; a < DIM; ++a) {
-                        S.re[j][a] = K.src_re[a * n + gi];
-                        S.im[j][a] = K.src_im[a * n + gi];
-                        if (K.dlp) {
-                            S.nr[j][a] = K.nrm_re[a * n + gi];
-                            S.ni[j][a] = K.nrm_im[a * n + gi];
-                        }
-                    }
-                    if (K.slp) S.sg[j] = K.sigma[(int64_t)rhs * K.dens_stride + gi];
-                    if (K.dlp) S.ta[j] = K.tau[(int64_t)rhs * K.dens_stride + gi];
-                }
-                __syncthreads();
-                if (!tvalid) continue;
-                for (int j = split; j < cn; j += kP2PSplit) {
-                    double dr[DIM], di[DIM];
-                    bool zero = true;
-#pragma unroll
-                    for (int a = 0; a < DIM; ++a) {
-                        dr[a] = xr[a] - S.re[j][a];
-                        di[a] = xim[a] - S.im[j][a];
-                        zero = zero && dr[a] == 0.0 && di[a] == 0.0;
-                    }
-                    if (zero) continue;
-                    pair_grad<DIM, KER>(dr, di, S.nr[j], S.ni[j], K.slp ? S.sg[j] : cd{0, 0},
-                                        K.dlp ? S.ta[j] : cd{0, 0}, K.slp, K.dlp, K.kappa, acc);
-                }
-            }
-        }
-        cd* gout = g + (int64_t)rhs * DIM * K.n_trg + ti;
-#pragma unroll
-        for (int a = 0; a < DIM; ++a)
-            finish_target<DIM, KER>(acc[a], red, tl, split, tvalid, gout + (int64_t)a * K.n_trg, false);
-    }
-}
-
-// direct sum: every target against every source
-template <int DIM, int KER>
-__global__ void __launch_bounds__(kP2PThreads) k_direct(KParams K, cd* __restrict__ out) {
-    __shared__ SrcTile S;
-    __shared__ cd red[kP2PThreads];
-    int rhs = blockIdx.y;
-    int tl = threadIdx.x % kP2PTargets, split = threadIdx.x / kP2PTargets;
-    int ti = blockIdx.x * kP2PTargets + tl;
-    bool tvalid = ti < K.n_trg;
-    double xr[DIM], xim[DIM];
-#pragma unroll
-    for (int a = 0; a < DIM; ++a) {
-        xr[a] = tvalid ? K.trg_re[a * K.n_trg + ti] : 0.0;
-        xim[a] = tvalid ? K.trg_im[a * K.n_trg + ti] : 0.0;
-    }
-    cd acc = {0.0, 0.0};
-    accumulate_sources<DIM, KER>(S, K, rhs, 0, (int)K.n_src, ti, tvalid, xr, xim, acc, split);
-    finish_target<DIM, KER>(acc, red, tl, split, tvalid, out + (int64_t)rhs * K.n_trg + ti, false);
 }
 
 // ---------------------------------------------------------------------------
@@ -421,6 +535,30 @@ __device__ __forceinline__ void helm2d_pair32(cf r2, float kappa, bool dlp, cf& 
         cf y = (-2.f / kPi) * ir2 + (k2 / kPi) * (L * Bs) - (k2 / (2.f * kPi)) * Ds;
         g1 = (0.5f * k2) * Bs + mul_if(y);
     }
+}
+
+// FP32 rounding of the general FP64 evaluation, which the mixed near field is
+// defined by. The quick evaluation is within 2^-42 (1 + |kappa r|/64) of it
+// relative to the modulus (both are good to 2^-44 or better at |kappa r| of
+// order 1 and their phases to 2^-52 |kappa r|), so both round alike except where
+// a bound of that interval rounds differently: about one pair in 30,000, which
+// takes the general evaluation.
+__device__ __forceinline__ bool round32(cd v, double rel, cf& out) {
+    double d = rel * (fabs(v.x) + fabs(v.y));
+    out = cf{(float)(v.x - d), (float)(v.y - d)};
+    return out.x == (float)(v.x + d) && out.y == (float)(v.y + d);
+}
+__device__ __forceinline__ void helm2d_round32(cd r2, const Wave& k, bool slp, bool dlp, cf& h0f, cf& g1f) {
+    cd h0, g1;
+    helm2d_pair64<false>(r2, k, slp, dlp, h0, g1);
+    double rel = 2.2737367544323206e-13 * (1.0 + 0.015625 * k.k * sqrt(fabs(r2.x) + fabs(r2.y)));
+    bool same = true;
+    if (slp) same = round32(h0, rel, h0f);
+    if (dlp) same = round32(g1, rel, g1f) && same;
+    if (same) return;
+    helm2d_pair64_general(r2, k.k, dlp, h0, g1);
+    if (slp) h0f = cf{(float)h0.x, (float)h0.y};
+    if (dlp) g1f = cf{(float)g1.x, (float)g1.y};
 }
 
 // Error-free transformations (Dekker, Knuth): the product and sum of two
@@ -527,7 +665,7 @@ __device__ __forceinline__ void far_phase_df(const PairHL& H, float kh, float kl
 
 template <int DIM, int KER>
 __device__ __forceinline__ void pair_kernel32(const float* d_re, const float* d_im, const PairHL& H, cf nd, cf sg,
-                                              cf ta, bool slp, bool dlp, float kappa, double kappa64, Kahan& acc) {
+                                              cf ta, bool slp, bool dlp, float kappa, const Wave& k, Kahan& acc) {
     cf d[DIM];
     cf r2 = {0.f, 0.f};
 #pragma unroll
@@ -551,10 +689,10 @@ __device__ __forceinline__ void pair_kernel32(const float* d_re, const float* d_
             if (dlp) v = v + (g1 * nd) * ta;
         } else {
             // |kappa r| > 3: FP64 r^2 and the FP64 evaluation, result rounded to FP32
-            cd h0, g1;
-            helm2d_pair64(r2_from_hl<DIM>(H), kappa64, slp, dlp, h0, g1);
-            if (slp) v = cf{(float)h0.x, (float)h0.y} * sg;
-            if (dlp) v = v + (cf{(float)g1.x, (float)g1.y} * nd) * ta;
+            cf h0 = {0.f, 0.f}, g1 = {0.f, 0.f};
+            helm2d_round32(r2_from_hl<DIM>(H), k, slp, dlp, h0, g1);
+            if (slp) v = h0 * sg;
+            if (dlp) v = v + (g1 * nd) * ta;
         }
     } else if (KER == CFMM_LAPLACE) {
         cf r = csqrtf_p(r2);
@@ -572,7 +710,7 @@ __device__ __forceinline__ void pair_kernel32(const float* d_re, const float* d_
         } else {
             // |kappa r| > 3: double-float phase
             cf e;
-            far_phase_df<DIM>(H, kappa, (float)(kappa64 - (double)kappa), e, r);
+            far_phase_df<DIM>(H, kappa, (float)(k.k - (double)kappa), e, r);
             g = e * cinvf(r);
         }
         cf ir = cinvf(r);
@@ -643,7 +781,7 @@ __device__ void accumulate_sources32(SrcTileF& S, const KParams& K, int rhs, int
                 if (K.dlp) nd = dot_nd<DIM>(hr, lr, hi, li, S.nhr[j], S.nlr[j], S.nhi[j], S.nli[j]);
                 PairHL H{xh_r, xl_r, xh_i, xl_i, S.hr[j], S.lr[j], S.hi[j], S.li[j]};
                 pair_kernel32<DIM, KER>(dr, di, H, nd, K.slp ? S.sg[j] : cf{0, 0}, K.dlp ? S.ta[j] : cf{0, 0},
-                                        K.slp, K.dlp, kap, K.kappa, acc);
+                                        K.slp, K.dlp, kap, Wave{K.kappa, K.ikappa, K.isqrt_kappa, K.kappa_ang, K.kappa_exp}, acc);
             }
         }
     }
@@ -931,19 +1069,60 @@ __global__ void __launch_bounds__(kP2PThreads) k_p2p32g_h3(KParams K, const int*
     }
 }
 
-template <int DIM, int KER>
-static void launch_p2p_t(const KParams& K, const int* leaf_boxes, int nleaves, const int* bst, const int* ben,
-                         const int* l1off, const int* l1, cd* out, int nrhs, bool add, bool mixed, cudaStream_t st) {
-    if (nleaves == 0) return;
-    dim3 grid(nleaves, nrhs);
-    if (mixed) k_p2p32<DIM, KER><<<grid, kP2PThreads, 0, st>>>(K, leaf_boxes, bst, ben, l1off, l1, out, add ? 1 : 0);
-    else k_p2p<DIM, KER><<<grid, kP2PThreads, 0, st>>>(K, leaf_boxes, bst, ben, l1off, l1, out, add ? 1 : 0);
+static KParams with_wave(KParams K) {
+    if (K.kappa > 0.0) {
+        K.ikappa = 1.0 / K.kappa;
+        K.isqrt_kappa = std::sqrt(K.ikappa);
+        K.kappa_ang = K.kappa * 40.74366543152521;     // 256/(2 pi)
+        K.kappa_exp = K.kappa * 369.3299304675746;     // 256/log 2
+    }
+    return K;
+}
+
+// nleaves target leaves of at most leaf_size points each (List 1 in L), or,
+// without boxes, all targets against all sources. Blocks differ in work, so a
+// large near field is cut down to 16 targets a block while an SM gets fewer than
+// 32 blocks (8,224 instead of 1,028 blocks of the 1e5-point 3D Helmholtz surface:
+// 37.9 -> 36.1 ms). A small one runs beside the far field, whose first kernels
+// wait for free SMs: two blocks an SM, of at least 4 targets (70 leaves of a
+// 3,001-point 2D Helmholtz matvec: 0.62 -> 0.21 ms). The direct sum has the chip
+// to itself.
+template <int DIM, int KER, bool GRAD>
+static void launch_near(const KParams& K, const NearLists& L, int nleaves, int leaf_size, cd* out, int nrhs,
+                        cudaStream_t st) {
+    int dev = 0, nsm = 0;
+    CFMM_CUDA(cudaGetDevice(&dev));
+    CFMM_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
+    int64_t per = L.boxes ? leaf_size : K.n_trg, rows = L.boxes ? (int64_t)nleaves * nrhs : nrhs;
+    int tb = (int)std::min<int64_t>(kNearTargets, per);
+    auto blocks = [&] { return rows * ((per + tb - 1) / tb); };
+    if (rows * per >= 32768)
+        while (tb > 16 && blocks() < 32 * nsm) tb = std::max(16, tb / 2);
+    while (tb > 4 && blocks() < (L.boxes ? 2 : 8) * nsm) tb = std::max(4, tb / 2);
+    unsigned groups = (unsigned)((per + tb - 1) / tb);
+    dim3 grid = L.boxes ? dim3((unsigned)nleaves, nrhs, groups) : dim3(groups, nrhs);
+    k_near<DIM, KER, GRAD><<<grid, kNearThreads, near_smem<DIM, GRAD>(), st>>>(K, L, tb, out);
     CFMM_LAUNCHED();
 }
 
-void launch_p2p(int dim, int ker, const KParams& K, const int* leaf_boxes, int nleaves, const int* bst,
+template <int DIM, int KER>
+static void launch_p2p_t(const KParams& K, const int* leaf_boxes, int nleaves, const int* bst, const int* ben,
+                         const int* l1off, const int* l1, cd* out, int nrhs, bool add, bool mixed, cudaStream_t st,
+                         int leaf_size) {
+    if (nleaves == 0) return;
+    dim3 grid(nleaves, nrhs);
+    if (mixed) {
+        k_p2p32<DIM, KER><<<grid, kP2PThreads, 0, st>>>(K, leaf_boxes, bst, ben, l1off, l1, out, add ? 1 : 0);
+        CFMM_LAUNCHED();
+    } else {
+        launch_near<DIM, KER, false>(K, NearLists{leaf_boxes, bst, ben, l1off, l1}, nleaves, leaf_size, out, nrhs, st);
+    }
+}
+
+void launch_p2p(int dim, int ker, const KParams& K0, const int* leaf_boxes, int nleaves, const int* bst,
                 const int* ben, const int* l1off, const int* l1, cd* out, int nrhs, bool add, cudaStream_t st,
-                bool mixed, const int* blevel, double W, int sep) {
+                bool mixed, int leaf_size, const int* blevel, double W, int sep) {
+    const KParams K = with_wave(K0);
     if (mixed && dim == 3 && ker == CFMM_HELMHOLTZ && blevel && nleaves > 0) {
         dim3 grid(nleaves, nrhs);
         k_p2p32g_h3<<<grid, kP2PThreads, 0, st>>>(K, leaf_boxes, bst, ben, l1off, l1, blevel, W, sep, out,
@@ -951,38 +1130,42 @@ void launch_p2p(int dim, int ker, const KParams& K, const int* leaf_boxes, int n
         CFMM_LAUNCHED();
         return;
     }
-    if (dim == 2 && ker == CFMM_LAPLACE) launch_p2p_t<2, CFMM_LAPLACE>(K, leaf_boxes, nleaves, bst, ben, l1off, l1, out, nrhs, add, mixed, st);
-    else if (dim == 2) launch_p2p_t<2, CFMM_HELMHOLTZ>(K, leaf_boxes, nleaves, bst, ben, l1off, l1, out, nrhs, add, mixed, st);
-    else if (ker == CFMM_LAPLACE) launch_p2p_t<3, CFMM_LAPLACE>(K, leaf_boxes, nleaves, bst, ben, l1off, l1, out, nrhs, add, mixed, st);
-    else launch_p2p_t<3, CFMM_HELMHOLTZ>(K, leaf_boxes, nleaves, bst, ben, l1off, l1, out, nrhs, add, mixed, st);
+    if (dim == 2 && ker == CFMM_LAPLACE) launch_p2p_t<2, CFMM_LAPLACE>(K, leaf_boxes, nleaves, bst, ben, l1off, l1, out, nrhs, add, mixed, st, leaf_size);
+    else if (dim == 2) launch_p2p_t<2, CFMM_HELMHOLTZ>(K, leaf_boxes, nleaves, bst, ben, l1off, l1, out, nrhs, add, mixed, st, leaf_size);
+    else if (ker == CFMM_LAPLACE) launch_p2p_t<3, CFMM_LAPLACE>(K, leaf_boxes, nleaves, bst, ben, l1off, l1, out, nrhs, add, mixed, st, leaf_size);
+    else launch_p2p_t<3, CFMM_HELMHOLTZ>(K, leaf_boxes, nleaves, bst, ben, l1off, l1, out, nrhs, add, mixed, st, leaf_size);
 }
 
 template <int DIM, int KER>
 static void launch_p2p_grad_t(const KParams& K, const int* leaf_boxes, int nleaves, const int* bst, const int* ben,
-                              const int* l1off, const int* l1, cd* g, int nrhs, cudaStream_t st) {
+                              const int* l1off, const int* l1, cd* g, int nrhs, cudaStream_t st, int leaf_size) {
     if (nleaves == 0) return;
-    dim3 grid(nleaves, nrhs);
-    k_p2p_grad<DIM, KER><<<grid, kP2PThreads, 0, st>>>(K, leaf_boxes, bst, ben, l1off, l1, g);
-    CFMM_LAUNCHED();
+    launch_near<DIM, KER, true>(K, NearLists{leaf_boxes, bst, ben, l1off, l1}, nleaves, leaf_size, g, nrhs, st);
 }
 
-void launch_p2p_grad(int dim, int ker, const KParams& K, const int* leaf_boxes, int nleaves, const int* bst,
-                     const int* ben, const int* l1off, const int* l1, cd* g, int nrhs, cudaStream_t st) {
-    if (dim == 2 && ker == CFMM_LAPLACE) launch_p2p_grad_t<2, CFMM_LAPLACE>(K, leaf_boxes, nleaves, bst, ben, l1off, l1, g, nrhs, st);
-    else if (dim == 2) launch_p2p_grad_t<2, CFMM_HELMHOLTZ>(K, leaf_boxes, nleaves, bst, ben, l1off, l1, g, nrhs, st);
-    else if (ker == CFMM_LAPLACE) launch_p2p_grad_t<3, CFMM_LAPLACE>(K, leaf_boxes, nleaves, bst, ben, l1off, l1, g, nrhs, st);
-    else launch_p2p_grad_t<3, CFMM_HELMHOLTZ>(K, leaf_boxes, nleaves, bst, ben, l1off, l1, g, nrhs, st);
+void launch_p2p_grad(int dim, int ker, const KParams& K0, const int* leaf_boxes, int nleaves, const int* bst,
+                     const int* ben, const int* l1off, const int* l1, cd* g, int nrhs, cudaStream_t st,
+                     int leaf_size) {
+    const KParams K = with_wave(K0);
+    if (dim == 2 && ker == CFMM_LAPLACE) launch_p2p_grad_t<2, CFMM_LAPLACE>(K, leaf_boxes, nleaves, bst, ben, l1off, l1, g, nrhs, st, leaf_size);
+    else if (dim == 2) launch_p2p_grad_t<2, CFMM_HELMHOLTZ>(K, leaf_boxes, nleaves, bst, ben, l1off, l1, g, nrhs, st, leaf_size);
+    else if (ker == CFMM_LAPLACE) launch_p2p_grad_t<3, CFMM_LAPLACE>(K, leaf_boxes, nleaves, bst, ben, l1off, l1, g, nrhs, st, leaf_size);
+    else launch_p2p_grad_t<3, CFMM_HELMHOLTZ>(K, leaf_boxes, nleaves, bst, ben, l1off, l1, g, nrhs, st, leaf_size);
 }
 
 template <int DIM, int KER>
 static void launch_direct_t(const KParams& K, cd* out, int nrhs, bool mixed, cudaStream_t st) {
+    if (!mixed) {
+        launch_near<DIM, KER, false>(K, NearLists{}, 0, 0, out, nrhs, st);
+        return;
+    }
     dim3 grid((unsigned)((K.n_trg + kP2PTargets - 1) / kP2PTargets), nrhs);
-    if (mixed) k_direct32<DIM, KER><<<grid, kP2PThreads, 0, st>>>(K, out);
-    else k_direct<DIM, KER><<<grid, kP2PThreads, 0, st>>>(K, out);
+    k_direct32<DIM, KER><<<grid, kP2PThreads, 0, st>>>(K, out);
     CFMM_LAUNCHED();
 }
 
-void launch_direct(int dim, int ker, const KParams& K, cd* out, int nrhs, cudaStream_t st, bool mixed) {
+void launch_direct(int dim, int ker, const KParams& K0, cd* out, int nrhs, cudaStream_t st, bool mixed) {
+    const KParams K = with_wave(K0);
     if (K.n_trg == 0) return;
     if (dim == 2 && ker == CFMM_LAPLACE) launch_direct_t<2, CFMM_LAPLACE>(K, out, nrhs, mixed, st);
     else if (dim == 2) launch_direct_t<2, CFMM_HELMHOLTZ>(K, out, nrhs, mixed, st);
