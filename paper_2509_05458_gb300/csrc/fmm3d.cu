@@ -562,8 +562,7 @@ void fmm3d_apply(cfmm_plan_s* P, const cd* sigma, const cd* tau, int64_t dstride
         lap3_tr_launch(S->tr, P, 0, l, Pu, S->exp_off.get(), S->ncoef, mp, mp, nrhs);
     rec(3);
     // (4) M2L
-    for (int l = S->l0; l < T.nlevels; ++l)
-        lap3_tr_launch(S->tr, P, 1, l, Pu, S->exp_off.get(), S->ncoef, mp, lc, nrhs);
+    lap3_m2l(S->tr, P, S->l0, T.nlevels, Pu, S->exp_off.get(), S->ncoef, mp, lc, nrhs);
     rec(4);
     // (6) P2L
     if (S->n_p2l > 0) {

@@ -56,6 +56,7 @@
 
 #include "cfmm_special.cuh"
 #include "kernels.cuh"
+#include "m2l3d.cuh"
 
 namespace cfmm {
 
@@ -81,6 +82,7 @@ constexpr size_t kTriBudget = (size_t)6 << 30;   // bytes of operators per M2L l
 struct H3Tables {
     int Pmax = -1;
     DevBuf<double> Dh;       // D_n[m][m'] for m, m' >= 0, column-major per order
+    DevBuf<double> Dg;       // the same scaled by (-1)^n/(2n+1)
     DevBuf<int64_t> Dhoff;   // [Pmax+2]
     DevBuf<double> inv2n1;   // 1/(2n+1), n <= 2Pmax+2
     DevBuf<double> zA, zB;   // [(2Pmax+3)^2] by nmi(n, m), m >= 0
@@ -195,6 +197,11 @@ static void host_rotation_tables(int P, std::vector<double>& D, std::vector<int6
     }
 }
 
+static Tr3Tables tr3_tables(const H3Tables* T) {
+    return Tr3Tables{T->Dh.get(), T->Dg.get(), T->Dhoff.get(), T->al.get(), T->be.get(), T->ibe.get(), T->mu.get(),
+                     T->nu.get(), T->lsm.get(), T->lsd.get(), T->fact.get()};
+}
+
 static H3Tables* tables(int P) {
     int dev = 0;
     CFMM_CUDA(cudaGetDevice(&dev));
@@ -250,6 +257,9 @@ static H3Tables* tables(int P) {
         CFMM_CUDA(cudaMemcpy(b.get(), v.data(), sizeof(double) * v.size(), cudaMemcpyHostToDevice));
     };
     up(T->Dh, Dh);
+    for (int n = 0; n <= Pm; ++n)
+        for (int64_t k = hoff[n]; k < hoff[n + 1]; ++k) Dh[k] *= ((n & 1) ? -1.0 : 1.0) / (2.0 * n + 1.0);
+    up(T->Dg, Dh);
     up(T->inv2n1, inv2n1);
     T->Dhoff.alloc(hoff.size());
     CFMM_CUDA(cudaMemcpy(T->Dhoff.get(), hoff.data(), sizeof(int64_t) * hoff.size(), cudaMemcpyHostToDevice));
@@ -1992,6 +2002,7 @@ struct Helm3dState {
     DevBuf<int> pre_fb;          // per pair: fixed frame k, or -1
     DevBuf<cd> pre_pw;           // per pair: e^m, e_a^m for m in [-Pm, Pm]
     DevBuf<cd> tri;              // coaxial operators of the M2L pairs of a launch range
+    PairSlots pairs;             // List-2 pairs of the M2L
     std::vector<int> level_off;
     int lvl_of_lo(int lo) const {
         for (size_t l = 0; l + 1 < level_off.size(); ++l)
@@ -2101,6 +2112,7 @@ void helm3d_setup(cfmm_plan_s* P) {
     }
     for (int b : T.leaf_boxes)
         if (lvl[b] >= S->l0) S->leaves_l0.push_back(b);
+    pair_slots_build(P, &S->pairs, l2, S->l0);
     S->d_leaves_l0.alloc(S->leaves_l0.size());
     CFMM_CUDA(cudaMemcpyAsync(S->d_leaves_l0.get(), S->leaves_l0.data(), sizeof(int) * S->leaves_l0.size(),
                               cudaMemcpyHostToDevice, st));
@@ -2373,19 +2385,8 @@ void helm3d_apply(cfmm_plan_s* P, const cd* sigma, const cd* tau, int64_t dstrid
     rec(3);
     // (4) M2L per level (overwrites L at levels >= l0)
     for (int l = S->l0; l < T.nlevels; ++l) {
-        int lo = T.level_off[l], nb = T.level_off[l + 1] - lo;
-        // long lists (the all-pairs top level) are split over several blocks,
-        // as far as the launch needs more blocks (many right-hand sides already
-        // give enough, and then no partials are written)
-        int nchunk = S->l2max[l] > 2 * kM2LChunk3 ? (S->l2max[l] + kM2LChunk3 - 1) / kM2LChunk3 : 1;
-        int64_t want = (int64_t)16 * nsm, base = (int64_t)std::max(1, nb) * nrhs;
-        if (nchunk > 1 && base * nchunk > want) nchunk = (int)std::max<int64_t>(1, (want + base - 1) / base);
-        // few boxes (a coarse top level): split their lists down to 4 entries
-        // so that every SM gets work
-        if (base * nchunk < want && S->l2max[l] > 4)
-            nchunk = (int)std::max<int64_t>(nchunk, std::min<int64_t>((S->l2max[l] + 3) / 4, (want + base - 1) / base));
-        int chunk = nchunk > 1 ? (S->l2max[l] + nchunk - 1) / nchunk : std::max(1, S->l2max[l]);
-        launch_tr(1, lo, nb, S->Plev[l], S->Plev[l], 1, mp, lc, nchunk, chunk);
+        m2l3d_launch(P, &S->pairs, tr3_tables(TB), l, l + 1, S->Plev[l], P->kappa, S->exp_off.get(), S->ncoef, mp, lc,
+                     nrhs);
     }
     rec(4);
     // (6) P2L, per level
@@ -2440,6 +2441,7 @@ struct Lap3Tr {
     DevBuf<int> qbox;
     DevBuf<cd> sc, tt;
     DevBuf<int> fb;
+    PairSlots pairs;
 };
 
 Lap3Tr* lap3_tr_create(cfmm_plan_s* P, int Pord) {
@@ -2462,6 +2464,7 @@ Lap3Tr* lap3_tr_create(cfmm_plan_s* P, int Pord) {
     CFMM_CUDA(cudaFuncSetAttribute((const void*)k_p2x3h_slp<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                    kH3Smem));
     L->Pord = Pord;
+    pair_slots_build(P, &L->pairs, L->l2off, T.l0);
     return L;
 }
 
@@ -2498,6 +2501,11 @@ void lap3_l2p32(Lap3Tr* L, cfmm_plan_s* P, const int* leaves, int cnt, int maxP,
 }
 
 void lap3_tr_destroy(Lap3Tr* L) { delete L; }
+
+void lap3_m2l(Lap3Tr* L, cfmm_plan_s* P, int l_lo, int l_hi, int Pord, const int64_t* eoff, int64_t ncoef, const cd* mp,
+              cd* lc, int nrhs) {
+    m2l3d_launch(P, &L->pairs, tr3_tables(L->tab), l_lo, l_hi, Pord, 0.0, eoff, ncoef, mp, lc, nrhs);
+}
 
 // mode 0: M2M into the non-leaf boxes of level l from level l+1; 1: M2L at
 // level l (writes L); 2: L2L into level l from level l-1 (adds)

@@ -1,0 +1,40 @@
+// 3D M2L over all List-2 pairs of a level, pairs on the lanes (m2l3d.cu).
+#pragma once
+
+#include "kernels.cuh"
+
+namespace cfmm {
+
+// Device tables of the 3D translations (helm3d.cu builds and owns them)
+struct Tr3Tables {
+    const double* Dh;       // D_n[m][m'], m, m' >= 0, column-major per order
+    const double* Dg;       // D_n scaled by (-1)^n/(2n+1)
+    const int64_t* Dhoff;
+    const double *al, *be, *ibe, *mu, *nu;   // coaxial recurrence coefficients by nmi(n, m >= 0)
+    const double *lsm, *lsd;                 // eps_m s_n^m, eps_m / s_n^m by nmi(n, m)
+    const double* fact;                      // j!
+};
+
+// The unordered List-2 pairs of a plan in slots of 32-lane tiles: level l owns
+// the tiles [tile0[l], tile0[l+1]). With one order at every level (Laplace) all
+// levels are translated in one go.
+struct PairSlots {
+    std::vector<int> tile0;
+    int64_t nslot = 0;
+    DevBuf<int> box_a, box_b;     // the pair's boxes (a < b), -1 for an empty slot
+    DevBuf<signed char> kind;     // kPairFlat, kPairGeneral, kPairIso + k
+    DevBuf<int> slot;             // per List-2 entry: 2 slot + (0: owner is box_a, 1: box_b)
+    DevBuf<int> count;            // per level: slots given to flat and to other pairs
+    // workspaces of an apply
+    DevBuf<cd> pw, fl, tri, vec;
+};
+
+// Builds the slots of the plan's List 2 (device work on the plan's stream)
+void pair_slots_build(cfmm_plan_s* P, PairSlots* S, const std::vector<int>& l2off, int l0);
+
+// M2L of the boxes of levels [l_lo, l_hi) at order Pord, all right-hand sides:
+// local expansions of those boxes are overwritten. Laplace when kappa == 0.
+void m2l3d_launch(cfmm_plan_s* P, PairSlots* S, const Tr3Tables& T, int l_lo, int l_hi, int Pord, double kappa,
+                  const int64_t* eoff, int64_t ncoef, const cd* mp, cd* lc, int nrhs);
+
+}  // namespace cfmm

@@ -1093,7 +1093,9 @@ static void launch_near(const KParams& K, const NearLists& L, int nleaves, int l
     int dev = 0, nsm = 0;
     CFMM_CUDA(cudaGetDevice(&dev));
     CFMM_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
-    int64_t per = L.boxes ? leaf_size : K.n_trg, rows = L.boxes ? (int64_t)nleaves * nrhs : nrhs;
+    // (nrhs stays out of the rule: the order of a target's sum depends on tb, and a
+    // right-hand side's result is the same alone and among others)
+    int64_t per = L.boxes ? leaf_size : K.n_trg, rows = L.boxes ? nleaves : 1;
     int tb = (int)std::min<int64_t>(kNearTargets, per);
     auto blocks = [&] { return rows * ((per + tb - 1) / tb); };
     if (rows * per >= 32768)
