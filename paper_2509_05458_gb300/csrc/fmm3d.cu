@@ -17,7 +17,7 @@
 //   L2L  L'_k^l = sum L_n^m U_{n-k}^{m-l}(c' - c)
 //   P2L  L_k^l = sum s (-1)^l T_k^{-l}(y - c)          L2P  u = sum L_k^l U_k^l(x - c)
 // The translations run as point-and-shoot (rotate the shift onto the z-axis,
-// translate along it, rotate back; O(P^3)), in helm3d.cu's k_tr3l.
+// translate along it, rotate back; O(P^3)), in pairs3d.cu.
 // Double layer: n.grad = nu+ d+ + nu- d- + n3 dz (nu+- = n1 +- i n2),
 //   d+ U_n^m = -U_{n-1}^{m-1}/2, d- U_n^m = U_{n-1}^{m+1}/2, dz U_n^m = U_{n-1}^m,
 //   d+ T_n^m = -T_{n+1}^{m-1}/2, d- T_n^m = T_{n+1}^{m+1}/2, dz T_n^m = -T_{n+1}^m.
@@ -559,7 +559,7 @@ void fmm3d_apply(cfmm_plan_s* P, const cd* sigma, const cd* tau, int64_t dstride
     int Pu = S->Plev[0];
     // (2) M2M
     for (int l = T.nlevels - 2; l >= S->l0; --l)
-        lap3_tr_launch(S->tr, P, 0, l, Pu, S->exp_off.get(), S->ncoef, mp, mp, nrhs);
+        lap3_m2m(S->tr, P, l, Pu, S->exp_off.get(), S->ncoef, mp, nrhs);
     rec(3);
     // (4) M2L
     lap3_m2l(S->tr, P, S->l0, T.nlevels, Pu, S->exp_off.get(), S->ncoef, mp, lc, nrhs);
@@ -575,8 +575,8 @@ void fmm3d_apply(cfmm_plan_s* P, const cd* sigma, const cd* tau, int64_t dstride
     }
     rec(5);
     // (7) L2L
-    for (int l = S->l0 + 1; l < T.nlevels; ++l)
-        lap3_tr_launch(S->tr, P, 2, l, Pu, S->exp_off.get(), S->ncoef, lc, lc, nrhs);
+    for (int l = S->l0; l + 1 < T.nlevels; ++l)
+        lap3_l2l(S->tr, P, l, Pu, S->exp_off.get(), S->ncoef, lc, nrhs);
     rec(6);
     rec(7);
     near_join(P);   // the near field has written u

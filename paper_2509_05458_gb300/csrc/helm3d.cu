@@ -56,7 +56,7 @@
 
 #include "cfmm_special.cuh"
 #include "kernels.cuh"
-#include "m2l3d.cuh"
+#include "pairs3d.cuh"
 
 namespace cfmm {
 
@@ -67,13 +67,6 @@ __host__ __device__ __forceinline__ int nmi(int n, int m) { return n * n + n + m
 constexpr int kH3Threads = 256;
 constexpr int kH3MaxP = kMaxP3Top;   // expansion order limit of this path
 constexpr int kH3Smem = 220 * 1024;  // dynamic shared memory ceiling per block
-constexpr int kM2LChunk3 = 32;       // List-2 entries per block when a list is split
-constexpr int kTr3FlatMaxP = 23;     // largest order of the flat coaxial work
-constexpr double kDegenTol = 1e-8;   // |d1^2 + d2^2| <= this * sum |d_i|^2: fixed-frame translation
-constexpr int kTriMaxP = 40;         // largest M2L order whose coaxial operators are built ahead (k_tr3h_tri)
-constexpr int kTriMaxPMulti = 56;    // the same with several right-hand sides (operators shared by all)
-constexpr int kTriThreads = 128;     // threads of k_tr3h_tri
-constexpr size_t kTriBudget = (size_t)6 << 30;   // bytes of operators per M2L launch range
 
 // ---------------------------------------------------------------------------
 // Per-device tables shared by all plans: D_n (row-major, n <= Pmax), the Z
@@ -84,9 +77,8 @@ struct H3Tables {
     DevBuf<double> Dh;       // D_n[m][m'] for m, m' >= 0, column-major per order
     DevBuf<double> Dg;       // the same scaled by (-1)^n/(2n+1)
     DevBuf<int64_t> Dhoff;   // [Pmax+2]
-    DevBuf<double> inv2n1;   // 1/(2n+1), n <= 2Pmax+2
     DevBuf<double> zA, zB;   // [(2Pmax+3)^2] by nmi(n, m), m >= 0
-    DevBuf<double> al, be, ibe, mu, nu;  // coaxial recurrence coefficients, nmi(n, m), m >= 0
+    DevBuf<double> al, be, ab, cg, smu, snu;   // coaxial recurrence coefficients (see Tr3Tables)
     DevBuf<double> g3, gp, gm;           // gradient coefficients c3, s+ c+, s- c- by nmi(n, m), all m
     DevBuf<double> dg, s21;  // sqrt((2m-1)/(2m)), sqrt(2m+1), m <= Pmax+1
     DevBuf<int> knm;         // k -> n * 256 + (m + 128), k < (Pmax+1)^2
@@ -198,8 +190,8 @@ static void host_rotation_tables(int P, std::vector<double>& D, std::vector<int6
 }
 
 static Tr3Tables tr3_tables(const H3Tables* T) {
-    return Tr3Tables{T->Dh.get(), T->Dg.get(), T->Dhoff.get(), T->al.get(), T->be.get(), T->ibe.get(), T->mu.get(),
-                     T->nu.get(), T->lsm.get(), T->lsd.get(), T->fact.get()};
+    return Tr3Tables{T->Dh.get(), T->Dg.get(), T->Dhoff.get(), T->al.get(), T->be.get(), T->ab.get(), T->cg.get(),
+                     T->smu.get(), T->snu.get(), T->lsm.get(), T->lsd.get(), T->fact.get(), T->ifact.get()};
 }
 
 static H3Tables* tables(int P) {
@@ -215,7 +207,7 @@ static H3Tables* tables(int P) {
     host_rotation_tables(Pm, D, off);
     int NN = 2 * Pm + 3;
     size_t NT = (size_t)NN * NN;
-    std::vector<double> zA(NT, 0.0), zB(NT, 0.0), al(NT, 0.0), be(NT, 0.0), ibe(NT, 0.0), mu(NT, 0.0),
+    std::vector<double> zA(NT, 0.0), zB(NT, 0.0), al(NT, 0.0), be(NT, 0.0), mu(NT, 0.0),
         nu(NT, 0.0), g3(NT, 0.0), gp(NT, 0.0), gm(NT, 0.0), dg(Pm + 2, 0.0), s21(Pm + 2, 0.0);
     for (int n = 0; n < NN; ++n) {
         for (int m = 0; m <= n; ++m) {
@@ -226,7 +218,6 @@ static H3Tables* tables(int P) {
             }
             al[k] = std::sqrt((double)(n - m) * (n + m)) / (2.0 * n + 1.0);
             be[k] = std::sqrt((double)(n + 1 - m) * (n + 1 + m)) / (2.0 * n + 1.0);
-            ibe[k] = 1.0 / be[k];
             mu[k] = std::sqrt((double)(n - m) * std::max(n - m - 1, 0)) / (2.0 * (2.0 * n + 1.0));
             nu[k] = std::sqrt((double)(n + m + 1) * (n + m + 2)) / (2.0 * (2.0 * n + 1.0));
         }
@@ -250,8 +241,20 @@ static H3Tables* tables(int P) {
         for (int m = 0; m <= n; ++m)
             for (int mp = 0; mp <= n; ++mp) Dh[hoff[n] + (int64_t)mp * (n + 1) + m] = D[off[n] + (int64_t)(m + n) * N + (mp + n)];
     }
-    std::vector<double> inv2n1(NN);
-    for (int n = 0; n < NN; ++n) inv2n1[n] = 1.0 / (2.0 * n + 1.0);
+    // products of the coaxial recurrence (see Tr3Tables)
+    std::vector<double> ab(NT, 0.0), cg(NT, 0.0), smu(NT, 0.0), snu(NT, 0.0);
+    for (int m = 0; m < NN; ++m) {
+        double gam = 1.0;
+        for (int n = m; n < NN; ++n) {
+            cg[nmi(n, m)] = ((n & 1) ? -(2.0 * n + 1.0) : 2.0 * n + 1.0) * gam;
+            gam /= be[nmi(n, m)];
+            if (n > m) ab[nmi(n, m)] = al[nmi(n, m)] * be[nmi(n - 1, m)];
+            if (m > 0 && n + 1 < NN) {
+                smu[nmi(n, m)] = mu[nmi(n + 1, m - 1)] / nu[nmi(m - 1, m - 1)];
+                snu[nmi(n, m)] = nu[nmi(n - 1, m - 1)] / nu[nmi(m - 1, m - 1)];
+            }
+        }
+    }
     auto up = [](DevBuf<double>& b, const std::vector<double>& v) {
         b.alloc(v.size());
         CFMM_CUDA(cudaMemcpy(b.get(), v.data(), sizeof(double) * v.size(), cudaMemcpyHostToDevice));
@@ -260,11 +263,14 @@ static H3Tables* tables(int P) {
     for (int n = 0; n <= Pm; ++n)
         for (int64_t k = hoff[n]; k < hoff[n + 1]; ++k) Dh[k] *= ((n & 1) ? -1.0 : 1.0) / (2.0 * n + 1.0);
     up(T->Dg, Dh);
-    up(T->inv2n1, inv2n1);
     T->Dhoff.alloc(hoff.size());
     CFMM_CUDA(cudaMemcpy(T->Dhoff.get(), hoff.data(), sizeof(int64_t) * hoff.size(), cudaMemcpyHostToDevice));
-    up(T->mu, mu);
-    up(T->nu, nu);
+    up(T->al, al);
+    up(T->be, be);
+    up(T->ab, ab);
+    up(T->cg, cg);
+    up(T->smu, smu);
+    up(T->snu, snu);
     up(T->g3, g3);
     up(T->gp, gp);
     up(T->gm, gm);
@@ -304,15 +310,9 @@ static H3Tables* tables(int P) {
 
     T->zA.alloc(zA.size());
     T->zB.alloc(zB.size());
-    T->al.alloc(al.size());
-    T->be.alloc(be.size());
-    T->ibe.alloc(ibe.size());
 
     CFMM_CUDA(cudaMemcpy(T->zA.get(), zA.data(), sizeof(double) * zA.size(), cudaMemcpyHostToDevice));
     CFMM_CUDA(cudaMemcpy(T->zB.get(), zB.data(), sizeof(double) * zB.size(), cudaMemcpyHostToDevice));
-    CFMM_CUDA(cudaMemcpy(T->al.get(), al.data(), sizeof(double) * al.size(), cudaMemcpyHostToDevice));
-    CFMM_CUDA(cudaMemcpy(T->be.get(), be.data(), sizeof(double) * be.size(), cudaMemcpyHostToDevice));
-    CFMM_CUDA(cudaMemcpy(T->ibe.get(), ibe.data(), sizeof(double) * ibe.size(), cudaMemcpyHostToDevice));
     T->Pmax = Pm;
     sets.push_back(T);
     return T;
@@ -1108,867 +1108,6 @@ static void launch_l2p3f(H3Tables* TB, bool helm, cfmm_plan_s* P, const int* lea
     CFMM_LAUNCHED();
 }
 
-// ---------------------------------------------------------------------------
-// translations
-// ---------------------------------------------------------------------------
-struct Tr3hArgs {
-    const double* cre;
-    const double* cim;
-    const int64_t* eoff;
-    int64_t ncoef;
-    const double* Dh;
-    const int64_t* Dhoff;
-    const double* inv2n1;
-    const double* al;
-    const double* be;
-    const double* ibe;
-    const double* mu;
-    const double* nu;
-    const int* knm;
-    double kappa;
-    // source enumeration (mode 0: children cbeg..cend; 1: List 2; 2: parent)
-    const int* cbeg;
-    const int* cend;
-    const int* loff;
-    const int* lent;
-    const int* parent;
-    const int* leaf;
-    const int* qbox;     // owner (destination) box of each List-2 entry
-};
-
-// i^e x for integer e (a permutation of the parts; no arithmetic)
-__device__ __forceinline__ cd mul_ipow(int e, cd x) {
-    switch (e & 3) {
-        case 0: return x;
-        case 1: return cd{-x.y, x.x};
-        case 2: return cd{-x.x, -x.y};
-        default: return cd{x.y, -x.x};
-    }
-}
-
-// The fixed matrices D_n satisfy D[-m][m'] = D[m][-m'] = (-1)^{n+m+m'} D[m][m']
-// and D^T = S D S, S = diag((-1)^m). With w+-_{m'} = x_{m'} +- (-1)^{m'} x_{-m'}
-// (m' > 0), row m >= 0 of D x and row -m follow from one half-row pass:
-//   n+m even:  y_{+-m} = D[m][0] x_0 + E +- O,   E, O = sum over even / odd m' > 0 of D[m][m'] w+_{m'}
-//   n+m odd:   y_m = E + O,  y_{-m} = O - E      (with w-; D[m][0] = 0)
-// Dh holds D[m][m'] for m, m' >= 0, column-major per order (Dh_n[m' (n+1) + m]).
-
-// w-pass: wb <- w+- of x, x_k = f_k in_k with the per-coefficient factor f
-// given by (i-power, sign, power table): x = i^{ip*m} sg^m pw[m + Pm] in
-__device__ __forceinline__ void w_pass(const int* knm, const cd* in, cd* wb, int P, int ip, int sgn_alt,
-                                       const cd* pw, int Pm) {
-    int W = (P + 1) * (P + 2) / 2;          // items (n, m >= 0)
-    for (int w = threadIdx.x; w < W; w += blockDim.x) {
-        int n = (int)((sqrtf(8.0f * w + 1.0f) - 1.0f) * 0.5f);
-        while ((n + 1) * (n + 2) / 2 <= w) ++n;
-        while (n * (n + 1) / 2 > w) --n;
-        int m = w - n * (n + 1) / 2;
-        int k = nmi(n, m);
-        auto xf = [&](int mm) {
-            cd v = in[nmi(n, mm)];
-            if (pw) v = v * pw[mm + Pm];
-            v = mul_ipow(ip * mm, v);
-            if (sgn_alt && (mm & 1)) v = -v;
-            return v;
-        };
-        cd xp = xf(m);
-        if (m == 0) {
-            wb[k] = xp;
-            continue;
-        }
-        cd xm = xf(-m);
-        if (m & 1) xm = -xm;
-        wb[nmi(n, m)] = xp + xm;
-        wb[nmi(n, -m)] = xp - xm;
-    }
-}
-
-// D-pass: y = D x from the w+- of x; out_k = g_k y_k with g = i^{op*m} (sgn_out:
-// times (-1)^m), optionally times pw_out[m + Pm], accumulated when acc != 0
-__device__ __forceinline__ void d_pass(const double* Dh, const int64_t* Dhoff, const cd* wb, cd* out, int P,
-                                       int op, int sgn_out, const cd* pwo, int Pm, int accum) {
-    int W = (P + 1) * (P + 2) / 2;          // work items (n, m >= 0)
-    for (int w = threadIdx.x; w < W; w += blockDim.x) {
-        int n = (int)((sqrtf(8.0f * w + 1.0f) - 1.0f) * 0.5f);
-        while ((n + 1) * (n + 2) / 2 <= w) ++n;
-        while (n * (n + 1) / 2 > w) --n;
-        int m = w - n * (n + 1) / 2;
-        const double* Dn = Dh + __ldg(Dhoff + n);
-        int N1 = n + 1;
-        bool odd = (n + m) & 1;
-        cd E = {0, 0}, O = {0, 0};
-        const cd* wv = wb + n * n + n;       // wv[m'] = w+_{m'}, wv[-m'] = w-_{m'}
-        for (int mp = 1; mp <= n; ++mp) {
-            double d = Dn[mp * N1 + m];
-            cd wq = odd ? wv[-mp] : wv[mp];
-            if (mp & 1) O = rmac(O, d, wq);
-            else E = rmac(E, d, wq);
-        }
-        cd yp, ym;
-        if (odd) {
-            yp = E + O;
-            ym = O - E;
-        } else {
-            cd d0 = Dn[m] * wv[0];
-            yp = d0 + E + O;
-            ym = d0 + E - O;
-        }
-        auto emit = [&](int mm, cd y) {
-            y = mul_ipow(op * mm, y);
-            if (sgn_out && (mm & 1)) y = -y;
-            if (accum && pwo) {
-                out[nmi(n, mm)] = cmac(out[nmi(n, mm)], y, pwo[mm + Pm]);
-                return;
-            }
-            if (pwo) y = y * pwo[mm + Pm];
-            if (accum) out[nmi(n, mm)] += y;
-            else out[nmi(n, mm)] = y;
-        };
-        emit(m, yp);
-        if (m > 0) emit(-m, ym);
-    }
-}
-
-// The fixed real rotation Q_k (k = 0, 1) of the fixed-frame translation,
-// applied in place to the coefficients x (order P) through wb and tmp: the
-// rotation sequence of the translation kernels with e = i^k and alpha = pi/2,
-// whose diagonal factors are powers of i (no tables). Ends with a barrier.
-__device__ void rot_fixed(const Tr3hArgs& A, const double* Dh, cd* x, cd* wb, cd* tmp, int P, int Pm, int k) {
-    w_pass(A.knm, x, wb, P, 1 + k, 0, nullptr, Pm);
-    __syncthreads();
-    d_pass(Dh, A.Dhoff, wb, tmp, P, 0, 0, nullptr, Pm, 0);
-    __syncthreads();
-    w_pass(A.knm, tmp, wb, P, 3, 0, nullptr, Pm);
-    __syncthreads();
-    d_pass(Dh, A.Dhoff, wb, x, P, 1, 0, nullptr, Pm, 0);
-    __syncthreads();
-}
-
-// Its inverse from x into out (added when accum != 0); x and tmp are
-// overwritten. Needs a barrier before (x written) and leaves out unsynchronised.
-__device__ void rot_fixed_inv(const Tr3hArgs& A, const double* Dh, cd* x, cd* wb, cd* tmp, cd* out, int P, int Pm,
-                              int k, int accum) {
-    w_pass(A.knm, x, wb, P, 1, 0, nullptr, Pm);
-    __syncthreads();
-    d_pass(Dh, A.Dhoff, wb, tmp, P, 0, 0, nullptr, Pm, 0);
-    __syncthreads();
-    w_pass(A.knm, tmp, wb, P, 1, 0, nullptr, Pm);
-    __syncthreads();
-    d_pass(Dh, A.Dhoff, wb, out, P, (1 - k) & 3, 0, nullptr, Pm, accum);
-}
-
-// Per-shift quantities of a launch, one thread per (destination, source)
-// pair: e = e^{i beta}, e_a = e^{i alpha} and f_l(kappa t), l <= NR. Pair p
-// of the launch is list entry qfirst + p (mode 1), child box qfirst + p
-// (mode 0) or destination box lo + p (mode 2).
-__global__ void k_tr3h_pre(Tr3hArgs A, int mode, int lo, int qfirst, int npair, int NR, int use_h,
-                           cd* __restrict__ sc, cd* __restrict__ fl, int* __restrict__ fb, int Pm,
-                           cd* __restrict__ pwt) {
-    int p = blockIdx.x * blockDim.x + threadIdx.x;
-    if (p >= npair) return;
-    int b, s;
-    if (mode == 1) {
-        int q = qfirst + p;
-        s = A.lent[q];
-        b = A.qbox[q];
-    } else if (mode == 0) {
-        s = qfirst + p;
-        b = A.parent[s];
-    } else {
-        b = lo + p;
-        s = A.parent[b];
-    }
-    cd d[3];
-    for (int k = 0; k < 3; ++k) d[k] = cd{A.cre[3 * b + k] - A.cre[3 * s + k], A.cim[3 * b + k] - A.cim[3 * s + k]};
-    cd s2 = d[0] * d[0] + d[1] * d[1];
-    // an isotropic complex direction in the xy-plane (s^2 = 0 or nearly, with
-    // (d1, d2) != 0) has no z-rotation angle: the pair is translated in the
-    // frame of the fixed real rotation Q_k (Q_0 d = (-d3, d2, d1), Q_1 d =
-    // (-d3, -d1, d2)), the one with the larger |(Q d)_1^2 + (Q d)_2^2|
-    int fr = -1;
-    {
-        double n2 = cabs2(d[0]) + cabs2(d[1]) + cabs2(d[2]);
-        bool xy = d[0].x != 0.0 || d[0].y != 0.0 || d[1].x != 0.0 || d[1].y != 0.0;
-        if (xy && cabs2(s2) <= (kDegenTol * n2) * (kDegenTol * n2)) {
-            cd a0 = d[2] * d[2] + d[1] * d[1], a1 = d[2] * d[2] + d[0] * d[0];
-            fr = cabs2(a0) >= cabs2(a1) ? 0 : 1;
-            cd q1 = fr == 0 ? d[1] : -d[0], q2 = fr == 0 ? d[0] : d[1];
-            d[0] = -d[2];
-            d[1] = q1;
-            d[2] = q2;
-            s2 = d[0] * d[0] + d[1] * d[1];
-        }
-    }
-    fb[p] = fr;
-    cd t = csqrt_p(s2 + d[2] * d[2]);
-    cd sq = {0, 0}, e = {1, 0};
-    if (!(s2.x == 0.0 && s2.y == 0.0)) {
-        sq = csqrt_p(s2);
-        e = (d[0] + mul_i(d[1])) / sq;
-    }
-    cd ea = (d[2] + mul_i(sq)) / t;
-    sc[2 * (size_t)p] = e;
-    sc[2 * (size_t)p + 1] = ea;
-    if (pwt) {
-        // e^m and e_a^m for m in [-Pm, Pm] (running products), for the
-        // translation kernel's diagonal factors
-        int W = 2 * Pm + 1;
-        cd* pe = pwt + (size_t)p * 2 * W;
-        for (int q = 0; q < 2; ++q) {
-            cd* dst = pe + q * W;
-            cd x = q ? ea : e, ix = cinv(x), v = {1, 0}, iv = {1, 0};
-            dst[Pm] = v;
-            for (int m = 1; m <= Pm; ++m) {
-                v = v * x;
-                iv = iv * ix;
-                dst[Pm + m] = v;
-                dst[Pm - m] = iv;
-            }
-        }
-    }
-    if (NR < 0) {                      // Laplace: only t
-        fl[p] = t;
-        return;
-    }
-    cd* f = fl + (size_t)p * (NR + 1);
-    cd z = A.kappa * t;
-    if (use_h) sph_h_seq(z, NR, f);
-    else sph_j_seq(z, NR, f);
-}
-
-// x^m for m = 0..M by binary exponentiation (one lane per m)
-__device__ __forceinline__ cd cpow_int(cd x, int m) {
-    cd r = {1, 0};
-    while (m) {
-        if (m & 1) r = r * x;
-        x = x * x;
-        m >>= 1;
-    }
-    return r;
-}
-
-// Coaxial translation with the work flattened over the block (equal input
-// and output orders P, all columns of T^m in shared memory at once):
-//   1. the columns of every m advance together: at step c' thread items are
-//      the (m, row) pairs of column c = m + c' + 1 (rows c..NR-c, NR = 2P),
-//      from the two previous columns of the same m (the recurrence of the
-//      file comment, in the stable direction);
-//   2. rows <= P of each column go to a compact lower triangle per m
-//      (rows r = m..P, columns c = m..r, at (r-m)(r-m+1)/2 + c - m, m-blocks
-//      one after the other);
-//   3. the product out_n^{+-m} = sum_{c<=n} T_{n c} a_c + (2n+1)(-1)^n
-//      sum_{r>n} T_{r n} a~_r, one thread item per (m, n, sign), m-major, so
-//      the lanes of a warp share a loop length.
-// The per-warp path below does the same work with one warp per m, whose lanes
-// idle as the columns shorten.
-__host__ __device__ inline size_t tr3h_tri_off(int P, int m) {
-    size_t o = 0;
-    for (int q = 0; q < m; ++q) o += (size_t)(P - q + 1) * (P - q + 2) / 2;
-    return o;
-}
-// g_c = (-1)^c (2c + 1), the column factor of the stored coaxial triangles
-__device__ __forceinline__ double coax_g(int c) { return (c & 1) ? -(2.0 * c + 1.0) : (2.0 * c + 1.0); }
-__host__ __device__ inline size_t tr3h_tri_size(int P) { return (size_t)(P + 1) * (P + 2) * (P + 3) / 6; }
-__host__ __device__ inline size_t tr3h_flat_cols(int P) {
-    return (size_t)3 * (P + 1) * (2 * P + 2) + tr3h_tri_off(P, P + 1);
-}
-
-// out_n^{+-m} = sum_{c<=n} T_{n c} a_c + (2n+1)(-1)^n sum_{r>n} T_{r n} a~_r from
-// the compact triangles tri (shared or global memory) holding T'_{r c} =
-// g_c T_{r c}, g_c = (-1)^c (2c+1): with a~_c = a_c / g_c both sums read the same
-// vector a~, out_n = sum_{c<=n} T'_{n c} a~_c + sum_{r>n} T'_{r n} a~_r, one loop of
-// P - m + 1 terms for every n of a given m (row n of the triangle, then its
-// column n). One thread item per (m >= 0, n) computes both signs of m from the
-// same operator entries and writes them as the first pass of the back rotation
-// would (w+- of Phi out, see w_pass), so that pass is not run. m-major items.
-__device__ void coax_product_w(int P, const cd* __restrict__ tri, const cd* __restrict__ wb, cd* __restrict__ wout) {
-    int nitem = (P + 1) * (P + 2) / 2;
-    for (int t = threadIdx.x; t < nitem; t += blockDim.x) {
-        int m = 0, rem = t;
-        while (rem >= P - m + 1) {
-            rem -= P - m + 1;
-            ++m;
-        }
-        int n = m + rem;
-        const cd* T = tri + tr3h_tri_off(P, m);
-        const int k0 = n - m;                               // row n holds columns m..n
-        const int rowb = k0 * (k0 + 1) / 2;
-        cd sp = {0, 0}, sn = {0, 0};
-        for (int j = 0; j <= P - m; ++j) {
-            int idx, k;
-            if (j <= k0) {
-                idx = rowb + j;                             // T'_{n, m+j}
-                k = m + j;
-            } else {
-                int r = n + (j - k0);                       // T'_{r, n}
-                idx = (r - m) * (r - m + 1) / 2 + k0;
-                k = r;
-            }
-            cd tv = T[idx];
-            sp = cmac(sp, tv, wb[nmi(k, m)]);
-            if (m > 0) sn = cmac(sn, tv, wb[nmi(k, -m)]);
-        }
-        // w+- of x = Phi out: x_{+-m} = i^{+-m} out_{+-m}
-        cd xp = mul_ipow(m, sp);
-        if (m == 0) {
-            wout[nmi(n, 0)] = xp;
-            continue;
-        }
-        cd xm = mul_ipow(-m, sn);
-        if (m & 1) xm = -xm;
-        wout[nmi(n, m)] = xp + xm;
-        wout[nmi(n, -m)] = xp - xm;
-    }
-}
-
-__device__ void coax_flat(const Tr3hArgs& A, int P, int NR, const cd* __restrict__ sect, cd* __restrict__ cols,
-                          const cd* __restrict__ a, const cd* __restrict__ wb, cd* __restrict__ bb) {
-    const int L = NR + 2;                       // column length
-    cd* tri = cols + (size_t)3 * (P + 1) * L;
-    auto col = [&](int k, int m) { return cols + ((size_t)k * (P + 1) + m) * L; };
-    // columns c = m (sectorial) in buffer 1, c = m - 1 (zero) in buffer 0
-    for (int t = threadIdx.x; t < (P + 1) * L; t += blockDim.x) {
-        int m = t / L, r = t - m * L;
-        col(0, m)[r] = cd{0, 0};
-        col(1, m)[r] = (r >= m && r <= NR - m) ? sect[(size_t)m * (NR + 1) + r] : cd{0, 0};
-    }
-    __syncthreads();
-    // column c = m into the triangles (rows m..P)
-    for (int t = threadIdx.x; t < (P + 1) * (P + 1); t += blockDim.x) {
-        int m = t / (P + 1), r = t - m * (P + 1);
-        if (r >= m) tri[tr3h_tri_off(P, m) + (size_t)(r - m) * (r - m + 1) / 2] = coax_g(m) * col(1, m)[r];
-    }
-    int kp = 0, kc = 1, kn = 2;
-    for (int cp = 0; cp < P; ++cp) {
-        // items (m, r): m <= P - 1 - cp, r in [m + cp + 1, NR - m - cp - 1]
-        int K = NR - 2 * cp - 1;                // rows of m = 0
-        int nitem = 0;
-        for (int m = 0; m <= P - 1 - cp; ++m) nitem += K - 2 * m;
-        for (int t = threadIdx.x; t < nitem; t += blockDim.x) {
-            int m = 0, rem = t;
-            while (rem >= K - 2 * m) {
-                rem -= K - 2 * m;
-                ++m;
-            }
-            int c = m + cp, r = c + 1 + rem;
-            const cd* prv = col(kp, m);
-            const cd* cur = col(kc, m);
-            double ac = __ldg(A.al + nmi(c, m)), ib = __ldg(A.ibe + nmi(c, m));
-            cd v = rmac(ac * prv[r], -__ldg(A.al + nmi(r + 1, m)), cur[r + 1]);
-            v = rmac(v, __ldg(A.be + nmi(r - 1, m)), cur[r - 1]);
-            col(kn, m)[r] = ib * v;
-        }
-        __syncthreads();
-        // rows c + 1 .. P of column c + 1 into the triangles
-        int ns = 0;
-        for (int m = 0; m <= P - 1 - cp; ++m) ns += P - (m + cp);
-        for (int t = threadIdx.x; t < ns; t += blockDim.x) {
-            int m = 0, rem = t;
-            while (rem >= P - (m + cp)) {
-                rem -= P - (m + cp);
-                ++m;
-            }
-            int c1 = m + cp + 1, r = c1 + rem;
-            tri[tr3h_tri_off(P, m) + (size_t)(r - m) * (r - m + 1) / 2 + (c1 - m)] = coax_g(c1) * col(kn, m)[r];
-        }
-        int k0 = kp;
-        kp = kc;
-        kc = kn;
-        kn = k0;
-    }
-    __syncthreads();
-    coax_product_w(P, tri, wb, bb);
-}
-
-// The coaxial operators of the M2L pairs of a launch (equal orders P), built
-// once per pair for every right-hand side: one block per pair writes the
-// compact triangles T^m (the layout of tr3h_tri_off, tr3h_tri_size entries)
-// to tri. The sectorial columns T_{r m}^m (r = m..NR - m) come from the
-// recurrence over m (one step per m, rows over the block's threads), then the
-// columns of every m advance together, two buffers per m: the next column
-// overwrites the one before the current one in place (each row reads only its
-// own entry of it). Shared memory: the radial sequence, 2 (P+1) (NR+2)
-// complex values and P+1 offsets.
-__global__ void k_tr3h_tri(Tr3hArgs A, int P, int npair, const cd* __restrict__ fl, cd* __restrict__ tri) {
-    extern __shared__ cd sm[];
-    const int NR = 2 * P, L = NR + 2;
-    cd* f = sm;
-    cd* cols = f + (NR + 1);
-    int* moff = (int*)(cols + (size_t)2 * (P + 1) * L);
-    auto col = [&](int k, int m) { return cols + ((size_t)k * (P + 1) + m) * L; };
-    const size_t tsz = tr3h_tri_size(P);
-    for (int p = blockIdx.x; p < npair; p += gridDim.x) {
-        __syncthreads();
-        cd* T = tri + (size_t)p * tsz;
-        for (int l = threadIdx.x; l <= NR; l += blockDim.x) f[l] = fl[(size_t)p * (NR + 1) + l];
-        for (int m = threadIdx.x; m <= P; m += blockDim.x) moff[m] = (int)tr3h_tri_off(P, m);
-        for (int t = threadIdx.x; t < 2 * (P + 1) * L; t += blockDim.x) cols[t] = cd{0, 0};
-        __syncthreads();
-        // sectorial columns into buffer 1 (buffer 0 stays zero: the column
-        // before the first)
-        for (int r = threadIdx.x; r <= NR; r += blockDim.x) {
-            double sg = (r & 1) ? -1.0 : 1.0;
-            col(1, 0)[r] = (sg * (2.0 * r + 1.0)) * f[r];
-        }
-        __syncthreads();
-        for (int m = 1; m <= P; ++m) {
-            const cd* pv = col(1, m - 1);
-            cd* cur = col(1, m);
-            int mm = m - 1;
-            double inu = 1.0 / __ldg(A.nu + nmi(mm, mm));
-            for (int r = m + threadIdx.x; r <= NR - m; r += blockDim.x) {
-                double mu1 = __ldg(A.mu + nmi(r + 1, mm)), nu1 = __ldg(A.nu + nmi(r - 1, mm));
-                cur[r] = inu * (mu1 * pv[r + 1] + nu1 * pv[r - 1]);
-            }
-            __syncthreads();
-        }
-        // column c = m of every m into the triangles (rows m..P)
-        for (int t = threadIdx.x; t < (P + 1) * (P + 1); t += blockDim.x) {
-            int m = t / (P + 1), r = t - m * (P + 1);
-            if (r >= m) T[moff[m] + (r - m) * (r - m + 1) / 2] = coax_g(m) * col(1, m)[r];
-        }
-        int kp = 0, kc = 1;
-        for (int cp = 0; cp < P; ++cp) {
-            // items (m, r): m <= P - 1 - cp, r in [m + cp + 1, NR - m - cp - 1]
-            int K = NR - 2 * cp - 1;
-            int nitem = (P - cp) * (K - (P - 1 - cp));
-            for (int t = threadIdx.x; t < nitem; t += blockDim.x) {
-                int m = 0, rem = t;
-                while (rem >= K - 2 * m) {
-                    rem -= K - 2 * m;
-                    ++m;
-                }
-                int c = m + cp, r = c + 1 + rem;
-                cd* prv = col(kp, m);
-                const cd* cur = col(kc, m);
-                double ac = __ldg(A.al + nmi(c, m)), ib = __ldg(A.ibe + nmi(c, m));
-                cd v = rmac(ac * prv[r], -__ldg(A.al + nmi(r + 1, m)), cur[r + 1]);
-                v = rmac(v, __ldg(A.be + nmi(r - 1, m)), cur[r - 1]);
-                prv[r] = ib * v;
-            }
-            __syncthreads();
-            // rows c + 1 .. P of column c + 1 into the triangles
-            int ns = 0;
-            for (int m = 0; m <= P - 1 - cp; ++m) ns += P - (m + cp);
-            for (int t = threadIdx.x; t < ns; t += blockDim.x) {
-                int m = 0, rem = t;
-                while (rem >= P - (m + cp)) {
-                    rem -= P - (m + cp);
-                    ++m;
-                }
-                int c1 = m + cp + 1, r = c1 + rem;
-                T[moff[m] + (r - m) * (r - m + 1) / 2 + (c1 - m)] = coax_g(c1) * col(kp, m)[r];
-            }
-            int k0 = kp;
-            kp = kc;
-            kc = k0;
-        }
-    }
-}
-
-// One translation per destination box and source; the destination box's
-// result is accumulated in shared memory and written (mode 0, 1) or added
-// (mode 2) at the end. Shared layout: acc[Ko], a[Km], bb[Km], wb[Km],
-// f[Pi+Po+1], pw_e[2Pm+1], pw_a[2Pm+1], pw_ai[2Pm+1], pw_ei[2Pm+1],
-// sect[(Pmin+1)(Pi+Po+1)], per-warp columns [nwarps][3][Pi+Po+2] (these two
-// in global scratch for large orders), then (when it fits) the Dh table.
-__global__ void k_tr3h(Tr3hArgs A, int mode, int lo, int nb, int Pi, int Po, int use_h, int d_in_smem,
-                       cd* __restrict__ gscr, const cd* __restrict__ in, cd* __restrict__ out, int chunk,
-                       cd* __restrict__ part, int qfirst, const cd* __restrict__ pwt, const cd* __restrict__ fl,
-                       int nrhs, int nchunk, int acc_glob, int flat, const int* __restrict__ fb,
-                       int ops_g, const cd* __restrict__ trig) {
-    extern __shared__ cd sm[];
-    int Pm = max(Pi, Po), Pn = min(Pi, Po);
-    int Ki = (Pi + 1) * (Pi + 1), Ko = (Po + 1) * (Po + 1), Km = (Pm + 1) * (Pm + 1);
-    int NR = Pi + Po;                   // rows 0..NR
-    int nwarp = blockDim.x >> 5, lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    // acc_glob (the largest orders): the destination accumulator lives after the
-    // work arrays in the block's global scratch slice
-    cd* acc = sm;
-    cd* a = acc_glob ? sm : acc + Ko;
-    cd* bb = a + Km;
-    cd* wb = bb + Km;
-    cd* f = wb + Km;
-    cd* pwe = f + (NR + 1);
-    cd* pwa = pwe + (2 * Pm + 1);
-    cd* pwai = pwa + (2 * Pm + 1);
-    cd* pwei = pwai + (2 * Pm + 1);
-    cd* sect = pwei + (2 * Pm + 1);
-    cd* cols = sect + (size_t)(Pn + 1) * (NR + 1);
-    size_t wsz = flat ? tr3h_flat_cols(Po) : (size_t)nwarp * ((size_t)3 * (NR + 2) + (size_t)(Pm + 1) * (Pn + 1));
-    double* Dsm = (double*)(cols + wsz);
-    // ops_g: the coaxial operators come from trig (the launch was sized without
-    // coaxial work arrays, also when it has no pairs and trig is null)
-    if (ops_g) Dsm = (double*)(pwei + (2 * Pm + 1));
-    if (gscr) {
-        // large orders: the coaxial work arrays live in this block's slice of
-        // global scratch instead of shared memory
-        size_t per = (size_t)(Pn + 1) * (NR + 1) + wsz + (acc_glob ? (size_t)Ko : 0);
-        sect = gscr + (size_t)blockIdx.x * per;
-        cols = sect + (size_t)(Pn + 1) * (NR + 1);
-        if (acc_glob) acc = cols + wsz;
-        Dsm = (double*)(pwei + (2 * Pm + 1));
-    }
-    const double* Dh = A.Dh;
-    if (d_in_smem) {
-        int64_t nd = __ldg(A.Dhoff + Pm + 1);
-        for (int64_t k = threadIdx.x; k < nd; k += blockDim.x) Dsm[k] = A.Dh[k];
-        Dh = Dsm;
-    }
-    // work items (destination box, rhs, list chunk), grid-stride: a block's
-    // global scratch slice is reused by its items
-    int64_t nitem = (int64_t)nb * nrhs * nchunk;
-    for (int64_t item = blockIdx.x; item < nitem; item += gridDim.x) {
-    // with operators from trig the right-hand sides of a box are neighbours,
-    // so the blocks that read a pair's operators run close together (L2)
-    int bx = ops_g ? (int)((item / nrhs) % nb) : (int)(item % nb);
-    int rhs = ops_g ? (int)(item % nrhs) : (int)((item / nb) % nrhs);
-    int zc = (int)(item / ((int64_t)nb * nrhs));
-    int b = lo + bx;
-    if (mode == 0 && A.leaf[b]) continue;    // a leaf keeps its P2M expansion
-    __syncthreads();
-    for (int k = threadIdx.x; k < Ko; k += blockDim.x) acc[k] = cd{0, 0};
-    int qa, qb;
-    if (mode == 0) {
-        qa = A.cbeg[b];
-        qb = A.cend[b];
-    } else if (mode == 1) {
-        qa = A.loff[b];
-        qb = A.loff[b + 1];
-        if (part) {
-            // chunked List 2: this block takes entries [qa + z chunk, qa + (z+1) chunk)
-            qa += zc * chunk;
-            qb = min(qb, qa + chunk);
-        }
-    } else {
-        qa = 0;
-        qb = 1;
-    }
-    for (int q = qa; q < qb; ++q) {
-        int s = mode == 0 ? q : mode == 1 ? A.lent[q] : A.parent[b];
-        __syncthreads();
-        // shift d = c_new - c_old: M2M new = parent b, old = child s; M2L new =
-        // target b, old = source s; L2L new = child b, old = parent s
-        // this pair's index in the launch's prologue arrays
-        int p = mode == 1 ? q - qfirst : mode == 0 ? q - qfirst : b - lo;
-        const cd* src = in + (int64_t)rhs * A.ncoef + A.eoff[s];
-        for (int k = threadIdx.x; k < Ki; k += blockDim.x) a[k] = src[k];
-        if (!ops_g)
-            for (int l = threadIdx.x; l <= NR; l += blockDim.x) f[l] = fl[(size_t)p * (NR + 1) + l];
-        {
-            // powers of e and e_a, m in [-Pm, Pm], from the prologue (pwe and pwa
-            // are adjacent)
-            const cd* pt = pwt + (size_t)p * 2 * (2 * Pm + 1);
-            for (int k = threadIdx.x; k < 2 * (2 * Pm + 1); k += blockDim.x) pwe[k] = pt[k];
-        }
-        __syncthreads();
-        for (int m = threadIdx.x - Pm; m <= Pm; m += blockDim.x) {
-            pwai[Pm + m] = pwa[Pm - m];
-            pwei[Pm + m] = pwe[Pm - m];
-        }
-        // (0) a pair in the fixed frame: turn the input into it
-        int fr = __ldg(fb + p);
-        if (fr >= 0) rot_fixed(A, Dh, a, wb, bb, Pi, Pm, fr);
-        // (1) forward rotation: x = Phi E(e) c; y = D x; x' = S E(e_a) y; u = D x'; c~ = i^m u
-        w_pass(A.knm, a, wb, Pi, 1, 0, pwe, Pm);
-        __syncthreads();
-        d_pass(Dh, A.Dhoff, wb, bb, Pi, 0, 0, nullptr, Pm, 0);
-        __syncthreads();
-        w_pass(A.knm, bb, wb, Pi, 0, 1, pwa, Pm);
-        __syncthreads();
-        d_pass(Dh, A.Dhoff, wb, a, Pi, 1, 0, nullptr, Pm, 0);
-        // (2) coaxial: a~ = (-1)^r a / (2r+1) for the symmetric half; sectorial
-        // columns (warp 0), then one warp per m
-        __syncthreads();
-        for (int k = threadIdx.x; k < Ki; k += blockDim.x) {
-            int n, m;
-            nm_tab(A.knm, k, n, m);
-            double sc = __ldg(A.inv2n1 + n);
-            wb[k] = ((n & 1) ? -sc : sc) * a[k];
-        }
-        for (int k = threadIdx.x; k < Ko; k += blockDim.x) bb[k] = cd{0, 0};
-        if (wid == 0 && !ops_g) {
-            for (int r = lane; r <= NR; r += 32) {
-                double sg = (r & 1) ? -1.0 : 1.0;
-                sect[r] = (sg * (2.0 * r + 1.0)) * f[r];
-            }
-            __syncwarp();
-            for (int m = 1; m <= Pn; ++m) {
-                const cd* pv = sect + (size_t)(m - 1) * (NR + 1);
-                cd* cur = sect + (size_t)m * (NR + 1);
-                int mm = m - 1;
-                double inu = 1.0 / __ldg(A.nu + nmi(mm, mm));
-                for (int r = m + lane; r <= NR - m; r += 32) {
-                    double mu1 = __ldg(A.mu + nmi(r + 1, mm)), nu1 = __ldg(A.nu + nmi(r - 1, mm));
-                    cur[r] = inu * (mu1 * pv[r + 1] + nu1 * pv[r - 1]);
-                }
-                __syncwarp();
-            }
-        }
-        __syncthreads();
-        if (ops_g) {
-            coax_product_w(Po, trig + (size_t)p * tr3h_tri_size(Po), wb, bb);
-        } else if (flat) {
-            coax_flat(A, Po, NR, sect, cols, a, wb, bb);
-        } else
-        for (int m = wid; m <= Pn; m += nwarp) {
-            cd* cm1 = cols + (size_t)wid * ((size_t)3 * (NR + 2) + (size_t)(Pm + 1) * (Pn + 1));
-            cd* c0 = cm1 + (NR + 2);
-            cd* c1 = c0 + (NR + 2);
-            cd* Tm = c1 + (NR + 2);              // lower triangle T[r][c], r <= Pm, c <= Pn
-            const cd* sc = sect + (size_t)m * (NR + 1);
-            for (int r = lane; r <= NR; r += 32) {
-                cm1[r] = cd{0, 0};
-                c0[r] = (r >= m && r <= NR - m) ? sc[r] : cd{0, 0};
-            }
-            __syncwarp();
-            for (int c = m; c <= Pn; ++c) {
-                // column c holds T_{r,c} for rows c <= r <= NR - c; keep rows <= Pm
-                for (int r = c + lane; r <= Pm; r += 32) Tm[r * (Pn + 1) + c] = c0[r];
-                if (c == Pn) break;
-                // next column c + 1, rows c + 1 .. NR - c - 1
-                double ac = __ldg(A.al + nmi(c, m)), ib = __ldg(A.ibe + nmi(c, m));
-                for (int r = c + 1 + lane; r <= NR - c - 1; r += 32) {
-                    cd v = rmac(ac * cm1[r], -__ldg(A.al + nmi(r + 1, m)), c0[r + 1]);
-                    if (r - 1 >= m) v = rmac(v, __ldg(A.be + nmi(r - 1, m)), c0[r - 1]);
-                    c1[r] = ib * v;
-                }
-                __syncwarp();
-                cd* tmp = cm1;
-                cm1 = c0;
-                c0 = c1;
-                c1 = tmp;
-            }
-            __syncwarp();
-            // out_n^{mm} = sum_{c <= min(n, Pi)} T_{n c} a_c^{mm}
-            //            + (2n+1)(-1)^n sum_{n < r <= Pi} T_{r n} a~_r^{mm},  mm = +-m;
-            // one lane per (n, sign)
-            int nout = Po - m + 1, nitems = m > 0 ? 2 * nout : nout;
-            for (int it = lane; it < nitems; it += 32) {
-                int n = m + (it % nout);
-                int mm = it < nout ? m : -m;
-                cd sp = {0, 0};
-                int ce = min(n, Pi);
-                const cd* Tr = Tm + n * (Pn + 1);
-                for (int c = m; c <= ce; ++c) sp = cmac(sp, Tr[c], a[nmi(c, mm)]);
-                if (n < Pi) {
-                    cd up = {0, 0};
-                    for (int r = n + 1; r <= Pi; ++r) up = cmac(up, Tm[r * (Pn + 1) + n], wb[nmi(r, mm)]);
-                    double g = (n & 1) ? -(2.0 * n + 1.0) : (2.0 * n + 1.0);
-                    sp += g * up;
-                }
-                bb[nmi(n, mm)] = sp;
-            }
-        }
-        __syncthreads();
-        // (3) back rotation: x = Phi c'; y = D x; x' = S E(1/e_a) y; u = D x'; acc += E(1/e) i^m u
-        // (the flat and operator paths left w+- of Phi c' in bb already)
-        if (ops_g || flat) {
-            d_pass(Dh, A.Dhoff, bb, a, Po, 0, 0, nullptr, Pm, 0);
-        } else {
-            w_pass(A.knm, bb, wb, Po, 1, 0, nullptr, Pm);
-            __syncthreads();
-            d_pass(Dh, A.Dhoff, wb, a, Po, 0, 0, nullptr, Pm, 0);
-        }
-        __syncthreads();
-        w_pass(A.knm, a, wb, Po, 0, 1, pwai, Pm);
-        __syncthreads();
-        if (fr >= 0) {
-            // (4) out of the fixed frame, added to the accumulator
-            d_pass(Dh, A.Dhoff, wb, a, Po, 1, 0, pwei, Pm, 0);
-            __syncthreads();
-            rot_fixed_inv(A, Dh, a, wb, bb, acc, Po, Pm, fr, 1);
-        } else {
-            d_pass(Dh, A.Dhoff, wb, acc, Po, 1, 0, pwei, Pm, 1);
-        }
-    }
-    __syncthreads();
-    if (part) {
-        cd* o = part + (((size_t)zc * nrhs + rhs) * nb + bx) * Ko;
-        for (int k = threadIdx.x; k < Ko; k += blockDim.x) o[k] = acc[k];
-        continue;
-    }
-    cd* o = out + (int64_t)rhs * A.ncoef + A.eoff[b];
-    for (int k = threadIdx.x; k < Ko; k += blockDim.x) {
-        if (mode == 2) o[k] += acc[k];
-        else o[k] = acc[k];
-    }
-    }
-}
-
-// sum of the chunk partials of a chunked M2L launch, in chunk order
-__global__ void k_tr3h_reduce(const cd* __restrict__ part, int nchunk, int nb, int Ko, int lo,
-                              const int64_t* __restrict__ eoff, int64_t ncoef, cd* __restrict__ out) {
-    int bi = blockIdx.x, rhs = blockIdx.y, nr = gridDim.y;
-    cd* o = out + (int64_t)rhs * ncoef + eoff[lo + bi];
-    for (int k = threadIdx.x; k < Ko; k += blockDim.x) {
-        cd s = {0, 0};
-        for (int z = 0; z < nchunk; ++z) s += part[(((size_t)z * nr + rhs) * nb + bi) * Ko + k];
-        o[k] = s;
-    }
-}
-
-// 3D Laplace translations by the same point-and-shoot scheme (Sec. 5.2,
-// Lemma 5.2.4's z-axis forms written for the solid harmonics of fmm3d.cu):
-// with U_n^m = Z_n^m / (eps_m s_n^m), T_n^m = eps_m s_n^m Y_n^m / rho^{n+1},
-// s_n^m = sqrt((n-|m|)! (n+|m|)!), the Y-basis coefficients of a multipole
-// are eps_m s_n^m M_n^m and of a local expansion eps_m L_n^m / s_n^m; the
-// rotations of the Helmholtz kernel act on them. Along the z-axis (new centre
-// at (0, 0, t) from the old, U_k^0(0,0,z) = z^k/k!, T_j^0(0,0,t) = j!/t^{j+1}):
-//   M2M  M'_n^m = sum_k ((-t)^k / k!) M_{n-k}^m
-//   M2L  L_k^m  = (-1)^{k+m} sum_n M_n^m (n+k)! / t^{n+k+1}
-//   L2L  L'_k^m = sum_{n >= k} L_n^m t^{n-k} / (n-k)!
-__global__ void k_tr3l(Tr3hArgs A, int mode, int lo, int P, int d_in_smem, const double* __restrict__ lsm,
-                       const double* __restrict__ lsd, const double* __restrict__ fact,
-                       const double* __restrict__ ifact, const cd* __restrict__ in, cd* __restrict__ out,
-                       int qfirst, const cd* __restrict__ sc, const cd* __restrict__ tt,
-                       const int* __restrict__ fb) {
-    extern __shared__ cd sm[];
-    int b = lo + blockIdx.x;
-    if (mode == 0 && A.leaf[b]) return;
-    int rhs = blockIdx.y;
-    int K = (P + 1) * (P + 1);
-    cd* acc = sm;
-    cd* a = acc + K;
-    cd* bb = a + K;
-    cd* wb = bb + K;
-    cd* g = wb + K;                     // 2P + 2
-    cd* pwe = g + (2 * P + 2);
-    cd* pwa = pwe + (2 * P + 1);
-    cd* pwai = pwa + (2 * P + 1);
-    cd* pwei = pwai + (2 * P + 1);
-    double* Dsm = (double*)(pwei + (2 * P + 1));
-    const double* Dh = A.Dh;
-    if (d_in_smem) {
-        int64_t nd = __ldg(A.Dhoff + P + 1);
-        for (int64_t k = threadIdx.x; k < nd; k += blockDim.x) Dsm[k] = A.Dh[k];
-        Dh = Dsm;
-    }
-    bool in_local = mode == 2, out_local = mode != 0;
-    for (int k = threadIdx.x; k < K; k += blockDim.x) acc[k] = cd{0, 0};
-    int qa, qb;
-    if (mode == 0) {
-        qa = A.cbeg[b];
-        qb = A.cend[b];
-    } else if (mode == 1) {
-        qa = A.loff[b];
-        qb = A.loff[b + 1];
-    } else {
-        qa = 0;
-        qb = 1;
-    }
-    for (int q = qa; q < qb; ++q) {
-        int s = mode == 0 ? q : mode == 1 ? A.lent[q] : A.parent[b];
-        int p = mode == 2 ? b - lo : q - qfirst;
-        __syncthreads();
-        const cd* src = in + (int64_t)rhs * A.ncoef + A.eoff[s];
-        // Y-basis input
-        for (int k = threadIdx.x; k < K; k += blockDim.x) a[k] = (in_local ? __ldg(lsd + k) : __ldg(lsm + k)) * src[k];
-        cd t = tt[p];
-        int w4 = threadIdx.x >> 5, ln = threadIdx.x & 31;
-        if (w4 < 4) {
-            cd x = sc[2 * (size_t)p + (w4 >> 1)];
-            if (w4 & 1) x = cinv(x);
-            cd* dst = (w4 >> 1) ? pwa : pwe;
-            for (int m = ln; m <= P; m += 32) dst[P + ((w4 & 1) ? -m : m)] = cpow_int(x, m);
-        } else if (w4 == 4) {
-            // coaxial factors g[j], j <= 2P+1
-            cd base = mode == 0 ? -t : mode == 1 ? cinv(t) : t;
-            for (int j = ln; j <= 2 * P + 1; j += 32) {
-                cd v = cpow_int(base, mode == 1 ? j + 1 : j);
-                g[j] = (mode == 1 ? __ldg(fact + j) : __ldg(ifact + j)) * v;
-            }
-        }
-        __syncthreads();
-        for (int m = threadIdx.x - P; m <= P; m += blockDim.x) {
-            pwai[P + m] = pwa[P - m];
-            pwei[P + m] = pwe[P - m];
-        }
-        int fr = __ldg(fb + p);
-        if (fr >= 0) rot_fixed(A, Dh, a, wb, bb, P, P, fr);
-        // forward rotation
-        w_pass(A.knm, a, wb, P, 1, 0, pwe, P);
-        __syncthreads();
-        d_pass(Dh, A.Dhoff, wb, bb, P, 0, 0, nullptr, P, 0);
-        __syncthreads();
-        w_pass(A.knm, bb, wb, P, 0, 1, pwa, P);
-        __syncthreads();
-        d_pass(Dh, A.Dhoff, wb, a, P, 1, 0, nullptr, P, 0);
-        __syncthreads();
-        // back to the solid-harmonic basis, z-axis translation, to the Y basis
-        for (int k = threadIdx.x; k < K; k += blockDim.x) a[k] = (in_local ? __ldg(lsm + k) : __ldg(lsd + k)) * a[k];
-        __syncthreads();
-        for (int k = threadIdx.x; k < K; k += blockDim.x) {
-            int n, m;
-            nm_tab(A.knm, k, n, m);
-            int am = m < 0 ? -m : m;
-            cd v = {0, 0};
-            if (mode == 0) {
-                for (int kk = 0; kk <= n - am; ++kk) v = cmac(v, g[kk], a[nmi(n - kk, m)]);
-            } else if (mode == 1) {
-                for (int nn = am; nn <= P; ++nn) v = cmac(v, g[nn + n], a[nmi(nn, m)]);
-                if ((n + m) & 1) v = -v;
-            } else {
-                for (int nn = n; nn <= P; ++nn) v = cmac(v, g[nn - n], a[nmi(nn, m)]);
-            }
-            bb[k] = (out_local ? __ldg(lsd + k) : __ldg(lsm + k)) * v;
-        }
-        __syncthreads();
-        // back rotation, accumulated in the solid-harmonic basis
-        w_pass(A.knm, bb, wb, P, 1, 0, nullptr, P);
-        __syncthreads();
-        d_pass(Dh, A.Dhoff, wb, a, P, 0, 0, nullptr, P, 0);
-        __syncthreads();
-        w_pass(A.knm, a, wb, P, 0, 1, pwai, P);
-        __syncthreads();
-        d_pass(Dh, A.Dhoff, wb, bb, P, 1, 0, pwei, P, 0);
-        __syncthreads();
-        if (fr >= 0) {
-            rot_fixed_inv(A, Dh, bb, wb, a, bb, P, P, fr, 0);
-            __syncthreads();
-        }
-        for (int k = threadIdx.x; k < K; k += blockDim.x) acc[k] += (out_local ? __ldg(lsm + k) : __ldg(lsd + k)) * bb[k];
-    }
-    __syncthreads();
-    cd* o = out + (int64_t)rhs * A.ncoef + A.eoff[b];
-    for (int k = threadIdx.x; k < K; k += blockDim.x) {
-        if (mode == 2) o[k] += acc[k];
-        else o[k] = acc[k];
-    }
-}
-
-// coaxial work arrays of one block (complex entries): sectorial columns and,
-// per warp, three recurrence columns and the lower triangle of T^m
-size_t tr3h_work(int Pi, int Po, int threads = kH3Threads) {
-    int Pn = std::min(Pi, Po), Pm = std::max(Pi, Po), NR = Pi + Po;
-    return (size_t)(Pn + 1) * (NR + 1) +
-           (size_t)(threads / 32) * ((size_t)3 * (NR + 2) + (size_t)(Pm + 1) * (Pn + 1));
-}
-
-size_t tr3h_dh(int P) {
-    size_t nd = 0;
-    for (int n = 0; n <= P; ++n) nd += (size_t)(n + 1) * (n + 1);
-    return nd;
-}
-
-size_t tr3h_smem(int Pi, int Po, bool d_in_smem, bool work_in_smem = true, bool acc_in_smem = true,
-                 bool flat = false) {
-    int Pm = std::max(Pi, Po);
-    size_t Km = (size_t)(Pm + 1) * (Pm + 1), Ko = (size_t)(Po + 1) * (Po + 1);
-    int NR = Pi + Po;
-    size_t work = flat ? (size_t)(Po + 1) * (NR + 1) + tr3h_flat_cols(Po) : tr3h_work(Pi, Po);
-    size_t c = (acc_in_smem ? Ko : 0) + 3 * Km + (NR + 1) + 4 * (2 * Pm + 1) + (work_in_smem ? work : 0);
-    size_t bytes = c * sizeof(cd);
-    if (d_in_smem) bytes += tr3h_dh(Pm) * sizeof(double);
-    return bytes;
-}
-
-// shared memory of k_tr3h_tri: radial sequence, two column buffers per m,
-// triangle offsets
-size_t tri_build_smem(int P) {
-    return sizeof(cd) * ((size_t)(2 * P + 1) + (size_t)2 * (P + 1) * (2 * P + 2)) + sizeof(int) * (size_t)(P + 1);
-}
-
 }  // namespace
 
 // ---------------------------------------------------------------------------
@@ -1993,22 +1132,7 @@ struct Helm3dState {
     std::vector<int64_t> p2m_rtot, p2l_rtot;    // per level: points in the level's launch
     DevBuf<cd> rad;
     H3Tables* tab = nullptr;
-    DevBuf<cd> gscr;             // coaxial work arrays of large-order translations
-    DevBuf<cd> part;             // partial results of chunked M2L launches
-    std::vector<int> l2max;      // longest List 2 per level
-    std::vector<int> l2off;      // host copy of the List-2 offsets
-    DevBuf<int> qbox;            // owner box of each List-2 entry
-    DevBuf<cd> pre_sc, pre_fl;   // per-pair prologue of a translation launch
-    DevBuf<int> pre_fb;          // per pair: fixed frame k, or -1
-    DevBuf<cd> pre_pw;           // per pair: e^m, e_a^m for m in [-Pm, Pm]
-    DevBuf<cd> tri;              // coaxial operators of the M2L pairs of a launch range
-    PairSlots pairs;             // List-2 pairs of the M2L
-    std::vector<int> level_off;
-    int lvl_of_lo(int lo) const {
-        for (size_t l = 0; l + 1 < level_off.size(); ++l)
-            if (level_off[l] == lo) return (int)l;
-        return -1;
-    }
+    PairSlots pairs;             // List-2 pairs, workspaces of the translations
 };
 
 static std::mutex g_mu;
@@ -2070,7 +1194,6 @@ void helm3d_setup(cfmm_plan_s* P) {
     }
     S->l0 = T.l0;
     S->nlev = T.nlevels;
-    S->level_off = T.level_off;
     S->Plev.resize(T.nlevels);
     for (int l = 0; l < T.nlevels; ++l) S->Plev[l] = nterms_helm3d(P->sep, P->eps * 0.01, P->kappa, P->W / (double)(1 << l));
     P->P = S->Plev;
@@ -2094,25 +1217,13 @@ void helm3d_setup(cfmm_plan_s* P) {
     P->ncoef = tot;
     S->exp_off.alloc(T.nboxes);
     CFMM_CUDA(cudaMemcpyAsync(S->exp_off.get(), off.data(), sizeof(int64_t) * T.nboxes, cudaMemcpyHostToDevice, st));
-    std::vector<int> lvl(T.nboxes), l4(T.nboxes + 1), l2(T.nboxes + 1), boxes;
+    std::vector<int> lvl(T.nboxes), l4(T.nboxes + 1), boxes;
     CFMM_CUDA(cudaMemcpyAsync(lvl.data(), T.level.get(), sizeof(int) * T.nboxes, cudaMemcpyDeviceToHost, st));
     CFMM_CUDA(cudaMemcpyAsync(l4.data(), T.loff[3].get(), sizeof(int) * (T.nboxes + 1), cudaMemcpyDeviceToHost, st));
-    CFMM_CUDA(cudaMemcpyAsync(l2.data(), T.loff[1].get(), sizeof(int) * (T.nboxes + 1), cudaMemcpyDeviceToHost, st));
     CFMM_CUDA(cudaStreamSynchronize(st));
-    S->l2max.assign(T.nlevels, 0);
-    for (int b = 0; b < T.nboxes; ++b) S->l2max[lvl[b]] = std::max(S->l2max[lvl[b]], l2[b + 1] - l2[b]);
-    S->l2off = l2;
-    {
-        std::vector<int> qb(std::max(1, l2[T.nboxes]));
-        for (int b = 0; b < T.nboxes; ++b)
-            for (int q = l2[b]; q < l2[b + 1]; ++q) qb[q] = b;
-        S->qbox.alloc(qb.size());
-        CFMM_CUDA(cudaMemcpyAsync(S->qbox.get(), qb.data(), sizeof(int) * qb.size(), cudaMemcpyHostToDevice, st));
-        CFMM_CUDA(cudaStreamSynchronize(st));
-    }
     for (int b : T.leaf_boxes)
         if (lvl[b] >= S->l0) S->leaves_l0.push_back(b);
-    pair_slots_build(P, &S->pairs, l2, S->l0);
+    pair_slots_build(P, &S->pairs, T.hloff[1], S->l0);
     S->d_leaves_l0.alloc(S->leaves_l0.size());
     CFMM_CUDA(cudaMemcpyAsync(S->d_leaves_l0.get(), S->leaves_l0.data(), sizeof(int) * S->leaves_l0.size(),
                               cudaMemcpyHostToDevice, st));
@@ -2170,8 +1281,8 @@ void helm3d_setup(cfmm_plan_s* P) {
         CFMM_CUDA(cudaMemcpyAsync(S->d_p2l_boxes.get(), boxes.data(), sizeof(int) * boxes.size(),
                                   cudaMemcpyHostToDevice, st));
     CFMM_CUDA(cudaStreamSynchronize(st));
-    for (auto f : {(const void*)k_p2x3h, (const void*)k_p2x3h_slp<false>, (const void*)k_eval3h, (const void*)k_tr3h,
-                   (const void*)k_eval3h_grad, (const void*)k_tr3h_tri})
+    for (auto f : {(const void*)k_p2x3h, (const void*)k_p2x3h_slp<false>, (const void*)k_eval3h,
+                   (const void*)k_eval3h_grad})
         CFMM_CUDA(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, kH3Smem));
 }
 
@@ -2267,127 +1378,14 @@ void helm3d_apply(cfmm_plan_s* P, const cd* sigma, const cd* tau, int64_t dstrid
         CFMM_LAUNCHED();
     }
     rec(2);
-    Tr3hArgs TA{T.cen_re.get(), T.cen_im.get(), S->exp_off.get(), S->ncoef, TB->Dh.get(), TB->Dhoff.get(),
-                TB->inv2n1.get(), TB->al.get(), TB->be.get(), TB->ibe.get(), TB->mu.get(), TB->nu.get(),
-                TB->knm.get(), P->kappa, T.cbeg.get(), T.cend.get(),
-                T.loff[1].get(), T.lent[1].get(), T.parent.get(), T.leaf.get(), S->qbox.get()};
-    int nsm = 0;
-    CFMM_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, P->device));
-    auto launch_range = [&](int mode, int lo, int nb, int Pi, int Po, int use_h, const cd* in, cd* out, int nchunk,
-                            int chunk, bool tri) {
-        if (nb <= 0) return;
-        // the flat coaxial work (equal orders, everything in shared memory with
-        // the rotation table) for the translations of the lower levels
-        int flat = (!tri && Pi == Po && Pi <= kTr3FlatMaxP &&
-                    tr3h_smem(Pi, Po, true, true, true, true) <= (size_t)kH3Smem) ? 1 : 0;
-        size_t smem = tri ? tr3h_smem(Pi, Po, true, false) : tr3h_smem(Pi, Po, true, true, true, flat != 0);
-        int dsm = 1;
-        cd* gs = nullptr;
-        if (smem > (size_t)kH3Smem) {
-            smem = tr3h_smem(Pi, Po, false, !tri);
-            dsm = 0;
-        }
-        int64_t nitem = (int64_t)nb * nrhs * nchunk, G = nitem;
-        int accg = 0, threads = kH3Threads;
-        if (!tri && smem > (size_t)kH3Smem) {
-            // coaxial work arrays (and for the largest orders the accumulator)
-            // in global scratch: one slice per resident block, the blocks
-            // stride over the work items
-            smem = tr3h_smem(Pi, Po, false, false);
-            if (smem > (size_t)kH3Smem) {
-                // one block per SM fits: twice the threads keep the FP64 pipe fed
-                smem = tr3h_smem(Pi, Po, false, false, false);
-                accg = 1;
-                threads = 2 * kH3Threads;
-            }
-            int per_sm = 0;
-            CFMM_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_tr3h, threads, smem));
-            G = std::min<int64_t>(nitem, (int64_t)std::max(1, per_sm) * nsm);
-            size_t per = tr3h_work(Pi, Po, threads) + (accg ? (size_t)(Po + 1) * (Po + 1) : 0);
-            S->gscr.alloc(per * (size_t)G);
-            gs = S->gscr.get();
-        }
-        CFMM_REQUIRE(smem <= (size_t)kH3Smem, CFMM_EUNSUPPORTED, "3D Helmholtz translation exceeds shared memory");
-        dim3 g((unsigned)G);
-        size_t Ko = (size_t)(Po + 1) * (Po + 1);
-        cd* pp = nullptr;
-        if (nchunk > 1) {
-            S->part.alloc(Ko * nb * nrhs * nchunk);
-            pp = S->part.get();
-        }
-        // per-pair prologue (shift, rotation scalars, radial sequence)
-        int qfirst, npair;
-        if (mode == 1) {
-            qfirst = S->l2off[lo];
-            npair = S->l2off[lo + nb] - qfirst;
-        } else if (mode == 0) {
-            int l = S->lvl_of_lo(lo);
-            qfirst = T.level_off[l + 1];
-            npair = T.level_off[l + 2] - qfirst;
-        } else {
-            qfirst = lo;
-            npair = nb;
-        }
-        int NR = Pi + Po;
-        S->pre_sc.alloc((size_t)2 * std::max(npair, 1));
-        S->pre_fl.alloc((size_t)(NR + 1) * std::max(npair, 1));
-        S->pre_fb.alloc((size_t)std::max(npair, 1));
-        int Pmx = std::max(Pi, Po);
-        S->pre_pw.alloc((size_t)2 * (2 * Pmx + 1) * std::max(npair, 1));
-        if (npair > 0) {
-            k_tr3h_pre<<<(npair + 127) / 128, 128, 0, st>>>(TA, mode, lo, qfirst, npair, NR, use_h, S->pre_sc.get(),
-                                                           S->pre_fl.get(), S->pre_fb.get(), Pmx, S->pre_pw.get());
-            CFMM_LAUNCHED();
-        }
-        const cd* trig = nullptr;
-        if (tri && npair > 0) {
-            S->tri.alloc(tr3h_tri_size(Pi) * (size_t)npair);
-            k_tr3h_tri<<<npair, kTriThreads, tri_build_smem(Pi), st>>>(TA, Pi, npair, S->pre_fl.get(), S->tri.get());
-            CFMM_LAUNCHED();
-            trig = S->tri.get();
-        }
-        k_tr3h<<<g, threads, smem, st>>>(TA, mode, lo, nb, Pi, Po, use_h, dsm, gs, in, out, chunk, pp,
-                                            qfirst, S->pre_pw.get(), S->pre_fl.get(), nrhs, nchunk, accg, flat,
-                                            S->pre_fb.get(), tri ? 1 : 0, trig);
-        CFMM_LAUNCHED();
-        if (nchunk > 1) {
-            k_tr3h_reduce<<<dim3(nb, nrhs), 256, 0, st>>>(pp, nchunk, nb, (int)Ko, lo, S->exp_off.get(), S->ncoef,
-                                                          out);
-            CFMM_LAUNCHED();
-        }
-    };
-    auto launch_tr = [&](int mode, int lo, int nb, int Pi, int Po, int use_h, const cd* in, cd* out, int nchunk,
-                         int chunk) {
-        // M2L at equal orders up to kTriMaxP (kTriMaxPMulti with several
-        // right-hand sides): the coaxial operators of the level's pairs are
-        // built first by k_tr3h_tri (in HBM, once for every right-hand side),
-        // over box ranges whose operators fit kTriBudget
-        bool tri = mode == 1 && Pi == Po && (Pi <= kTriMaxP || (nrhs > 1 && Pi <= kTriMaxPMulti)) &&
-                   tri_build_smem(Pi) <= (size_t)kH3Smem && tr3h_smem(Pi, Po, false, false) <= (size_t)kH3Smem;
-        if (!tri) {
-            launch_range(mode, lo, nb, Pi, Po, use_h, in, out, nchunk, chunk, false);
-            return;
-        }
-        int64_t cap = std::max<int64_t>(1, (int64_t)(kTriBudget / (tr3h_tri_size(Pi) * sizeof(cd))));
-        for (int b0 = lo; b0 < lo + nb;) {
-            int b1 = b0 + 1;
-            while (b1 < lo + nb && S->l2off[b1 + 1] - S->l2off[b0] <= cap) ++b1;
-            launch_range(mode, b0, b1 - b0, Pi, Po, use_h, in, out, nchunk, chunk, true);
-            b0 = b1;
-        }
-    };
-    // (2) M2M: parents at level l from children at l + 1 (leaf parents get zeros
-    // from an empty child range)
-    for (int l = T.nlevels - 2; l >= S->l0; --l) {
-        int lo = T.level_off[l], nb = T.level_off[l + 1] - lo;
-        launch_tr(0, lo, nb, S->Plev[l + 1], S->Plev[l], 0, mp, mp, 1, 1);
-    }
+    const Tr3Tables tr = tr3_tables(TB);
+    // (2) M2M: parents at level l from children at l + 1
+    for (int l = T.nlevels - 2; l >= S->l0; --l)
+        pairs3d_m2m(P, &S->pairs, tr, l, S->Plev[l + 1], S->Plev[l], P->kappa, S->exp_off.get(), S->ncoef, mp, nrhs);
     rec(3);
     // (4) M2L per level (overwrites L at levels >= l0)
-    for (int l = S->l0; l < T.nlevels; ++l) {
-        m2l3d_launch(P, &S->pairs, tr3_tables(TB), l, l + 1, S->Plev[l], P->kappa, S->exp_off.get(), S->ncoef, mp, lc,
-                     nrhs);
-    }
+    for (int l = S->l0; l < T.nlevels; ++l)
+        pairs3d_m2l(P, &S->pairs, tr, l, l + 1, S->Plev[l], P->kappa, S->exp_off.get(), S->ncoef, mp, lc, nrhs);
     rec(4);
     // (6) P2L, per level
     for (int l = S->l0; l < T.nlevels; ++l) {
@@ -2407,10 +1405,8 @@ void helm3d_apply(cfmm_plan_s* P, const cd* sigma, const cd* tau, int64_t dstrid
     }
     rec(5);
     // (7) L2L
-    for (int l = S->l0 + 1; l < T.nlevels; ++l) {
-        int lo = T.level_off[l], nb = T.level_off[l + 1] - lo;
-        launch_tr(2, lo, nb, S->Plev[l - 1], S->Plev[l], 0, lc, lc, 1, 1);
-    }
+    for (int l = S->l0; l + 1 < T.nlevels; ++l)
+        pairs3d_l2l(P, &S->pairs, tr, l, S->Plev[l], S->Plev[l + 1], P->kappa, S->exp_off.get(), S->ncoef, lc, nrhs);
     rec(6);
     rec(7);
     near_join(P);   // the near field has written u
@@ -2432,39 +1428,22 @@ void helm3d_apply(cfmm_plan_s* P, const cd* sigma, const cd* tau, int64_t dstrid
 }
 
 // ---------------------------------------------------------------------------
-// 3D Laplace translations through k_tr3l (used by fmm3d.cu)
+// 3D Laplace translations (used by fmm3d.cu)
 // ---------------------------------------------------------------------------
 struct Lap3Tr {
     H3Tables* tab = nullptr;
     int Pord = 0;
-    std::vector<int> l2off, level_off;
-    DevBuf<int> qbox;
-    DevBuf<cd> sc, tt;
-    DevBuf<int> fb;
     PairSlots pairs;
 };
 
 Lap3Tr* lap3_tr_create(cfmm_plan_s* P, int Pord) {
     TreeDev& T = P->tree;
-    cudaStream_t st = P->stream;
     Lap3Tr* L = new Lap3Tr();
     L->tab = tables(Pord);
-    L->level_off = T.level_off;
-    L->l2off.resize(T.nboxes + 1);
-    CFMM_CUDA(cudaMemcpyAsync(L->l2off.data(), T.loff[1].get(), sizeof(int) * (T.nboxes + 1), cudaMemcpyDeviceToHost,
-                              st));
-    CFMM_CUDA(cudaStreamSynchronize(st));
-    std::vector<int> qb(std::max(1, L->l2off[T.nboxes]));
-    for (int b = 0; b < T.nboxes; ++b)
-        for (int q = L->l2off[b]; q < L->l2off[b + 1]; ++q) qb[q] = b;
-    L->qbox.alloc(qb.size());
-    CFMM_CUDA(cudaMemcpyAsync(L->qbox.get(), qb.data(), sizeof(int) * qb.size(), cudaMemcpyHostToDevice, st));
-    CFMM_CUDA(cudaStreamSynchronize(st));
-    CFMM_CUDA(cudaFuncSetAttribute((const void*)k_tr3l, cudaFuncAttributeMaxDynamicSharedMemorySize, kH3Smem));
     CFMM_CUDA(cudaFuncSetAttribute((const void*)k_p2x3h_slp<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                    kH3Smem));
     L->Pord = Pord;
-    pair_slots_build(P, &L->pairs, L->l2off, T.l0);
+    pair_slots_build(P, &L->pairs, T.hloff[1], T.l0);
     return L;
 }
 
@@ -2504,51 +1483,15 @@ void lap3_tr_destroy(Lap3Tr* L) { delete L; }
 
 void lap3_m2l(Lap3Tr* L, cfmm_plan_s* P, int l_lo, int l_hi, int Pord, const int64_t* eoff, int64_t ncoef, const cd* mp,
               cd* lc, int nrhs) {
-    m2l3d_launch(P, &L->pairs, tr3_tables(L->tab), l_lo, l_hi, Pord, 0.0, eoff, ncoef, mp, lc, nrhs);
+    pairs3d_m2l(P, &L->pairs, tr3_tables(L->tab), l_lo, l_hi, Pord, 0.0, eoff, ncoef, mp, lc, nrhs);
 }
 
-// mode 0: M2M into the non-leaf boxes of level l from level l+1; 1: M2L at
-// level l (writes L); 2: L2L into level l from level l-1 (adds)
-void lap3_tr_launch(Lap3Tr* L, cfmm_plan_s* P, int mode, int l, int Pord, const int64_t* eoff, int64_t ncoef,
-                    const cd* in, cd* out, int nrhs) {
-    TreeDev& T = P->tree;
-    cudaStream_t st = P->stream;
-    int lo = T.level_off[l], nb = T.level_off[l + 1] - lo;
-    if (nb <= 0) return;
-    H3Tables* TB = L->tab;
-    Tr3hArgs TA{T.cen_re.get(), T.cen_im.get(), eoff, ncoef, TB->Dh.get(), TB->Dhoff.get(),
-                TB->inv2n1.get(), TB->al.get(), TB->be.get(), TB->ibe.get(), TB->mu.get(), TB->nu.get(),
-                TB->knm.get(), 0.0, T.cbeg.get(), T.cend.get(), T.loff[1].get(), T.lent[1].get(), T.parent.get(),
-                T.leaf.get(), L->qbox.get()};
-    int qfirst, npair;
-    if (mode == 1) {
-        qfirst = L->l2off[lo];
-        npair = L->l2off[lo + nb] - qfirst;
-    } else if (mode == 0) {
-        qfirst = T.level_off[l + 1];
-        npair = T.level_off[l + 2] - qfirst;
-    } else {
-        qfirst = lo;
-        npair = nb;
-    }
-    L->sc.alloc((size_t)2 * std::max(npair, 1));
-    L->tt.alloc((size_t)std::max(npair, 1));
-    L->fb.alloc((size_t)std::max(npair, 1));
-    if (npair > 0) {
-        k_tr3h_pre<<<(npair + 127) / 128, 128, 0, st>>>(TA, mode, lo, qfirst, npair, -1, 0, L->sc.get(), L->tt.get(),
-                                                       L->fb.get(), 0, nullptr);
-        CFMM_LAUNCHED();
-    }
-    size_t K = (size_t)(Pord + 1) * (Pord + 1);
-    size_t smem = sizeof(cd) * (4 * K + (2 * Pord + 2) + 4 * (2 * Pord + 1));
-    size_t nd = tr3h_dh(Pord) * sizeof(double);
-    int dsm = smem + nd <= (size_t)kH3Smem;
-    if (dsm) smem += nd;
-    CFMM_REQUIRE(smem <= (size_t)kH3Smem, CFMM_EUNSUPPORTED, "3D Laplace translation exceeds shared memory");
-    dim3 g(nb, nrhs);
-    k_tr3l<<<g, kH3Threads, smem, st>>>(TA, mode, lo, Pord, dsm, TB->lsm.get(), TB->lsd.get(), TB->fact.get(),
-                                        TB->ifact.get(), in, out, qfirst, L->sc.get(), L->tt.get(), L->fb.get());
-    CFMM_LAUNCHED();
+void lap3_m2m(Lap3Tr* L, cfmm_plan_s* P, int l, int Pord, const int64_t* eoff, int64_t ncoef, cd* mp, int nrhs) {
+    pairs3d_m2m(P, &L->pairs, tr3_tables(L->tab), l, Pord, Pord, 0.0, eoff, ncoef, mp, nrhs);
+}
+
+void lap3_l2l(Lap3Tr* L, cfmm_plan_s* P, int l, int Pord, const int64_t* eoff, int64_t ncoef, cd* lc, int nrhs) {
+    pairs3d_l2l(P, &L->pairs, tr3_tables(L->tab), l, Pord, Pord, 0.0, eoff, ncoef, lc, nrhs);
 }
 
 }  // namespace cfmm

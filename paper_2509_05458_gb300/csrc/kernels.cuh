@@ -97,8 +97,7 @@ void helm3d_apply(cfmm_plan_s* P, const cd* sigma, const cd* tau, int64_t dens_s
 int nterms_helm3d(int k, double eps, double kappa, double w);
 // 3D Laplace point-and-shoot translations (helm3d.cu, used by fmm3d.cu)
 // largest 3D Helmholtz expansion order: the limit of the translation tables
-// (the translation kernel keeps 3 (P+1)^2 + 10 P + 5 complex values in shared
-// memory, the rest in global scratch, which fits up to here)
+// (pairs3d.cu keeps 3 (2P+2) rows of 512 bytes in shared memory, which fits up to here)
 constexpr int kMaxP3Top = 63;
 struct Lap3Tr;
 Lap3Tr* lap3_tr_create(cfmm_plan_s* P, int Pord);
@@ -107,8 +106,9 @@ void lap3_tr_destroy(Lap3Tr* L);
 // the order does not fit the kernel (the caller then uses the general P2M)
 bool lap3_p2m_slp(Lap3Tr* L, cfmm_plan_s* P, const int* leaves, int cnt, int maxP, const int* dPlev,
                   const int64_t* eoff, int64_t ncoef, const cd* sigma, int64_t dstride, cd* out, int nrhs);
-void lap3_tr_launch(Lap3Tr* L, cfmm_plan_s* P, int mode, int l, int Pord, const int64_t* eoff, int64_t ncoef,
-                    const cd* in, cd* out, int nrhs);
+// M2M into the non-leaf boxes of level l from level l + 1; L2L from level l, added to level l + 1
+void lap3_m2m(Lap3Tr* L, cfmm_plan_s* P, int l, int Pord, const int64_t* eoff, int64_t ncoef, cd* mp, int nrhs);
+void lap3_l2l(Lap3Tr* L, cfmm_plan_s* P, int l, int Pord, const int64_t* eoff, int64_t ncoef, cd* lc, int nrhs);
 // M2L of levels [l_lo, l_hi) (overwrites their local expansions)
 void lap3_m2l(Lap3Tr* L, cfmm_plan_s* P, int l_lo, int l_hi, int Pord, const int64_t* eoff, int64_t ncoef, const cd* mp,
               cd* lc, int nrhs);
