@@ -1,0 +1,413 @@
+// FP64 evaluation of 3D expansions at points: M2P over List 3 and L2P, potential
+// and target gradient, Laplace and Helmholtz.
+//
+// The expansion functions (file comments of fmm3d.cu and helm3d.cu) share their
+// dependence on z and rho^2 between +m and -m:
+//   H_n^{+-m}(x) = F_n xi_{+-}^m q_n^m,  q_m^m = D_m,  q_n^m = A_n^m (zeta q_{n-1}^m) - B_n^m (w q_{n-2}^m),
+//   Helmholtz      zeta = z, w = rho^2, xi+- = x+-,            F_n = f_n(kappa rho)/rho^n  (q from Z)
+//   Laplace L2P    zeta = z, w = rho^2, xi+ = x+, xi- = -x-,   F_n = 1                     (q from U)
+//   Laplace M2P    the same over rho^2, w = 1/rho^2,           F_n = 1/rho                 (q from T)
+// so sum c_n^{+-m} H_n^{+-m} = sum_m xi+^m (sum_n F_n q_n c_n^m) + xi-^m (sum_n F_n q_n
+// c_n^{-m}): 24 FP64 instructions per (n, m >= 0) for both signs instead of 20 for
+// each, which is what bounds it (the FP64 pipe).
+//
+// A warp evaluates one expansion (a leaf's own, or one List-3 entry) at up to 32
+// targets of a leaf. Fewer targets leave room for groups of lanes that take every
+// G-th m each (a shell of leaves of one or two points has most List-3 entries of a
+// small surface: 2.4 of 32 lanes were in use with a thread per target and a block
+// per leaf, and the entries of a leaf ran one after the other). Each result goes to
+// its own slot and k_eval3_sum adds a target's slots in list order.
+#include <algorithm>
+#include <cmath>
+
+#include "cfmm_special.cuh"
+#include "eval3d.cuh"
+
+namespace cfmm {
+
+namespace {
+
+__host__ __device__ __forceinline__ int nmi(int n, int m) { return n * n + n + m; }
+
+__device__ __forceinline__ cd ldc(const cd* p) {
+    double2 v = __ldg(reinterpret_cast<const double2*>(p));
+    return cd{v.x, v.y};
+}
+
+constexpr int kEvalWarps = 4;
+constexpr int64_t kEvalItems = (int64_t)1 << 27;   // slots of a launch over all right-hand sides, about
+
+struct EvalK {
+    const double *xr, *xi;
+    int64_t n;
+    Eval3Args E;
+    const int *tst, *ten, *l3off, *l3, *blevel;
+    const double *cre, *cim;
+    const int64_t* ioff;
+    const int* own;
+    int64_t nslot;                // slots per right-hand side (and component): n for L2P, then the items
+    int l2p;                      // 0: List 3 only
+    Eval3Tables T;
+    const cd* gco;                // Helmholtz gradient: derived coefficients [3][2][ncoef] (multipole, local)
+    cd* val;                      // [rhs][1 or 3][nslot]
+    int nleaf_tasks, ntask;
+};
+
+// F_n = f_n(kappa rho)/rho^n, n = 0..N, of one lane into rows F[32 n]: h by forward
+// recurrence, j by Miller's (both as in cfmm_special.cuh; the overflow test reads the
+// exponent bits)
+__device__ void radial_rows(bool sing, double kappa, cd r2, int N, cd* F) {
+    cd rho = csqrt_p(r2);
+    if (rho.x == 0.0 && rho.y == 0.0) {
+        double v = 1.0;
+        for (int n = 0; n <= N; ++n) {
+            F[n * 32] = cd{v, 0};
+            v *= kappa / (2.0 * n + 3.0);
+        }
+        return;
+    }
+    cd z = kappa * rho, ir = cinv(rho), p = {1, 0};
+    if (sing) {
+        cd e = cexp_i(z), zi = cinv(z);
+        cd h0 = -mul_i(e * zi), h1 = -(e * (z + cd{0.0, 1.0})) * (zi * zi);
+        double c = 3.0;
+        for (int n = 0; n <= N; ++n, c += 2.0) {
+            F[n * 32] = h0 * p;
+            p = p * ir;
+            cd h2 = rmac(-h0, c, zi * h1);
+            h0 = h1;
+            h1 = h2;
+        }
+        return;
+    }
+    double az = hypot(z.x, z.y);
+    double big = az > (double)N ? az : (double)N;
+    int N0 = az <= 2.0 ? N + 13 + (int)(4.0 * az) : (int)big + 24 + (int)sqrt(32.0 * big);
+    bool up = z.y >= 0.0;
+    cd zi = cinv(z), fp = {0.0, 0.0}, f = {1e-200, 0.0}, S = {0.0, 0.0};
+    double c2 = 2.0 * N0 + 1.0;
+    for (int n = N0; n >= 1; --n, c2 -= 2.0) {
+        if (n <= N) F[n * 32] = f;
+        // (-+i)^n f
+        int r = up ? n & 3 : (4 - n) & 3;
+        cd w = r == 0 ? f : r == 1 ? cd{f.y, -f.x} : r == 2 ? -f : cd{-f.y, f.x};
+        S = rmac(S, c2, w);
+        cd fm = rmac(-fp, c2, zi * f);
+        fp = f;
+        f = fm;
+        // |f| beyond 2^500: everything so far is scaled down
+        unsigned hx = (unsigned)__double2hiint(f.x) & 0x7fffffffu, hy = (unsigned)__double2hiint(f.y) & 0x7fffffffu;
+        if (max(hx, hy) >= 0x5f300000u) {
+            const double sc = 3.0549363634996047e-151;     // 2^-500
+            f = sc * f;
+            fp = sc * fp;
+            S = sc * S;
+            for (int m = n; m <= min(N, N0); ++m) F[m * 32] = sc * F[m * 32];
+        }
+    }
+    F[0] = f;
+    S += f;
+    cd s = (up ? cexp_i(-z) : cexp_i(z)) / S;
+    for (int n = 0; n <= N; ++n) {
+        F[n * 32] = F[n * 32] * s;
+        s = s * ir;
+    }
+}
+
+// Columns m = g, g + G, .. of the sums of one target. POT: u = sum c H. GRAD, Laplace:
+// dz, dp, dm from the shifted coefficients (d+ U_n^m = -U_{n-1}^{m-1}/2 etc.), order
+// Q = P - 1 (L2P) or P + 1 (M2P); Helmholtz: dz, dp, dm, b of eval with F_{n+1} from
+// the derived coefficients (k_grad_coef).
+template <bool LAP, bool GRAD>
+__device__ __forceinline__ void eval_columns(const QTables& q, bool sing, cd zeta, cd w, cd xp, cd xm, int P,
+                                             const cd* __restrict__ F, const cd* __restrict__ c,
+                                             const cd* __restrict__ dc, int64_t dstride, int g, int G, cd* out) {
+    constexpr int NS = !GRAD ? 1 : LAP ? 3 : 4;        // sums
+    const int Q = GRAD && LAP ? (sing ? P + 1 : P - 1) : P;
+    cd pp = {1, 0}, pm = {1, 0}, sp = {1, 0}, sm = {1, 0};
+    for (int i = 0; i < G; ++i) {
+        if (i == g) {
+            pp = sp;
+            pm = sm;
+        }
+        sp = sp * xp;
+        sm = sm * xm;
+    }
+    for (int m = g; m <= Q; m += G) {
+        cd a[NS], b[NS];
+#pragma unroll
+        for (int k = 0; k < NS; ++k) a[k] = b[k] = cd{0, 0};
+        cd q2 = {0, 0}, q1 = {__ldg(q.D + m), 0};
+        for (int n = m; n <= Q; ++n) {
+            if (GRAD && LAP) {
+                // H_n^{+-m} meets c_k^{+-m}, c_k^{+-m+1}, c_k^{+-m-1} with k = n + 1 (L2P) or n - 1
+                const int k = sing ? n - 1 : n + 1;
+                auto at = [&](int mm) -> cd { return k >= 0 && mm <= k && -mm <= k ? ldc(c + nmi(k, mm)) : cd{0, 0}; };
+                a[0] = cmac(a[0], q1, at(m));
+                a[1] = cmac(a[1], q1, at(m + 1));
+                a[2] = cmac(a[2], q1, at(m - 1));
+                b[0] = cmac(b[0], q1, at(-m));
+                b[1] = cmac(b[1], q1, at(-m + 1));
+                b[2] = cmac(b[2], q1, at(-m - 1));
+            } else if (GRAD) {
+                cd t = F[(n + 1) * 32] * q1;
+#pragma unroll
+                for (int k = 0; k < 3; ++k) {
+                    a[k] = cmac(a[k], t, ldc(dc + k * dstride + nmi(n, m)));
+                    b[k] = cmac(b[k], t, ldc(dc + k * dstride + nmi(n, -m)));
+                }
+                a[3] = cmac(a[3], t, ldc(c + nmi(n, m)));
+                b[3] = cmac(b[3], t, ldc(c + nmi(n, -m)));
+            } else {
+                cd t = LAP ? q1 : F[n * 32] * q1;
+                a[0] = cmac(a[0], t, ldc(c + nmi(n, m)));
+                b[0] = cmac(b[0], t, ldc(c + nmi(n, -m)));
+            }
+            if (n == Q) break;
+            double A = __ldg(q.A + nmi(n + 1, m)), B = __ldg(q.B + nmi(n + 1, m));
+            cd v = rmac(A * (zeta * q1), -B, w * q2);
+            q2 = q1;
+            q1 = v;
+        }
+#pragma unroll
+        for (int k = 0; k < NS; ++k) {
+            out[k] = cmac(out[k], pp, a[k]);
+            if (m > 0) out[k] = cmac(out[k], pm, b[k]);
+        }
+        pp = pp * sp;
+        pm = pm * sm;
+    }
+}
+
+// One warp per (task, 32 targets): tasks are the leaves (L2P) and then the List-3
+// entries. Grid (tasks / warps, target groups, rhs).
+template <bool LAP, bool GRAD>
+__global__ void __launch_bounds__(kEvalWarps * 32) k_eval3_items(EvalK A) {
+    extern __shared__ cd sm[];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, rhs = blockIdx.z;
+    const int task = blockIdx.x * kEvalWarps + wid;
+    if (task >= A.ntask) return;
+    const bool sing = task >= A.nleaf_tasks;
+    int b, s, li;
+    int64_t slot;
+    if (!sing) {
+        li = task;
+        b = s = A.E.leaves[li];
+        slot = A.tst[b];
+    } else {
+        const int e = task - A.nleaf_tasks;
+        li = A.own[e];
+        b = A.E.leaves[li];
+        s = A.l3[e];
+        slot = A.n + A.ioff[li] + (int64_t)(e - A.l3off[b]) * (A.ten[b] - A.tst[b]);
+    }
+    const int P = A.E.Plev[A.blevel[s]], t0 = A.tst[b], cnt = A.ten[b] - t0;
+    const int64_t co = (int64_t)rhs * A.E.ncoef + A.E.eoff[s];
+    const cd* c = (sing ? A.E.mp : A.E.loc) + co;
+    cd* F = sm + (size_t)wid * (A.E.maxP + 2) * 32;
+    const cd cen[3] = {{A.cre[3 * s], A.cim[3 * s]}, {A.cre[3 * s + 1], A.cim[3 * s + 1]},
+                       {A.cre[3 * s + 2], A.cim[3 * s + 2]}};
+    for (int k0 = blockIdx.y * 32; k0 < cnt; k0 += gridDim.y * 32) {
+        const int nt = min(32, cnt - k0), G = min(32 / nt, P + 1), g = lane / nt, t = lane - g * nt;
+        const bool on = g < G;
+        const int64_t i = t0 + k0 + t;
+        cd x[3];
+#pragma unroll
+        for (int a = 0; a < 3; ++a) x[a] = cd{A.xr[a * A.n + i], A.xi[a * A.n + i]} - cen[a];
+        cd xp = x[0] + mul_i(x[1]), xm = x[0] - mul_i(x[1]), zeta = x[2];
+        cd w = xp * xm + zeta * zeta, ir = {1, 0};
+        if (LAP) {
+            xm = -xm;
+            if (sing) {
+                ir = cinv(csqrt_p(w));
+                w = cinv(w);
+                xp = xp * w;
+                xm = xm * w;
+                zeta = zeta * w;
+            }
+        } else {
+            __syncwarp();
+            if (g == 0) radial_rows(sing, A.E.kappa, w, GRAD ? P + 1 : P, F + t);
+            __syncwarp();
+        }
+        constexpr int NS = !GRAD ? 1 : LAP ? 3 : 4;
+        cd o[NS];
+#pragma unroll
+        for (int k = 0; k < NS; ++k) o[k] = cd{0, 0};
+        if (on)
+            eval_columns<LAP, GRAD>(LAP ? (sing ? A.T.T : A.T.U) : A.T.Z, sing, zeta, w, xp, xm, P, F + t, c,
+                                    GRAD && !LAP ? A.gco + (sing ? 0 : A.E.ncoef) + (int64_t)rhs * 6 * A.E.ncoef + A.E.eoff[s]
+                                                 : nullptr,
+                                    2 * A.E.ncoef, g, G, o);
+        // the groups' sums in order
+#pragma unroll
+        for (int k = 0; k < NS; ++k) {
+            cd sum = o[k];
+            for (int j = 1; j < G; ++j) {
+                double px = __shfl_sync(0xffffffffu, o[k].x, min(31, t + j * nt));
+                double py = __shfl_sync(0xffffffffu, o[k].y, min(31, t + j * nt));
+                sum += cd{px, py};
+            }
+            o[k] = sum;
+        }
+        if (lane >= nt) continue;
+        cd* v = A.val + (int64_t)rhs * (GRAD ? 3 : 1) * A.nslot + slot + k0 + t;
+        if (!GRAD) {
+            v[0] = LAP ? ir * o[0] : o[0];
+        } else if (LAP) {
+            // dz U_n = U_{n-1}, d+ U_n^m = -U_{n-1}^{m-1}/2, d- U_n^m = U_{n-1}^{m+1}/2; dz T has the other sign
+            cd dz = ir * o[0], dp = -0.5 * (ir * o[1]), dm = 0.5 * (ir * o[2]);
+            v[0] = dp + dm;
+            v[A.nslot] = mul_i(dp - dm);
+            v[2 * A.nslot] = sing ? -dz : dz;
+        } else {
+            const double k = A.E.kappa;
+            v[0] = o[1] + o[2] - k * (x[0] * o[3]);
+            v[A.nslot] = mul_i(o[1] - o[2]) - k * (x[1] * o[3]);
+            v[2 * A.nslot] = o[0] - k * (x[2] * o[3]);
+        }
+    }
+}
+
+// Derived coefficients of the Helmholtz gradient, one block per box of [lo, lo + grid):
+// dz_n^m = g3(n+1,m) c_{n+1}^m, dp_n^m = -gp(n+1,m+1) c_{n+1}^{m+1}, dm_n^m =
+// gm(n+1,m-1) c_{n+1}^{m-1} (0 for n = P), for the multipole (x) and local expansion;
+// out [rhs][3][2][ncoef]
+__global__ void k_grad_coef(EvalK A, int lo, cd* __restrict__ out) {
+    const int b = lo + blockIdx.x, rhs = blockIdx.y, kind = blockIdx.z, P = A.E.Plev[A.blevel[b]];
+    const cd* c = (kind ? A.E.loc : A.E.mp) + (int64_t)rhs * A.E.ncoef + A.E.eoff[b];
+    cd* o = out + (int64_t)rhs * 6 * A.E.ncoef + kind * A.E.ncoef + A.E.eoff[b];
+    const int64_t st = 2 * A.E.ncoef;
+    for (int k = threadIdx.x; k < (P + 1) * (P + 1); k += blockDim.x) {
+        int n = (int)sqrtf((float)k);
+        while (n * n > k) --n;
+        while ((n + 1) * (n + 1) <= k) ++n;
+        const int m = k - n * n - n, n1 = n + 1;
+        const bool in = n1 <= P;
+        auto at = [&](const double* f, int mm) -> cd {
+            return in && mm <= n1 && -mm <= n1 ? __ldg(f + nmi(n1, mm)) * c[nmi(n1, mm)] : cd{0, 0};
+        };
+        o[k] = at(A.T.g3, m);
+        o[st + k] = -at(A.T.gp, m + 1);
+        o[2 * st + k] = at(A.T.gm, m - 1);
+    }
+}
+
+__global__ void k_eval3_own(int nleaf, const int* __restrict__ leaves, const int* __restrict__ l3off,
+                            int* __restrict__ own) {
+    int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= nleaf) return;
+    int b = leaves[i];
+    for (int e = l3off[b]; e < l3off[b + 1]; ++e) own[e] = i;
+}
+
+// u [rhs][comp][n] += the slots of each target: L2P and its leaf's List 3 in order
+__global__ void k_eval3_sum(EvalK A, int ncomp, cd* __restrict__ u) {
+    const int li = blockIdx.x, row = blockIdx.y, b = A.E.leaves[li];
+    const int t0 = A.tst[b], cnt = A.ten[b] - t0, ne = A.l3off[b + 1] - A.l3off[b];
+    if (!A.l2p && ne == 0) return;
+    const cd* v = A.val + (int64_t)row * A.nslot;
+    const int64_t first = A.n + A.ioff[li];
+    for (int t = threadIdx.x; t < cnt; t += blockDim.x) {
+        cd s = A.l2p ? v[t0 + t] : cd{0, 0};
+        for (int e = 0; e < ne; ++e) s += v[first + (int64_t)e * cnt + t];
+        u[(int64_t)row * A.n + t0 + t] += s;
+    }
+}
+
+template <bool LAP, bool GRAD>
+void launch_items(EvalK A, cudaStream_t st, int nrhs, int groups) {
+    const size_t smem = LAP ? 0 : sizeof(cd) * kEvalWarps * (size_t)(A.E.maxP + 2) * 32;
+    if (smem > 48 * 1024)
+        CFMM_CUDA(cudaFuncSetAttribute((const void*)k_eval3_items<LAP, GRAD>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       (int)smem));
+    if (A.ntask <= 0) return;
+    dim3 g((unsigned)((A.ntask + kEvalWarps - 1) / kEvalWarps), groups, nrhs);
+    k_eval3_items<LAP, GRAD><<<g, kEvalWarps * 32, smem, st>>>(A);
+    CFMM_LAUNCHED();
+}
+
+}  // namespace
+
+void eval3_qtable(int kind, int N, double* A, double* B, double* D) {
+    double d = 1.0;
+    for (int m = 0; m <= N; ++m) {
+        if (m > 0) d *= kind == 0 ? -std::sqrt((2.0 * m - 1.0) / (2.0 * m)) : kind == 1 ? -0.5 / m : -(2.0 * m - 1.0);
+        D[m] = d;
+        for (int n = m; n <= N; ++n) {
+            double& a = A[nmi(n, m)];
+            double& b = B[nmi(n, m)];
+            a = b = 0.0;
+            if (n == m) continue;
+            double nn = (double)(n - m) * (n + m);
+            a = kind == 0 ? (2.0 * n - 1.0) / std::sqrt(nn) : kind == 1 ? (2.0 * n - 1.0) / nn : 2.0 * n - 1.0;
+            if (n >= m + 2)
+                b = kind == 0 ? std::sqrt((double)(n - m - 1) * (n + m - 1) / nn) : kind == 1 ? 1.0 / nn
+                                                                                   : (double)(n - 1) * (n - 1) - (double)m * m;
+        }
+    }
+}
+
+void eval3_build(Eval3* E, const std::vector<int>& leaves, const std::vector<int>& l3off, const std::vector<int>& st,
+                 const std::vector<int>& en, const int* d_leaves, const int* d_l3off, cudaStream_t stream) {
+    std::vector<int64_t> off(leaves.size() + 1, 0);
+    for (size_t i = 0; i < leaves.size(); ++i) {
+        int b = leaves[i];
+        off[i + 1] = off[i] + (int64_t)(l3off[b + 1] - l3off[b]) * (en[b] - st[b]);
+    }
+    E->total = off.back();
+    E->ioff.alloc(off.size());
+    upload(E->ioff.get(), off.data(), sizeof(int64_t) * off.size(), stream);
+    if (l3off.back() == 0) return;
+    E->own.alloc(l3off.back());
+    k_eval3_own<<<((int)leaves.size() + 127) / 128, 128, 0, stream>>>((int)leaves.size(), d_leaves, d_l3off, E->own.get());
+    CFMM_LAUNCHED();
+}
+
+void eval3_apply(cfmm_plan_s* P, Eval3* E, const Eval3Tables& T, const Eval3Args& A, bool l2p, cd* u, cd* g, int nrhs) {
+    TreeDev& Tr = P->tree;
+    cudaStream_t st = P->stream;
+    if (A.nleaf == 0) return;
+    const bool lap = A.kappa == 0.0;
+    const int nl3 = Tr.hloff[2].back();
+    EvalK K{P->xr.get(), P->xi.get(), P->n, A, Tr.start.get(), Tr.end.get(), Tr.loff[2].get(), Tr.lent[2].get(),
+            Tr.level.get(), Tr.cen_re.get(), Tr.cen_im.get(), E->ioff.get(), E->own.get(), P->n + E->total, 0, T, nullptr, nullptr, 0, 0};
+    const int groups = std::max(1, std::min(64, (P->leaf_size + 31) / 32));
+    // right-hand sides whose slots fit
+    const int ncomp = g ? 3 : 1;
+    const int batch = (int)std::max<int64_t>(1, std::min<int64_t>(nrhs, kEvalItems / (K.nslot * ncomp)));
+    E->val.alloc((size_t)batch * ncomp * K.nslot);
+    if (g && !lap) E->gco.alloc((size_t)6 * A.ncoef * batch);
+    K.val = E->val.get();
+    for (int r = 0; r < nrhs; r += batch) {
+        const int nr = std::min(batch, nrhs - r);
+        K.E.mp = A.mp + (int64_t)r * A.ncoef;
+        K.E.loc = A.loc + (int64_t)r * A.ncoef;
+        if (u && (l2p || nl3 > 0)) {
+            K.l2p = l2p ? 1 : 0;
+            K.nleaf_tasks = l2p ? A.nleaf : 0;
+            K.ntask = K.nleaf_tasks + nl3;
+            if (lap) launch_items<true, false>(K, st, nr, groups);
+            else launch_items<false, false>(K, st, nr, groups);
+            k_eval3_sum<<<dim3(A.nleaf, nr), 64, 0, st>>>(K, 1, u + (int64_t)r * P->n);
+            CFMM_LAUNCHED();
+        }
+        if (!g) continue;
+        K.l2p = 1;
+        K.nleaf_tasks = A.nleaf;
+        K.ntask = K.nleaf_tasks + nl3;
+        if (lap) {
+            launch_items<true, true>(K, st, nr, groups);
+        } else {
+            const int lo = Tr.level_off[Tr.l0];
+            k_grad_coef<<<dim3(Tr.nboxes - lo, nr, 2), 128, 0, st>>>(K, lo, E->gco.get());
+            CFMM_LAUNCHED();
+            K.gco = E->gco.get();
+            launch_items<false, true>(K, st, nr, groups);
+        }
+        k_eval3_sum<<<dim3(A.nleaf, 3 * nr), 64, 0, st>>>(K, 3, g + (int64_t)r * 3 * P->n);
+        CFMM_LAUNCHED();
+    }
+}
+
+}  // namespace cfmm

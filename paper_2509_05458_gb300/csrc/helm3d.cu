@@ -55,6 +55,7 @@
 #include <mutex>
 
 #include "cfmm_special.cuh"
+#include "eval3d.cuh"
 #include "kernels.cuh"
 #include "pairs3d.cuh"
 
@@ -84,6 +85,7 @@ struct H3Tables {
     DevBuf<int> knm;         // k -> n * 256 + (m + 128), k < (Pmax+1)^2
     DevBuf<double> lsm, lsd; // eps_m s_n^m and eps_m / s_n^m, s = sqrt((n-|m|)! (n+|m|)!)
     DevBuf<double> fact, ifact;  // j! and 1/j!, j <= 2 Pmax + 2
+    DevBuf<double> q[3][3];  // A, B, D of Z, U, T (eval3d.cuh), orders <= Pmax + 2
     DevBuf<float> zAf, zBf, dgf, s21f;   // FP32 copies of zA, zB, dg, s21 (mixed-precision L2P)
 };
 
@@ -194,6 +196,11 @@ static Tr3Tables tr3_tables(const H3Tables* T) {
                      T->smu.get(), T->snu.get(), T->lsm.get(), T->lsd.get(), T->fact.get(), T->ifact.get()};
 }
 
+static Eval3Tables eval3_tables(const H3Tables* T) {
+    auto q = [&](int k) { return QTables{T->q[k][0].get(), T->q[k][1].get(), T->q[k][2].get()}; };
+    return Eval3Tables{q(0), q(1), q(2), T->g3.get(), T->gp.get(), T->gm.get()};
+}
+
 static H3Tables* tables(int P) {
     int dev = 0;
     CFMM_CUDA(cudaGetDevice(&dev));
@@ -293,6 +300,14 @@ static H3Tables* tables(int P) {
         up(T->ifact, fi);
         up(T->lsm, lm);
         up(T->lsd, ld);
+    }
+    for (int kind = 0; kind < 3; ++kind) {
+        int N = Pm + 2;
+        std::vector<double> A((size_t)(N + 1) * (N + 1), 0.0), B = A, Dq(N + 1, 0.0);
+        eval3_qtable(kind, N, A.data(), B.data(), Dq.data());
+        up(T->q[kind][0], A);
+        up(T->q[kind][1], B);
+        up(T->q[kind][2], Dq);
     }
     T->knm.alloc(knm.size());
     CFMM_CUDA(cudaMemcpy(T->knm.get(), knm.data(), sizeof(int) * knm.size(), cudaMemcpyHostToDevice));
@@ -640,189 +655,6 @@ __global__ void k_p2x3h_slp(Exp3hArgs A, const int* __restrict__ boxes, const in
     }
 }
 
-// Sum over n, m of coef_n^m F[n] Z_n^m(x) with Z generated column by column.
-__device__ cd eval_wave(ZCoef zc, cd a0, cd a1, cd a2, int P, const cd* F, const cd* coef) {
-    cd xp = a0 + mul_i(a1), xm = a0 - mul_i(a1), z = a2;
-    cd r2 = xp * xm + z * z;
-    cd acc = {0, 0};
-    for (int sgn = 0; sgn < 2; ++sgn) {
-        cd xs = sgn ? xm : xp;
-        cd d = {1, 0};
-        for (int m = 0; m <= P; ++m) {
-            if (m > 0) d = (-__ldg(zc.dg + m)) * (xs * d);
-            if (sgn == 1 && m == 0) continue;
-            int mi = sgn ? -m : m;
-            acc = cmac(acc, F[m], d * coef[nmi(m, mi)]);
-            if (m + 1 > P) continue;
-            cd p2 = d, p1 = __ldg(zc.s21 + m) * (z * d);
-            acc = cmac(acc, F[m + 1], p1 * coef[nmi(m + 1, mi)]);
-            for (int n = m + 2; n <= P; ++n) {
-                int k = nmi(n, m);
-                cd cur = zc.A[k] * (z * p1) - zc.B[k] * (r2 * p2);
-                acc = cmac(acc, F[n], cur * coef[nmi(n, mi)]);
-                p2 = p1;
-                p1 = cur;
-            }
-        }
-    }
-    return acc;
-}
-
-// Target gradient of sum c_n^m F_n Z_n^m (F_n = f_n(k rho)/rho^n, f = j or h):
-// grad(F_n Z) = F_n grad Z - k F_{n+1} Z x with dz Z_n^m = g3 Z_{n-1}^m,
-// d+ Z_n^m = -gp Z_{n-1}^{m-1}, d- Z_n^m = gm Z_{n-1}^{m+1} (the tables g3, gp,
-// gm of the double layer), so in one pass over Z_{n'}^{m'}, n' <= P (F given
-// for n <= P + 1):
-//   Dz = sum g3(n'+1, m') c_{n'+1}^{m'} F_{n'+1} Z,  D+ = sum -gp(n'+1, m'+1)
-//   c_{n'+1}^{m'+1} F_{n'+1} Z,  D- = sum gm(n'+1, m'-1) c_{n'+1}^{m'-1} F_{n'+1} Z,
-//   B = sum c_{n'}^{m'} F_{n'+1} Z;
-// grad = (D+ + D- - k x1 B, i (D+ - D-) - k x2 B, Dz - k x3 B).
-__device__ void eval_wave_grad(ZCoef zc, cd a0, cd a1, cd a2, int P, const cd* F, const cd* coef, cd& Dz, cd& Dp,
-                               cd& Dm, cd& B) {
-    cd xp = a0 + mul_i(a1), xm = a0 - mul_i(a1), z = a2;
-    cd r2 = xp * xm + z * z;
-    auto c = [&](int n, int m) -> cd {
-        if (n > P || m > n || -m > n) return cd{0, 0};
-        return coef[nmi(n, m)];
-    };
-    Dz = Dp = Dm = B = cd{0, 0};
-    auto add = [&](int n, int mi, cd zv) {
-        cd t = F[n + 1] * zv;
-        B = cmac(B, t, coef[nmi(n, mi)]);
-        if (n + 1 > P) return;
-        int k1 = n + 1;
-        Dz = cmac(Dz, t, __ldg(zc.g3 + nmi(k1, mi)) * c(k1, mi));
-        if (mi + 1 <= k1) Dp = cmac(Dp, t, (-__ldg(zc.gp + nmi(k1, mi + 1))) * c(k1, mi + 1));
-        if (mi - 1 >= -k1) Dm = cmac(Dm, t, __ldg(zc.gm + nmi(k1, mi - 1)) * c(k1, mi - 1));
-    };
-    for (int sgn = 0; sgn < 2; ++sgn) {
-        cd xs = sgn ? xm : xp;
-        cd d = {1, 0};
-        for (int m = 0; m <= P; ++m) {
-            if (m > 0) d = (-__ldg(zc.dg + m)) * (xs * d);
-            if (sgn == 1 && m == 0) continue;
-            int mi = sgn ? -m : m;
-            add(m, mi, d);
-            if (m + 1 > P) continue;
-            cd p2 = d, p1 = __ldg(zc.s21 + m) * (z * d);
-            add(m + 1, mi, p1);
-            for (int n = m + 2; n <= P; ++n) {
-                int k = nmi(n, m);
-                cd cur = zc.A[k] * (z * p1) - zc.B[k] * (r2 * p2);
-                add(n, mi, cur);
-                p2 = p1;
-                p1 = cur;
-            }
-        }
-    }
-}
-
-// target gradients of M2P (List 3, S waves) and L2P (R waves), FP64, added to
-// g [rhs][3][n]
-__global__ void k_eval3h_grad(Exp3hArgs A, const int* __restrict__ leaves, const int* __restrict__ l3off,
-                              const int* __restrict__ l3, const cd* __restrict__ mp, const cd* __restrict__ loc,
-                              cd* __restrict__ g) {
-    extern __shared__ cd sm[];
-    int b = leaves[blockIdx.x];
-    int rhs = blockIdx.y;
-    int P = A.Plev[A.blevel[b]];
-    int nc = (P + 1) * (P + 1);
-    cd* coef = sm;
-    int s0 = A.bst[b], s1 = A.ben[b];
-    cd F[kH3MaxP + 3];
-    for (int t0 = s0; t0 < s1; t0 += blockDim.x) {
-        int i = t0 + threadIdx.x;
-        bool valid = i < s1;
-        cd x[3] = {{0, 0}, {0, 0}, {0, 0}};
-        if (valid) load3(A.xr, A.xi, A.n, i, x);
-        cd G[3] = {{0, 0}, {0, 0}, {0, 0}};
-        auto accum = [&](const cd* d, int Pq) {
-            cd Dz, Dp, Dm, B;
-            eval_wave_grad(A.zc, d[0], d[1], d[2], Pq, F, coef, Dz, Dp, Dm, B);
-            G[0] += Dp + Dm - A.kappa * (d[0] * B);
-            G[1] += mul_i(Dp - Dm) - A.kappa * (d[1] * B);
-            G[2] += Dz - A.kappa * (d[2] * B);
-        };
-        for (int q = l3off[b]; q < l3off[b + 1]; ++q) {
-            int s = l3[q];
-            int Ps = A.Plev[A.blevel[s]];
-            __syncthreads();
-            const cd* m = mp + (int64_t)rhs * A.ncoef + A.eoff[s];
-            for (int c = threadIdx.x; c < (Ps + 1) * (Ps + 1); c += blockDim.x) coef[c] = m[c];
-            __syncthreads();
-            if (valid) {
-                cd d[3];
-                for (int a = 0; a < 3; ++a) d[a] = x[a] - cd{A.cre[3 * s + a], A.cim[3 * s + a]};
-                radial_seq(false, A.kappa, d[0] * d[0] + d[1] * d[1] + d[2] * d[2], Ps + 1, F);
-                accum(d, Ps);
-            }
-        }
-        __syncthreads();
-        const cd* lc = loc + (int64_t)rhs * A.ncoef + A.eoff[b];
-        for (int c = threadIdx.x; c < nc; c += blockDim.x) coef[c] = lc[c];
-        __syncthreads();
-        if (valid) {
-            cd d[3];
-            for (int a = 0; a < 3; ++a) d[a] = x[a] - cd{A.cre[3 * b + a], A.cim[3 * b + a]};
-            radial_seq(true, A.kappa, d[0] * d[0] + d[1] * d[1] + d[2] * d[2], P + 1, F);
-            accum(d, P);
-            cd* go = g + (int64_t)rhs * 3 * A.n + i;
-            for (int a = 0; a < 3; ++a) go[(int64_t)a * A.n] += G[a];
-        }
-    }
-}
-
-// M2P over List 3 (S waves) and L2P (R waves); one thread per target.
-__global__ void k_eval3h(Exp3hArgs A, const int* __restrict__ leaves, const int* __restrict__ l3off,
-                         const int* __restrict__ l3, const cd* __restrict__ mp, const cd* __restrict__ loc,
-                         cd* __restrict__ u, int do_l2p) {
-    extern __shared__ cd sm[];
-    int b = leaves[blockIdx.x];
-    int rhs = blockIdx.y;
-    int P = A.Plev[A.blevel[b]];
-    int nc = (P + 1) * (P + 1);
-    cd* coef = sm;
-    int s0 = A.bst[b], s1 = A.ben[b];
-    cd F[kH3MaxP + 2];
-    for (int t0 = s0; t0 < s1; t0 += blockDim.x) {
-        int i = t0 + threadIdx.x;
-        bool valid = i < s1;
-        cd x[3] = {{0, 0}, {0, 0}, {0, 0}};
-        if (valid) load3(A.xr, A.xi, A.n, i, x);
-        cd acc = {0, 0};
-        for (int q = l3off[b]; q < l3off[b + 1]; ++q) {
-            int s = l3[q];
-            int Ps = A.Plev[A.blevel[s]];
-            __syncthreads();
-            const cd* m = mp + (int64_t)rhs * A.ncoef + A.eoff[s];
-            for (int c = threadIdx.x; c < (Ps + 1) * (Ps + 1); c += blockDim.x) coef[c] = m[c];
-            __syncthreads();
-            if (valid) {
-                cd d[3];
-                for (int a = 0; a < 3; ++a) d[a] = x[a] - cd{A.cre[3 * s + a], A.cim[3 * s + a]};
-                radial_seq(false, A.kappa, d[0] * d[0] + d[1] * d[1] + d[2] * d[2], Ps, F);
-                acc += eval_wave(A.zc, d[0], d[1], d[2], Ps, F, coef);
-            }
-        }
-        if (!do_l2p) {
-            // M2P only (the L2P runs in complex64): leaves without List 3 add nothing
-            if (valid && l3off[b + 1] > l3off[b]) u[(int64_t)rhs * A.n + i] += acc;
-            continue;
-        }
-        __syncthreads();
-        const cd* lc = loc + (int64_t)rhs * A.ncoef + A.eoff[b];
-        for (int c = threadIdx.x; c < nc; c += blockDim.x) coef[c] = lc[c];
-        __syncthreads();
-        if (valid) {
-            cd d[3];
-            for (int a = 0; a < 3; ++a) d[a] = x[a] - cd{A.cre[3 * b + a], A.cim[3 * b + a]};
-            radial_seq(true, A.kappa, d[0] * d[0] + d[1] * d[1] + d[2] * d[2], P, F);
-            acc += eval_wave(A.zc, d[0], d[1], d[2], P, F, coef);
-            u[(int64_t)rhs * A.n + i] += acc;
-        }
-    }
-}
-
 // ---------------------------------------------------------------------------
 // L2P in complex64 arithmetic (mixed precision), 3D Helmholtz and Laplace.
 //
@@ -1133,6 +965,8 @@ struct Helm3dState {
     DevBuf<cd> rad;
     H3Tables* tab = nullptr;
     PairSlots pairs;             // List-2 pairs, workspaces of the translations
+    Eval3 eval;                  // M2P, L2P
+    int maxP_eval = 0;           // largest order at a leaf's level
 };
 
 static std::mutex g_mu;
@@ -1251,6 +1085,8 @@ void helm3d_setup(cfmm_plan_s* P) {
             CFMM_CUDA(cudaMemcpyAsync(l4e.data(), T.lent[3].get(), sizeof(int) * l4[T.nboxes], cudaMemcpyDeviceToHost,
                                       st));
         CFMM_CUDA(cudaStreamSynchronize(st));
+        eval3_build(&S->eval, S->leaves_l0, T.hloff[2], hst, hen, S->d_leaves_l0.get(), T.loff[2].get(), st);
+        for (int b : S->leaves_l0) S->maxP_eval = std::max(S->maxP_eval, S->Plev[lvl[b]]);
         std::vector<int> ro(byl.size()), rl(boxes.size());
         S->p2m_rtot.assign(T.nlevels, 0);
         S->p2l_rtot.assign(T.nlevels, 0);
@@ -1281,8 +1117,7 @@ void helm3d_setup(cfmm_plan_s* P) {
         CFMM_CUDA(cudaMemcpyAsync(S->d_p2l_boxes.get(), boxes.data(), sizeof(int) * boxes.size(),
                                   cudaMemcpyHostToDevice, st));
     CFMM_CUDA(cudaStreamSynchronize(st));
-    for (auto f : {(const void*)k_p2x3h, (const void*)k_p2x3h_slp<false>, (const void*)k_eval3h,
-                   (const void*)k_eval3h_grad})
+    for (auto f : {(const void*)k_p2x3h, (const void*)k_p2x3h_slp<false>})
         CFMM_CUDA(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, kH3Smem));
 }
 
@@ -1412,17 +1247,11 @@ void helm3d_apply(cfmm_plan_s* P, const cd* sigma, const cd* tau, int64_t dstrid
     near_join(P);   // the near field has written u
     // (5) M2P, (8) L2P (complex64 in mixed precision)
     {
-        dim3 gr((unsigned)S->leaves_l0.size(), nrhs);
-        k_eval3h<<<gr, 128, sizeof(cd) * (size_t)(maxP + 1) * (maxP + 1), st>>>(
-            A, S->d_leaves_l0.get(), T.loff[2].get(), T.lent[2].get(), mp, lc, u, mixed ? 0 : 1);
-        CFMM_LAUNCHED();
+        Eval3Args E{S->d_leaves_l0.get(), (int)S->leaves_l0.size(), S->dPlev.get(), S->maxP_eval, S->exp_off.get(),
+                    S->ncoef, P->kappa, mp, lc};
+        eval3_apply(P, &S->eval, eval3_tables(TB), E, !mixed, u, g, nrhs);
         if (mixed) launch_l2p3f(TB, true, P, S->d_leaves_l0.get(), (int)S->leaves_l0.size(), maxP, S->dPlev.get(),
                                 S->exp_off.get(), S->ncoef, lc, u, nrhs);
-        if (g && gr.x) {
-            k_eval3h_grad<<<gr, 128, sizeof(cd) * (size_t)(maxP + 1) * (maxP + 1), st>>>(
-                A, S->d_leaves_l0.get(), T.loff[2].get(), T.lent[2].get(), mp, lc, g);
-            CFMM_LAUNCHED();
-        }
     }
     rec(8);
 }
@@ -1484,6 +1313,10 @@ void lap3_tr_destroy(Lap3Tr* L) { delete L; }
 void lap3_m2l(Lap3Tr* L, cfmm_plan_s* P, int l_lo, int l_hi, int Pord, const int64_t* eoff, int64_t ncoef, const cd* mp,
               cd* lc, int nrhs) {
     pairs3d_m2l(P, &L->pairs, tr3_tables(L->tab), l_lo, l_hi, Pord, 0.0, eoff, ncoef, mp, lc, nrhs);
+}
+
+void lap3_eval(Lap3Tr* L, cfmm_plan_s* P, Eval3* E, const Eval3Args& A, bool l2p, cd* u, cd* g, int nrhs) {
+    eval3_apply(P, E, eval3_tables(L->tab), A, l2p, u, g, nrhs);
 }
 
 void lap3_m2m(Lap3Tr* L, cfmm_plan_s* P, int l, int Pord, const int64_t* eoff, int64_t ncoef, cd* mp, int nrhs) {

@@ -106,6 +106,10 @@ void lap3_tr_destroy(Lap3Tr* L);
 // the order does not fit the kernel (the caller then uses the general P2M)
 bool lap3_p2m_slp(Lap3Tr* L, cfmm_plan_s* P, const int* leaves, int cnt, int maxP, const int* dPlev,
                   const int64_t* eoff, int64_t ncoef, const cd* sigma, int64_t dstride, cd* out, int nrhs);
+// M2P and L2P in FP64 (eval3d.cuh)
+struct Eval3;
+struct Eval3Args;
+void lap3_eval(Lap3Tr* L, cfmm_plan_s* P, Eval3* E, const Eval3Args& A, bool l2p, cd* u, cd* g, int nrhs);
 // M2M into the non-leaf boxes of level l from level l + 1; L2L from level l, added to level l + 1
 void lap3_m2m(Lap3Tr* L, cfmm_plan_s* P, int l, int Pord, const int64_t* eoff, int64_t ncoef, cd* mp, int nrhs);
 void lap3_l2l(Lap3Tr* L, cfmm_plan_s* P, int l, int Pord, const int64_t* eoff, int64_t ncoef, cd* lc, int nrhs);
