@@ -35,6 +35,17 @@ static inline void upload_lag_rule_local() {
     CFMM_CUDA(cudaMemcpyToSymbol(c_lag, &host_lag_rule(), sizeof(LagRule)));
 }
 
+// |f|^2 > 1e300 for the Miller recurrences. On the device an FP64 slot is dear: the
+// exponent bits tell whether a component is beyond 2^498 (3e149).
+CFMM_HD bool miller_big(cd f) {
+#ifdef __CUDA_ARCH__
+    int hx = __double2hiint(f.x) & 0x7fffffff, hy = __double2hiint(f.y) & 0x7fffffff;
+    return (hx > hy ? hx : hy) >= 0x5f100000;
+#else
+    return cabs2(f) > 1e300;
+#endif
+}
+
 CFMM_HD cd csqrt_p(cd z) {
     double a = z.x, b = z.y;
     if (a == 0.0 && b == 0.0) return cd{0.0, 0.0};
@@ -134,6 +145,7 @@ CFMM_HD void bessel_j_seq(cd z, int nmax, cd* out) {
     cd fp = {0.0, 0.0}, f = {1e-200, 0.0};
     cd S = {0.0, 0.0};
     for (int n = 0; n <= nmax; ++n) out[n] = cd{0.0, 0.0};
+    double c2 = 2.0 * N0;
     for (int n = N0; n >= 1; --n) {
         if (n <= nmax) out[n] = f;
         // (-i)^n or i^n times 2 f
@@ -143,10 +155,11 @@ CFMM_HD void bessel_j_seq(cd z, int nmax, cd* out) {
         else    w = (r == 0) ? f : (r == 1) ? cd{-f.y, f.x} : (r == 2) ? -f : cd{f.y, -f.x};
         S = cd{fma(2.0, w.x, S.x), fma(2.0, w.y, S.y)};
         cd t = zi * f;
-        cd fm = {fma(2.0 * n, t.x, -fp.x), fma(2.0 * n, t.y, -fp.y)};
+        cd fm = {fma(c2, t.x, -fp.x), fma(c2, t.y, -fp.y)};
+        c2 -= 2.0;
         fp = f;
         f = fm;
-        if (cabs2(f) > 1e300) {
+        if (miller_big(f)) {
             const double sc = 1e-150;
             f = sc * f;
             fp = sc * fp;
@@ -188,19 +201,20 @@ CFMM_HD void sph_j_seq(cd z, int nmax, cd* out) {
     cd fp = {0.0, 0.0}, f = {1e-200, 0.0};
     cd S = {0.0, 0.0};
     for (int n = 0; n <= nmax; ++n) out[n] = cd{0.0, 0.0};
+    double c2 = 2.0 * N0 + 1.0;
     for (int n = N0; n >= 1; --n) {
         if (n <= nmax) out[n] = f;
         cd w;
         int r = n & 3;
         if (up) w = (r == 0) ? f : (r == 1) ? cd{f.y, -f.x} : (r == 2) ? -f : cd{-f.y, f.x};
         else    w = (r == 0) ? f : (r == 1) ? cd{-f.y, f.x} : (r == 2) ? -f : cd{f.y, -f.x};
-        double c2 = 2.0 * n + 1.0;
         S = cd{fma(c2, w.x, S.x), fma(c2, w.y, S.y)};
         cd t = zi * f;
         cd fm = {fma(c2, t.x, -fp.x), fma(c2, t.y, -fp.y)};   // j_{n-1} = ((2n+1)/z) j_n - j_{n+1}
+        c2 -= 2.0;
         fp = f;
         f = fm;
-        if (cabs2(f) > 1e300) {
+        if (miller_big(f)) {
             const double sc = 1e-150;
             f = sc * f;
             fp = sc * fp;

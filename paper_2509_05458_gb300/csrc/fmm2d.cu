@@ -29,14 +29,27 @@
 #include <cstdlib>
 #include <mutex>
 
-#include "cfmm_special.cuh"
 #include "kernels.cuh"
+#include "pair64.cuh"
 
 namespace cfmm {
 
-void upload_lag_rule_fmm2d() { upload_lag_rule_local(); }
+// 1/k (an FP64 division costs ten FP64 instructions)
+constexpr int kInvTab = 128;
+static __constant__ double c_inv[kInvTab];
+__device__ __forceinline__ double inv_of(int k) { return k < kInvTab ? c_inv[k] : 1.0 / k; }
+
+void upload_lag_rule_fmm2d() {
+    upload_lag_rule_local();
+    double inv[kInvTab] = {0.0};
+    for (int k = 1; k < kInvTab; ++k) inv[k] = 1.0 / k;
+    CFMM_CUDA(cudaMemcpyToSymbol(c_inv, inv, sizeof(inv)));
+}
 
 constexpr int kExpThreads = 64;
+constexpr int kP2eThreads = 128;   // k_point_to_exp
+// its accumulator entries at orders up to P
+static size_t p2e_acc(int P) { return std::max<size_t>(2 * (size_t)P + 1, kP2eThreads); }
 constexpr int kMaxSmem = 200 * 1024;
 
 // per-plan constants of the 2D expansions
@@ -51,6 +64,8 @@ struct Fmm2dState {
     // Laplace: binomial table C(n, k), n, k <= NB
     int NB = 0;
     DevBuf<double> binom;
+    // Laplace, (maxP+1)^2 by [n][k]: C(k-1, n-1) and C(n+k-1, k)
+    DevBuf<double> cm2m, cm2l;
     // Helmholtz translation tables
     DevBuf<cd> t_m2l;                      // per List-2 entry: S_j(c_t - c_s), j = -2P..2P
     std::vector<int64_t> m2l_base;         // per level: table base (complex units)
@@ -91,9 +106,33 @@ __device__ __forceinline__ void zeta_eta(cd d0, cd d1, cd& z, cd& e) {
 
 __device__ __forceinline__ cd load_pt(const double* a, int64_t n, int axis, int64_t i) { return cd{a[axis * n + i], 0}; }
 
+// tables and wavenumber constants of the quick Hankel functions (pair64.cuh)
+struct HankelArgs {
+    const PairTab* T;
+    Wave w;
+};
+
+// H_0^(1), H_1^(1) of kappa r, r^2 given: the Taylor cells of pair64.cuh (about 150
+// FP64 instructions), or hankel01 outside them (its quadrature beyond |z| = 6 takes
+// 6000, which a lone warp issues in 0.2 ms)
+__device__ void hankel01_r2(const HankelArgs& H, cd r2, cd* h0, cd* h1) {
+    cd y = crsqrt64(r2), ds;
+    int cell = hankel_cell(H.w.ik * y, ds);
+    if (cell < 0) {
+        hankel01(H.w.k * csqrt_p(r2), h0, h1);
+        return;
+    }
+    cd r;
+    cd e = wave64(H.T, H.w, r2, y, r);
+    e = e * (H.w.isk * crsqrt64(r));
+    *h0 = e * hankel_factor(H.T->hk[cell][0], ds);
+    *h1 = e * hankel_factor(H.T->hk[cell][1], ds);
+}
+
 // Fill row[0 .. 2P+2] with T_m(d), m = -P-1..P+1 (index m + P + 1), where
 // T = G (kind 0, regular) or S (kind 1, singular) of the displacement d.
-__device__ void cyl_row(int kind, cd zeta, cd eta, double kappa, int P, cd* row) {
+__device__ void cyl_row(int kind, cd zeta, cd eta, const HankelArgs& H, int P, cd* row) {
+    const double kappa = H.w.k;
     cd r2 = zeta * eta;
     cd r = csqrt_p(r2);
     int M = P + 1;
@@ -107,7 +146,7 @@ __device__ void cyl_row(int kind, cd zeta, cd eta, double kappa, int P, cd* row)
     } else {
         cd h0, h1;
         cd z = kappa * r;
-        hankel01(z, &h0, &h1);
+        hankel01_r2(H, r2, &h0, &h1);
         pos[0] = h0;
         if (M >= 1) pos[1] = h1;
         cd zi = cinv(z);
@@ -131,7 +170,7 @@ __device__ void cyl_row(int kind, cd zeta, cd eta, double kappa, int P, cd* row)
 __global__ void k_leaf_rows(const int* __restrict__ leaves, const int* __restrict__ blevel,
                             const int* __restrict__ bst, const int* __restrict__ ben, const int* __restrict__ Plev,
                             const double* __restrict__ xr, const double* __restrict__ xi, int64_t n,
-                            const double* __restrict__ cre, const double* __restrict__ cim, double kappa, int RL,
+                            const double* __restrict__ cre, const double* __restrict__ cim, HankelArgs H, int RL,
                             cd* __restrict__ lrow) {
     int b = leaves[blockIdx.x];
     int P = Plev[blevel[b]];
@@ -140,7 +179,7 @@ __global__ void k_leaf_rows(const int* __restrict__ leaves, const int* __restric
         cd y0 = {xr[j], xi[j]}, y1 = {xr[n + j], xi[n + j]};
         cd z, e;
         zeta_eta(cen0 - y0, cen1 - y1, z, e);   // D = c - y
-        cyl_row(0, z, e, kappa, P, lrow + (int64_t)j * RL);
+        cyl_row(0, z, e, H, P, lrow + (int64_t)j * RL);
     }
 }
 
@@ -166,57 +205,57 @@ struct ExpArgs {
     const int* Plev;
     const int64_t* eoff;
     int64_t ncoef;
+    HankelArgs H;
 };
 
-// term row (Laplace) for a source at d = y - c, regular (P2M) or singular (P2L)
-__device__ void lap_terms(bool sing, cd zeta, cd eta, cd s, cd t, cd nu, cd nut, int P, bool slp, bool dlp,
-                          cd* row) {
-    if (!sing) {
-        row[0] = slp ? s : cd{0, 0};
-        cd ep = {1, 0}, zp = {1, 0};
-        for (int k = 1; k <= P; ++k) {
-            cd a = {0, 0}, b = {0, 0};
-            if (slp) {
-                a = (-0.5 / k) * (ep * eta) * s;
-                b = (-0.5 / k) * (zp * zeta) * s;
-            }
-            if (dlp) {
-                a -= 0.5 * (nut * ep) * t;
-                b -= 0.5 * (nu * zp) * t;
-            }
-            row[k] = a;
-            row[P + k] = b;
-            ep = ep * eta;
-            zp = zp * zeta;
+// term row (Laplace) for a source at d = y - c, regular (P2M) or singular (P2L):
+//   P2M  row_k = -s eta^k/(2k) - nut t eta^{k-1}/2          (k <= P; P + k: zeta, nu)
+//   P2L  row_k = -s zeta^-k/(2k) + nu t zeta^{-k-1}/2       (P + k: eta, nut)
+// as two running products a series, 10 FP64 instructions a term
+__device__ void lap_terms(const PairTab* T, bool sing, cd zeta, cd eta, cd s, cd t, cd nu, cd nut, int P, bool slp,
+                          bool dlp, cd* row) {
+    cd x = eta, y = zeta, nx = nut, ny = nu;           // series 1..P in x, P+1..2P in y
+    double h = -0.5;
+    cd v0 = slp ? s : cd{0, 0};
+    if (sing) {
+        x = crcp64(zeta);
+        y = crcp64(eta);
+        nx = nu;
+        ny = nut;
+        h = 0.5;
+        v0 = slp ? (0.5 * clog64(T, zeta * eta)) * s : cd{0, 0};
+        if (dlp) v0 = cmac(v0, 0.5 * (nu * x + nut * y), t);
+    }
+    row[0] = v0;
+    cd ax = -0.5 * (s * x), ay = -0.5 * (s * y), bx = h * (nx * t), by = h * (ny * t);
+    if (sing) {
+        bx = bx * x * x;
+        by = by * y * y;
+    }
+    for (int k = 1; k <= P; ++k) {
+        double ik = inv_of(k);
+        cd a = dlp ? bx : cd{0, 0}, b = dlp ? by : cd{0, 0};
+        if (slp) {
+            a = rmac(a, ik, ax);
+            b = rmac(b, ik, ay);
+            ax = ax * x;
+            ay = ay * y;
         }
-    } else {
-        cd iz = cinv(zeta), ie = cinv(eta);
-        cd v0 = {0, 0};
-        if (slp) v0 = (0.5 * clog_p(zeta * eta)) * s;
-        if (dlp) v0 += (0.5 * (nu * iz + nut * ie)) * t;
-        row[0] = v0;
-        cd zp = iz, ep = ie;   // zeta^-k, eta^-k
-        for (int k = 1; k <= P; ++k) {
-            cd a = {0, 0}, b = {0, 0};
-            if (slp) {
-                a = (-0.5 / k) * zp * s;
-                b = (-0.5 / k) * ep * s;
-            }
-            if (dlp) {
-                a += 0.5 * (nu * (zp * iz)) * t;
-                b += 0.5 * (nut * (ep * ie)) * t;
-            }
-            row[k] = a;
-            row[P + k] = b;
-            zp = zp * iz;
-            ep = ep * ie;
+        row[k] = a;
+        row[P + k] = b;
+        if (dlp) {
+            bx = bx * x;
+            by = by * y;
         }
     }
 }
 
 // One CTA per target box; sources = the box's own points (P2M, list == null)
-// or the points of the List-4 leaves (P2L). Result added to (P2L) or stored
-// in (P2M) out[rhs][eoff[b] + c].
+// or the points of the List-4 leaves (P2L), taken `chunk` at a time over the whole
+// list (leaves of a point or two share a chunk: a source's row is a chain of 700
+// FP64 instructions). Thread (c, s) owns coefficient c for every S-th source: with
+// one thread per coefficient 41 of 64 lanes were in use at order 20. Result added to
+// (P2L) or stored in (P2M) out[rhs][eoff[b] + c].
 template <int KER>
 __global__ void k_point_to_exp(ExpArgs A, const int* __restrict__ boxes, const int* __restrict__ loff,
                                const int* __restrict__ lent, int sing, cd* __restrict__ out, int chunk,
@@ -227,78 +266,97 @@ __global__ void k_point_to_exp(ExpArgs A, const int* __restrict__ boxes, const i
     int P = A.Plev[A.blevel[b]];
     int nc = 2 * P + 1;
     int R = KER == CFMM_LAPLACE ? nc : nc + 2;
-    cd* acc = sm;
-    cd* rows = sm + nc;
+    const int S = max(1, min((int)blockDim.x / nc, 4));
+    cd* acc = sm;                              // [S][nc]
+    cd* rows = sm + S * nc;
     cd* wts = rows + (size_t)chunk * R;        // Helmholtz: per source (s, -k/2 nu t, k/2 nu~ t)
-    for (int c = threadIdx.x; c < nc; c += blockDim.x) acc[c] = cd{0, 0};
+    for (int c = threadIdx.x; c < S * nc; c += blockDim.x) acc[c] = cd{0, 0};
     cd cen0 = {A.cre[2 * b], A.cim[2 * b]}, cen1 = {A.cre[2 * b + 1], A.cim[2 * b + 1]};
-    int qa = loff ? loff[b] : 0, qb = loff ? loff[b + 1] : 1;
-    for (int q = qa; q < qb; ++q) {
-        int src = loff ? lent[q] : b;
-        int s0 = A.bst[src], s1 = A.ben[src];
-        for (int c0 = s0; c0 < s1; c0 += chunk) {
-            int cn = min(chunk, s1 - c0);
-            __syncthreads();
-            if (threadIdx.x < cn) {
-                int64_t j = c0 + threadIdx.x;
-                cd y0 = {A.xr[j], A.xi[j]}, y1 = {A.xr[A.n + j], A.xi[A.n + j]};
-                cd s = A.slp ? A.sigma[rhs * A.dstride + j] : cd{0, 0};
-                cd t = A.dlp ? A.tau[rhs * A.dstride + j] : cd{0, 0};
-                cd nu = {0, 0}, nut = {0, 0};
-                if (A.dlp) {
-                    cd n0 = {A.nr[j], A.ni[j]}, n1 = {A.nr[A.n + j], A.ni[A.n + j]};
-                    nu = n0 + mul_i(n1);
-                    nut = n0 - mul_i(n1);
-                }
-                cd* row = rows + (size_t)threadIdx.x * R;
-                cd z, e;
-                if (KER == CFMM_LAPLACE) {
-                    zeta_eta(y0 - cen0, y1 - cen1, z, e);   // d = y - c
-                    lap_terms(sing != 0, z, e, s, t, nu, nut, P, A.slp, A.dlp, row);
-                } else {
-                    if (lrow && !sing) {
-                        // the plan's row of this point about its own leaf (this box)
-                        const cd* src = lrow + j * RL;
-                        for (int q = 0; q < R; ++q) row[q] = src[q];
-                    } else {
-                        zeta_eta(cen0 - y0, cen1 - y1, z, e);   // D = c - y
-                        cyl_row(sing ? 1 : 0, z, e, A.kappa, P, row);
-                    }
-                    double hk = 0.5 * A.kappa;
-                    cd* w = wts + 3 * threadIdx.x;
-                    w[0] = s;
-                    w[1] = (-hk) * (nu * t);
-                    w[2] = hk * (nut * t);
-                }
-            }
-            __syncthreads();
-            for (int c = threadIdx.x; c < nc; c += blockDim.x) {
-                cd a = acc[c];
-                if (KER == CFMM_LAPLACE) {
-                    for (int tt = 0; tt < cn; ++tt) a += rows[(size_t)tt * R + c];
-                } else {
-                    // coefficient n = c - P: s T_{-n} - (k/2)(nu T_{-n-1} - nu~ T_{-n+1}) t,
-                    // T_k at row index k + P + 1
-                    int i0 = 2 * P + 1 - c;
-                    if (A.dlp) {
-                        for (int tt = 0; tt < cn; ++tt) {
-                            const cd* r = rows + (size_t)tt * R + i0;
-                            const cd* w = wts + 3 * tt;
-                            a = cmac(cmac(cmac(a, w[0], r[0]), w[1], r[-1]), w[2], r[1]);
-                        }
-                    } else {
-                        for (int tt = 0; tt < cn; ++tt) a = cmac(a, wts[3 * tt], rows[(size_t)tt * R + i0]);
-                    }
-                }
-                acc[c] = a;
+    // first source of the next chunk: point j0 of list entry qn
+    int qn = loff ? loff[b] : 0, j0 = 0;
+    const int qb = loff ? loff[b + 1] : 1;
+    while (qn < qb) {
+        // the thread's source, and (the same for all) where the chunk ends
+        int64_t j = -1;
+        int cn = 0, q = qn, jn = j0;
+        while (q < qb && cn < chunk) {
+            const int src = loff ? lent[q] : b;
+            const int s0 = A.bst[src] + jn, m = min(A.ben[src] - s0, chunk - cn);
+            if ((int)threadIdx.x >= cn && (int)threadIdx.x < cn + m) j = s0 + (threadIdx.x - cn);
+            cn += m;
+            if (s0 + m == A.ben[src]) {
+                ++q;
+                jn = 0;
+            } else {
+                jn += m;
             }
         }
+        __syncthreads();
+        if (j >= 0) {
+            cd y0 = {A.xr[j], A.xi[j]}, y1 = {A.xr[A.n + j], A.xi[A.n + j]};
+            cd s = A.slp ? A.sigma[rhs * A.dstride + j] : cd{0, 0};
+            cd t = A.dlp ? A.tau[rhs * A.dstride + j] : cd{0, 0};
+            cd nu = {0, 0}, nut = {0, 0};
+            if (A.dlp) {
+                cd n0 = {A.nr[j], A.ni[j]}, n1 = {A.nr[A.n + j], A.ni[A.n + j]};
+                nu = n0 + mul_i(n1);
+                nut = n0 - mul_i(n1);
+            }
+            cd* row = rows + (size_t)threadIdx.x * R;
+            cd z, e;
+            if (KER == CFMM_LAPLACE) {
+                zeta_eta(y0 - cen0, y1 - cen1, z, e);   // d = y - c
+                lap_terms(A.H.T, sing != 0, z, e, s, t, nu, nut, P, A.slp, A.dlp, row);
+            } else {
+                if (!lrow || sing) {
+                    zeta_eta(cen0 - y0, cen1 - y1, z, e);   // D = c - y
+                    cyl_row(sing ? 1 : 0, z, e, A.H, P, row);
+                }
+                double hk = 0.5 * A.kappa;
+                cd* w = wts + 3 * threadIdx.x;
+                w[0] = s;
+                w[1] = (-hk) * (nu * t);
+                w[2] = hk * (nut * t);
+            }
+        }
+        // the plan's rows of the points about their own leaf (this box), a warp a row
+        if (KER == CFMM_HELMHOLTZ && lrow && !sing)
+            for (int tt = threadIdx.x >> 5; tt < cn; tt += blockDim.x >> 5) {
+                const cd* src = lrow + (int64_t)(A.bst[b] + j0 + tt) * RL;
+                for (int i = threadIdx.x & 31; i < R; i += 32) rows[(size_t)tt * R + i] = src[i];
+            }
+        __syncthreads();
+        for (int i = threadIdx.x; i < S * nc; i += blockDim.x) {
+            const int sl = i / nc, c = i - sl * nc;
+            cd a = acc[i];
+            if (KER == CFMM_LAPLACE) {
+                for (int tt = sl; tt < cn; tt += S) a += rows[(size_t)tt * R + c];
+            } else {
+                // coefficient n = c - P: s T_{-n} - (k/2)(nu T_{-n-1} - nu~ T_{-n+1}) t,
+                // T_k at row index k + P + 1
+                int i0 = 2 * P + 1 - c;
+                if (A.dlp) {
+                    for (int tt = sl; tt < cn; tt += S) {
+                        const cd* r = rows + (size_t)tt * R + i0;
+                        const cd* w = wts + 3 * tt;
+                        a = cmac(cmac(cmac(a, w[0], r[0]), w[1], r[-1]), w[2], r[1]);
+                    }
+                } else {
+                    for (int tt = sl; tt < cn; tt += S) a = cmac(a, wts[3 * tt], rows[(size_t)tt * R + i0]);
+                }
+            }
+            acc[i] = a;
+        }
+        qn = q;
+        j0 = jn;
     }
     __syncthreads();
     cd* o = out + (int64_t)rhs * A.ncoef + A.eoff[b];
     for (int c = threadIdx.x; c < nc; c += blockDim.x) {
-        if (sing) o[c] += acc[c];
-        else o[c] = acc[c];
+        cd v = acc[c];
+        for (int sl = 1; sl < S; ++sl) v += acc[sl * nc + c];
+        if (sing) o[c] += v;
+        else o[c] = v;
     }
 }
 
@@ -321,139 +379,178 @@ struct TransArgs {
     const int64_t* shoff;
 };
 
-__device__ __forceinline__ double binom_at(const TransArgs& T, int n, int k) { return T.binom[n * (T.NB + 1) + k]; }
+// The Laplace translations with the binomials as real matrices between diagonal
+// scalings (z = zeta or eta of the shift, per series):
+//   M2M  M'_k = z^k (sum_{n<=k} C(k-1,n-1) z^-n M_n - M_0/(2k))
+//   M2L  L_k  = z^-k (sum_n C(n+k-1,k) (-z)^-n M_n - M_0/(2k))
+//   L2L  L'_k = z^-k sum_{n>=k} C(n,k) z^n L_n
+// 2 FP64 instructions a term instead of 8. What bounds a level is the chain of FP64
+// instructions one warp issues (one in 64 cycles), so threads are (shift, k): a
+// group of warps takes a shift (its last warp the constant coefficient), and the
+// groups of a block work side by side.
+__device__ __forceinline__ cd cpow_k(cd z, int k) {
+    cd r = {1, 0};
+    for (; k; k >>= 1) {
+        if (k & 1) r = r * z;
+        if (k > 1) z = z * z;
+    }
+    return r;
+}
+__host__ __device__ inline int lap_group(int P) { return (2 * P + 31) / 32 * 32 + 32; }   // threads of a shift
 
 // M2M: parent b gathers its children
-template <int KER>
-__global__ void k_m2m(TransArgs T, int lo, const cd* __restrict__ mp_in, cd* __restrict__ mp_out, const int* __restrict__ leaf) {
+__global__ void k_m2m_lap(TransArgs T, int lo, const cd* __restrict__ mp_in, cd* __restrict__ mp_out,
+                          const int* __restrict__ leaf, int P, const double* __restrict__ cm2m) {
     extern __shared__ cd sm[];
-    int b = lo + blockIdx.x;
+    const int b = lo + blockIdx.x, rhs = blockIdx.y, nc = 2 * P + 1;
     if (leaf[b]) return;
-    int rhs = blockIdx.y;
-    int Pp = T.Plev[T.blevel[b]];
-    int ncp = 2 * Pp + 1;
-    int Pc = T.Plev[T.blevel[b] + 1];      // every child sits one level finer
-    int ncc = 2 * Pc + 1;
-    cd* acc = sm;
-    cd* src = sm + ncp;
-    cd* pw = src + ncc;                    // Laplace: 2(Pp+1) powers; Helmholtz: 2(Pc+Pp)+1 table
-    for (int c = threadIdx.x; c < ncp; c += blockDim.x) acc[c] = cd{0, 0};
+    const int gs = lap_group(P), ng = blockDim.x / gs, g = threadIdx.x / gs, i = threadIdx.x - g * gs;
+    cd *x = sm + g * nc, *red = sm + ng * nc + g * nc;
+    const int c = i < 2 * P ? i + 1 : 0, k = c > P ? c - P : c;
+    cd acc = {0, 0};
+    for (int c0 = T.cbeg[b]; c0 < T.cend[b]; c0 += ng) {
+        const int ch = c0 + g;
+        const bool on = ch < T.cend[b];
+        cd pk = {1, 0}, m0 = {0, 0};
+        bool nz = true;
+        __syncthreads();
+        if (on) {
+            const cd* m = mp_in + (int64_t)rhs * T.ncoef + T.eoff[ch];
+            m0 = m[0];
+            if (c) {
+                // a = c_child - c_parent
+                cd z, e;
+                zeta_eta(cd{T.cre[2 * ch] - T.cre[2 * b], T.cim[2 * ch] - T.cim[2 * b]},
+                         cd{T.cre[2 * ch + 1] - T.cre[2 * b + 1], T.cim[2 * ch + 1] - T.cim[2 * b + 1]}, z, e);
+                if (c <= P) z = e;
+                nz = z.x != 0.0 || z.y != 0.0;
+                if (nz) pk = cpow_k(z, k);
+                x[c] = nz ? m[c] * crcp64(pk) : m[c];
+            }
+        }
+        __syncthreads();
+        if (on && c) {
+            const cd* xs = x + (c > P ? P : 0);
+            if (nz) {
+                cd y = (-0.5 * inv_of(k)) * m0;
+                for (int n = 1; n <= P; ++n) y = rmac(y, __ldg(cm2m + n * (P + 1) + k), xs[n]);   // 0 for n > k
+                acc = cmac(acc, pk, y);
+            } else {
+                acc += xs[k];
+            }
+        } else if (on && i == 2 * P) {
+            acc += m0;
+        }
+    }
+    __syncthreads();
+    if (c || i == 2 * P) red[c] = acc;
+    __syncthreads();
+    cd* o = mp_out + (int64_t)rhs * T.ncoef + T.eoff[b];
+    for (int q = threadIdx.x; q < nc; q += blockDim.x) {
+        cd v = sm[ng * nc + q];
+        for (int j = 1; j < ng; ++j) v += sm[(ng + j) * nc + q];
+        o[q] = v;
+    }
+}
+
+// L2L: child b (at level lo..) receives its parent's local expansion
+__global__ void k_l2l_lap(TransArgs T, int lo, cd* __restrict__ loc, int P) {
+    extern __shared__ cd sm[];
+    const int b = lo + blockIdx.x, rhs = blockIdx.y, p = T.parent[b], i = threadIdx.x;
+    const int c = i < 2 * P ? i + 1 : 0, k = c > P ? c - P : c;
+    const cd* lp = loc + (int64_t)rhs * T.ncoef + T.eoff[p];
+    cd* o = loc + (int64_t)rhs * T.ncoef + T.eoff[b];
+    cd pk = {1, 0};
+    bool nz = true;
+    if (c) {
+        // powers of -zeta0, -eta0 with a = c_parent - c_child: of the child's offset
+        cd z, e;
+        zeta_eta(cd{T.cre[2 * b] - T.cre[2 * p], T.cim[2 * b] - T.cim[2 * p]},
+                 cd{T.cre[2 * b + 1] - T.cre[2 * p + 1], T.cim[2 * b + 1] - T.cim[2 * p + 1]}, z, e);
+        if (c > P) z = e;
+        nz = z.x != 0.0 || z.y != 0.0;
+        if (nz) pk = cpow_k(z, k);
+        // (a zero shift leaves the coefficients; they do not reach L_0)
+        sm[c] = pk * lp[c];
+        sm[2 * P + c] = nz ? sm[c] : cd{0, 0};
+    }
+    __syncthreads();
+    if (c) {
+        const cd* xs = sm + (c > P ? P : 0);
+        if (nz) {
+            cd y = {0, 0};
+            for (int n = 1; n <= P; ++n) y = rmac(y, __ldg(T.binom + n * (T.NB + 1) + k), xs[n]);   // 0 for n < k
+            o[c] = cmac(o[c], crcp64(pk), y);
+        } else {
+            o[c] += xs[k];
+        }
+    } else if (i >= (int)blockDim.x - 32) {
+        // the constant: the last warp sums L_0 and every scaled coefficient
+        const int lane = i & 31;
+        cd v = {0, 0};
+        for (int q = 1 + lane; q <= 2 * P; q += 32) v += sm[2 * P + q];
+        for (int d = 16; d > 0; d >>= 1) {
+            v.x += __shfl_xor_sync(0xffffffffu, v.x, d);
+            v.y += __shfl_xor_sync(0xffffffffu, v.y, d);
+        }
+        if (lane == 0) o[0] += lp[0] + v;
+    }
+}
+
+// The Helmholtz M2M and L2L: Toeplitz products with the plan's tables; item (c, s)
+// takes every S-th term of coefficient c, so that a block's warps share the chain.
+__global__ void k_m2m_helm(TransArgs T, int lo, const cd* __restrict__ mp_in, cd* __restrict__ mp_out,
+                           const int* __restrict__ leaf, int Pc, int Pp, int S) {
+    extern __shared__ cd sm[];
+    const int b = lo + blockIdx.x, rhs = blockIdx.y, ncp = 2 * Pp + 1, ncc = 2 * Pc + 1, off = Pc + Pp;
+    if (leaf[b]) return;
+    cd *src = sm, *pw = src + ncc, *red = pw + 2 * off + 1;
+    for (int i = threadIdx.x; i < S * ncp; i += blockDim.x) red[i] = cd{0, 0};
     for (int ch = T.cbeg[b]; ch < T.cend[b]; ++ch) {
         __syncthreads();
         const cd* m = mp_in + (int64_t)rhs * T.ncoef + T.eoff[ch];
-        for (int c = threadIdx.x; c < ncc; c += blockDim.x) src[c] = m[c];
-        if (KER == CFMM_LAPLACE) {
-            // powers of zeta0, eta0 of a = c_child - c_parent, up to Pp
-            if (threadIdx.x == 0) {
-                cd a0 = {T.cre[2 * ch] - T.cre[2 * b], T.cim[2 * ch] - T.cim[2 * b]};
-                cd a1 = {T.cre[2 * ch + 1] - T.cre[2 * b + 1], T.cim[2 * ch + 1] - T.cim[2 * b + 1]};
-                cd z, e;
-                zeta_eta(a0, a1, z, e);
-                cd zp = {1, 0}, ep = {1, 0};
-                for (int k = 0; k <= Pp; ++k) {
-                    pw[k] = zp;
-                    pw[Pp + 1 + k] = ep;
-                    zp = zp * z;
-                    ep = ep * e;
-                }
-            }
-        } else {
-            const cd* tb = T.tshift + T.shoff[ch];
-            int nt = 2 * (Pc + Pp) + 1;
-            for (int c = threadIdx.x; c < nt; c += blockDim.x) pw[c] = tb[c];
-        }
+        const cd* tb = T.tshift + T.shoff[ch];
+        for (int q = threadIdx.x; q < ncc; q += blockDim.x) src[q] = m[q];
+        for (int q = threadIdx.x; q < 2 * off + 1; q += blockDim.x) pw[q] = tb[q];
         __syncthreads();
-        for (int c = threadIdx.x; c < ncp; c += blockDim.x) {
-            cd a = acc[c];
-            if (KER == CFMM_LAPLACE) {
-                if (c == 0) {
-                    a += src[0];
-                } else {
-                    bool isz = c > Pp;
-                    int k = isz ? c - Pp : c;
-                    const cd* pk = isz ? pw : pw + Pp + 1;      // zeta or eta powers
-                    a += (-0.5 / k) * pk[k] * src[0];
-                    int top = k < Pc ? k : Pc;
-                    for (int nn = 1; nn <= top; ++nn) {
-                        cd mn = isz ? src[Pc + nn] : src[nn];
-                        a += binom_at(T, k - 1, k - nn) * (pk[k - nn] * mn);
-                    }
-                }
-            } else {
-                int m = c - Pp;
-                int off = Pc + Pp;
-                for (int nn = -Pc; nn <= Pc; ++nn) a = cmac(a, pw[nn - m + off], src[nn + Pc]);
-            }
-            acc[c] = a;
+        for (int i = threadIdx.x; i < S * ncp; i += blockDim.x) {
+            const int s = i / ncp, c = i - s * ncp;
+            cd a = red[i];
+            for (int q = s; q < ncc; q += S) a = cmac(a, pw[q - Pc - (c - Pp) + off], src[q]);
+            red[i] = a;
         }
     }
     __syncthreads();
     cd* o = mp_out + (int64_t)rhs * T.ncoef + T.eoff[b];
-    for (int c = threadIdx.x; c < ncp; c += blockDim.x) o[c] = acc[c];
+    for (int q = threadIdx.x; q < ncp; q += blockDim.x) {
+        cd v = red[q];
+        for (int j = 1; j < S; ++j) v += red[j * ncp + q];
+        o[q] = v;
+    }
 }
 
-// L2L: child b (at level lo..) receives its parent's local expansion
-template <int KER>
-__global__ void k_l2l(TransArgs T, int lo, cd* __restrict__ loc) {
+__global__ void k_l2l_helm(TransArgs T, int lo, cd* __restrict__ loc, int Pp, int Pc, int S) {
     extern __shared__ cd sm[];
-    int b = lo + blockIdx.x;
-    int rhs = blockIdx.y;
-    int p = T.parent[b];
-    int Pc = T.Plev[T.blevel[b]], Pp = T.Plev[T.blevel[p]];
-    int ncc = 2 * Pc + 1, ncp = 2 * Pp + 1;
-    cd* src = sm;
-    cd* pw = sm + ncp;
+    const int b = lo + blockIdx.x, rhs = blockIdx.y, p = T.parent[b], ncp = 2 * Pp + 1, ncc = 2 * Pc + 1, off = Pc + Pp;
+    cd *src = sm, *pw = src + ncp, *red = pw + 2 * off + 1;
     const cd* lp = loc + (int64_t)rhs * T.ncoef + T.eoff[p];
-    for (int c = threadIdx.x; c < ncp; c += blockDim.x) src[c] = lp[c];
-    if (KER == CFMM_LAPLACE) {
-        if (threadIdx.x == 0) {
-            // powers of -zeta0, -eta0 with a = c_parent - c_child
-            cd a0 = {T.cre[2 * p] - T.cre[2 * b], T.cim[2 * p] - T.cim[2 * b]};
-            cd a1 = {T.cre[2 * p + 1] - T.cre[2 * b + 1], T.cim[2 * p + 1] - T.cim[2 * b + 1]};
-            cd z, e;
-            zeta_eta(a0, a1, z, e);
-            z = -z;
-            e = -e;
-            cd zp = {1, 0}, ep = {1, 0};
-            for (int k = 0; k <= Pp; ++k) {
-                pw[k] = zp;
-                pw[Pp + 1 + k] = ep;
-                zp = zp * z;
-                ep = ep * e;
-            }
-        }
-    } else {
-        // table holds G_j(c_parent - c_child); L2L needs G_j(c_child - c_parent) = (-1)^j G_j(...)
-        const cd* tb = T.tshift + T.shoff[b];
-        int off = Pc + Pp;
-        for (int c = threadIdx.x; c < 2 * off + 1; c += blockDim.x) {
-            int j = c - off;
-            pw[c] = (j & 1) ? -tb[c] : tb[c];
-        }
+    // table holds G_j(c_parent - c_child); L2L needs G_j(c_child - c_parent) = (-1)^j G_j(...)
+    const cd* tb = T.tshift + T.shoff[b];
+    for (int q = threadIdx.x; q < ncp; q += blockDim.x) src[q] = lp[q];
+    for (int q = threadIdx.x; q < 2 * off + 1; q += blockDim.x) pw[q] = ((q - off) & 1) ? -tb[q] : tb[q];
+    __syncthreads();
+    for (int i = threadIdx.x; i < S * ncc; i += blockDim.x) {
+        const int s = i / ncc, c = i - s * ncc;
+        cd a = {0, 0};
+        for (int q = s; q < ncp; q += S) a = cmac(a, pw[q - Pp - (c - Pc) + off], src[q]);
+        red[i] = a;
     }
     __syncthreads();
     cd* o = loc + (int64_t)rhs * T.ncoef + T.eoff[b];
-    for (int c = threadIdx.x; c < ncc; c += blockDim.x) {
-        cd a = {0, 0};
-        if (KER == CFMM_LAPLACE) {
-            if (c == 0) {
-                a = src[0];
-                for (int nn = 1; nn <= Pp; ++nn) a += pw[nn] * src[nn] + pw[Pp + 1 + nn] * src[Pp + nn];
-            } else {
-                bool isz = c > Pc;
-                int k = isz ? c - Pc : c;
-                const cd* pk = isz ? pw + Pp + 1 : pw;          // Lm (eta) uses eta powers
-                for (int nn = k; nn <= Pp; ++nn) {
-                    cd ln = isz ? src[Pp + nn] : src[nn];
-                    a += binom_at(T, nn, k) * (pk[nn - k] * ln);
-                }
-            }
-        } else {
-            int m = c - Pc;
-            int off = Pc + Pp;
-            for (int nn = -Pp; nn <= Pp; ++nn) a = cmac(a, pw[nn - m + off], src[nn + Pp]);
-        }
-        o[c] += a;
+    for (int q = threadIdx.x; q < ncc; q += blockDim.x) {
+        cd v = red[q];
+        for (int j = 1; j < S; ++j) v += red[j * ncc + q];
+        o[q] += v;
     }
 }
 
@@ -469,17 +566,71 @@ struct M2LArgs {
     int64_t ncoef;
     const int* loff;
     const int* lent;
-    const double* binom;
-    int NB;
     const cd* tab;
     const int64_t* tbase;
     const int* tq0;
 };
 
-__device__ __forceinline__ double binom_at_m2l(const M2LArgs& A, int n, int k) { return A.binom[n * (A.NB + 1) + k]; }
+// Laplace M2L (see the comment above k_m2m_lap): a block per box, groups of warps
+// side by side on its List-2 entries
+__global__ void k_m2l_lap(M2LArgs A, int first_box, const cd* __restrict__ mp, cd* __restrict__ loc, int P,
+                          const double* __restrict__ cm2l, const PairTab* __restrict__ T) {
+    extern __shared__ cd sm[];
+    const int b = first_box + blockIdx.x, rhs = blockIdx.y, nc = 2 * P + 1;
+    const int gs = lap_group(P), ng = blockDim.x / gs, g = threadIdx.x / gs, i = threadIdx.x - g * gs;
+    cd *x = sm + g * nc, *red = sm + ng * nc + g * nc;
+    const int c = i < 2 * P ? i + 1 : 0, k = c > P ? c - P : c, q1 = A.loff[b + 1];
+    const bool last = i >= gs - 32;                     // the group's last warp: the constant
+    cd acc = {0, 0};
+    for (int q0 = A.loff[b]; q0 < q1; q0 += ng) {
+        const bool on = q0 + g < q1;
+        cd pk = {0, 0}, m0 = {0, 0}, z = {1, 0}, e = {1, 0};
+        __syncthreads();
+        if (on) {
+            const int s = A.lent[q0 + g];
+            const cd* m = mp + (int64_t)rhs * A.ncoef + A.eoff[s];
+            m0 = m[0];
+            // a = c_s - c_t
+            zeta_eta(cd{A.cre[2 * s] - A.cre[2 * b], A.cim[2 * s] - A.cim[2 * b]},
+                     cd{A.cre[2 * s + 1] - A.cre[2 * b + 1], A.cim[2 * s + 1] - A.cim[2 * b + 1]}, z, e);
+            if (c) {
+                // L_1.. in zeta from the source's zeta series (entries P+1..), L_P+1.. in eta from 1..P
+                pk = cpow_k(crcp64(c <= P ? z : e), k);
+                cd v = pk * m[c <= P ? P + c : c - P];
+                x[c] = (k & 1) ? -v : v;
+            }
+        }
+        __syncthreads();
+        if (!on) continue;
+        if (c) {
+            const cd* xs = x + (c > P ? P : 0);
+            cd y = (-0.5 * inv_of(k)) * m0;
+            for (int n = 1; n <= P; ++n) y = rmac(y, __ldg(cm2l + n * (P + 1) + k), xs[n]);
+            acc = cmac(acc, pk, y);
+        } else if (last) {
+            for (int n = 1 + (i & 31); n <= 2 * P; n += 32) acc += x[n];
+            if (i == gs - 1) acc = cmac(acc, 0.5 * clog64(T, z * e), m0);
+        }
+    }
+    __syncthreads();
+    if (last) {
+        for (int d = 16; d > 0; d >>= 1) {
+            acc.x += __shfl_xor_sync(0xffffffffu, acc.x, d);
+            acc.y += __shfl_xor_sync(0xffffffffu, acc.y, d);
+        }
+    }
+    if (c || i == gs - 1) red[c] = acc;
+    __syncthreads();
+    cd* o = loc + (int64_t)rhs * A.ncoef + A.eoff[b];
+    for (int q = threadIdx.x; q < nc; q += blockDim.x) {
+        cd v = sm[ng * nc + q];
+        for (int j = 1; j < ng; ++j) v += sm[(ng + j) * nc + q];
+        o[q] = v;
+    }
+}
 
-template <int KER>
-__global__ void k_m2l(M2LArgs A, int first_box, const cd* __restrict__ mp, cd* __restrict__ loc) {
+// Helmholtz M2L of orders beyond the chunked kernel's block: one block per box
+__global__ void k_m2l_helm(M2LArgs A, int first_box, const cd* __restrict__ mp, cd* __restrict__ loc) {
     extern __shared__ cd sm[];
     int b = first_box + blockIdx.x;
     int rhs = blockIdx.y;
@@ -488,68 +639,20 @@ __global__ void k_m2l(M2LArgs A, int first_box, const cd* __restrict__ mp, cd* _
     int nc = 2 * P + 1;
     cd* acc = sm;
     cd* src = sm + nc;
-    cd* tb = src + nc;     // 4P+1 (Helmholtz) or 2*(2P+1) powers + log (Laplace)
+    cd* tb = src + nc;     // 4P+1
     for (int c = threadIdx.x; c < nc; c += blockDim.x) acc[c] = cd{0, 0};
     for (int q = A.loff[b]; q < A.loff[b + 1]; ++q) {
         int s = A.lent[q];
         __syncthreads();
         const cd* m = mp + (int64_t)rhs * A.ncoef + A.eoff[s];
         for (int c = threadIdx.x; c < nc; c += blockDim.x) src[c] = m[c];
-        if (KER == CFMM_LAPLACE) {
-            // inverse powers of zeta0, eta0 (a = c_s - c_t), j = 0..2P, and log r0
-            cd a0 = {A.cre[2 * s] - A.cre[2 * b], A.cim[2 * s] - A.cim[2 * b]};
-            cd a1 = {A.cre[2 * s + 1] - A.cre[2 * b + 1], A.cim[2 * s + 1] - A.cim[2 * b + 1]};
-            cd z, e;
-            zeta_eta(a0, a1, z, e);
-            cd iz = cinv(z), ie = cinv(e);
-            for (int j = threadIdx.x; j <= 2 * P; j += blockDim.x) {
-                // binary powering
-                cd pz = {1, 0}, pe = {1, 0}, bz = iz, be = ie;
-                int ee = j;
-                while (ee) {
-                    if (ee & 1) {
-                        pz = pz * bz;
-                        pe = pe * be;
-                    }
-                    bz = bz * bz;
-                    be = be * be;
-                    ee >>= 1;
-                }
-                tb[j] = pz;
-                tb[2 * P + 1 + j] = pe;
-            }
-            if (threadIdx.x == 0) tb[4 * P + 2] = 0.5 * clog_p(z * e);
-        } else {
-            const cd* t = A.tab + A.tbase[l] + (int64_t)(q - A.tq0[l]) * (4 * P + 1);
-            for (int c = threadIdx.x; c < 4 * P + 1; c += blockDim.x) tb[c] = t[c];
-        }
+        const cd* t = A.tab + A.tbase[l] + (int64_t)(q - A.tq0[l]) * (4 * P + 1);
+        for (int c = threadIdx.x; c < 4 * P + 1; c += blockDim.x) tb[c] = t[c];
         __syncthreads();
         for (int c = threadIdx.x; c < nc; c += blockDim.x) {
             cd a = acc[c];
-            if (KER == CFMM_LAPLACE) {
-                const cd* zi = tb;             // zeta0^-j
-                const cd* ei = tb + 2 * P + 1; // eta0^-j
-                if (c == 0) {
-                    a += tb[4 * P + 2] * src[0];
-                    for (int nn = 1; nn <= P; ++nn) {
-                        cd t = ei[nn] * src[nn] + zi[nn] * src[P + nn];
-                        a += (nn & 1) ? -t : t;
-                    }
-                } else {
-                    bool ise = c > P;                 // Lm (eta) from Mp; Lp (zeta) from Mm
-                    int k = ise ? c - P : c;
-                    const cd* pk = ise ? ei : zi;
-                    a += (-0.5 / k) * pk[k] * src[0];
-                    for (int nn = 1; nn <= P; ++nn) {
-                        cd mn = ise ? src[nn] : src[P + nn];
-                        cd t = binom_at_m2l(A, nn + k - 1, k) * (pk[nn + k] * mn);
-                        a += (nn & 1) ? -t : t;
-                    }
-                }
-            } else {
-                int j = c - P;
-                for (int nn = -P; nn <= P; ++nn) a = cmac(a, tb[nn - j + 2 * P], src[nn + P]);
-            }
+            int j = c - P;
+            for (int nn = -P; nn <= P; ++nn) a = cmac(a, tb[nn - j + 2 * P], src[nn + P]);
             acc[c] = a;
         }
     }
@@ -642,7 +745,7 @@ __global__ void k_eval(ExpArgs A, const int* __restrict__ leaves, const int* __r
     int P = A.Plev[A.blevel[b]];
     int nc = 2 * P + 1;
     cd* coef = sm;                                  // 2*maxP+1
-    cd* rows = sm + 2 * maxP + 1;                   // per thread: maxP+2 (Helmholtz L2P)
+    cd* rows = sm + 2 * maxP + 1;                   // per thread: maxP+2 (Helmholtz L2P), 1 (M2P)
     int s0 = A.bst[b], s1 = A.ben[b];
     for (int t0 = s0; t0 < s1; t0 += blockDim.x) {
         int i = t0 + threadIdx.x;
@@ -653,45 +756,55 @@ __global__ void k_eval(ExpArgs A, const int* __restrict__ leaves, const int* __r
             x1 = cd{A.xr[A.n + i], A.xi[A.n + i]};
         }
         cd acc = {0, 0};
-        // M2P over List 3
-        for (int q = l3off[b]; q < l3off[b + 1]; ++q) {
-            int s = l3[q];
-            int Ps = A.Plev[A.blevel[s]];
-            int ns = 2 * Ps + 1;
-            __syncthreads();
-            const cd* m = mp + (int64_t)rhs * A.ncoef + A.eoff[s];
-            for (int c = threadIdx.x; c < ns; c += blockDim.x) coef[c] = m[c];
-            __syncthreads();
-            if (!valid) continue;
-            cd z, e;
-            zeta_eta(x0 - cd{A.cre[2 * s], A.cim[2 * s]}, x1 - cd{A.cre[2 * s + 1], A.cim[2 * s + 1]}, z, e);
-            if (KER == CFMM_LAPLACE) {
-                acc += (0.5 * clog_p(z * e)) * coef[0];
-                cd iz = cinv(z), ie = cinv(e), zp = iz, ep = ie;
-                for (int nn = 1; nn <= Ps; ++nn) {
-                    acc += coef[nn] * ep + coef[Ps + nn] * zp;
-                    zp = zp * iz;
-                    ep = ep * ie;
-                }
-            } else {
-                // S_n(x - c) by forward recurrence in registers
-                cd r = csqrt_p(z * e);
-                cd zz = A.kappa * r;
-                cd h0, h1;
-                hankel01(zz, &h0, &h1);
-                cd ir = cinv(r), uu = z * ir, vv = e * ir, zi = cinv(zz);
-                acc += coef[Ps] * h0;
-                cd hm = h0, hn = h1, up = uu, vp = vv;
-                for (int nn = 1; nn <= Ps; ++nn) {
-                    cd neg = (nn & 1) ? -hn : hn;
-                    acc = cmac(cmac(acc, coef[Ps + nn], hn * up), coef[Ps - nn], neg * vp);
-                    cd hp = rmac(-hm, 2.0 * nn, zi * hn);
-                    hm = hn;
-                    hn = hp;
-                    up = up * uu;
-                    vp = vp * vv;
+        // M2P over List 3: items (entry, target), a thread each, so that the entries
+        // of a leaf of few points (a chain of 700 FP64 instructions each) run side by
+        // side; a target adds its items in list order
+        const int nt = min((int)blockDim.x, s1 - t0), q0 = l3off[b], items = (l3off[b + 1] - q0) * nt;
+        for (int base = 0; base < items; base += blockDim.x) {
+            const int item = base + threadIdx.x;
+            cd v = {0, 0};
+            if (item < items) {
+                const int s = l3[q0 + item / nt], it = t0 + item % nt, Ps = A.Plev[A.blevel[s]];
+                const cd* m = mp + (int64_t)rhs * A.ncoef + A.eoff[s];
+                cd z, e;
+                zeta_eta(cd{A.xr[it], A.xi[it]} - cd{A.cre[2 * s], A.cim[2 * s]},
+                         cd{A.xr[A.n + it], A.xi[A.n + it]} - cd{A.cre[2 * s + 1], A.cim[2 * s + 1]}, z, e);
+                if (KER == CFMM_LAPLACE) {
+                    // Horner in 1/eta and 1/zeta
+                    cd iz = crcp64(z), ie = crcp64(e), vz = m[2 * Ps], ve = m[Ps];
+                    for (int nn = Ps - 1; nn >= 1; --nn) {
+                        ve = cmac(m[nn], ve, ie);
+                        vz = cmac(m[Ps + nn], vz, iz);
+                    }
+                    v = cmac(cmac((0.5 * clog64(A.H.T, z * e)) * m[0], ve, ie), vz, iz);
+                } else {
+                    // S_n(x - c) by forward recurrence in registers
+                    cd r = csqrt_p(z * e);
+                    cd zz = A.kappa * r;
+                    cd h0, h1;
+                    hankel01_r2(A.H, z * e, &h0, &h1);
+                    cd ir = cinv(r), uu = z * ir, vv = e * ir, zi = cinv(zz);
+                    v = m[Ps] * h0;
+                    cd hm = h0, hn = h1, up = uu, vp = vv;
+                    for (int nn = 1; nn <= Ps; ++nn) {
+                        cd neg = (nn & 1) ? -hn : hn;
+                        v = cmac(cmac(v, m[Ps + nn], hn * up), m[Ps - nn], neg * vp);
+                        cd hp = rmac(-hm, 2.0 * nn, zi * hn);
+                        hm = hn;
+                        hn = hp;
+                        up = up * uu;
+                        vp = vp * vv;
+                    }
                 }
             }
+            __syncthreads();
+            rows[threadIdx.x] = v;
+            __syncthreads();
+            // the pass's items of this target: base + k with (base + k) % nt == its index
+            if ((int)threadIdx.x < nt)
+                for (int k = ((int)threadIdx.x - base % nt + nt) % nt; k < (int)blockDim.x && base + k < items; k += nt)
+                    acc += rows[k];
+            __syncthreads();
         }
         if (!do_l2p) {
             // M2P only (the L2P runs in complex64): leaves without List 3 add nothing
@@ -707,13 +820,12 @@ __global__ void k_eval(ExpArgs A, const int* __restrict__ leaves, const int* __r
             cd z, e;
             zeta_eta(x0 - cd{A.cre[2 * b], A.cim[2 * b]}, x1 - cd{A.cre[2 * b + 1], A.cim[2 * b + 1]}, z, e);
             if (KER == CFMM_LAPLACE) {
-                acc += coef[0];
-                cd zp = z, ep = e;
-                for (int nn = 1; nn <= P; ++nn) {
-                    acc += coef[nn] * zp + coef[P + nn] * ep;
-                    zp = zp * z;
-                    ep = ep * e;
+                cd vz = coef[P], ve = coef[2 * P];
+                for (int nn = P - 1; nn >= 1; --nn) {
+                    vz = cmac(coef[nn], vz, z);
+                    ve = cmac(coef[P + nn], ve, e);
                 }
+                acc += cmac(cmac(coef[0], vz, z), ve, e);
             } else if (lrow) {
                 // T_k(x - c) = (-1)^k T_k(c - x), the plan's row of this point
                 const cd* t = lrow + (int64_t)i * RL + (P + 1);
@@ -802,7 +914,7 @@ __global__ void k_eval_grad(ExpArgs A, const int* __restrict__ leaves, const int
                     ep = ep * ie;
                 }
             } else {
-                cyl_row(1, z, e, A.kappa, Ps, row);          // S_n, n = -Ps-1..Ps+1
+                cyl_row(1, z, e, A.H, Ps, row);          // S_n, n = -Ps-1..Ps+1
                 for (int nn = -Ps; nn <= Ps; ++nn) {
                     cd c = coef[Ps + nn];
                     dz = cmac(dz, c, row[nn + Ps + 1 - 1]);
@@ -827,7 +939,7 @@ __global__ void k_eval_grad(ExpArgs A, const int* __restrict__ leaves, const int
                 ep = ep * e;
             }
         } else {
-            cyl_row(0, z, e, A.kappa, P, row);               // G_n, n = -P-1..P+1
+            cyl_row(0, z, e, A.H, P, row);               // G_n, n = -P-1..P+1
             for (int nn = -P; nn <= P; ++nn) {
                 cd c = coef[P + nn];
                 lz = cmac(lz, c, row[nn + P + 1 - 1]);
@@ -935,7 +1047,7 @@ __global__ void __launch_bounds__(kExpThreads) k_l2p2f(ExpArgs A, const int* __r
 __global__ void k_tab_m2l(int nq, const int* __restrict__ qbox, const int* __restrict__ lent,
                           const int* __restrict__ blevel, const int* __restrict__ Plev, const int64_t* __restrict__ tbase,
                           const int* __restrict__ tq0, const double* __restrict__ cre, const double* __restrict__ cim,
-                          double kappa, cd* __restrict__ tab, int q_first) {
+                          HankelArgs H, cd* __restrict__ tab, int q_first) {
     int qi = blockIdx.x * blockDim.x + threadIdx.x;
     if (qi >= nq) return;
     int q = q_first + qi;
@@ -948,9 +1060,9 @@ __global__ void k_tab_m2l(int nq, const int* __restrict__ qbox, const int* __res
     zeta_eta(cd{cre[2 * b] - cre[2 * s], cim[2 * b] - cim[2 * s]},
              cd{cre[2 * b + 1] - cre[2 * s + 1], cim[2 * b + 1] - cim[2 * s + 1]}, z, e);
     cd r = csqrt_p(z * e);
-    cd zz = kappa * r;
+    cd zz = H.w.k * r;
     cd h0, h1;
-    hankel01(zz, &h0, &h1);
+    hankel01_r2(H, z * e, &h0, &h1);
     cd ir = cinv(r), uu = z * ir, vv = e * ir, zi = cinv(zz);
     int M = 2 * P;
     t[M] = h0;
@@ -1079,9 +1191,12 @@ static int nterms_helm2d(int k, double eps, double kappa, double w) {
 constexpr double kPHeadroom = 0.1;
 constexpr double kPHeadroomHelm = 0.01;
 
+static HankelArgs hankel_args(double kappa) { return HankelArgs{pair_tab_device(), make_wave(kappa)}; }
+
 // First part of the setup, run before the lists are built: orders, offsets,
-// the leaves and (Helmholtz) the per-point row table, launched on the side
-// stream so that it overlaps the construction of the lists.
+// the leaves and (Helmholtz) the per-point row table and the children's shift
+// tables, launched on the side stream so that they overlap the construction of the
+// lists.
 void fmm2d_presetup(cfmm_plan_s* P) {
     TreeDev& T = P->tree;
     cudaStream_t st = P->stream;
@@ -1146,15 +1261,36 @@ void fmm2d_presetup(cfmm_plan_s* P) {
     S->d_leaves_l0.alloc(S->leaves_l0.size());
     upload(S->d_leaves_l0.get(), S->leaves_l0.data(), sizeof(int) * S->leaves_l0.size(), st);
     pt.mark("setup:leaves");
-    if (P->kernel == CFMM_HELMHOLTZ && !S->leaves_l0.empty()) {
-        // on the side stream, beside the lists and the translation tables
+    if (P->kernel == CFMM_HELMHOLTZ) {   // (a tree of several boxes has leaves below l0)
+        // on the side stream, beside the lists: the rows and the shift tables
         S->RL = 2 * S->maxP_leaf + 3;
         S->lrow.alloc((size_t)P->n * S->RL);
         S->rows_side = true;
-        k_leaf_rows<<<(unsigned)S->leaves_l0.size(), 64, 0, near_fork(P)>>>(
+        // (its offsets are uploaded on the plan's stream, before the fork)
+        std::vector<int64_t> so(T.nboxes, -1);
+        int64_t sb = 0;
+        for (int l = S->l0 + 1; l < T.nlevels; ++l)
+            for (int b = T.level_off[l]; b < T.level_off[l + 1]; ++b) {
+                so[b] = sb;
+                sb += 2 * (S->Plev[l] + S->Plev[l - 1]) + 1;
+            }
+        S->t_shift.alloc(sb > 0 ? sb : 1);
+        S->shift_off.alloc(T.nboxes);
+        upload(S->shift_off.get(), so.data(), sizeof(int64_t) * T.nboxes, st);
+        cudaStream_t side = near_fork(P);
+        if (!S->leaves_l0.empty())
+            k_leaf_rows<<<(unsigned)S->leaves_l0.size(), 64, 0, side>>>(
             S->d_leaves_l0.get(), T.level.get(), T.start.get(), T.end.get(), S->dPlev.get(), P->xr.get(),
-            P->xi.get(), P->n, T.cen_re.get(), T.cen_im.get(), P->kappa, S->RL, S->lrow.get());
+            P->xi.get(), P->n, T.cen_re.get(), T.cen_im.get(), hankel_args(P->kappa), S->RL, S->lrow.get());
         CFMM_LAUNCHED();
+        // translation tables of the child boxes (levels > l0)
+        int lo = T.level_off[std::min(S->l0 + 1, T.nlevels)], hi = T.nboxes;
+        if (hi > lo) {
+            k_tab_shift<<<(hi - lo + 31) / 32, 32, 0, side>>>(lo, hi, T.parent.get(), T.level.get(), S->dPlev.get(),
+                                                             S->shift_off.get(), T.cen_re.get(), T.cen_im.get(),
+                                                             P->kappa, S->t_shift.get());
+            CFMM_LAUNCHED();
+        }
     }
 }
 
@@ -1193,6 +1329,19 @@ void fmm2d_setup(cfmm_plan_s* P) {
         S->binom.alloc(bt.size());
         // (a copy from pageable memory returns once the source is staged)
         upload(S->binom.get(), bt.data(), sizeof(double) * bt.size(), st);
+        if (P->kernel == CFMM_LAPLACE) {
+            size_t w = maxP + 1;
+            std::vector<double> a(w * w, 0.0), c(w * w, 0.0);
+            for (int n = 1; n <= maxP; ++n)
+                for (int k = 1; k <= maxP; ++k) {
+                    if (n <= k) a[n * w + k] = bt[(size_t)(k - 1) * (NB + 1) + n - 1];
+                    c[n * w + k] = bt[(size_t)(n + k - 1) * (NB + 1) + k];
+                }
+            S->cm2m.alloc(a.size());
+            S->cm2l.alloc(c.size());
+            upload(S->cm2m.get(), a.data(), sizeof(double) * a.size(), st);
+            upload(S->cm2l.get(), c.data(), sizeof(double) * c.size(), st);
+        }
     }
     if (P->kernel == CFMM_HELMHOLTZ) {
         // M2L tables, level-major like List 2 itself
@@ -1224,7 +1373,7 @@ void fmm2d_setup(cfmm_plan_s* P) {
             // every SM instead of filling a fraction of them with larger blocks
             k_tab_m2l<<<(nq + 31) / 32, 32, 0, st>>>(nq, dq, T.lent[1].get(), T.level.get(), S->dPlev.get(),
                                                        S->d_m2l_base.get(), S->d_m2l_q0.get(), T.cen_re.get(),
-                                                       T.cen_im.get(), P->kappa, S->t_m2l.get(), qf);
+                                                       T.cen_im.get(), hankel_args(P->kappa), S->t_m2l.get(), qf);
             CFMM_LAUNCHED();
         }
         pt.mark("setup:m2ltab");
@@ -1268,32 +1417,12 @@ void fmm2d_setup(cfmm_plan_s* P) {
             upload(S->box_chunk0.get(), bc0.data(), sizeof(int) * (T.nboxes + 1), st);
         }
         pt.mark("setup:chunks");
-        // shift tables for boxes at levels > l0
-        std::vector<int64_t> so(T.nboxes, -1);
-        int64_t sb = 0;
-        for (int l = S->l0 + 1; l < T.nlevels; ++l)
-            for (int b = T.level_off[l]; b < T.level_off[l + 1]; ++b) {
-                so[b] = sb;
-                sb += 2 * (S->Plev[l] + S->Plev[l - 1]) + 1;
-            }
-        S->t_shift.alloc(sb > 0 ? sb : 1);
-        S->shift_off.alloc(T.nboxes);
-        upload(S->shift_off.get(), so.data(), sizeof(int64_t) * T.nboxes, st);
-        int lo = T.level_off[std::min(S->l0 + 1, T.nlevels)], hi = T.nboxes;
-        if (hi > lo) {
-            k_tab_shift<<<(hi - lo + 31) / 32, 32, 0, st>>>(lo, hi, T.parent.get(), T.level.get(), S->dPlev.get(),
-                                                           S->shift_off.get(), T.cen_re.get(), T.cen_im.get(),
-                                                           P->kappa, S->t_shift.get());
-            CFMM_LAUNCHED();
-        }
     }
-    pt.mark("setup:shift");
     if (S->rows_side) near_join(P);
     pt.mark("setup:rowsjoin");
     for (auto f : {(const void*)k_point_to_exp<CFMM_LAPLACE>, (const void*)k_point_to_exp<CFMM_HELMHOLTZ>,
-                   (const void*)k_m2m<CFMM_LAPLACE>, (const void*)k_m2m<CFMM_HELMHOLTZ>,
-                   (const void*)k_l2l<CFMM_LAPLACE>, (const void*)k_l2l<CFMM_HELMHOLTZ>,
-                   (const void*)k_m2l<CFMM_LAPLACE>, (const void*)k_m2l<CFMM_HELMHOLTZ>,
+                   (const void*)k_m2m_lap, (const void*)k_m2m_helm, (const void*)k_l2l_lap, (const void*)k_l2l_helm,
+                   (const void*)k_m2l_lap, (const void*)k_m2l_helm,
                    (const void*)k_m2l_chunk,
                    (const void*)k_eval<CFMM_LAPLACE>, (const void*)k_eval<CFMM_HELMHOLTZ>,
                    (const void*)k_eval_grad<CFMM_LAPLACE>, (const void*)k_eval_grad<CFMM_HELMHOLTZ>})
@@ -1328,7 +1457,7 @@ static void apply_t(cfmm_plan_s* P, Fmm2dState* S, const cd* sigma, const cd* ta
     cd* lc = P->local.get();
     ExpArgs A{P->xr.get(), P->xi.get(), P->nr.get(), P->ni.get(), P->n, sigma, tau, dstride, P->slp, P->dlp,
               P->kappa, T.level.get(), T.start.get(), T.end.get(), T.cen_re.get(), T.cen_im.get(),
-              S->dPlev.get(), S->exp_off.get(), S->ncoef};
+              S->dPlev.get(), S->exp_off.get(), S->ncoef, hankel_args(P->kappa)};
     int maxP = S->maxP;
     // (3) P2P over List 1 (writes u) on the side stream, beside the far field
     {
@@ -1345,10 +1474,10 @@ static void apply_t(cfmm_plan_s* P, Fmm2dState* S, const cd* sigma, const cd* ta
         int PL = S->maxP_leaf;
         int R = KER == CFMM_LAPLACE ? 2 * PL + 1 : 2 * PL + 3;
         int chunk = std::max(1, std::min(kExpThreads, (int)((96 * 1024) / ((R + 3) * sizeof(cd)))));
-        size_t smem = sizeof(cd) * ((size_t)(2 * PL + 1) + (size_t)chunk * (R + 3));
+        size_t smem = sizeof(cd) * (p2e_acc(PL) + (size_t)chunk * (R + 3));
         dim3 g((unsigned)S->leaves_l0.size(), nrhs);
         if (g.x) {
-            k_point_to_exp<KER><<<g, kExpThreads, smem, st>>>(A, S->d_leaves_l0.get(), nullptr, nullptr, 0, mp, chunk,
+            k_point_to_exp<KER><<<g, kP2eThreads, smem, st>>>(A, S->d_leaves_l0.get(), nullptr, nullptr, 0, mp, chunk,
                                                              S->lrow.get(), S->RL);
             CFMM_LAUNCHED();
         }
@@ -1358,20 +1487,29 @@ static void apply_t(cfmm_plan_s* P, Fmm2dState* S, const cd* sigma, const cd* ta
     TransArgs TA{T.level.get(), T.parent.get(), T.cbeg.get(), T.cend.get(), T.cen_re.get(), T.cen_im.get(),
                  S->dPlev.get(), S->exp_off.get(), S->ncoef, S->binom.get(), S->NB, S->t_shift.get(),
                  S->shift_off.get()};
+    // Helmholtz: parts of a coefficient's sum, threads of a block
+    auto split = [](int nc) { return std::max(1, std::min(8, 512 / nc)); };
+    auto threads = [](int nc, int S2) { return std::min(512, (nc * S2 + 31) / 32 * 32); };
     for (int l = T.nlevels - 2; l >= S->l0; --l) {
         int lo = T.level_off[l], nb = T.level_off[l + 1] - lo;
         int Pp = S->Plev[l], Pc = S->Plev[l + 1];
-        size_t smem = sizeof(cd) * ((2 * Pp + 1) + (2 * Pc + 1) + 2 * (Pc + Pp) + 2);
         dim3 g(nb, nrhs);
-        k_m2m<KER><<<g, kExpThreads, smem, st>>>(TA, lo, mp, mp, T.leaf.get());
+        if (KER == CFMM_LAPLACE) {
+            const int ng = 2;
+            k_m2m_lap<<<g, ng * lap_group(Pp), sizeof(cd) * 2 * ng * (2 * Pp + 1), st>>>(TA, lo, mp, mp, T.leaf.get(),
+                                                                                      Pp, S->cm2m.get());
+        } else {
+            const int S2 = split(2 * Pp + 1);
+            k_m2m_helm<<<g, threads(2 * Pp + 1, S2), sizeof(cd) * ((2 * Pc + 1) + 2 * (Pc + Pp) + 1 + S2 * (2 * Pp + 1)),
+                         st>>>(TA, lo, mp, mp, T.leaf.get(), Pc, Pp, S2);
+        }
         CFMM_LAUNCHED();
     }
     rec(3);
     // (4) M2L over List 2 (all levels >= l0)
     {
         M2LArgs MA{T.level.get(), T.cen_re.get(), T.cen_im.get(), S->dPlev.get(), S->exp_off.get(), S->ncoef,
-                   T.loff[1].get(), T.lent[1].get(), S->binom.get(), S->NB, S->t_m2l.get(), S->d_m2l_base.get(),
-                   S->d_m2l_q0.get()};
+                   T.loff[1].get(), T.lent[1].get(), S->t_m2l.get(), S->d_m2l_base.get(), S->d_m2l_q0.get()};
         int first = T.level_off[S->l0], nb = T.nboxes - first;
         if (KER == CFMM_HELMHOLTZ && maxP <= 255) {
             // chunks of List-2 entries, one launch per level (P fixed per level), then
@@ -1400,8 +1538,14 @@ static void apply_t(cfmm_plan_s* P, Fmm2dState* S, const cd* sigma, const cd* ta
             }
         } else {
             dim3 g(nb, nrhs);
-            size_t smem = sizeof(cd) * (2 * (2 * maxP + 1) + 4 * maxP + 3);
-            k_m2l<KER><<<g, 128, smem, st>>>(MA, first, mp, lc);
+            if (KER == CFMM_LAPLACE) {
+                const int ng = 3;
+                k_m2l_lap<<<g, ng * lap_group(maxP), sizeof(cd) * 2 * ng * (2 * maxP + 1), st>>>(
+                    MA, first, mp, lc, maxP, S->cm2l.get(), pair_tab_device());
+            } else {
+                size_t smem = sizeof(cd) * (2 * (2 * maxP + 1) + 4 * maxP + 3);
+                k_m2l_helm<<<g, 128, smem, st>>>(MA, first, mp, lc);
+            }
             CFMM_LAUNCHED();
         }
     }
@@ -1410,10 +1554,10 @@ static void apply_t(cfmm_plan_s* P, Fmm2dState* S, const cd* sigma, const cd* ta
     {
         int R = KER == CFMM_LAPLACE ? 2 * maxP + 1 : 2 * maxP + 3;
         int chunk = std::max(1, std::min(kExpThreads, (int)((96 * 1024) / ((R + 3) * sizeof(cd)))));
-        size_t smem = sizeof(cd) * ((size_t)(2 * maxP + 1) + (size_t)chunk * (R + 3));
+        size_t smem = sizeof(cd) * (p2e_acc(maxP) + (size_t)chunk * (R + 3));
         if (S->n_p2l > 0) {
             dim3 g(S->n_p2l, nrhs);
-            k_point_to_exp<KER><<<g, kExpThreads, smem, st>>>(A, S->d_p2l_boxes.get(), T.loff[3].get(),
+            k_point_to_exp<KER><<<g, kP2eThreads, smem, st>>>(A, S->d_p2l_boxes.get(), T.loff[3].get(),
                                                              T.lent[3].get(), 1, lc, chunk, nullptr, 0);
             CFMM_LAUNCHED();
         }
@@ -1423,9 +1567,14 @@ static void apply_t(cfmm_plan_s* P, Fmm2dState* S, const cd* sigma, const cd* ta
     for (int l = S->l0 + 1; l < T.nlevels; ++l) {
         int lo = T.level_off[l], nb = T.level_off[l + 1] - lo;
         int Pp = S->Plev[l - 1], Pc = S->Plev[l];
-        size_t smem = sizeof(cd) * ((2 * Pp + 1) + 2 * (Pc + Pp) + 2);
         dim3 g(nb, nrhs);
-        k_l2l<KER><<<g, kExpThreads, smem, st>>>(TA, lo, lc);
+        if (KER == CFMM_LAPLACE) {
+            k_l2l_lap<<<g, lap_group(Pc), sizeof(cd) * (4 * Pc + 1), st>>>(TA, lo, lc, Pc);
+        } else {
+            const int S2 = split(2 * Pc + 1);
+            k_l2l_helm<<<g, threads(2 * Pc + 1, S2), sizeof(cd) * ((2 * Pp + 1) + 2 * (Pc + Pp) + 1 + S2 * (2 * Pc + 1)),
+                         st>>>(TA, lo, lc, Pp, Pc, S2);
+        }
         CFMM_LAUNCHED();
     }
     rec(6);
@@ -1434,7 +1583,7 @@ static void apply_t(cfmm_plan_s* P, Fmm2dState* S, const cd* sigma, const cd* ta
     // (5) M2P and (8) L2P (add to u; L2P in complex64 in mixed precision)
     {
         // with the plan's rows, L2P needs no per-thread row space
-        size_t smem = sizeof(cd) * ((size_t)(2 * maxP + 1) + (S->lrow.get() ? 0 : (size_t)kExpThreads * (maxP + 2)));
+        size_t smem = sizeof(cd) * ((size_t)(2 * maxP + 1) + (size_t)kExpThreads * (S->lrow.get() ? 1 : maxP + 2));
         dim3 gr((unsigned)S->leaves_l0.size(), nrhs);
         bool l2p32 = P->precision == CFMM_MIXED && S->maxP_leaf <= kL2p2fMaxP;
         k_eval<KER><<<gr, kExpThreads, smem, st>>>(A, S->d_leaves_l0.get(), T.loff[2].get(), T.lent[2].get(), mp, lc,

@@ -86,6 +86,17 @@ void make_pair_tab(PairTab* T) {
     }
 }
 
+const PairTab* pair_tab_device() {
+    void* d = nullptr;
+    CFMM_CUDA(cudaGetSymbolAddress(&d, d_pair));
+    return static_cast<const PairTab*>(d);
+}
+
+Wave make_wave(double k) {
+    if (!(k > 0.0)) return Wave{0.0, 0.0, 0.0, 0.0, 0.0};
+    return Wave{k, 1.0 / k, std::sqrt(1.0 / k), k * 40.74366543152521, k * 369.3299304675746};   // 256/(2 pi), 256/log 2
+}
+
 void upload_lag_rule_p2p() {
     upload_lag_rule_local();
     SeriesTab T = make_series_tab();
@@ -1070,12 +1081,11 @@ __global__ void __launch_bounds__(kP2PThreads) k_p2p32g_h3(KParams K, const int*
 }
 
 static KParams with_wave(KParams K) {
-    if (K.kappa > 0.0) {
-        K.ikappa = 1.0 / K.kappa;
-        K.isqrt_kappa = std::sqrt(K.ikappa);
-        K.kappa_ang = K.kappa * 40.74366543152521;     // 256/(2 pi)
-        K.kappa_exp = K.kappa * 369.3299304675746;     // 256/log 2
-    }
+    Wave w = make_wave(K.kappa);
+    K.ikappa = w.ik;
+    K.isqrt_kappa = w.isk;
+    K.kappa_ang = w.ka;
+    K.kappa_exp = w.kb;
     return K;
 }
 

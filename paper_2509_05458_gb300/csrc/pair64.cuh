@@ -206,6 +206,10 @@ __device__ __forceinline__ cd hankel_factor(const double2* __restrict__ c, cd d)
     return p;
 }
 
+// Device pointer of the current device's tables (p2p.cu), constants of a wavenumber
+const PairTab* pair_tab_device();
+Wave make_wave(double kappa);
+
 // Tables of the current device: the host part (make_pair_tab, p2p.cu) and the
 // Hankel cells (k_pair_hankel).
 void make_pair_tab(PairTab* T);

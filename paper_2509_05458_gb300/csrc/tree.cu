@@ -758,11 +758,9 @@ __global__ void k_leaf_stats(int nb, const int* __restrict__ bleaf, const int* _
     }
 }
 
-__global__ void k_parent_stats(int lo, int hi, const int* __restrict__ bleaf, const int* __restrict__ cbeg,
-                               const int* __restrict__ cend, int dim, double* __restrict__ sum,
-                               double* __restrict__ mn, double* __restrict__ mx) {
-    int b = lo + blockIdx.x * blockDim.x + threadIdx.x;
-    if (b >= hi || bleaf[b]) return;
+__device__ void parent_stats(int b, const int* __restrict__ bleaf, const int* __restrict__ cbeg,
+                             const int* __restrict__ cend, int dim, double* sum, double* mn, double* mx) {
+    if (bleaf[b]) return;
     for (int d = 0; d < dim; ++d) {
         double s = 0.0, a = INFINITY, z = -INFINITY;
         for (int c = cbeg[b]; c < cend[b]; ++c) {
@@ -773,6 +771,26 @@ __global__ void k_parent_stats(int lo, int hi, const int* __restrict__ bleaf, co
         sum[b * dim + d] = s;
         mn[b * dim + d] = a;
         mx[b * dim + d] = z;
+    }
+}
+
+__global__ void k_parent_stats(int lo, int hi, const int* __restrict__ bleaf, const int* __restrict__ cbeg,
+                               const int* __restrict__ cend, int dim, double* sum, double* mn, double* mx) {
+    int b = lo + blockIdx.x * blockDim.x + threadIdx.x;
+    if (b < hi) parent_stats(b, bleaf, cbeg, cend, dim, sum, mn, mx);
+}
+
+// the coarse levels top .. 0 (at most a block's threads of boxes each) one after the
+// other in one block: a launch a level took 7 us each (12 of them in a 100,000-point
+// 2D plan)
+constexpr int kStatsTail = 1024;
+__global__ void k_parent_stats_tail(int top, const int* __restrict__ level_off, const int* __restrict__ bleaf,
+                                    const int* __restrict__ cbeg, const int* __restrict__ cend, int dim, double* sum,
+                                    double* mn, double* mx) {
+    for (int m = top; m >= 0; --m) {
+        for (int b = level_off[m] + threadIdx.x; b < level_off[m + 1]; b += blockDim.x)
+            parent_stats(b, bleaf, cbeg, cend, dim, sum, mn, mx);
+        __syncthreads();
     }
 }
 
@@ -1039,10 +1057,17 @@ static void box_stats(cfmm_plan_s* P, cudaStream_t st, std::vector<double>* spre
     k_leaf_stats<<<blocks_for((int64_t)nb * 32, 256), 256, 0, st>>>(nb, T.leaf.get(), T.start.get(), T.end.get(),
                                                                    P->xi.get(), P->n, dim, sum, mn, mx);
     CFMM_LAUNCHED();
-    for (int m = T.nlevels - 2; m >= 0; --m) {
+    int top = -1;   // coarsest levels of at most kStatsTail boxes
+    while (top + 1 <= T.nlevels - 2 && T.level_off[top + 2] - T.level_off[top + 1] <= kStatsTail) ++top;
+    for (int m = T.nlevels - 2; m > top; --m) {
         int lo = T.level_off[m], hi = T.level_off[m + 1];
         k_parent_stats<<<blocks_for(hi - lo, 128), 128, 0, st>>>(lo, hi, T.leaf.get(), T.cbeg.get(), T.cend.get(),
                                                                 dim, sum, mn, mx);
+        CFMM_LAUNCHED();
+    }
+    if (top >= 0) {
+        k_parent_stats_tail<<<1, kStatsTail, 0, st>>>(top, T.d_level_off.get(), T.leaf.get(), T.cbeg.get(),
+                                                     T.cend.get(), dim, sum, mn, mx);
         CFMM_LAUNCHED();
     }
     T.cen_re.alloc((size_t)nb * dim);
