@@ -434,6 +434,8 @@ static void destroy_plan(cfmm_plan_s* P) {
         if (e) cudaEventDestroy(e);
     for (auto& e : P->ev_p2p)
         if (e) cudaEventDestroy(e);
+    for (auto& e : P->ev_far)
+        if (e) cudaEventDestroy(e);
     if (P->ev_fork) cudaEventDestroy(P->ev_fork);
     if (P->ev_join) cudaEventDestroy(P->ev_join);
     if (P->side) {
@@ -535,6 +537,8 @@ static cfmm_plan_t plan_common(int dim, int kernel, double k, double eps, const 
         for (auto& e : P->ev_p2p) CFMM_CUDA(cudaEventCreate(&e));
         CFMM_CUDA(cudaEventCreateWithFlags(&P->ev_fork, cudaEventDisableTiming));
         CFMM_CUDA(cudaEventCreateWithFlags(&P->ev_join, cudaEventDisableTiming));
+        if (dim == 2)
+            for (auto& e : P->ev_far) CFMM_CUDA(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
         CFMM_CUDA(cudaStreamCreateWithFlags(&P->side, cudaStreamNonBlocking));
         Scratch& scr = plan_scratch();
         scr.rewind();

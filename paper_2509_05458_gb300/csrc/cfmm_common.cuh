@@ -322,6 +322,7 @@ struct cfmm_plan_s {
     // evaluated into the same output
     cudaStream_t side = nullptr;
     cudaEvent_t ev_fork = nullptr, ev_join = nullptr, ev_p2p[2] = {};
+    cudaEvent_t ev_far[2] = {};      // far-field work on the side stream (2D): P2L done, multipoles ready
     bool p2p_side = false;           // the last apply ran the near field on `side`
     bool p2p_serial = false;         // the last apply ran it in line (timing mode 2)
     // captured apply

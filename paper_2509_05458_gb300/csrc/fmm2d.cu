@@ -88,9 +88,9 @@ struct Fmm2dState {
     int n_p2l = 0;                         // boxes with a non-empty List 4
     DevBuf<int> d_p2l_boxes;
     // Helmholtz M2L work split: chunks of at most kM2LChunk List-2 entries
-    std::vector<int> lvl_chunk0;           // per level: first chunk (levels >= l0), size nlev+1
-    std::vector<int64_t> lvl_part0;        // per level: first partial-sum slot (complex units)
     DevBuf<int> chunk_box, chunk_q0, chunk_q1, box_chunk0;   // box_chunk0: [nboxes+1]
+    DevBuf<int64_t> chunk_part;            // per chunk: its partial sum's first slot
+    int nchunk = 0;
     int64_t npart = 0;                     // partial-sum slots per rhs
     DevBuf<cd> part;
 };
@@ -574,7 +574,7 @@ struct M2LArgs {
 // Laplace M2L (see the comment above k_m2m_lap): a block per box, groups of warps
 // side by side on its List-2 entries
 __global__ void k_m2l_lap(M2LArgs A, int first_box, const cd* __restrict__ mp, cd* __restrict__ loc, int P,
-                          const double* __restrict__ cm2l, const PairTab* __restrict__ T) {
+                          const double* __restrict__ cm2l, const PairTab* __restrict__ T, int add) {
     extern __shared__ cd sm[];
     const int b = first_box + blockIdx.x, rhs = blockIdx.y, nc = 2 * P + 1;
     const int gs = lap_group(P), ng = blockDim.x / gs, g = threadIdx.x / gs, i = threadIdx.x - g * gs;
@@ -625,12 +625,12 @@ __global__ void k_m2l_lap(M2LArgs A, int first_box, const cd* __restrict__ mp, c
     for (int q = threadIdx.x; q < nc; q += blockDim.x) {
         cd v = sm[ng * nc + q];
         for (int j = 1; j < ng; ++j) v += sm[(ng + j) * nc + q];
-        o[q] = v;
+        o[q] = add ? o[q] + v : v;
     }
 }
 
 // Helmholtz M2L of orders beyond the chunked kernel's block: one block per box
-__global__ void k_m2l_helm(M2LArgs A, int first_box, const cd* __restrict__ mp, cd* __restrict__ loc) {
+__global__ void k_m2l_helm(M2LArgs A, int first_box, const cd* __restrict__ mp, cd* __restrict__ loc, int add) {
     extern __shared__ cd sm[];
     int b = first_box + blockIdx.x;
     int rhs = blockIdx.y;
@@ -658,7 +658,7 @@ __global__ void k_m2l_helm(M2LArgs A, int first_box, const cd* __restrict__ mp, 
     }
     __syncthreads();
     cd* o = loc + (int64_t)rhs * A.ncoef + A.eoff[b];
-    for (int c = threadIdx.x; c < nc; c += blockDim.x) o[c] = acc[c];
+    for (int c = threadIdx.x; c < nc; c += blockDim.x) o[c] = add ? o[c] + acc[c] : acc[c];
 }
 
 // Helmholtz M2L split into chunks of List-2 entries: one CTA per chunk, thread
@@ -668,15 +668,21 @@ __global__ void k_m2l_helm(M2LArgs A, int first_box, const cd* __restrict__ mp, 
 // of the top level are spread over many CTAs).
 constexpr int kM2LChunk = 32;
 
-__global__ void k_m2l_chunk(M2LArgs A, int ch0, const int* __restrict__ chunk_box, const int* __restrict__ cq0,
-                            const int* __restrict__ cq1, int P, int S, cd* __restrict__ part, int64_t part_stride,
-                            const cd* __restrict__ mp) {
+// All levels share one launch (the orders and so the split over S come from the
+// box's level): the coarse levels' few, long blocks run beside the fine levels'.
+__host__ __device__ inline int m2l_lanes(int nc, int threads) { return nc > threads ? 1 : threads / nc < 8 ? threads / nc : 8; }
+
+__global__ void k_m2l_chunk(M2LArgs A, const int* __restrict__ chunk_box, const int* __restrict__ cq0,
+                            const int* __restrict__ cq1, const int64_t* __restrict__ cpart, cd* __restrict__ part,
+                            int64_t part_stride, const cd* __restrict__ mp) {
     extern __shared__ cd sm[];
-    int ch = ch0 + blockIdx.x;
+    int ch = blockIdx.x;
     int rhs = blockIdx.y;
     int b = chunk_box[ch];
     int l = A.blevel[b];
+    const int P = A.Plev[l];
     int nc = 2 * P + 1, nt = 4 * P + 1;
+    const int S = m2l_lanes(nc, blockDim.x);
     int t = threadIdx.x;
     int c = t % nc, sl = t / nc;
     bool act = sl < S;
@@ -713,22 +719,24 @@ __global__ void k_m2l_chunk(M2LArgs A, int ch0, const int* __restrict__ chunk_bo
     if (t < nc) {
         cd v = red[t];
         for (int ss = 1; ss < S; ++ss) v += red[(size_t)ss * nc + t];
-        part[(int64_t)rhs * part_stride + (int64_t)(ch - ch0) * nc + t] = v;
+        part[(int64_t)rhs * part_stride + cpart[ch] + t] = v;
     }
 }
 
-__global__ void k_m2l_reduce(int lo, int nbl, const int* __restrict__ box_chunk0, int ch0, int nc,
+// chunk sums of a box in order, added to what P2L left there (add) or stored
+__global__ void k_m2l_reduce(int first_box, const int* __restrict__ blevel, const int* __restrict__ Plev,
+                             const int* __restrict__ box_chunk0, const int64_t* __restrict__ cpart,
                              const cd* __restrict__ part, int64_t part_stride, const int64_t* __restrict__ eoff,
-                             int64_t ncoef, cd* __restrict__ loc) {
-    int b = lo + blockIdx.x;
+                             int64_t ncoef, int add, cd* __restrict__ loc) {
+    int b = first_box + blockIdx.x;
     int rhs = blockIdx.y;
-    int c0 = box_chunk0[b], c1 = box_chunk0[b + 1];
+    int c0 = box_chunk0[b], c1 = box_chunk0[b + 1], nc = 2 * Plev[blevel[b]] + 1;
     cd* out = loc + (int64_t)rhs * ncoef + eoff[b];
     const cd* pp = part + (int64_t)rhs * part_stride;
     for (int c = threadIdx.x; c < nc; c += blockDim.x) {
         cd v = {0, 0};
-        for (int k = c0; k < c1; ++k) v += pp[(int64_t)(k - ch0) * nc + c];
-        out[c] = v;
+        for (int k = c0; k < c1; ++k) v += pp[cpart[k] + c];
+        out[c] = add ? out[c] + v : v;
     }
 }
 
@@ -1380,12 +1388,9 @@ void fmm2d_setup(cfmm_plan_s* P) {
         // List-2 chunks per box (levels >= l0)
         {
             std::vector<int> cb, c0v, c1v, bc0(T.nboxes + 1, 0);
-            S->lvl_chunk0.assign(T.nlevels + 1, 0);
-            S->lvl_part0.assign(T.nlevels + 1, 0);
+            std::vector<int64_t> cp;
             int64_t pslot = 0;
             for (int l = 0; l < T.nlevels; ++l) {
-                S->lvl_chunk0[l] = (int)cb.size();
-                S->lvl_part0[l] = pslot;
                 // chunks of kM2LChunk entries (shorter chunks fill more SMs at a coarse
                 // top level but spread each block's fixed per-coefficient work over
                 // fewer sources: measured slower)
@@ -1397,22 +1402,24 @@ void fmm2d_setup(cfmm_plan_s* P) {
                         cb.push_back(b);
                         c0v.push_back(q);
                         c1v.push_back(std::min(q + clen, loff[b + 1]));
+                        cp.push_back(pslot);
+                        pslot += 2 * S->Plev[l] + 1;
                     }
                 }
-                if (l >= S->l0) pslot += (int64_t)((int)cb.size() - S->lvl_chunk0[l]) * (2 * S->Plev[l] + 1);
             }
-            S->lvl_chunk0[T.nlevels] = (int)cb.size();
-            S->lvl_part0[T.nlevels] = pslot;
+            S->nchunk = (int)cb.size();
             bc0[T.nboxes] = (int)cb.size();
             S->npart = pslot;
             S->chunk_box.alloc(cb.size());
             S->chunk_q0.alloc(cb.size());
             S->chunk_q1.alloc(cb.size());
+            S->chunk_part.alloc(cb.size());
             S->box_chunk0.alloc(T.nboxes + 1);
             if (!cb.empty()) {
                 upload(S->chunk_box.get(), cb.data(), sizeof(int) * cb.size(), st);
                 upload(S->chunk_q0.get(), c0v.data(), sizeof(int) * cb.size(), st);
                 upload(S->chunk_q1.get(), c1v.data(), sizeof(int) * cb.size(), st);
+                upload(S->chunk_part.get(), cp.data(), sizeof(int64_t) * cp.size(), st);
             }
             upload(S->box_chunk0.get(), bc0.data(), sizeof(int) * (T.nboxes + 1), st);
         }
@@ -1459,9 +1466,42 @@ static void apply_t(cfmm_plan_s* P, Fmm2dState* S, const cd* sigma, const cd* ta
               P->kappa, T.level.get(), T.start.get(), T.end.get(), T.cen_re.get(), T.cen_im.get(),
               S->dPlev.get(), S->exp_off.get(), S->ncoef, hankel_args(P->kappa)};
     int maxP = S->maxP;
+    // (6) P2L over List 4, added to the local expansions
+    auto p2l = [&](cudaStream_t s) {
+        if (S->n_p2l == 0) return;
+        int R = KER == CFMM_LAPLACE ? 2 * maxP + 1 : 2 * maxP + 3;
+        int chunk = std::max(1, std::min(kExpThreads, (int)((96 * 1024) / ((R + 3) * sizeof(cd)))));
+        size_t smem = sizeof(cd) * (p2e_acc(maxP) + (size_t)chunk * (R + 3));
+        k_point_to_exp<KER><<<dim3(S->n_p2l, nrhs), kP2eThreads, smem, s>>>(
+            A, S->d_p2l_boxes.get(), T.loff[3].get(), T.lent[3].get(), 1, lc, chunk, nullptr, 0);
+        CFMM_LAUNCHED();
+    };
+    // (5) M2P over List 3, added to u
+    bool l2p32 = P->precision == CFMM_MIXED && S->maxP_leaf <= kL2p2fMaxP;
+    // P2L and (mixed) M2P are short chains on a few blocks that need nothing of the
+    // M2L: they run on the side stream, P2L into zeroed expansions before the near
+    // field and M2P after it (0.08 and 0.13 of 1.43 ms of a 100,000-point mixed 2D
+    // Helmholtz apply). An FP64 near field of more than 2^21 pairs (1 ms) is itself the
+    // longer branch, and P2L stays in its place.
+    const bool side_work = !(P->timing && P->serial);
+    const bool p2l_first = side_work && S->n_p2l > 0 && (P->precision == CFMM_MIXED || P->p2p_pairs <= (1 << 21));
+    const bool m2p_side = side_work && l2p32 && T.llen[2] > 0;
+    auto eval = [&](cudaStream_t s, int do_l2p) {
+        // with the plan's rows, L2P needs no per-thread row space
+        size_t smem = sizeof(cd) * ((size_t)(2 * maxP + 1) + (size_t)kExpThreads * (S->lrow.get() ? 1 : maxP + 2));
+        dim3 gr((unsigned)S->leaves_l0.size(), nrhs);
+        k_eval<KER><<<gr, kExpThreads, smem, s>>>(A, S->d_leaves_l0.get(), T.loff[2].get(), T.lent[2].get(), mp, lc, u,
+                                                 maxP, S->lrow.get(), S->RL, do_l2p);
+        CFMM_LAUNCHED();
+    };
     // (3) P2P over List 1 (writes u) on the side stream, beside the far field
+    cudaStream_t ns = near_fork(P);
     {
-        cudaStream_t ns = near_fork(P);
+        if (p2l_first) {
+            CFMM_CUDA(cudaMemsetAsync(lc, 0, sizeof(cd) * need, ns));
+            p2l(ns);
+            CFMM_CUDA(cudaEventRecord(P->ev_far[0], ns));
+        }
         launch_p2p(2, KER, K, S->d_leaves_l0.get(), (int)S->leaves_l0.size(), T.start.get(), T.end.get(),
                    T.loff[0].get(), T.lent[0].get(), u, nrhs, false, ns, P->precision == CFMM_MIXED, P->leaf_size);
         if (g)
@@ -1506,62 +1546,52 @@ static void apply_t(cfmm_plan_s* P, Fmm2dState* S, const cd* sigma, const cd* ta
         CFMM_LAUNCHED();
     }
     rec(3);
+    if (m2p_side) {
+        CFMM_CUDA(cudaEventRecord(P->ev_far[1], st));
+        CFMM_CUDA(cudaStreamWaitEvent(ns, P->ev_far[1], 0));
+        eval(ns, 0);
+    }
+    if (p2l_first) CFMM_CUDA(cudaStreamWaitEvent(st, P->ev_far[0], 0));
     // (4) M2L over List 2 (all levels >= l0)
     {
         M2LArgs MA{T.level.get(), T.cen_re.get(), T.cen_im.get(), S->dPlev.get(), S->exp_off.get(), S->ncoef,
                    T.loff[1].get(), T.lent[1].get(), S->t_m2l.get(), S->d_m2l_base.get(), S->d_m2l_q0.get()};
         int first = T.level_off[S->l0], nb = T.nboxes - first;
         if (KER == CFMM_HELMHOLTZ && maxP <= 255) {
-            // chunks of List-2 entries, one launch per level (P fixed per level), then
-            // the per-box reduction of the chunk sums
+            // chunks of List-2 entries, then the per-box reduction of the chunk sums
             P->m2l_part.alloc((size_t)S->npart * nrhs + 1);
             cd* part = P->m2l_part.get();
-            for (int l = S->l0; l < T.nlevels; ++l) {
-                int lo = T.level_off[l], nbl = T.level_off[l + 1] - lo;
-                int ch0 = S->lvl_chunk0[l], nch = S->lvl_chunk0[l + 1] - ch0;
-                if (nbl == 0) continue;
-                int Pl = S->Plev[l], ncl = 2 * Pl + 1;
-                cd* pl = part + S->lvl_part0[l];
-                if (nch > 0) {
-                    int Sl = std::max(1, std::min(8, 256 / ncl));
-                    int threads = ((ncl * Sl + 31) / 32) * 32;
-                    size_t smem = sizeof(cd) * (size_t)Sl * (ncl + 4 * Pl + 1);
-                    dim3 gl(nch, nrhs);
-                    k_m2l_chunk<<<gl, threads, smem, st>>>(MA, ch0, S->chunk_box.get(), S->chunk_q0.get(),
-                                                            S->chunk_q1.get(), Pl, Sl, pl, S->npart, mp);
-                    CFMM_LAUNCHED();
+            if (S->nchunk > 0) {
+                int threads = std::max(256, (2 * maxP + 1 + 31) / 32 * 32);
+                size_t smem = 0;
+                for (int l = S->l0; l < T.nlevels; ++l) {
+                    int ncl = 2 * S->Plev[l] + 1;
+                    smem = std::max(smem, sizeof(cd) * (size_t)m2l_lanes(ncl, threads) * (ncl + 4 * S->Plev[l] + 1));
                 }
-                dim3 gr(nbl, nrhs);
-                k_m2l_reduce<<<gr, 64, 0, st>>>(lo, nbl, S->box_chunk0.get(), ch0, ncl, pl, S->npart,
-                                                S->exp_off.get(), S->ncoef, lc);
+                k_m2l_chunk<<<dim3(S->nchunk, nrhs), threads, smem, st>>>(MA, S->chunk_box.get(), S->chunk_q0.get(),
+                                                                        S->chunk_q1.get(), S->chunk_part.get(), part,
+                                                                        S->npart, mp);
                 CFMM_LAUNCHED();
             }
+            k_m2l_reduce<<<dim3(nb, nrhs), 64, 0, st>>>(first, T.level.get(), S->dPlev.get(), S->box_chunk0.get(),
+                                                       S->chunk_part.get(), part, S->npart, S->exp_off.get(), S->ncoef,
+                                                       p2l_first ? 1 : 0, lc);
+            CFMM_LAUNCHED();
         } else {
             dim3 g(nb, nrhs);
             if (KER == CFMM_LAPLACE) {
                 const int ng = 3;
                 k_m2l_lap<<<g, ng * lap_group(maxP), sizeof(cd) * 2 * ng * (2 * maxP + 1), st>>>(
-                    MA, first, mp, lc, maxP, S->cm2l.get(), pair_tab_device());
+                    MA, first, mp, lc, maxP, S->cm2l.get(), pair_tab_device(), p2l_first ? 1 : 0);
             } else {
                 size_t smem = sizeof(cd) * (2 * (2 * maxP + 1) + 4 * maxP + 3);
-                k_m2l_helm<<<g, 128, smem, st>>>(MA, first, mp, lc);
+                k_m2l_helm<<<g, 128, smem, st>>>(MA, first, mp, lc, p2l_first ? 1 : 0);
             }
             CFMM_LAUNCHED();
         }
     }
     rec(4);
-    // (6) P2L over List 4
-    {
-        int R = KER == CFMM_LAPLACE ? 2 * maxP + 1 : 2 * maxP + 3;
-        int chunk = std::max(1, std::min(kExpThreads, (int)((96 * 1024) / ((R + 3) * sizeof(cd)))));
-        size_t smem = sizeof(cd) * (p2e_acc(maxP) + (size_t)chunk * (R + 3));
-        if (S->n_p2l > 0) {
-            dim3 g(S->n_p2l, nrhs);
-            k_point_to_exp<KER><<<g, kP2eThreads, smem, st>>>(A, S->d_p2l_boxes.get(), T.loff[3].get(),
-                                                             T.lent[3].get(), 1, lc, chunk, nullptr, 0);
-            CFMM_LAUNCHED();
-        }
-    }
+    if (!p2l_first) p2l(st);   // (6)
     rec(5);
     // (7) L2L, coarsest level first
     for (int l = S->l0 + 1; l < T.nlevels; ++l) {
@@ -1582,13 +1612,8 @@ static void apply_t(cfmm_plan_s* P, Fmm2dState* S, const cd* sigma, const cd* ta
     near_join(P);   // the near field has written u
     // (5) M2P and (8) L2P (add to u; L2P in complex64 in mixed precision)
     {
-        // with the plan's rows, L2P needs no per-thread row space
-        size_t smem = sizeof(cd) * ((size_t)(2 * maxP + 1) + (size_t)kExpThreads * (S->lrow.get() ? 1 : maxP + 2));
         dim3 gr((unsigned)S->leaves_l0.size(), nrhs);
-        bool l2p32 = P->precision == CFMM_MIXED && S->maxP_leaf <= kL2p2fMaxP;
-        k_eval<KER><<<gr, kExpThreads, smem, st>>>(A, S->d_leaves_l0.get(), T.loff[2].get(), T.lent[2].get(), mp, lc,
-                                                  u, maxP, S->lrow.get(), S->RL, l2p32 ? 0 : 1);
-        CFMM_LAUNCHED();
+        if (!m2p_side && !(l2p32 && T.llen[2] == 0)) eval(st, l2p32 ? 0 : 1);
         if (l2p32 && gr.x) {
             k_l2p2f<KER><<<gr, kExpThreads, sizeof(cf) * (2 * S->maxP_leaf + 1), st>>>(A, S->d_leaves_l0.get(), lc,
                                                                                         u, P->W);
