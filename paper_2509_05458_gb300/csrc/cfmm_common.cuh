@@ -270,12 +270,23 @@ struct TreeDev {
     DevBuf<int> level, start, end, parent, cbeg, cend, leaf;
     DevBuf<uint64_t> prefix;
     DevBuf<double> cen_re, cen_im;  // [nboxes][dim]
+    // separate targets: per box, the range of its sources and targets among all
+    // sources (targets), and the sorted point of each (see SubRange); wsen (wten): the
+    // end of a box that holds a source (a target), the start of any other
+    DevBuf<int> sst, sen, tst, ten, sidx, tidx, wsen, wten;
     DevBuf<int> loff[4];            // CSR offsets [nboxes+1]
     std::vector<int> hloff[4];      // host copies of the offsets
     DevBuf<int> lent[4];            // CSR entries
     int64_t llen[4] = {0, 0, 0, 0};
     std::vector<int> leaf_boxes;    // host: box index of every leaf, Morton order
     DevBuf<int> d_leaf_boxes;
+};
+
+// Points of a box that a kernel goes over: k in [st[b], en[b]) is sorted point
+// map[k], or k itself without a map (every point is a source and a target).
+struct SubRange {
+    const int *st, *en, *map;
+    __device__ __forceinline__ int64_t at(int64_t k) const { return map ? map[k] : k; }
 };
 
 }  // namespace cfmm

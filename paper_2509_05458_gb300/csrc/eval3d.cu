@@ -41,7 +41,8 @@ struct EvalK {
     const double *xr, *xi;
     int64_t n;
     Eval3Args E;
-    const int *tst, *ten, *l3off, *l3, *blevel;
+    SubRange trg;
+    const int *l3off, *l3, *blevel;
     const double *cre, *cim;
     const int64_t* ioff;
     const int* own;
@@ -193,15 +194,15 @@ __global__ void __launch_bounds__(kEvalWarps * 32) k_eval3_items(EvalK A) {
     if (!sing) {
         li = task;
         b = s = A.E.leaves[li];
-        slot = A.tst[b];
+        slot = A.trg.st[b];
     } else {
         const int e = task - A.nleaf_tasks;
         li = A.own[e];
         b = A.E.leaves[li];
         s = A.l3[e];
-        slot = A.n + A.ioff[li] + (int64_t)(e - A.l3off[b]) * (A.ten[b] - A.tst[b]);
+        slot = A.n + A.ioff[li] + (int64_t)(e - A.l3off[b]) * (A.trg.en[b] - A.trg.st[b]);
     }
-    const int P = A.E.Plev[A.blevel[s]], t0 = A.tst[b], cnt = A.ten[b] - t0;
+    const int P = A.E.Plev[A.blevel[s]], t0 = A.trg.st[b], cnt = A.trg.en[b] - t0;
     const int64_t co = (int64_t)rhs * A.E.ncoef + A.E.eoff[s];
     const cd* c = (sing ? A.E.mp : A.E.loc) + co;
     cd* F = sm + (size_t)wid * (A.E.maxP + 2) * 32;
@@ -210,7 +211,7 @@ __global__ void __launch_bounds__(kEvalWarps * 32) k_eval3_items(EvalK A) {
     for (int k0 = blockIdx.y * 32; k0 < cnt; k0 += gridDim.y * 32) {
         const int nt = min(32, cnt - k0), G = min(32 / nt, P + 1), g = lane / nt, t = lane - g * nt;
         const bool on = g < G;
-        const int64_t i = t0 + k0 + t;
+        const int64_t i = A.trg.at(t0 + k0 + t);
         cd x[3];
 #pragma unroll
         for (int a = 0; a < 3; ++a) x[a] = cd{A.xr[a * A.n + i], A.xi[a * A.n + i]} - cen[a];
@@ -304,14 +305,14 @@ __global__ void k_eval3_own(int nleaf, const int* __restrict__ leaves, const int
 // u [rhs][comp][n] += the slots of each target: L2P and its leaf's List 3 in order
 __global__ void k_eval3_sum(EvalK A, int ncomp, cd* __restrict__ u) {
     const int li = blockIdx.x, row = blockIdx.y, b = A.E.leaves[li];
-    const int t0 = A.tst[b], cnt = A.ten[b] - t0, ne = A.l3off[b + 1] - A.l3off[b];
+    const int t0 = A.trg.st[b], cnt = A.trg.en[b] - t0, ne = A.l3off[b + 1] - A.l3off[b];
     if (!A.l2p && ne == 0) return;
     const cd* v = A.val + (int64_t)row * A.nslot;
     const int64_t first = A.n + A.ioff[li];
     for (int t = threadIdx.x; t < cnt; t += blockDim.x) {
         cd s = A.l2p ? v[t0 + t] : cd{0, 0};
         for (int e = 0; e < ne; ++e) s += v[first + (int64_t)e * cnt + t];
-        u[(int64_t)row * A.n + t0 + t] += s;
+        u[(int64_t)row * A.n + A.trg.at(t0 + t)] += s;
     }
 }
 
@@ -370,7 +371,7 @@ void eval3_apply(cfmm_plan_s* P, Eval3* E, const Eval3Tables& T, const Eval3Args
     if (A.nleaf == 0) return;
     const bool lap = A.kappa == 0.0;
     const int nl3 = Tr.hloff[2].back();
-    EvalK K{P->xr.get(), P->xi.get(), P->n, A, Tr.start.get(), Tr.end.get(), Tr.loff[2].get(), Tr.lent[2].get(),
+    EvalK K{P->xr.get(), P->xi.get(), P->n, A, target_range(P), Tr.loff[2].get(), Tr.lent[2].get(),
             Tr.level.get(), Tr.cen_re.get(), Tr.cen_im.get(), E->ioff.get(), E->own.get(), P->n + E->total, 0, T, nullptr, nullptr, 0, 0};
     const int groups = std::max(1, std::min(64, (P->leaf_size + 31) / 32));
     // right-hand sides whose slots fit

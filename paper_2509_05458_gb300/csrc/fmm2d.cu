@@ -198,8 +198,7 @@ struct ExpArgs {
     bool slp, dlp;
     double kappa;
     const int* blevel;
-    const int* bst;
-    const int* ben;
+    SubRange src, trg;
     const double* cre;
     const double* cim;
     const int* Plev;
@@ -281,10 +280,10 @@ __global__ void k_point_to_exp(ExpArgs A, const int* __restrict__ boxes, const i
         int cn = 0, q = qn, jn = j0;
         while (q < qb && cn < chunk) {
             const int src = loff ? lent[q] : b;
-            const int s0 = A.bst[src] + jn, m = min(A.ben[src] - s0, chunk - cn);
-            if ((int)threadIdx.x >= cn && (int)threadIdx.x < cn + m) j = s0 + (threadIdx.x - cn);
+            const int s0 = A.src.st[src] + jn, m = min(A.src.en[src] - s0, chunk - cn);
+            if ((int)threadIdx.x >= cn && (int)threadIdx.x < cn + m) j = A.src.at(s0 + (threadIdx.x - cn));
             cn += m;
-            if (s0 + m == A.ben[src]) {
+            if (s0 + m == A.src.en[src]) {
                 ++q;
                 jn = 0;
             } else {
@@ -322,7 +321,7 @@ __global__ void k_point_to_exp(ExpArgs A, const int* __restrict__ boxes, const i
         // the plan's rows of the points about their own leaf (this box), a warp a row
         if (KER == CFMM_HELMHOLTZ && lrow && !sing)
             for (int tt = threadIdx.x >> 5; tt < cn; tt += blockDim.x >> 5) {
-                const cd* src = lrow + (int64_t)(A.bst[b] + j0 + tt) * RL;
+                const cd* src = lrow + A.src.at(A.src.st[b] + j0 + tt) * RL;
                 for (int i = threadIdx.x & 31; i < R; i += 32) rows[(size_t)tt * R + i] = src[i];
             }
         __syncthreads();
@@ -754,10 +753,10 @@ __global__ void k_eval(ExpArgs A, const int* __restrict__ leaves, const int* __r
     int nc = 2 * P + 1;
     cd* coef = sm;                                  // 2*maxP+1
     cd* rows = sm + 2 * maxP + 1;                   // per thread: maxP+2 (Helmholtz L2P), 1 (M2P)
-    int s0 = A.bst[b], s1 = A.ben[b];
+    int s0 = A.trg.st[b], s1 = A.trg.en[b];
     for (int t0 = s0; t0 < s1; t0 += blockDim.x) {
-        int i = t0 + threadIdx.x;
-        bool valid = i < s1;
+        bool valid = t0 + (int)threadIdx.x < s1;
+        const int64_t i = valid ? A.trg.at(t0 + threadIdx.x) : 0;
         cd x0 = {0, 0}, x1 = {0, 0};
         if (valid) {
             x0 = cd{A.xr[i], A.xi[i]};
@@ -772,7 +771,8 @@ __global__ void k_eval(ExpArgs A, const int* __restrict__ leaves, const int* __r
             const int item = base + threadIdx.x;
             cd v = {0, 0};
             if (item < items) {
-                const int s = l3[q0 + item / nt], it = t0 + item % nt, Ps = A.Plev[A.blevel[s]];
+                const int s = l3[q0 + item / nt], Ps = A.Plev[A.blevel[s]];
+                const int64_t it = A.trg.at(t0 + item % nt);
                 const cd* m = mp + (int64_t)rhs * A.ncoef + A.eoff[s];
                 cd z, e;
                 zeta_eta(cd{A.xr[it], A.xi[it]} - cd{A.cre[2 * s], A.cim[2 * s]},
@@ -888,11 +888,11 @@ __global__ void k_eval_grad(ExpArgs A, const int* __restrict__ leaves, const int
     int P = A.Plev[A.blevel[b]];
     cd* coef = sm;                                  // 2*maxP+1
     cd* rows = sm + 2 * maxP + 1;                   // per thread: 2*maxP+3 (Helmholtz rows n = -P-1..P+1)
-    int s0 = A.bst[b], s1 = A.ben[b];
+    int s0 = A.trg.st[b], s1 = A.trg.en[b];
     const double kh = 0.5 * A.kappa;
     for (int t0 = s0; t0 < s1; t0 += blockDim.x) {
-        int i = t0 + threadIdx.x;
-        bool valid = i < s1;
+        bool valid = t0 + (int)threadIdx.x < s1;
+        const int64_t i = valid ? A.trg.at(t0 + threadIdx.x) : 0;
         cd x0 = {0, 0}, x1 = {0, 0};
         if (valid) {
             x0 = cd{A.xr[i], A.xi[i]};
@@ -1008,7 +1008,8 @@ __global__ void __launch_bounds__(kExpThreads) k_l2p2f(ExpArgs A, const int* __r
     double irb = 1.0 / rb;
     cd c0 = {A.cre[2 * b], A.cim[2 * b]}, c1 = {A.cre[2 * b + 1], A.cim[2 * b + 1]};
     cf G[kL2p2fMaxP + 1];
-    for (int i = A.bst[b] + threadIdx.x; i < A.ben[b]; i += blockDim.x) {
+    for (int k = A.trg.st[b] + threadIdx.x; k < A.trg.en[b]; k += blockDim.x) {
+        const int64_t i = A.trg.at(k);
         cd d0 = irb * (cd{A.xr[i], A.xi[i]} - c0), d1 = irb * (cd{A.xr[A.n + i], A.xi[A.n + i]} - c1);
         cf zt = to_cf(d0 + mul_i(d1)), et = to_cf(d0 - mul_i(d1));
         Kahan acc;
@@ -1448,10 +1449,10 @@ static void apply_t(cfmm_plan_s* P, Fmm2dState* S, const cd* sigma, const cd* ta
               sigma, tau, dstride, P->slp, P->dlp, P->kappa};
     if (T.nboxes <= 1) {
         for (int i = 2; i <= 6; ++i) rec(i);
-        launch_p2p(2, KER, K, T.d_leaf_boxes.get(), T.nleaves, T.start.get(), T.end.get(), T.loff[0].get(),
+        launch_p2p(2, KER, K, T.d_leaf_boxes.get(), T.nleaves, near_ranges(P), T.loff[0].get(),
                    T.lent[0].get(), u, nrhs, false, st, P->precision == CFMM_MIXED, P->leaf_size);
         if (g)
-            launch_p2p_grad(2, KER, K, T.d_leaf_boxes.get(), T.nleaves, T.start.get(), T.end.get(), T.loff[0].get(),
+            launch_p2p_grad(2, KER, K, T.d_leaf_boxes.get(), T.nleaves, near_ranges(P), T.loff[0].get(),
                             T.lent[0].get(), g, nrhs, st, P->leaf_size);
         rec(7);
         rec(8);
@@ -1463,7 +1464,7 @@ static void apply_t(cfmm_plan_s* P, Fmm2dState* S, const cd* sigma, const cd* ta
     cd* mp = P->mpole.get();
     cd* lc = P->local.get();
     ExpArgs A{P->xr.get(), P->xi.get(), P->nr.get(), P->ni.get(), P->n, sigma, tau, dstride, P->slp, P->dlp,
-              P->kappa, T.level.get(), T.start.get(), T.end.get(), T.cen_re.get(), T.cen_im.get(),
+              P->kappa, T.level.get(), source_range(P), target_range(P), T.cen_re.get(), T.cen_im.get(),
               S->dPlev.get(), S->exp_off.get(), S->ncoef, hankel_args(P->kappa)};
     int maxP = S->maxP;
     // (6) P2L over List 4, added to the local expansions
@@ -1502,10 +1503,10 @@ static void apply_t(cfmm_plan_s* P, Fmm2dState* S, const cd* sigma, const cd* ta
             p2l(ns);
             CFMM_CUDA(cudaEventRecord(P->ev_far[0], ns));
         }
-        launch_p2p(2, KER, K, S->d_leaves_l0.get(), (int)S->leaves_l0.size(), T.start.get(), T.end.get(),
+        launch_p2p(2, KER, K, S->d_leaves_l0.get(), (int)S->leaves_l0.size(), near_ranges(P),
                    T.loff[0].get(), T.lent[0].get(), u, nrhs, false, ns, P->precision == CFMM_MIXED, P->leaf_size);
         if (g)
-            launch_p2p_grad(2, KER, K, S->d_leaves_l0.get(), (int)S->leaves_l0.size(), T.start.get(), T.end.get(),
+            launch_p2p_grad(2, KER, K, S->d_leaves_l0.get(), (int)S->leaves_l0.size(), near_ranges(P),
                             T.loff[0].get(), T.lent[0].get(), g, nrhs, ns, P->leaf_size);
     }
     near_launched(P);

@@ -93,8 +93,7 @@ struct Exp3Args {
     int64_t dstride;
     bool slp, dlp;
     const int* blevel;
-    const int* bst;
-    const int* ben;
+    SubRange src;                // sources
     const double* cre;
     const double* cim;
     const int* Plev;
@@ -127,7 +126,7 @@ __global__ void k_point_to_exp3(Exp3Args A, const int* __restrict__ boxes, const
     int qa = loff ? loff[b] : 0, qb = loff ? loff[b + 1] : 1;
     for (int q = qa; q < qb; ++q) {
         int src = loff ? lent[q] : b;
-        int s0 = A.bst[src], s1 = A.ben[src];
+        int s0 = A.src.st[src], s1 = A.src.en[src];
         for (int c0 = s0; c0 < s1; c0 += chunk) {
             int cn = min(chunk, s1 - c0);
             __syncthreads();
@@ -135,7 +134,7 @@ __global__ void k_point_to_exp3(Exp3Args A, const int* __restrict__ boxes, const
             int cols = 2 * PT + 1;
             for (int w = threadIdx.x; w < cn * cols; w += blockDim.x) {
                 int s = w / cols, col = w - s * cols;
-                int64_t j = c0 + s;
+                const int64_t j = A.src.at(c0 + s);
                 cd y[3];
                 load3(A.xr, A.xi, A.n, j, y);
                 solid_table(!sing, y[0] - cen[0], y[1] - cen[1], y[2] - cen[2], PT, tabs + (size_t)s * nt, col, cols);
@@ -281,8 +280,9 @@ void fmm3d_setup(cfmm_plan_s* P) {
     S->exp_off.alloc(T.nboxes);
     CFMM_CUDA(cudaMemcpyAsync(S->exp_off.get(), off.data(), sizeof(int64_t) * T.nboxes, cudaMemcpyHostToDevice, st));
     std::vector<int> lvl(T.nboxes), l4(T.nboxes + 1), hst(T.nboxes), hen(T.nboxes), boxes;
-    CFMM_CUDA(cudaMemcpyAsync(hst.data(), T.start.get(), sizeof(int) * T.nboxes, cudaMemcpyDeviceToHost, st));
-    CFMM_CUDA(cudaMemcpyAsync(hen.data(), T.end.get(), sizeof(int) * T.nboxes, cudaMemcpyDeviceToHost, st));
+    const SubRange tr = target_range(P);
+    CFMM_CUDA(cudaMemcpyAsync(hst.data(), tr.st, sizeof(int) * T.nboxes, cudaMemcpyDeviceToHost, st));
+    CFMM_CUDA(cudaMemcpyAsync(hen.data(), tr.en, sizeof(int) * T.nboxes, cudaMemcpyDeviceToHost, st));
     CFMM_CUDA(cudaMemcpyAsync(lvl.data(), T.level.get(), sizeof(int) * T.nboxes, cudaMemcpyDeviceToHost, st));
     CFMM_CUDA(cudaMemcpyAsync(l4.data(), T.loff[3].get(), sizeof(int) * (T.nboxes + 1), cudaMemcpyDeviceToHost, st));
     CFMM_CUDA(cudaStreamSynchronize(st));
@@ -320,11 +320,10 @@ void fmm3d_apply(cfmm_plan_s* P, const cd* sigma, const cd* tau, int64_t dstride
                  "3D Helmholtz translations are not built yet");
     if (T.nboxes <= 1) {
         for (int i = 2; i <= 6; ++i) rec(i);
-        launch_p2p(3, P->kernel, K, T.d_leaf_boxes.get(), T.nleaves, T.start.get(), T.end.get(), T.loff[0].get(),
+        launch_p2p(3, P->kernel, K, T.d_leaf_boxes.get(), T.nleaves, near_ranges(P), T.loff[0].get(),
                    T.lent[0].get(), u, nrhs, false, st, mixed, P->leaf_size);
         if (g)
-            launch_p2p_grad(3, P->kernel, K, T.d_leaf_boxes.get(), T.nleaves, T.start.get(), T.end.get(),
-                            T.loff[0].get(), T.lent[0].get(), g, nrhs, st, P->leaf_size);
+            launch_p2p_grad(3, P->kernel, K, T.d_leaf_boxes.get(), T.nleaves, near_ranges(P), T.loff[0].get(), T.lent[0].get(), g, nrhs, st, P->leaf_size);
         rec(7);
         rec(8);
         return;
@@ -336,7 +335,7 @@ void fmm3d_apply(cfmm_plan_s* P, const cd* sigma, const cd* tau, int64_t dstride
     cd* lc = P->local.get();
     int maxP = S->maxP;
     Exp3Args A{P->xr.get(), P->xi.get(), P->nr.get(), P->ni.get(), P->n, sigma, tau, dstride, P->slp, P->dlp,
-               T.level.get(), T.start.get(), T.end.get(), T.cen_re.get(), T.cen_im.get(), S->dPlev.get(),
+               T.level.get(), source_range(P), T.cen_re.get(), T.cen_im.get(), S->dPlev.get(),
                S->exp_off.get(), S->ncoef};
     auto p2x_smem = [&](int PT, int& chunk) {
         size_t nt = (size_t)(PT + 1) * (PT + 1);
@@ -346,11 +345,9 @@ void fmm3d_apply(cfmm_plan_s* P, const cd* sigma, const cd* tau, int64_t dstride
     // (3) P2P (writes u) on the side stream, beside the far field
     {
         cudaStream_t ns = near_fork(P);
-        launch_p2p(3, P->kernel, K, S->d_leaves_l0.get(), (int)S->leaves_l0.size(), T.start.get(), T.end.get(),
-                   T.loff[0].get(), T.lent[0].get(), u, nrhs, false, ns, mixed, P->leaf_size);
+        launch_p2p(3, P->kernel, K, S->d_leaves_l0.get(), (int)S->leaves_l0.size(), near_ranges(P), T.loff[0].get(), T.lent[0].get(), u, nrhs, false, ns, mixed, P->leaf_size);
         if (g)
-            launch_p2p_grad(3, P->kernel, K, S->d_leaves_l0.get(), (int)S->leaves_l0.size(), T.start.get(),
-                            T.end.get(), T.loff[0].get(), T.lent[0].get(), g, nrhs, ns, P->leaf_size);
+            launch_p2p_grad(3, P->kernel, K, S->d_leaves_l0.get(), (int)S->leaves_l0.size(), near_ranges(P), T.loff[0].get(), T.lent[0].get(), g, nrhs, ns, P->leaf_size);
     }
     near_launched(P);
     // (1) P2M (single layer: one lane per harmonic column; complex64 products

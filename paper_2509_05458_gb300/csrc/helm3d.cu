@@ -417,8 +417,7 @@ struct Exp3hArgs {
     int64_t dstride;
     bool slp, dlp;
     const int* blevel;
-    const int* bst;
-    const int* ben;
+    SubRange pts;                // sources (Exp3hArgs, k_p2m3f) or targets (k_l2p3f)
     const double* cre;
     const double* cim;
     const int* Plev;
@@ -453,14 +452,14 @@ __global__ void k_p2x3h(Exp3hArgs A, const int* __restrict__ boxes, const int* _
     int qa = loff ? loff[b] : 0, qb = loff ? loff[b + 1] : 1;
     for (int q = qa; q < qb; ++q) {
         int src = loff ? lent[q] : b;
-        int s0 = A.bst[src], s1 = A.ben[src];
+        int s0 = A.pts.st[src], s1 = A.pts.en[src];
         for (int c0 = s0; c0 < s1; c0 += chunk) {
             int cn = min(chunk, s1 - c0);
             __syncthreads();
             int cols = 2 * P + 1;
             for (int w = threadIdx.x; w < cn * (cols + 1); w += blockDim.x) {
                 int s = w / (cols + 1), col = w - s * (cols + 1);
-                int64_t j = c0 + s;
+                const int64_t j = A.pts.at(c0 + s);
                 cd y[3];
                 load3(A.xr, A.xi, A.n, j, y);
                 for (int a = 0; a < 3; ++a) y[a] = y[a] - cen[a];
@@ -538,10 +537,10 @@ __global__ void k_radial3h(Exp3hArgs A, const int* __restrict__ boxes, int nboxe
     int64_t o = roff[bi];
     for (int q = qa; q < qb; ++q) {
         int src = loff ? lent[q] : b;
-        int s0 = A.bst[src], s1 = A.ben[src];
+        int s0 = A.pts.st[src], s1 = A.pts.en[src];
         for (int j = s0 + threadIdx.x; j < s1; j += blockDim.x) {
             cd y[3];
-            load3(A.xr, A.xi, A.n, j, y);
+            load3(A.xr, A.xi, A.n, A.pts.at(j), y);
             for (int a = 0; a < 3; ++a) y[a] = y[a] - cen[a];
             radial_seq(!sing, A.kappa, y[0] * y[0] + y[1] * y[1] + y[2] * y[2], P,
                        rad + (o + (j - s0)) * (int64_t)(P + 1));
@@ -607,14 +606,14 @@ __global__ void k_p2x3h_slp(Exp3hArgs A, const int* __restrict__ boxes, const in
     int64_t o = roff ? roff[bi] : 0;
     for (int q = qa; q < qb; ++q) {
         int src = loff ? lent[q] : b;
-        int s0 = A.bst[src], s1 = A.ben[src];
+        int s0 = A.pts.st[src], s1 = A.pts.en[src];
         if (C >= 32) {
             int items = (s1 - s0) * C;
             for (int base = wid * 32; base < items; base += nwarp * 32) {
                 int it = base + lane;
                 if (it < items) {
                     int js = it / C, col = it - js * C;
-                    int j = s0 + js;
+                    const int64_t j = A.pts.at(s0 + js);
                     cd y[3];
                     load3(A.xr, A.xi, A.n, j, y);
                     for (int a = 0; a < 3; ++a) y[a] = y[a] - cen[a];
@@ -625,14 +624,15 @@ __global__ void k_p2x3h_slp(Exp3hArgs A, const int* __restrict__ boxes, const in
                 __syncwarp();
             }
         } else {
-            for (int j = s0 + wid; j < s1; j += nwarp) {
+            for (int k = s0 + wid; k < s1; k += nwarp) {
+                const int64_t j = A.pts.at(k);
                 if (lane < C) {
                     cd y[3];
                     load3(A.xr, A.xi, A.n, j, y);
                     for (int a = 0; a < 3; ++a) y[a] = y[a] - cen[a];
                     cd xp = y[0] + mul_i(y[1]), xm = y[0] - mul_i(y[1]), z = y[2];
                     p2x_column<LAP>(A.zc, P, lane, xp, xm, z, xp * xm + z * z, A.sigma[rhs * A.dstride + j],
-                                    LAP ? nullptr : rad + (o + (j - s0)) * (int64_t)(P + 1), accw);
+                                    LAP ? nullptr : rad + (o + (k - s0)) * (int64_t)(P + 1), accw);
                 }
             }
         }
@@ -680,8 +680,7 @@ struct L2p3fArgs {
     const double* xi;
     int64_t n;
     const int* blevel;
-    const int* bst;
-    const int* ben;
+    SubRange pts;                // sources (Exp3hArgs, k_p2m3f) or targets (k_l2p3f)
     const double* cre;
     const double* cim;
     const int* Plev;
@@ -757,7 +756,8 @@ __global__ void __launch_bounds__(128) k_l2p3f(L2p3fArgs A, const int* __restric
     cd cen[3];
     for (int a = 0; a < 3; ++a) cen[a] = cd{A.cre[3 * b + a], A.cim[3 * b + a]};
     cf G[kH3MaxP + 1];
-    for (int i = A.bst[b] + threadIdx.x; i < A.ben[b]; i += blockDim.x) {
+    for (int k = A.pts.st[b] + threadIdx.x; k < A.pts.en[b]; k += blockDim.x) {
+        const int64_t i = A.pts.at(k);
         cf x[3];
         for (int a = 0; a < 3; ++a)
             x[a] = to_cf(irb * (cd{A.xr[a * A.n + i], A.xi[a * A.n + i]} - cen[a]));
@@ -837,12 +837,12 @@ __global__ void __launch_bounds__(kP2m3fWarps * 32) k_p2m3f(L2p3fArgs A, const i
     cd cen[3];
     for (int a = 0; a < 3; ++a) cen[a] = cd{A.cre[3 * b + a], A.cim[3 * b + a]};
     float kr = (float)(A.kappa * rb);
-    int s0 = A.bst[b], s1 = A.ben[b];
+    int s0 = A.pts.st[b], s1 = A.pts.en[b];
     for (int base = s0 + wid * 32; base < s1; base += kP2m3fWarps * 32) {
         int cnt = min(32, s1 - base);
         __syncwarp();
         if (lane < cnt) {
-            int j = base + lane;
+            const int64_t j = A.pts.at(base + lane);
             cf y[3];
             for (int a = 0; a < 3; ++a) y[a] = to_cf(irb * (cd{A.xr[a * A.n + j], A.xi[a * A.n + j]} - cen[a]));
             cf xp = y[0] + mul_if(y[1]), xm = y[0] - mul_if(y[1]);
@@ -911,7 +911,7 @@ static void launch_p2m3f(H3Tables* TB, bool helm, cfmm_plan_s* P, const int* box
                          cd* out, int nrhs) {
     if (cnt <= 0) return;
     TreeDev& T = P->tree;
-    L2p3fArgs A{P->xr.get(), P->xi.get(), P->n, T.level.get(), T.start.get(), T.end.get(), T.cen_re.get(),
+    L2p3fArgs A{P->xr.get(), P->xi.get(), P->n, T.level.get(), source_range(P), T.cen_re.get(),
                 T.cen_im.get(), dPlev, eoff, ncoef, P->kappa, P->W, TB->zAf.get(), TB->zBf.get(),
                 TB->dgf.get(), TB->s21f.get(), TB->knm.get(), TB->lsd.get()};
     size_t smem = p2m3f_smem(PL);
@@ -930,7 +930,7 @@ static void launch_l2p3f(H3Tables* TB, bool helm, cfmm_plan_s* P, const int* lea
                          const int* dPlev, const int64_t* eoff, int64_t ncoef, const cd* loc, cd* u, int nrhs) {
     if (cnt == 0) return;
     TreeDev& T = P->tree;
-    L2p3fArgs A{P->xr.get(), P->xi.get(), P->n, T.level.get(), T.start.get(), T.end.get(), T.cen_re.get(),
+    L2p3fArgs A{P->xr.get(), P->xi.get(), P->n, T.level.get(), target_range(P), T.cen_re.get(),
                 T.cen_im.get(), dPlev, eoff, ncoef, P->kappa, P->W, TB->zAf.get(), TB->zBf.get(),
                 TB->dgf.get(), TB->s21f.get(), TB->knm.get(), TB->lsd.get()};
     size_t smem = sizeof(double) * (size_t)(maxP + 1) + sizeof(cf) * (size_t)(maxP + 1) * (maxP + 1);
@@ -1078,14 +1078,17 @@ void helm3d_setup(cfmm_plan_s* P) {
     S->n_p2l = (int)boxes.size();
     {
         // radial-buffer offsets of the single-layer P2M / P2L launches
-        std::vector<int> hst(T.nboxes), hen(T.nboxes), l4e(std::max(1, l4[T.nboxes]));
-        CFMM_CUDA(cudaMemcpyAsync(hst.data(), T.start.get(), sizeof(int) * T.nboxes, cudaMemcpyDeviceToHost, st));
-        CFMM_CUDA(cudaMemcpyAsync(hen.data(), T.end.get(), sizeof(int) * T.nboxes, cudaMemcpyDeviceToHost, st));
+        std::vector<int> hst(T.nboxes), hen(T.nboxes), tst(T.nboxes), ten(T.nboxes), l4e(std::max(1, l4[T.nboxes]));
+        const SubRange sr = source_range(P), tr = target_range(P);
+        CFMM_CUDA(cudaMemcpyAsync(hst.data(), sr.st, sizeof(int) * T.nboxes, cudaMemcpyDeviceToHost, st));
+        CFMM_CUDA(cudaMemcpyAsync(hen.data(), sr.en, sizeof(int) * T.nboxes, cudaMemcpyDeviceToHost, st));
+        CFMM_CUDA(cudaMemcpyAsync(tst.data(), tr.st, sizeof(int) * T.nboxes, cudaMemcpyDeviceToHost, st));
+        CFMM_CUDA(cudaMemcpyAsync(ten.data(), tr.en, sizeof(int) * T.nboxes, cudaMemcpyDeviceToHost, st));
         if (l4[T.nboxes] > 0)
             CFMM_CUDA(cudaMemcpyAsync(l4e.data(), T.lent[3].get(), sizeof(int) * l4[T.nboxes], cudaMemcpyDeviceToHost,
                                       st));
         CFMM_CUDA(cudaStreamSynchronize(st));
-        eval3_build(&S->eval, S->leaves_l0, T.hloff[2], hst, hen, S->d_leaves_l0.get(), T.loff[2].get(), st);
+        eval3_build(&S->eval, S->leaves_l0, T.hloff[2], tst, ten, S->d_leaves_l0.get(), T.loff[2].get(), st);
         for (int b : S->leaves_l0) S->maxP_eval = std::max(S->maxP_eval, S->Plev[lvl[b]]);
         std::vector<int> ro(byl.size()), rl(boxes.size());
         S->p2m_rtot.assign(T.nlevels, 0);
@@ -1134,11 +1137,10 @@ void helm3d_apply(cfmm_plan_s* P, const cd* sigma, const cd* tau, int64_t dstrid
     bool mixed = P->precision == CFMM_MIXED;
     if (T.nboxes <= 1) {
         for (int i = 2; i <= 6; ++i) rec(i);
-        launch_p2p(3, P->kernel, K, T.d_leaf_boxes.get(), T.nleaves, T.start.get(), T.end.get(), T.loff[0].get(),
+        launch_p2p(3, P->kernel, K, T.d_leaf_boxes.get(), T.nleaves, near_ranges(P), T.loff[0].get(),
                    T.lent[0].get(), u, nrhs, false, st, mixed, P->leaf_size);
         if (g)
-            launch_p2p_grad(3, P->kernel, K, T.d_leaf_boxes.get(), T.nleaves, T.start.get(), T.end.get(),
-                            T.loff[0].get(), T.lent[0].get(), g, nrhs, st, P->leaf_size);
+            launch_p2p_grad(3, P->kernel, K, T.d_leaf_boxes.get(), T.nleaves, near_ranges(P), T.loff[0].get(), T.lent[0].get(), g, nrhs, st, P->leaf_size);
         rec(7);
         rec(8);
         return;
@@ -1152,18 +1154,16 @@ void helm3d_apply(cfmm_plan_s* P, const cd* sigma, const cd* tau, int64_t dstrid
     ZCoef zc{TB->zA.get(), TB->zB.get(), TB->dg.get(), TB->s21.get(), TB->knm.get(),
              TB->g3.get(), TB->gp.get(), TB->gm.get()};
     Exp3hArgs A{P->xr.get(), P->xi.get(), P->nr.get(), P->ni.get(), P->n, sigma, tau, dstride, P->slp, P->dlp,
-                T.level.get(), T.start.get(), T.end.get(), T.cen_re.get(), T.cen_im.get(), S->dPlev.get(),
+                T.level.get(), source_range(P), T.cen_re.get(), T.cen_im.get(), S->dPlev.get(),
                 S->exp_off.get(), S->ncoef, P->kappa, zc};
     int maxP = S->maxP;
     // (3) P2P (writes u) on the side stream, beside the far field
     {
         cudaStream_t ns = near_fork(P);
-        launch_p2p(3, P->kernel, K, S->d_leaves_l0.get(), (int)S->leaves_l0.size(), T.start.get(), T.end.get(),
-                   T.loff[0].get(), T.lent[0].get(), u, nrhs, false, ns, mixed, P->leaf_size, T.level.get(), P->W,
+        launch_p2p(3, P->kernel, K, S->d_leaves_l0.get(), (int)S->leaves_l0.size(), near_ranges(P), T.loff[0].get(), T.lent[0].get(), u, nrhs, false, ns, mixed, P->leaf_size, T.level.get(), P->W,
                    P->sep);
         if (g)
-            launch_p2p_grad(3, P->kernel, K, S->d_leaves_l0.get(), (int)S->leaves_l0.size(), T.start.get(),
-                            T.end.get(), T.loff[0].get(), T.lent[0].get(), g, nrhs, ns, P->leaf_size);
+            launch_p2p_grad(3, P->kernel, K, S->d_leaves_l0.get(), (int)S->leaves_l0.size(), near_ranges(P), T.loff[0].get(), T.lent[0].get(), g, nrhs, ns, P->leaf_size);
     }
     near_launched(P);
     auto p2x_smem = [&](int PL, int& chunk) {
@@ -1286,7 +1286,7 @@ bool lap3_p2m_slp(Lap3Tr* L, cfmm_plan_s* P, const int* leaves, int cnt, int max
     ZCoef zc{TB->zA.get(), TB->zB.get(), TB->dg.get(), TB->s21.get(), TB->knm.get(),
              TB->g3.get(), TB->gp.get(), TB->gm.get()};
     Exp3hArgs A{P->xr.get(), P->xi.get(), nullptr, nullptr, P->n, sigma, nullptr, dstride, true, false,
-                T.level.get(), T.start.get(), T.end.get(), T.cen_re.get(), T.cen_im.get(), dPlev, eoff, ncoef,
+                T.level.get(), source_range(P), T.cen_re.get(), T.cen_im.get(), dPlev, eoff, ncoef,
                 0.0, zc};
     dim3 g((unsigned)cnt, nrhs);
     k_p2x3h_slp<true><<<g, kH3Threads, smem, P->stream>>>(A, leaves, nullptr, nullptr, 0, nullptr, nullptr, out,

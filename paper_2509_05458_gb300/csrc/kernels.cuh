@@ -25,6 +25,35 @@ struct KParams {
     double ikappa = 0.0, isqrt_kappa = 0.0, kappa_ang = 0.0, kappa_exp = 0.0;
 };
 
+// Source and target ranges of a plan's boxes: all points, or with separate targets
+// only the sources (the others carry no density) and only the targets (nothing else
+// is read)
+inline SubRange source_range(const cfmm_plan_s* P) {
+    const TreeDev& T = P->tree;
+    return P->n_trg > 0 ? SubRange{T.sst.get(), T.sen.get(), T.sidx.get()}
+                        : SubRange{T.start.get(), T.end.get(), nullptr};
+}
+inline SubRange target_range(const cfmm_plan_s* P) {
+    const TreeDev& T = P->tree;
+    return P->n_trg > 0 ? SubRange{T.tst.get(), T.ten.get(), T.tidx.get()}
+                        : SubRange{T.start.get(), T.end.get(), nullptr};
+}
+// Near field. FP64 goes over the sources and the targets; mixed precision over the
+// whole boxes that hold a source (a target), [st, sen) and [st, ten): its compensated
+// FP32 sums depend on which thread adds which term (1.4e-8 relative l2 between going
+// over the sources of a shared box and over all its points).
+struct NearRanges {
+    SubRange src, trg;
+    const int* first;             // first point of the boxes
+};
+inline NearRanges near_ranges(const cfmm_plan_s* P) {
+    const TreeDev& T = P->tree;
+    const int* st = T.start.get();
+    if (P->n_trg > 0 && P->precision == CFMM_MIXED)
+        return NearRanges{SubRange{st, T.wsen.get(), nullptr}, SubRange{st, T.wten.get(), nullptr}, st};
+    return NearRanges{source_range(P), target_range(P), st};
+}
+
 // near field of an apply on the plan's side stream: near_fork() makes the
 // side stream wait for what the plan's stream has queued and returns it;
 // near_join() makes the plan's stream wait for the side stream. In the
@@ -37,13 +66,13 @@ void near_join(cfmm_plan_s* P);
 // blevel/W/sep: the tree's box levels, root width and separation (the mixed
 // 3D Helmholtz near field sizes its coordinate grid from them; NULL = unknown);
 // leaf_size bounds the points of a leaf
-void launch_p2p(int dim, int ker, const KParams& K, const int* leaf_boxes, int nleaves, const int* bst,
-                const int* ben, const int* l1off, const int* l1, cd* out, int nrhs, bool add, cudaStream_t st,
+void launch_p2p(int dim, int ker, const KParams& K, const int* leaf_boxes, int nleaves, const NearRanges& R,
+                const int* l1off, const int* l1, cd* out, int nrhs, bool add, cudaStream_t st,
                 bool mixed, int leaf_size, const int* blevel = nullptr, double W = 0.0, int sep = 1);
 void launch_direct(int dim, int ker, const KParams& K, cd* out, int nrhs, cudaStream_t st, bool mixed = false);
 // near-field target gradient over List 1 in FP64: g = sorted [nrhs][dim][n], overwritten
-void launch_p2p_grad(int dim, int ker, const KParams& K, const int* leaf_boxes, int nleaves, const int* bst,
-                     const int* ben, const int* l1off, const int* l1, cd* g, int nrhs, cudaStream_t st,
+void launch_p2p_grad(int dim, int ker, const KParams& K, const int* leaf_boxes, int nleaves, const NearRanges& R,
+                     const int* l1off, const int* l1, cd* g, int nrhs, cudaStream_t st,
                      int leaf_size);
 
 // tree construction (tree.cu)
