@@ -20,8 +20,8 @@
 #include <algorithm>
 #include <cmath>
 
-#include "cfmm_special.cuh"
 #include "eval3d.cuh"
+#include "pair64.cuh"
 
 namespace cfmm {
 
@@ -54,15 +54,15 @@ struct EvalK {
     int nleaf_tasks, ntask;
 };
 
-// F_n = f_n(kappa rho)/rho^n, n = 0..N, of one lane into rows F[32 n]: h by forward
+// F_n = f_n(kappa rho)/rho^n, n = 0..N, of one lane into rows F[ld n]: h by forward
 // recurrence, j by Miller's (both as in cfmm_special.cuh; the overflow test reads the
 // exponent bits)
-__device__ void radial_rows(bool sing, double kappa, cd r2, int N, cd* F) {
+__device__ void radial_rows(bool sing, double kappa, cd r2, int N, cd* F, int ld = 32) {
     cd rho = csqrt_p(r2);
     if (rho.x == 0.0 && rho.y == 0.0) {
         double v = 1.0;
         for (int n = 0; n <= N; ++n) {
-            F[n * 32] = cd{v, 0};
+            F[n * ld] = cd{v, 0};
             v *= kappa / (2.0 * n + 3.0);
         }
         return;
@@ -73,7 +73,7 @@ __device__ void radial_rows(bool sing, double kappa, cd r2, int N, cd* F) {
         cd h0 = -mul_i(e * zi), h1 = -(e * (z + cd{0.0, 1.0})) * (zi * zi);
         double c = 3.0;
         for (int n = 0; n <= N; ++n, c += 2.0) {
-            F[n * 32] = h0 * p;
+            F[n * ld] = h0 * p;
             p = p * ir;
             cd h2 = rmac(-h0, c, zi * h1);
             h0 = h1;
@@ -88,7 +88,7 @@ __device__ void radial_rows(bool sing, double kappa, cd r2, int N, cd* F) {
     cd zi = cinv(z), fp = {0.0, 0.0}, f = {1e-200, 0.0}, S = {0.0, 0.0};
     double c2 = 2.0 * N0 + 1.0;
     for (int n = N0; n >= 1; --n, c2 -= 2.0) {
-        if (n <= N) F[n * 32] = f;
+        if (n <= N) F[n * ld] = f;
         // (-+i)^n f
         int r = up ? n & 3 : (4 - n) & 3;
         cd w = r == 0 ? f : r == 1 ? cd{f.y, -f.x} : r == 2 ? -f : cd{-f.y, f.x};
@@ -103,14 +103,14 @@ __device__ void radial_rows(bool sing, double kappa, cd r2, int N, cd* F) {
             f = sc * f;
             fp = sc * fp;
             S = sc * S;
-            for (int m = n; m <= min(N, N0); ++m) F[m * 32] = sc * F[m * 32];
+            for (int m = n; m <= min(N, N0); ++m) F[m * ld] = sc * F[m * ld];
         }
     }
     F[0] = f;
     S += f;
     cd s = (up ? cexp_i(-z) : cexp_i(z)) / S;
     for (int n = 0; n <= N; ++n) {
-        F[n * 32] = F[n * 32] * s;
+        F[n * ld] = F[n * ld] * s;
         s = s * ir;
     }
 }
@@ -316,6 +316,219 @@ __global__ void k_eval3_sum(EvalK A, int ncomp, cd* __restrict__ u) {
     }
 }
 
+// ---------------------------------------------------------------------------
+// P2M and P2L, single and double layer. With the harmonics H_n^mu = F_n xi^|mu| q_n
+// of the source's offset y, the expansions need four sums over the sources, each
+// over all (n, mu):
+//   W = sum s F_n Z - k t (y.nu) F_{n+1} Z   (Laplace sum s H),
+//   C3, C+, C- = sum t n3 G, t nu+ G, t nu- G,  G = F_{n+1} Z (Laplace H),
+// from which (mu = -m)
+//   Helmholtz    M_n^m = ik(2n+1) [W_n^mu + g3 C3_{n-1}^mu - gp C+_{n-1}^{mu-1} + gm C-_{n-1}^{mu+1}]
+//   Laplace P2M  M_n^m = (-1)^m [W_n^mu + C3_{n-1}^mu - C+_{n-1}^{mu-1}/2 + C-_{n-1}^{mu+1}/2]
+//   Laplace P2L  L_n^m = (-1)^m [W_n^mu - C3_{n+1}^mu - C+_{n+1}^{mu-1}/2 + C-_{n+1}^{mu+1}/2]
+// (g3, gp, gm the tables of the gradient): the double layer's derivative costs three
+// products a coefficient once per box instead of per source, and a source 4 FP64
+// instructions per sum and coefficient beside its own harmonics, which +-m share.
+// The FP64 pipe bounds it: 32 instructions per (n, m >= 0) pair and source for a single
+// layer. Sum over the leaves, before -> after: 1e5-point 3D Helmholtz single layer,
+// orders 23 and 36, 5.8 -> 3.6 ms; 3e4 points 1.2 -> 0.76 ms; 2e5-point 3D Laplace
+// single and double layer, order 16, 12.1 -> 3.6 ms.
+//
+// A block per box. The sources (of the whole List 4) come in groups of 32 (or 8), whose
+// offsets, radial functions and weights one warp computes, and in chunks of `cs` of
+// them: first the harmonics (a warp takes cs sources and 32 / cs columns m), then the
+// sums (thread = sum and (n, mu), consecutive lanes on consecutive entries of a
+// source's table). Where the sums do not fit in shared memory together (a double
+// layer at orders above 38, Laplace 48), each product is a pass of its own.
+// ---------------------------------------------------------------------------
+constexpr int kP2xThreads = 256;
+constexpr size_t kP2xSmem = 220 * 1024;
+
+struct P2xK {
+    const double *xr, *xi, *nr, *ni;
+    int64_t n;
+    const cd *sigma, *tau;        // nullptr: no such layer
+    int64_t dstride;
+    const int* boxes;
+    const int *loff, *lent;       // List 4 (P2L) or nullptr (P2M)
+    SubRange src;
+    const int *Plev, *blevel;
+    const double *cre, *cim;
+    const int64_t* eoff;
+    int64_t ncoef;
+    double kappa;
+    Eval3Tables T;
+    int cs, gs;                   // sources of a chunk and of a group
+    bool all;                     // all sums in one pass, or one product a pass
+    cd* out;
+};
+
+// order of the harmonics
+__host__ __device__ inline int p2x_order(bool lap, bool sing, bool dlp, int P) { return lap && sing && dlp ? P + 1 : P; }
+
+template <bool LAP>
+__global__ void __launch_bounds__(kP2xThreads) k_p2x3(P2xK A) {
+    extern __shared__ cd sm[];
+    const int b = A.boxes[blockIdx.x], rhs = blockIdx.y, P = A.Plev[A.blevel[b]];
+    const bool sing = A.loff != nullptr, slp = A.sigma != nullptr, dlp = A.tau != nullptr;
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const int qb = sing ? A.loff[b] : 0, qe = sing ? A.loff[b + 1] : 1;
+    if (sing) {
+        int q = qb;
+        while (q < qe && A.src.st[A.lent[q]] == A.src.en[A.lent[q]]) ++q;
+        if (q == qe) return;
+    }
+    const int Q = p2x_order(LAP, sing, dlp, P), KQ = (Q + 1) * (Q + 1), cs = A.cs;
+    const bool both = !LAP && dlp && A.all;
+    const int nsum = dlp && A.all ? 4 : 1, gs = A.gs;
+    cd* acc = sm;                                       // [nsum][KQ]
+    cd* Y0 = acc + nsum * KQ;                           // [cs][KQ] F_n Z (Laplace H)
+    cd* Y1 = Y0 + (both ? (size_t)cs * KQ : 0);         // [cs][KQ] F_{n+1} Z (Helmholtz double layer)
+    cd* F = Y1 + (size_t)cs * KQ;                       // Helmholtz [P + 2][gs]
+    cd* geo = F + (LAP ? 0 : (size_t)(P + 2) * gs);     // [5][32]: x+, x-, zeta, w, radial factor
+    cd* wt = geo + 5 * 32;                              // [32][5]: s, -k t (y.nu), t n3, t nu+, t nu-
+    const QTables& q = LAP ? (sing ? A.T.T : A.T.U) : A.T.Z;
+    cd* o = A.out + (int64_t)rhs * A.ncoef + A.eoff[b];
+    // the columns of a warp: the four schedulers of an SM get equal shares
+    const int per = 32 / cs, src = lane & (cs - 1), col = (wid < 4 ? wid : 11 - wid) * per + lane / cs;
+    // products of a weight and a table: s F_n Z and -k t (y.nu) F_{n+1} Z into W, the
+    // others into C3, C+, C-
+    const int p0 = slp ? 0 : LAP ? 2 : 1, p1 = dlp ? 5 : 1;
+    for (int pass = p0; pass < p1; pass += A.all ? 5 : LAP && pass == 0 ? 2 : 1) {
+    const int off = !LAP && !both && pass > 0 ? 1 : 0;  // F_{n+1} in the one table
+    __syncthreads();
+    for (int i = threadIdx.x; i < nsum * KQ; i += kP2xThreads) acc[i] = cd{0, 0};
+    int qn = qb, j0 = 0;
+    while (qn < qe) {
+        // the lane's source of the next 32, and where these end
+        int64_t j = -1;
+        int gn = 0;
+        while (qn < qe && gn < gs) {
+            const int box = sing ? A.lent[qn] : b;
+            const int k0 = A.src.st[box] + j0, m = min(A.src.en[box] - k0, gs - gn);
+            if (lane >= gn && lane < gn + m) j = A.src.at(k0 + (lane - gn));
+            gn += m;
+            if (k0 + m == A.src.en[box]) {
+                ++qn;
+                j0 = 0;
+            } else {
+                j0 += m;
+            }
+        }
+        __syncthreads();                                // the last group has been used
+        if (wid == 0 && j >= 0) {
+            cd y[3];
+            for (int a = 0; a < 3; ++a)
+                y[a] = cd{A.xr[a * A.n + j], A.xi[a * A.n + j]} - cd{A.cre[3 * b + a], A.cim[3 * b + a]};
+            cd xp = y[0] + mul_i(y[1]), xm = y[0] - mul_i(y[1]), zeta = y[2], w = xp * xm + zeta * zeta, f0 = {1, 0};
+            if (LAP) {
+                xm = -xm;
+                if (sing) {
+                    f0 = crcp_general(csqrt_p(w));
+                    w = crcp_general(w);
+                    xp = xp * w;
+                    xm = xm * w;
+                    zeta = zeta * w;
+                }
+            } else {
+                radial_rows(sing, A.kappa, w, P + 1, F + lane, gs);
+            }
+            geo[lane] = xp;
+            geo[32 + lane] = xm;
+            geo[64 + lane] = zeta;
+            geo[96 + lane] = w;
+            geo[128 + lane] = f0;
+            cd* v = wt + 5 * lane;
+            v[0] = slp ? A.sigma[(int64_t)rhs * A.dstride + j] : cd{0, 0};
+            if (dlp) {
+                cd t = A.tau[(int64_t)rhs * A.dstride + j], nn[3];
+                for (int a = 0; a < 3; ++a) nn[a] = cd{A.nr[a * A.n + j], A.ni[a * A.n + j]};
+                v[1] = (-A.kappa) * ((y[0] * nn[0] + y[1] * nn[1] + y[2] * nn[2]) * t);
+                v[2] = nn[2] * t;
+                v[3] = (nn[0] + mul_i(nn[1])) * t;
+                v[4] = (nn[0] - mul_i(nn[1])) * t;
+            }
+        }
+        for (int g0 = 0; g0 < gn; g0 += cs) {
+            const int cn = min(cs, gn - g0), s = g0 + src;
+            __syncthreads();                            // group ready, last chunk summed
+            if (src < cn) {
+                const cd xp = geo[s], xm = geo[32 + s], zeta = geo[64 + s], w = geo[96 + s], f0 = geo[128 + s];
+                cd *y0 = Y0 + (size_t)src * KQ, *y1 = Y1 + (size_t)src * KQ;
+                for (int m = col; m <= Q; m += kP2xThreads / cs) {
+                    cd pp = f0, pm = f0, bp = xp, bm = xm;
+                    for (int e = m; e; e >>= 1) {
+                        if (e & 1) {
+                            pp = pp * bp;
+                            pm = pm * bm;
+                        }
+                        if (e > 1) {
+                            bp = bp * bp;
+                            bm = bm * bm;
+                        }
+                    }
+                    cd q2 = {0, 0}, q1 = {__ldg(q.D + m), 0};
+                    for (int n = m; n <= Q; ++n) {
+                        cd t = LAP ? q1 : F[(n + off) * gs + s] * q1;
+                        y0[nmi(n, m)] = t * pp;
+                        if (m) y0[nmi(n, -m)] = t * pm;
+                        if (both) {
+                            t = F[(n + 1) * gs + s] * q1;
+                            y1[nmi(n, m)] = t * pp;
+                            if (m) y1[nmi(n, -m)] = t * pm;
+                        }
+                        if (n == Q) break;
+                        cd v = rmac(__ldg(q.A + nmi(n + 1, m)) * (zeta * q1), -__ldg(q.B + nmi(n + 1, m)), w * q2);
+                        q2 = q1;
+                        q1 = v;
+                    }
+                }
+            }
+            __syncthreads();
+            const cd* wc = wt + 5 * g0;
+            for (int i = threadIdx.x; i < nsum * KQ; i += kP2xThreads) {
+                const int sum = i / KQ, k = i - sum * KQ;
+                cd a = acc[i];
+                if (!A.all) {
+                    for (int s2 = 0; s2 < cn; ++s2) a = cmac(a, wc[5 * s2 + pass], Y0[(size_t)s2 * KQ + k]);
+                } else if (sum == 0) {
+                    if (slp)
+                        for (int s2 = 0; s2 < cn; ++s2) a = cmac(a, wc[5 * s2], Y0[(size_t)s2 * KQ + k]);
+                    if (both)
+                        for (int s2 = 0; s2 < cn; ++s2) a = cmac(a, wc[5 * s2 + 1], Y1[(size_t)s2 * KQ + k]);
+                } else {
+                    const cd* Y = LAP ? Y0 : Y1;
+                    for (int s2 = 0; s2 < cn; ++s2) a = cmac(a, wc[5 * s2 + 1 + sum], Y[(size_t)s2 * KQ + k]);
+                }
+                acc[i] = a;
+            }
+        }
+    }
+    __syncthreads();
+    for (int k = threadIdx.x; k < (P + 1) * (P + 1); k += kP2xThreads) {
+        int n = (int)sqrtf((float)k);
+        while (n * n > k) --n;
+        while ((n + 1) * (n + 1) <= k) ++n;
+        const int m = k - n * n - n, mu = -m, nn = LAP && sing ? n + 1 : n - 1;
+        auto at = [&](int sum, int mm) -> cd {
+            const int nx = sum ? nn : n;
+            if (!A.all && sum != max(pass - 1, 0)) return cd{0, 0};
+            if (nx < 0 || mm > nx || -mm > nx) return cd{0, 0};
+            return acc[(A.all ? sum * KQ : 0) + nmi(nx, mm)];
+        };
+        cd v = at(0, mu);
+        if (dlp) {
+            const double g3 = LAP ? (sing ? -1.0 : 1.0) : __ldg(A.T.g3 + nmi(n, mu));
+            const double gp = LAP ? 0.5 : __ldg(A.T.gp + nmi(n, mu)), gm = LAP ? 0.5 : __ldg(A.T.gm + nmi(n, mu));
+            v += g3 * at(1, mu) - gp * at(2, mu - 1) + gm * at(3, mu + 1);
+        }
+        if (LAP) v = (m & 1) ? -v : v;
+        else v = mul_i(A.kappa * (2.0 * n + 1.0) * v);
+        o[k] = sing || pass > p0 ? o[k] + v : v;
+    }
+    }
+}
+
 template <bool LAP, bool GRAD>
 void launch_items(EvalK A, cudaStream_t st, int nrhs, int groups) {
     const size_t smem = LAP ? 0 : sizeof(cd) * kEvalWarps * (size_t)(A.E.maxP + 2) * 32;
@@ -363,6 +576,45 @@ void eval3_build(Eval3* E, const std::vector<int>& leaves, const std::vector<int
     E->own.alloc(l3off.back());
     k_eval3_own<<<((int)leaves.size() + 127) / 128, 128, 0, stream>>>((int)leaves.size(), d_leaves, d_l3off, E->own.get());
     CFMM_LAUNCHED();
+}
+
+bool p2x3_apply(cfmm_plan_s* P, const Eval3Tables& T, const P2x3Args& A, const cd* sigma, const cd* tau, int64_t dstride,
+                cd* out, int nrhs) {
+    if (A.cnt <= 0) return true;
+    TreeDev& Tr = P->tree;
+    const bool lap = A.kappa == 0.0, dlp = tau != nullptr;
+    const int Q = p2x_order(lap, A.sing, dlp, A.P);
+    const size_t KQ = (size_t)(Q + 1) * (Q + 1);
+    P2xK K{P->xr.get(), P->xi.get(), P->nr.get(), P->ni.get(), P->n, sigma, tau, dstride, A.boxes,
+           A.sing ? Tr.loff[3].get() : nullptr, A.sing ? Tr.lent[3].get() : nullptr, source_range(P), A.Plev,
+           Tr.level.get(), Tr.cen_re.get(), Tr.cen_im.get(), A.eoff, A.ncoef, A.kappa, T, 0, 32, true, out};
+    auto bytes = [&](bool all, int cs, int gs) {
+        return sizeof(cd) * ((all && dlp ? 4 : 1) * KQ + cs * (all && dlp && !lap ? 2 : 1) * KQ +
+                             (lap ? 0 : (size_t)(A.P + 2) * gs) + 10 * 32);
+    };
+    auto fit = [&](size_t limit, bool all, int gs, int least) {
+        for (int cs = gs; cs >= least && !K.cs; cs /= 2)
+            if (bytes(all, cs, gs) <= limit) {
+                K.cs = cs;
+                K.gs = gs;
+                K.all = all;
+            }
+    };
+    // the largest chunk that leaves two blocks an SM, or one; a product a pass where
+    // the sums leave no room for two sources; the least that any order needs
+    fit(kP2xSmem / 2, true, 32, 4);
+    fit(kP2xSmem, true, 32, 2);
+    fit(kP2xSmem, false, 32, 2);
+    fit(kP2xSmem, !dlp, 8, 1);
+    if (!K.cs) return false;
+    const size_t smem = bytes(K.all, K.cs, K.gs);
+    const void* f = lap ? (const void*)k_p2x3<true> : (const void*)k_p2x3<false>;
+    CFMM_CUDA(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kP2xSmem));
+    dim3 g(A.cnt, nrhs);
+    if (lap) k_p2x3<true><<<g, kP2xThreads, smem, P->stream>>>(K);
+    else k_p2x3<false><<<g, kP2xThreads, smem, P->stream>>>(K);
+    CFMM_LAUNCHED();
+    return true;
 }
 
 void eval3_apply(cfmm_plan_s* P, Eval3* E, const Eval3Tables& T, const Eval3Args& A, bool l2p, cd* u, cd* g, int nrhs) {

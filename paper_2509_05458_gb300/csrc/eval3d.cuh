@@ -1,5 +1,5 @@
-// FP64 evaluation of 3D expansions at points: M2P (List 3) and L2P, and their
-// gradients (eval3d.cu).
+// FP64 expansions of and at points, 3D: P2M, P2L, M2P (List 3), L2P and gradients of
+// the last two (eval3d.cu).
 #pragma once
 
 #include "kernels.cuh"
@@ -40,6 +40,20 @@ struct Eval3Args {
     double kappa;                 // 0: Laplace
     const cd *mp, *loc;
 };
+// P2M of `cnt` leaves (written), or P2L into `cnt` boxes over their List 4 (added), FP64,
+// single layer (sigma) and/or double layer (tau); P: the largest order among the boxes
+struct P2x3Args {
+    const int* boxes;
+    int cnt;
+    bool sing;                    // P2L
+    int P;
+    const int* Plev;
+    const int64_t* eoff;
+    int64_t ncoef;
+    double kappa;                 // 0: Laplace
+};
+bool p2x3_apply(cfmm_plan_s* P, const Eval3Tables& T, const P2x3Args& A, const cd* sigma, const cd* tau, int64_t dstride,
+                cd* out, int nrhs);
 // u [rhs][n] += M2P, and L2P when l2p; g [rhs][3][n] += gradients of both (either may be null)
 void eval3_apply(cfmm_plan_s* P, Eval3* E, const Eval3Tables& T, const Eval3Args& A, bool l2p, cd* u, cd* g, int nrhs);
 

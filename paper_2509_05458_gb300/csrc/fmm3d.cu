@@ -31,169 +31,6 @@
 
 namespace cfmm {
 
-__host__ __device__ __forceinline__ int nm_idx(int n, int m) { return n * n + n + m; }
-
-// Table of U_n^m (reg = true) or T_n^m (reg = false), n <= P, of the complex
-// 3-vector (a0, a1, a2), written to tab[nm_idx(n, m)]. Column m of each sign is
-// computed by the threads t = lane0 .. in parallel (one column per thread).
-__device__ void solid_table(bool reg, cd a0, cd a1, cd a2, int P, cd* tab, int t0, int nthreads) {
-    cd xp = a0 + mul_i(a1), xm = a0 - mul_i(a1), z = a2;
-    cd r2 = xp * xm + z * z;
-    cd ir2 = {0, 0}, irho = {0, 0};
-    if (!reg) {
-        ir2 = cinv(r2);
-        irho = cinv(csqrt_p(r2));
-    }
-    for (int col = t0; col < 2 * P + 1; col += nthreads) {
-        int m = col <= P ? col : col - P;     // col 0..P: m >= 0 with x+; P+1..2P: m = 1..P with x-
-        bool neg = col > P;
-        cd xs = neg ? xm : xp;
-        // diagonal value
-        cd d;
-        if (reg) {
-            // U_m^m = (-x/2)^m / m!
-            d = cd{1, 0};
-            cd f = -0.5 * xs;
-            for (int j = 1; j <= m; ++j) d = d * f * (1.0 / j);
-        } else {
-            // T_m^m = (-1)^m (2m-1)!! x^m / rho^{2m+1}
-            d = irho;
-            for (int j = 1; j <= m; ++j) d = d * (-(2.0 * j - 1.0)) * (xs * ir2);
-        }
-        double sg = (neg && (m & 1)) ? -1.0 : 1.0;
-        tab[nm_idx(m, neg ? -m : m)] = sg * d;
-        if (m + 1 > P) continue;
-        cd p2 = d;
-        cd p1 = reg ? z * d : (2.0 * m + 1.0) * (z * ir2) * d;
-        tab[nm_idx(m + 1, neg ? -m : m)] = sg * p1;
-        for (int n = m + 2; n <= P; ++n) {
-            cd cur;
-            if (reg) cur = ((2.0 * n - 1.0) * (z * p1) - r2 * p2) * (1.0 / ((n - m) * (double)(n + m)));
-            else cur = ((2.0 * n - 1.0) * (z * p1) - ((double)(n - 1) * (n - 1) - (double)m * m) * p2) * ir2;
-            tab[nm_idx(n, neg ? -m : m)] = sg * cur;
-            p2 = p1;
-            p1 = cur;
-        }
-    }
-}
-
-__device__ __forceinline__ cd tab_get(const cd* tab, int n, int m) {
-    if (n < 0 || m > n || -m > n) return cd{0, 0};
-    return tab[nm_idx(n, m)];
-}
-
-struct Exp3Args {
-    const double* xr;
-    const double* xi;
-    const double* nr;
-    const double* ni;
-    int64_t n;
-    const cd* sigma;
-    const cd* tau;
-    int64_t dstride;
-    bool slp, dlp;
-    const int* blevel;
-    SubRange src;                // sources
-    const double* cre;
-    const double* cim;
-    const int* Plev;
-    const int64_t* eoff;
-    int64_t ncoef;
-};
-
-__device__ __forceinline__ void load3(const double* re, const double* im, int64_t n, int64_t j, cd* x) {
-    for (int a = 0; a < 3; ++a) x[a] = cd{re[a * n + j], im[a * n + j]};
-}
-
-// P2M (sing = 0) over a box's own points, or P2L (sing = 1) over its List-4 leaves.
-// chunk sources at a time: their U (or T) tables in shared memory; each thread
-// owns coefficients c and adds the sources' terms in source order.
-__global__ void k_point_to_exp3(Exp3Args A, const int* __restrict__ boxes, const int* __restrict__ loff,
-                                const int* __restrict__ lent, int sing, cd* __restrict__ out, int chunk) {
-    extern __shared__ cd sm[];
-    int b = boxes[blockIdx.x];
-    int rhs = blockIdx.y;
-    int P = A.Plev[A.blevel[b]];
-    int nc = (P + 1) * (P + 1);
-    int PT = sing ? P + 1 : P;                 // table order (P2L's dipole needs T_{k+1})
-    int nt = (PT + 1) * (PT + 1);
-    cd* acc = sm;
-    cd* tabs = sm + nc;                        // [chunk][nt]
-    cd* srcv = tabs + (size_t)chunk * nt;      // [chunk][6]: sigma, tau, nu+, nu-, n3
-    for (int c = threadIdx.x; c < nc; c += blockDim.x) acc[c] = cd{0, 0};
-    cd cen[3];
-    for (int a = 0; a < 3; ++a) cen[a] = cd{A.cre[3 * b + a], A.cim[3 * b + a]};
-    int qa = loff ? loff[b] : 0, qb = loff ? loff[b + 1] : 1;
-    for (int q = qa; q < qb; ++q) {
-        int src = loff ? lent[q] : b;
-        int s0 = A.src.st[src], s1 = A.src.en[src];
-        for (int c0 = s0; c0 < s1; c0 += chunk) {
-            int cn = min(chunk, s1 - c0);
-            __syncthreads();
-            // tables: threads split (source, column)
-            int cols = 2 * PT + 1;
-            for (int w = threadIdx.x; w < cn * cols; w += blockDim.x) {
-                int s = w / cols, col = w - s * cols;
-                const int64_t j = A.src.at(c0 + s);
-                cd y[3];
-                load3(A.xr, A.xi, A.n, j, y);
-                solid_table(!sing, y[0] - cen[0], y[1] - cen[1], y[2] - cen[2], PT, tabs + (size_t)s * nt, col, cols);
-                if (col == 0) {
-                    cd* v = srcv + (size_t)s * 6;
-                    v[0] = A.slp ? A.sigma[rhs * A.dstride + j] : cd{0, 0};
-                    v[1] = A.dlp ? A.tau[rhs * A.dstride + j] : cd{0, 0};
-                    if (A.dlp) {
-                        cd nn[3];
-                        load3(A.nr, A.ni, A.n, j, nn);
-                        v[2] = nn[0] + mul_i(nn[1]);
-                        v[3] = nn[0] - mul_i(nn[1]);
-                        v[4] = nn[2];
-                    }
-                }
-            }
-            __syncthreads();
-            for (int c = threadIdx.x; c < nc; c += blockDim.x) {
-                int n = (int)sqrt((double)c);
-                while (n * n > c) --n;
-                while ((n + 1) * (n + 1) <= c) ++n;
-                int m = c - n * n - n;
-                double sg = (m & 1) ? -1.0 : 1.0;
-                cd a = acc[c];
-                for (int s = 0; s < cn; ++s) {
-                    const cd* tb = tabs + (size_t)s * nt;
-                    const cd* v = srcv + (size_t)s * 6;
-                    cd term = {0, 0};
-                    if (!sing) {
-                        // (-1)^m [sigma U_n^{-m} + tau n.grad U_n^{-m}]
-                        if (A.slp) term = v[0] * tb[nm_idx(n, -m)];
-                        if (A.dlp) {
-                            cd g = (-0.5 * v[2]) * tab_get(tb, n - 1, -m - 1) + (0.5 * v[3]) * tab_get(tb, n - 1, -m + 1) +
-                                   v[4] * tab_get(tb, n - 1, -m);
-                            term += v[1] * g;
-                        }
-                    } else {
-                        // (-1)^l [sigma T_k^{-l} + tau n.grad T_k^{-l}]
-                        if (A.slp) term = v[0] * tb[nm_idx(n, -m)];
-                        if (A.dlp) {
-                            cd g = (-0.5 * v[2]) * tab_get(tb, n + 1, -m - 1) + (0.5 * v[3]) * tab_get(tb, n + 1, -m + 1) -
-                                   v[4] * tab_get(tb, n + 1, -m);
-                            term += v[1] * g;
-                        }
-                    }
-                    a += sg * term;
-                }
-                acc[c] = a;
-            }
-        }
-    }
-    __syncthreads();
-    cd* o = out + (int64_t)rhs * A.ncoef + A.eoff[b];
-    for (int c = threadIdx.x; c < nc; c += blockDim.x) {
-        if (sing) o[c] += acc[c];
-        else o[c] = acc[c];
-    }
-}
-
 // ---------------------------------------------------------------------------
 // host side
 // ---------------------------------------------------------------------------
@@ -244,9 +81,6 @@ static int nterms_laplace3(int k, double eps) {
         if (t <= eps) return n;
     }
 }
-
-constexpr int kExp3Threads = 128;
-constexpr int kMax3Smem = 200 * 1024;
 
 void fmm3d_setup(cfmm_plan_s* P) {
     TreeDev& T = P->tree;
@@ -300,8 +134,6 @@ void fmm3d_setup(cfmm_plan_s* P) {
                                   cudaMemcpyHostToDevice, st));
     CFMM_CUDA(cudaStreamSynchronize(st));
     eval3_build(&S->eval, S->leaves_l0, T.hloff[2], hst, hen, S->d_leaves_l0.get(), T.loff[2].get(), st);
-    for (auto f : {(const void*)k_point_to_exp3})
-        CFMM_CUDA(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, kMax3Smem));
     S->tr = lap3_tr_create(P, maxP);
 }
 
@@ -334,14 +166,6 @@ void fmm3d_apply(cfmm_plan_s* P, const cd* sigma, const cd* tau, int64_t dstride
     cd* mp = P->mpole.get();
     cd* lc = P->local.get();
     int maxP = S->maxP;
-    Exp3Args A{P->xr.get(), P->xi.get(), P->nr.get(), P->ni.get(), P->n, sigma, tau, dstride, P->slp, P->dlp,
-               T.level.get(), source_range(P), T.cen_re.get(), T.cen_im.get(), S->dPlev.get(),
-               S->exp_off.get(), S->ncoef};
-    auto p2x_smem = [&](int PT, int& chunk) {
-        size_t nt = (size_t)(PT + 1) * (PT + 1);
-        chunk = (int)std::max<size_t>(1, std::min<size_t>(16, (96 * 1024) / (nt * sizeof(cd))));
-        return sizeof(cd) * ((size_t)(maxP + 1) * (maxP + 1) + (size_t)chunk * nt + (size_t)chunk * 6);
-    };
     // (3) P2P (writes u) on the side stream, beside the far field
     {
         cudaStream_t ns = near_fork(P);
@@ -350,22 +174,14 @@ void fmm3d_apply(cfmm_plan_s* P, const cd* sigma, const cd* tau, int64_t dstride
             launch_p2p_grad(3, P->kernel, K, S->d_leaves_l0.get(), (int)S->leaves_l0.size(), near_ranges(P), T.loff[0].get(), T.lent[0].get(), g, nrhs, ns, P->leaf_size);
     }
     near_launched(P);
-    // (1) P2M (single layer: one lane per harmonic column; complex64 products
-    // with FP64 sums in mixed precision)
+    // (1) P2M (single layer: complex64 products with FP64 sums in mixed precision)
     bool slp1 = P->slp && !P->dlp;
     bool p2m_done = slp1 && mixed &&
                     lap3_p2m32(S->tr, P, S->d_leaves_l0.get(), (int)S->leaves_l0.size(), maxP, S->dPlev.get(),
                                S->exp_off.get(), S->ncoef, sigma, dstride, mp, nrhs);
-    if (!p2m_done && !(slp1 && lap3_p2m_slp(S->tr, P, S->d_leaves_l0.get(), (int)S->leaves_l0.size(), maxP,
-                                            S->dPlev.get(), S->exp_off.get(), S->ncoef, sigma, dstride, mp, nrhs))) {
-        int chunk;
-        size_t smem = p2x_smem(maxP, chunk);
-        dim3 g((unsigned)S->leaves_l0.size(), nrhs);
-        if (g.x) {
-            k_point_to_exp3<<<g, kExp3Threads, smem, st>>>(A, S->d_leaves_l0.get(), nullptr, nullptr, 0, mp, chunk);
-            CFMM_LAUNCHED();
-        }
-    }
+    P2x3Args X{S->d_leaves_l0.get(), (int)S->leaves_l0.size(), false, maxP, S->dPlev.get(), S->exp_off.get(), S->ncoef,
+               0.0};
+    if (!p2m_done) lap3_p2x(S->tr, P, X, sigma, tau, dstride, mp, nrhs);
     rec(2);
     int Pu = S->Plev[0];
     // (2) M2M
@@ -376,14 +192,10 @@ void fmm3d_apply(cfmm_plan_s* P, const cd* sigma, const cd* tau, int64_t dstride
     lap3_m2l(S->tr, P, S->l0, T.nlevels, Pu, S->exp_off.get(), S->ncoef, mp, lc, nrhs);
     rec(4);
     // (6) P2L
-    if (S->n_p2l > 0) {
-        int chunk;
-        size_t smem = p2x_smem(maxP + 1, chunk);
-        dim3 g(S->n_p2l, nrhs);
-        k_point_to_exp3<<<g, kExp3Threads, smem, st>>>(A, S->d_p2l_boxes.get(), T.loff[3].get(), T.lent[3].get(), 1,
-                                                       lc, chunk);
-        CFMM_LAUNCHED();
-    }
+    X.boxes = S->d_p2l_boxes.get();
+    X.cnt = S->n_p2l;
+    X.sing = true;
+    lap3_p2x(S->tr, P, X, sigma, tau, dstride, lc, nrhs);
     rec(5);
     // (7) L2L
     for (int l = S->l0; l + 1 < T.nlevels; ++l)

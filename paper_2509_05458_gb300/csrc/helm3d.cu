@@ -65,7 +65,6 @@ namespace {
 
 __host__ __device__ __forceinline__ int nmi(int n, int m) { return n * n + n + m; }
 
-constexpr int kH3Threads = 256;
 constexpr int kH3MaxP = kMaxP3Top;   // expansion order limit of this path
 constexpr int kH3Smem = 220 * 1024;  // dynamic shared memory ceiling per block
 
@@ -336,323 +335,10 @@ static H3Tables* tables(int P) {
 // ---------------------------------------------------------------------------
 // device helpers
 // ---------------------------------------------------------------------------
-struct ZCoef {
-    const double* A;
-    const double* B;
-    const double* dg;    // sqrt((2m-1)/(2m))
-    const double* s21;   // sqrt(2m+1)
-    const int* knm;      // k -> n * 256 + (m + 128)
-    const double* g3;    // gradient coefficients by nmi(n, m)
-    const double* gp;
-    const double* gm;
-};
-
 __device__ __forceinline__ void nm_tab(const int* knm, int k, int& n, int& m) {
     int v = __ldg(knm + k);
     n = v >> 8;
     m = (v & 255) - 128;
-}
-
-// Z table of (a0, a1, a2) up to order P into tab[nmi(n, m)]; columns split
-// over threads t0, t0 + nthreads, ...
-__device__ void z_table(ZCoef zc, cd a0, cd a1, cd a2, int P, cd* tab, int t0, int nthreads) {
-    cd xp = a0 + mul_i(a1), xm = a0 - mul_i(a1), z = a2;
-    cd r2 = xp * xm + z * z;
-    for (int col = t0; col < 2 * P + 1; col += nthreads) {
-        int m = col <= P ? col : col - P;
-        bool neg = col > P;
-        cd xs = neg ? xm : xp;
-        cd d = {1, 0};
-        for (int j = 1; j <= m; ++j) d = (-__ldg(zc.dg + j)) * (xs * d);
-        int mi = neg ? -m : m;
-        tab[nmi(m, mi)] = d;
-        if (m + 1 > P) continue;
-        cd p2 = d, p1 = __ldg(zc.s21 + m) * (z * d);
-        tab[nmi(m + 1, mi)] = p1;
-        for (int n = m + 2; n <= P; ++n) {
-            int k = nmi(n, m);
-            cd cur = zc.A[k] * (z * p1) - zc.B[k] * (r2 * p2);
-            tab[nmi(n, mi)] = cur;
-            p2 = p1;
-            p1 = cur;
-        }
-    }
-}
-
-// F[n] = f_n(k rho) / rho^n for n = 0..N (f = j if reg, else h); rho = 0 (reg
-// only) gives the limits k^n / (2n+1)!!
-__device__ void radial_seq(bool reg, double kappa, cd r2, int N, cd* F) {
-    cd rho = csqrt_p(r2);
-    if (rho.x == 0.0 && rho.y == 0.0) {
-        double v = 1.0;
-        for (int n = 0; n <= N; ++n) {
-            F[n] = cd{v, 0};
-            v *= kappa / (2.0 * n + 3.0);
-        }
-        return;
-    }
-    cd z = kappa * rho;
-    if (reg) sph_j_seq(z, N, F);
-    else sph_h_seq(z, N, F);
-    cd ir = cinv(rho), p = {1, 0};
-    for (int n = 0; n <= N; ++n) {
-        F[n] = F[n] * p;
-        p = p * ir;
-    }
-}
-
-__device__ __forceinline__ cd zget(const cd* tab, int n, int m) {
-    if (n < 0 || m > n || -m > n) return cd{0, 0};
-    return tab[nmi(n, m)];
-}
-
-struct Exp3hArgs {
-    const double* xr;
-    const double* xi;
-    const double* nr;
-    const double* ni;
-    int64_t n;
-    const cd* sigma;
-    const cd* tau;
-    int64_t dstride;
-    bool slp, dlp;
-    const int* blevel;
-    SubRange pts;                // sources (Exp3hArgs, k_p2m3f) or targets (k_l2p3f)
-    const double* cre;
-    const double* cim;
-    const int* Plev;
-    const int64_t* eoff;
-    int64_t ncoef;
-    double kappa;
-    ZCoef zc;
-};
-
-__device__ __forceinline__ void load3(const double* re, const double* im, int64_t n, int64_t j, cd* x) {
-    for (int a = 0; a < 3; ++a) x[a] = cd{re[a * n + j], im[a * n + j]};
-}
-
-// P2M (sing = 0: R waves, the box's own points) or P2L (sing = 1: S waves,
-// the box's List-4 leaves). Sources are staged chunk by chunk: Z table, radial
-// factors and (sigma, tau, nu+, nu-, n3, y.n) per source; each thread owns
-// coefficients and adds the sources' terms in source order.
-__global__ void k_p2x3h(Exp3hArgs A, const int* __restrict__ boxes, const int* __restrict__ loff,
-                        const int* __restrict__ lent, int sing, cd* __restrict__ out, int chunk) {
-    extern __shared__ cd sm[];
-    int b = boxes[blockIdx.x];
-    int rhs = blockIdx.y;
-    int P = A.Plev[A.blevel[b]];
-    int nc = (P + 1) * (P + 1);
-    cd* acc = sm;
-    cd* tabs = acc + nc;                           // [chunk][nc]
-    cd* rad = tabs + (size_t)chunk * nc;           // [chunk][P+2]
-    cd* srcv = rad + (size_t)chunk * (P + 2);      // [chunk][6]
-    for (int c = threadIdx.x; c < nc; c += blockDim.x) acc[c] = cd{0, 0};
-    cd cen[3];
-    for (int a = 0; a < 3; ++a) cen[a] = cd{A.cre[3 * b + a], A.cim[3 * b + a]};
-    int qa = loff ? loff[b] : 0, qb = loff ? loff[b + 1] : 1;
-    for (int q = qa; q < qb; ++q) {
-        int src = loff ? lent[q] : b;
-        int s0 = A.pts.st[src], s1 = A.pts.en[src];
-        for (int c0 = s0; c0 < s1; c0 += chunk) {
-            int cn = min(chunk, s1 - c0);
-            __syncthreads();
-            int cols = 2 * P + 1;
-            for (int w = threadIdx.x; w < cn * (cols + 1); w += blockDim.x) {
-                int s = w / (cols + 1), col = w - s * (cols + 1);
-                const int64_t j = A.pts.at(c0 + s);
-                cd y[3];
-                load3(A.xr, A.xi, A.n, j, y);
-                for (int a = 0; a < 3; ++a) y[a] = y[a] - cen[a];
-                if (col < cols) {
-                    z_table(A.zc, y[0], y[1], y[2], P, tabs + (size_t)s * nc, col, cols);
-                } else {
-                    cd r2 = y[0] * y[0] + y[1] * y[1] + y[2] * y[2];
-                    radial_seq(!sing, A.kappa, r2, P + 1, rad + (size_t)s * (P + 2));
-                    cd* v = srcv + (size_t)s * 6;
-                    v[0] = A.slp ? A.sigma[rhs * A.dstride + j] : cd{0, 0};
-                    v[1] = A.dlp ? A.tau[rhs * A.dstride + j] : cd{0, 0};
-                    if (A.dlp) {
-                        cd nn[3];
-                        load3(A.nr, A.ni, A.n, j, nn);
-                        v[2] = nn[0] + mul_i(nn[1]);
-                        v[3] = nn[0] - mul_i(nn[1]);
-                        v[4] = nn[2];
-                        v[5] = y[0] * nn[0] + y[1] * nn[1] + y[2] * nn[2];
-                    }
-                }
-            }
-            __syncthreads();
-            for (int c = threadIdx.x; c < nc; c += blockDim.x) {
-                int n, m;
-                nm_tab(A.zc.knm, c, n, m);
-                int mu = -m;
-                cd a = acc[c];
-                for (int s = 0; s < cn; ++s) {
-                    const cd* tb = tabs + (size_t)s * nc;
-                    const cd* F = rad + (size_t)s * (P + 2);
-                    const cd* v = srcv + (size_t)s * 6;
-                    cd Zv = tb[nmi(n, mu)];
-                    cd term = {0, 0};
-                    if (A.slp) term = v[0] * (F[n] * Zv);
-                    if (A.dlp) {
-                        cd g = {0, 0};
-                        if (n >= 1) {
-                            int kk = nmi(n, mu);
-                            g = (__ldg(A.zc.g3 + kk) * v[4]) * zget(tb, n - 1, mu);
-                            g = g - __ldg(A.zc.gp + kk) * (v[2] * zget(tb, n - 1, mu - 1));
-                            g = g + __ldg(A.zc.gm + kk) * (v[3] * zget(tb, n - 1, mu + 1));
-                        }
-                        cd dw = F[n] * g - A.kappa * (F[n + 1] * (Zv * v[5]));
-                        term += v[1] * dw;
-                    }
-                    a += term;
-                }
-                acc[c] = a;
-            }
-        }
-    }
-    __syncthreads();
-    cd* o = out + (int64_t)rhs * A.ncoef + A.eoff[b];
-    for (int c = threadIdx.x; c < nc; c += blockDim.x) {
-        int n, m;
-        nm_tab(A.zc.knm, c, n, m);
-        cd v = mul_i(A.kappa * (2.0 * n + 1.0) * acc[c]);
-        if (sing) o[c] += v;
-        else o[c] = v;
-    }
-}
-
-// Radial factors f_n(kappa rho)/rho^n, n <= P, of every point of the listed
-// boxes relative to a box centre (one thread per point): the centre is the
-// box itself (P2M, f = j) or, for P2L, the target box of List-4 entry q.
-__global__ void k_radial3h(Exp3hArgs A, const int* __restrict__ boxes, int nboxes, const int* __restrict__ loff,
-                           const int* __restrict__ lent, int sing, int P, const int* __restrict__ roff,
-                           cd* __restrict__ rad) {
-    int bi = blockIdx.x;
-    if (bi >= nboxes) return;
-    int b = boxes[bi];
-    cd cen[3];
-    for (int a = 0; a < 3; ++a) cen[a] = cd{A.cre[3 * b + a], A.cim[3 * b + a]};
-    int qa = loff ? loff[b] : 0, qb = loff ? loff[b + 1] : 1;
-    int64_t o = roff[bi];
-    for (int q = qa; q < qb; ++q) {
-        int src = loff ? lent[q] : b;
-        int s0 = A.pts.st[src], s1 = A.pts.en[src];
-        for (int j = s0 + threadIdx.x; j < s1; j += blockDim.x) {
-            cd y[3];
-            load3(A.xr, A.xi, A.n, A.pts.at(j), y);
-            for (int a = 0; a < 3; ++a) y[a] = y[a] - cen[a];
-            radial_seq(!sing, A.kappa, y[0] * y[0] + y[1] * y[1] + y[2] * y[2], P,
-                       rad + (o + (j - s0)) * (int64_t)(P + 1));
-        }
-        o += s1 - s0;
-    }
-}
-
-// One harmonic column of a single-layer source: Z_n^{mu}(y) sigma for
-// n = |mu|..P (mu >= 0 from x+, mu < 0 from x-, col = mu or P - mu), times
-// the radial factor F[n] (Helmholtz; none for Laplace), added into acc at
-// coefficient (n, -mu).
-template <bool LAP>
-__device__ __forceinline__ void p2x_column(const ZCoef& zc, int P, int col, cd xp, cd xm, cd z, cd r2, cd sg,
-                                           const cd* __restrict__ F, cd* acc) {
-    int am = col <= P ? col : col - P;
-    bool neg = col > P;
-    int m = neg ? am : -am;
-    cd xs = neg ? xm : xp;
-    cd d = sg;
-    for (int i = 1; i <= am; ++i) d = (-__ldg(zc.dg + i)) * (xs * d);
-    acc[nmi(am, m)] = LAP ? acc[nmi(am, m)] + d : cmac(acc[nmi(am, m)], F[am], d);
-    if (am + 1 > P) return;
-    cd p2 = d, p1 = __ldg(zc.s21 + am) * (z * d);
-    acc[nmi(am + 1, m)] = LAP ? acc[nmi(am + 1, m)] + p1 : cmac(acc[nmi(am + 1, m)], F[am + 1], p1);
-    for (int n = am + 2; n <= P; ++n) {
-        int k = nmi(n, am);
-        cd cur = __ldg(zc.A + k) * (z * p1) - __ldg(zc.B + k) * (r2 * p2);
-        acc[nmi(n, m)] = LAP ? acc[nmi(n, m)] + cur : cmac(acc[nmi(n, m)], F[n], cur);
-        p2 = p1;
-        p1 = cur;
-    }
-}
-
-// Single-layer P2M (sing = 0) / P2L (sing = 1). Each warp owns an accumulator
-// row in shared memory and takes the (source, column) items of its box in
-// rounds of 32 consecutive items, one per lane; with 2P+1 >= 32 columns the
-// lanes of a round hold distinct columns, so they touch disjoint coefficients,
-// and __syncwarp orders the rounds. With fewer columns a warp takes one source
-// at a time, one lane per column. The warp rows are summed in warp order at
-// the end, so the result does not depend on timing.
-// LAP: the 3D Laplace P2M, M_n^m = (-1)^m sum sigma U_n^{-m}(y) with the
-// regular solid harmonics U; since Z_n^{-m} = e s U_n^{-m} (s = sqrt((n-|m|)!
-// (n+|m|)!), e = +-1 as in lsd), M_n^m = lsd_n^m sum sigma Z_n^{-m}(y).
-template <bool LAP>
-__global__ void k_p2x3h_slp(Exp3hArgs A, const int* __restrict__ boxes, const int* __restrict__ loff,
-                            const int* __restrict__ lent, int sing, const int* __restrict__ roff,
-                            const cd* __restrict__ rad, cd* __restrict__ out, const double* __restrict__ lsd) {
-    extern __shared__ cd sm[];
-    int bi = blockIdx.x;
-    int b = boxes[bi];
-    int rhs = blockIdx.y;
-    int P = A.Plev[A.blevel[b]];
-    int nc = (P + 1) * (P + 1);
-    int C = 2 * P + 1;
-    int nwarp = blockDim.x >> 5, lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    cd* accw = sm + (size_t)wid * nc;
-    for (int c = lane; c < nc; c += 32) accw[c] = cd{0, 0};
-    __syncwarp();
-    cd cen[3];
-    for (int a = 0; a < 3; ++a) cen[a] = cd{A.cre[3 * b + a], A.cim[3 * b + a]};
-    int qa = loff ? loff[b] : 0, qb = loff ? loff[b + 1] : 1;
-    int64_t o = roff ? roff[bi] : 0;
-    for (int q = qa; q < qb; ++q) {
-        int src = loff ? lent[q] : b;
-        int s0 = A.pts.st[src], s1 = A.pts.en[src];
-        if (C >= 32) {
-            int items = (s1 - s0) * C;
-            for (int base = wid * 32; base < items; base += nwarp * 32) {
-                int it = base + lane;
-                if (it < items) {
-                    int js = it / C, col = it - js * C;
-                    const int64_t j = A.pts.at(s0 + js);
-                    cd y[3];
-                    load3(A.xr, A.xi, A.n, j, y);
-                    for (int a = 0; a < 3; ++a) y[a] = y[a] - cen[a];
-                    cd xp = y[0] + mul_i(y[1]), xm = y[0] - mul_i(y[1]), z = y[2];
-                    p2x_column<LAP>(A.zc, P, col, xp, xm, z, xp * xm + z * z, A.sigma[rhs * A.dstride + j],
-                                    LAP ? nullptr : rad + (o + js) * (int64_t)(P + 1), accw);
-                }
-                __syncwarp();
-            }
-        } else {
-            for (int k = s0 + wid; k < s1; k += nwarp) {
-                const int64_t j = A.pts.at(k);
-                if (lane < C) {
-                    cd y[3];
-                    load3(A.xr, A.xi, A.n, j, y);
-                    for (int a = 0; a < 3; ++a) y[a] = y[a] - cen[a];
-                    cd xp = y[0] + mul_i(y[1]), xm = y[0] - mul_i(y[1]), z = y[2];
-                    p2x_column<LAP>(A.zc, P, lane, xp, xm, z, xp * xm + z * z, A.sigma[rhs * A.dstride + j],
-                                    LAP ? nullptr : rad + (o + (k - s0)) * (int64_t)(P + 1), accw);
-                }
-            }
-        }
-        o += s1 - s0;
-    }
-    __syncthreads();
-    cd* op = out + (int64_t)rhs * A.ncoef + A.eoff[b];
-    for (int c = threadIdx.x; c < nc; c += blockDim.x) {
-        cd v = {0, 0};
-        for (int w = 0; w < nwarp; ++w) v += sm[(size_t)w * nc + c];
-        if (LAP) {
-            v = __ldg(lsd + c) * v;
-        } else {
-            int n, m;
-            nm_tab(A.zc.knm, c, n, m);
-            v = mul_i(A.kappa * (2.0 * n + 1.0) * v);
-        }
-        if (sing) op[c] += v;
-        else op[c] = v;
-    }
 }
 
 // ---------------------------------------------------------------------------
@@ -958,11 +644,6 @@ struct Helm3dState {
     std::vector<int> p2l_off;    // List-4 targets by level, likewise
     int n_p2l = 0;
     DevBuf<int> d_p2l_boxes;
-    // single-layer P2M / P2L: per listed box, the offset of its source points in
-    // the radial-factor buffer (prefix over the level's boxes)
-    DevBuf<int> d_p2m_roff, d_p2l_roff;
-    std::vector<int64_t> p2m_rtot, p2l_rtot;    // per level: points in the level's launch
-    DevBuf<cd> rad;
     H3Tables* tab = nullptr;
     PairSlots pairs;             // List-2 pairs, workspaces of the translations
     Eval3 eval;                  // M2P, L2P
@@ -1077,51 +758,19 @@ void helm3d_setup(cfmm_plan_s* P) {
     for (int l = 0; l < T.nlevels; ++l) S->p2l_off[l + 1] += S->p2l_off[l];
     S->n_p2l = (int)boxes.size();
     {
-        // radial-buffer offsets of the single-layer P2M / P2L launches
-        std::vector<int> hst(T.nboxes), hen(T.nboxes), tst(T.nboxes), ten(T.nboxes), l4e(std::max(1, l4[T.nboxes]));
-        const SubRange sr = source_range(P), tr = target_range(P);
-        CFMM_CUDA(cudaMemcpyAsync(hst.data(), sr.st, sizeof(int) * T.nboxes, cudaMemcpyDeviceToHost, st));
-        CFMM_CUDA(cudaMemcpyAsync(hen.data(), sr.en, sizeof(int) * T.nboxes, cudaMemcpyDeviceToHost, st));
+        std::vector<int> tst(T.nboxes), ten(T.nboxes);
+        const SubRange tr = target_range(P);
         CFMM_CUDA(cudaMemcpyAsync(tst.data(), tr.st, sizeof(int) * T.nboxes, cudaMemcpyDeviceToHost, st));
         CFMM_CUDA(cudaMemcpyAsync(ten.data(), tr.en, sizeof(int) * T.nboxes, cudaMemcpyDeviceToHost, st));
-        if (l4[T.nboxes] > 0)
-            CFMM_CUDA(cudaMemcpyAsync(l4e.data(), T.lent[3].get(), sizeof(int) * l4[T.nboxes], cudaMemcpyDeviceToHost,
-                                      st));
         CFMM_CUDA(cudaStreamSynchronize(st));
         eval3_build(&S->eval, S->leaves_l0, T.hloff[2], tst, ten, S->d_leaves_l0.get(), T.loff[2].get(), st);
         for (int b : S->leaves_l0) S->maxP_eval = std::max(S->maxP_eval, S->Plev[lvl[b]]);
-        std::vector<int> ro(byl.size()), rl(boxes.size());
-        S->p2m_rtot.assign(T.nlevels, 0);
-        S->p2l_rtot.assign(T.nlevels, 0);
-        for (int l = 0; l < T.nlevels; ++l) {
-            int64_t acc = 0;
-            for (int i = S->p2m_off[l]; i < S->p2m_off[l + 1]; ++i) {
-                ro[i] = (int)acc;
-                acc += hen[byl[i]] - hst[byl[i]];
-            }
-            S->p2m_rtot[l] = acc;
-            acc = 0;
-            for (int i = S->p2l_off[l]; i < S->p2l_off[l + 1]; ++i) {
-                rl[i] = (int)acc;
-                int b = boxes[i];
-                for (int q = l4[b]; q < l4[b + 1]; ++q) acc += hen[l4e[q]] - hst[l4e[q]];
-            }
-            S->p2l_rtot[l] = acc;
-        }
-        S->d_p2m_roff.alloc(std::max<size_t>(1, ro.size()));
-        S->d_p2l_roff.alloc(std::max<size_t>(1, rl.size()));
-        if (!ro.empty())
-            CFMM_CUDA(cudaMemcpyAsync(S->d_p2m_roff.get(), ro.data(), sizeof(int) * ro.size(), cudaMemcpyHostToDevice, st));
-        if (!rl.empty())
-            CFMM_CUDA(cudaMemcpyAsync(S->d_p2l_roff.get(), rl.data(), sizeof(int) * rl.size(), cudaMemcpyHostToDevice, st));
     }
     S->d_p2l_boxes.alloc(boxes.size());
     if (!boxes.empty())
         CFMM_CUDA(cudaMemcpyAsync(S->d_p2l_boxes.get(), boxes.data(), sizeof(int) * boxes.size(),
                                   cudaMemcpyHostToDevice, st));
     CFMM_CUDA(cudaStreamSynchronize(st));
-    for (auto f : {(const void*)k_p2x3h, (const void*)k_p2x3h_slp<false>})
-        CFMM_CUDA(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, kH3Smem));
 }
 
 void helm3d_apply(cfmm_plan_s* P, const cd* sigma, const cd* tau, int64_t dstride, cd* u, int nrhs, cd* g) {
@@ -1151,11 +800,6 @@ void helm3d_apply(cfmm_plan_s* P, const cd* sigma, const cd* tau, int64_t dstrid
     cd* mp = P->mpole.get();
     cd* lc = P->local.get();
     H3Tables* TB = S->tab;
-    ZCoef zc{TB->zA.get(), TB->zB.get(), TB->dg.get(), TB->s21.get(), TB->knm.get(),
-             TB->g3.get(), TB->gp.get(), TB->gm.get()};
-    Exp3hArgs A{P->xr.get(), P->xi.get(), P->nr.get(), P->ni.get(), P->n, sigma, tau, dstride, P->slp, P->dlp,
-                T.level.get(), source_range(P), T.cen_re.get(), T.cen_im.get(), S->dPlev.get(),
-                S->exp_off.get(), S->ncoef, P->kappa, zc};
     int maxP = S->maxP;
     // (3) P2P (writes u) on the side stream, beside the far field
     {
@@ -1166,31 +810,11 @@ void helm3d_apply(cfmm_plan_s* P, const cd* sigma, const cd* tau, int64_t dstrid
             launch_p2p_grad(3, P->kernel, K, S->d_leaves_l0.get(), (int)S->leaves_l0.size(), near_ranges(P), T.loff[0].get(), T.lent[0].get(), g, nrhs, ns, P->leaf_size);
     }
     near_launched(P);
-    auto p2x_smem = [&](int PL, int& chunk) {
-        size_t nc = (size_t)(PL + 1) * (PL + 1);
-        size_t per = nc + (PL + 2) + 6;
-        chunk = (int)std::max<size_t>(1, std::min<size_t>(32, (96 * 1024 / sizeof(cd) - nc) / per));
-        return sizeof(cd) * (nc + (size_t)chunk * per);
-    };
     bool slp_only = P->slp && !P->dlp;
-    auto slp_fits = [&](int l) {
-        size_t K = (size_t)(S->Plev[l] + 1) * (S->Plev[l] + 1);
-        return sizeof(cd) * (kH3Threads / 32) * K <= (size_t)kH3Smem;
-    };
-    // single-layer P2M / P2L of one level: radial factors of every source point,
-    // then one warp per source and one lane per harmonic column
-    auto p2x_slp = [&](int l, int sing, const int* boxes, int cnt, const int* roff, int64_t rtot, cd* dst) {
-        int PL = S->Plev[l];
-        S->rad.alloc((size_t)std::max<int64_t>(1, rtot) * (PL + 1));
-        k_radial3h<<<cnt, 128, 0, st>>>(A, boxes, cnt, sing ? T.loff[3].get() : nullptr,
-                                         sing ? T.lent[3].get() : nullptr, sing, PL, roff, S->rad.get());
-        CFMM_LAUNCHED();
-        size_t smem = sizeof(cd) * (size_t)(kH3Threads / 32) * (PL + 1) * (PL + 1);
-        dim3 g((unsigned)cnt, nrhs);
-        k_p2x3h_slp<false><<<g, kH3Threads, smem, st>>>(A, boxes, sing ? T.loff[3].get() : nullptr,
-                                                        sing ? T.lent[3].get() : nullptr, sing, roff, S->rad.get(),
-                                                        dst, nullptr);
-        CFMM_LAUNCHED();
+    auto p2x = [&](int l, bool sing, const int* boxes, int cnt, cd* dst) {
+        P2x3Args X{boxes, cnt, sing, S->Plev[l], S->dPlev.get(), S->exp_off.get(), S->ncoef, P->kappa};
+        CFMM_REQUIRE(p2x3_apply(P, eval3_tables(TB), X, sigma, tau, dstride, dst, nrhs), CFMM_EUNSUPPORTED,
+                     "3D Helmholtz P2M/P2L exceeds shared memory");
     };
     // (1) P2M, one launch per level (shared memory sized by that level's P)
     for (int l = S->l0; l < T.nlevels; ++l) {
@@ -1202,15 +826,7 @@ void helm3d_apply(cfmm_plan_s* P, const cd* sigma, const cd* tau, int64_t dstrid
                          S->exp_off.get(), S->ncoef, sigma, dstride, mp, nrhs);
             continue;
         }
-        if (slp_only && slp_fits(l)) {
-            p2x_slp(l, 0, S->d_p2m.get() + S->p2m_off[l], cnt, S->d_p2m_roff.get() + S->p2m_off[l], S->p2m_rtot[l], mp);
-            continue;
-        }
-        int chunk;
-        size_t smem = p2x_smem(S->Plev[l], chunk);
-        dim3 g((unsigned)cnt, nrhs);
-        k_p2x3h<<<g, kH3Threads, smem, st>>>(A, S->d_p2m.get() + S->p2m_off[l], nullptr, nullptr, 0, mp, chunk);
-        CFMM_LAUNCHED();
+        p2x(l, false, S->d_p2m.get() + S->p2m_off[l], cnt, mp);
     }
     rec(2);
     const Tr3Tables tr = tr3_tables(TB);
@@ -1226,17 +842,7 @@ void helm3d_apply(cfmm_plan_s* P, const cd* sigma, const cd* tau, int64_t dstrid
     for (int l = S->l0; l < T.nlevels; ++l) {
         int cnt = S->p2l_off[l + 1] - S->p2l_off[l];
         if (cnt <= 0) continue;
-        if (slp_only && slp_fits(l)) {
-            p2x_slp(l, 1, S->d_p2l_boxes.get() + S->p2l_off[l], cnt, S->d_p2l_roff.get() + S->p2l_off[l],
-                    S->p2l_rtot[l], lc);
-            continue;
-        }
-        int chunk;
-        size_t smem = p2x_smem(S->Plev[l], chunk);
-        dim3 g((unsigned)cnt, nrhs);
-        k_p2x3h<<<g, kH3Threads, smem, st>>>(A, S->d_p2l_boxes.get() + S->p2l_off[l], T.loff[3].get(),
-                                             T.lent[3].get(), 1, lc, chunk);
-        CFMM_LAUNCHED();
+        p2x(l, true, S->d_p2l_boxes.get() + S->p2l_off[l], cnt, lc);
     }
     rec(5);
     // (7) L2L
@@ -1269,30 +875,15 @@ Lap3Tr* lap3_tr_create(cfmm_plan_s* P, int Pord) {
     TreeDev& T = P->tree;
     Lap3Tr* L = new Lap3Tr();
     L->tab = tables(Pord);
-    CFMM_CUDA(cudaFuncSetAttribute((const void*)k_p2x3h_slp<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                   kH3Smem));
     L->Pord = Pord;
     pair_slots_build(P, &L->pairs, T.hloff[1], T.l0);
     return L;
 }
 
-bool lap3_p2m_slp(Lap3Tr* L, cfmm_plan_s* P, const int* leaves, int cnt, int maxP, const int* dPlev,
-                  const int64_t* eoff, int64_t ncoef, const cd* sigma, int64_t dstride, cd* out, int nrhs) {
-    size_t smem = sizeof(cd) * (size_t)(kH3Threads / 32) * (maxP + 1) * (maxP + 1);
-    if (smem > (size_t)kH3Smem || maxP > L->Pord) return false;
-    if (cnt <= 0) return true;
-    TreeDev& T = P->tree;
-    H3Tables* TB = L->tab;
-    ZCoef zc{TB->zA.get(), TB->zB.get(), TB->dg.get(), TB->s21.get(), TB->knm.get(),
-             TB->g3.get(), TB->gp.get(), TB->gm.get()};
-    Exp3hArgs A{P->xr.get(), P->xi.get(), nullptr, nullptr, P->n, sigma, nullptr, dstride, true, false,
-                T.level.get(), source_range(P), T.cen_re.get(), T.cen_im.get(), dPlev, eoff, ncoef,
-                0.0, zc};
-    dim3 g((unsigned)cnt, nrhs);
-    k_p2x3h_slp<true><<<g, kH3Threads, smem, P->stream>>>(A, leaves, nullptr, nullptr, 0, nullptr, nullptr, out,
-                                                          TB->lsd.get());
-    CFMM_LAUNCHED();
-    return true;
+void lap3_p2x(Lap3Tr* L, cfmm_plan_s* P, const P2x3Args& A, const cd* sigma, const cd* tau, int64_t dstride, cd* out,
+              int nrhs) {
+    CFMM_REQUIRE(p2x3_apply(P, eval3_tables(L->tab), A, sigma, tau, dstride, out, nrhs), CFMM_EUNSUPPORTED,
+                 "3D Laplace P2M/P2L exceeds shared memory");
 }
 
 bool lap3_p2m32(Lap3Tr* L, cfmm_plan_s* P, const int* leaves, int cnt, int maxP, const int* dPlev,

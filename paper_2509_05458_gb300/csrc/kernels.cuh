@@ -131,10 +131,10 @@ constexpr int kMaxP3Top = 63;
 struct Lap3Tr;
 Lap3Tr* lap3_tr_create(cfmm_plan_s* P, int Pord);
 void lap3_tr_destroy(Lap3Tr* L);
-// single-layer 3D Laplace P2M over `leaves` (one column per lane); false when
-// the order does not fit the kernel (the caller then uses the general P2M)
-bool lap3_p2m_slp(Lap3Tr* L, cfmm_plan_s* P, const int* leaves, int cnt, int maxP, const int* dPlev,
-                  const int64_t* eoff, int64_t ncoef, const cd* sigma, int64_t dstride, cd* out, int nrhs);
+// P2M, P2L in FP64 (eval3d.cuh)
+struct P2x3Args;
+void lap3_p2x(Lap3Tr* L, cfmm_plan_s* P, const P2x3Args& A, const cd* sigma, const cd* tau, int64_t dstride, cd* out,
+              int nrhs);
 // M2P and L2P in FP64 (eval3d.cuh)
 struct Eval3;
 struct Eval3Args;
