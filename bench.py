@@ -122,7 +122,7 @@ def profile_figures(name, files):
 # the source file of each profiled kernel (a summary is used only while its
 # recorded hash matches this file)
 P2P_SOURCES = ("p2p.cu",)
-TR3H_SOURCES = ("helm3d.cu",)
+PAIRS3D_SOURCES = ("pairs3d.cu",)
 
 
 def _peaks():
@@ -391,7 +391,7 @@ def rooflines(W, r):
     mixed = r["mixed"]
     kt, work = mixed["kt"], mixed["work"]
     out = []
-    m2l = {"kernel": "M2L" + (" (k_tr3h, modes M2L)" if W["DIM"] == 3 and W["KERNEL"] else ""),
+    m2l = {"kernel": "M2L" + (" (k_pair_*)" if W["DIM"] == 3 and W["KERNEL"] else ""),
            "bound": "alu", "unit": "GFLOP/s", "ms": float(kt[3]), "peak": FP64_PEAK_GFLOPS,
            "peak_source": "FP64 FMA units x max SM clock (152 SMs x 2 FMA/clk x 2 flops x 2.07 GHz); "
                           "MEASURED_PEAKS.json has no FP64 figure",
@@ -399,7 +399,7 @@ def rooflines(W, r):
     m2l["achieved"] = work["m2l_flops"] / (kt[3] / 1e3) / 1e9 if kt[3] > 0 else None
     m2l["frac"] = m2l["achieved"] / FP64_PEAK_GFLOPS if m2l["achieved"] else None
     if W["DIM"] == 3 and W["KERNEL"]:
-        prof = profile_figures("m2l_traffic_helm3d_k10_n1e6.txt", TR3H_SOURCES)
+        prof = profile_figures("m2l_traffic_helm3d_k10_n1e6.txt", PAIRS3D_SOURCES)
         if prof and "dram_bytes_per_apply" in prof:
             m2l["traffic"] = int(float(prof["dram_bytes_per_apply"]))
             m2l["traffic_source"] = prof["_path"]
@@ -917,7 +917,7 @@ def work_model(p, W=None):
                 m2l_flops += npairs * (m2l_flops_pair_3d(int(P[l])) if W["KERNEL"]
                                        else m2l_flops_pair_lap3d(int(P[l])))
                 if W["KERNEL"] and int(P[l]) <= 40:
-                    # the coaxial operators of these pairs are built once (k_tr3h_tri)
+                    # the coaxial operators of these pairs are built once (k_pair_tri)
                     m2l_shared += npairs * m2l_flops_coax_3d(int(P[l]))
     return {"p2p_pairs": int(inf["p2p_pairs"]), "m2l_pairs": int(inf["m2l_pairs"]),
             "m2l_pairs_per_level": pairs_per_level, "orders": [int(x) for x in P],

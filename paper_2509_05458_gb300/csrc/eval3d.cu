@@ -1,5 +1,5 @@
-// FP64 evaluation of 3D expansions at points: M2P over List 3 and L2P, potential
-// and target gradient, Laplace and Helmholtz.
+// FP64 expansions of and at points in 3D, Laplace and Helmholtz: P2M and P2L (their own
+// comment below), M2P over List 3 and L2P, potential and target gradient.
 //
 // The expansion functions (file comments of fmm3d.cu and helm3d.cu) share their
 // dependence on z and rho^2 between +m and -m:

@@ -485,7 +485,7 @@ __global__ void __launch_bounds__(128) k_l2p3f(L2p3fArgs A, const int* __restric
 // Laplace. With y~ = (y - c)/rho_b,
 //   Helmholtz  M_n^m = i k (2n+1) (k rho_b)^n/(2n+1)!! sum s jh_n(k rho) Z_n^{-m}(y~)
 //   Laplace    M_n^m = lsd_n^m rho_b^n sum s Z_n^{-m}(y~)
-// (the forms of k_p2x3h_slp rewritten as in k_l2p3f). Each warp stages 32
+// (scaled as in k_l2p3f). Each warp stages 32
 // sources (their jh table, x+, x-, x3 and density) and then takes (source,
 // harmonic column) items in rounds of 32, one per lane; a column owns the
 // coefficients (n, -mu), n >= |mu|, so with 2P+1 >= 32 columns the lanes of a
