@@ -450,15 +450,16 @@ __global__ void __launch_bounds__(kNearThreads) k_near(KParams K, NearLists L, i
                 // lanes without a source and pairs with x == y (self pair, coincident
                 // point) take a harmless distance and store nothing: the warp stays whole
                 double dr[DIM], di[DIM];
-                int bits = 0;                           // 0 when every difference is (FP64 compares cost an FP64 slot)
+                int hi = 0, lo = 0;                     // the differences' bits (FP64 compares cost an FP64 slot)
 #pragma unroll
                 for (int a = 0; a < DIM; ++a) {
                     dr[a] = tx[a * kNearTargets + t] - yr[a];
                     di[a] = tx[(DIM + a) * kNearTargets + t] - yi[a];
-                    bits |= __double2hiint(dr[a]) | __double2loint(dr[a]) | __double2hiint(di[a]) | __double2loint(di[a]);
+                    hi |= __double2hiint(dr[a]) | __double2hiint(di[a]);
+                    lo |= __double2loint(dr[a]) | __double2loint(di[a]);
                 }
-                // (x - x is +0 in every rounding but one, which is not in use)
-                const bool skip = !valid || bits == 0;
+                // (the difference of -0 and +0 is -0)
+                const bool skip = !valid || ((hi & 0x7fffffff) | lo) == 0;
                 if (skip) {
                     dr[0] = wave.k > 0.0 ? wave.ik : 1.0;
                     di[0] = 0.0;
