@@ -232,10 +232,11 @@ constexpr int kP2PTargets = 32;
 constexpr int kP2PSplit = kP2PThreads / kP2PTargets;
 constexpr int kP2PChunk = 128;
 
-// r^2 = sum d_a^2 of the complex differences (3 DIM + 1 FP64 instructions)
+// r^2 = sum d_a^2 of the complex differences (3 DIM + 1 FP64 instructions). Its imaginary
+// part starts from +0: a sum of zero products is +0, the upper side of the branch cut
 template <int DIM>
 __device__ __forceinline__ cd pair_r2(const double* dr, const double* di) {
-    double x = dr[0] * dr[0], y = dr[0] * di[0];
+    double x = dr[0] * dr[0], y = fma(dr[0], di[0], 0.0);
     x = fma(-di[0], di[0], x);
 #pragma unroll
     for (int a = 1; a < DIM; ++a) {

@@ -40,12 +40,13 @@ struct PairTab {
     double2 hk[kHkGrids * kHkNx * kHkNy][2][kHkDeg + 1];   // Taylor coefficients of the H_0 and H_1 factors
 };
 
-// double -> float by truncation of the bits, for |v| < 2^127 (below 2^-126: 0)
+// double -> float by truncation of the bits, for |v| < 2^127 (below 2^-126: 0 of v's sign,
+// which tells the side of the branch cut)
 __device__ __forceinline__ float seed_f32(double v) {
     unsigned hi = (unsigned)__double2hiint(v), lo = (unsigned)__double2loint(v);
     unsigned f = __funnelshift_l(lo, hi, 3) + 0x40000000u;
     f = (f & 0x7fffffffu) | (hi & 0x80000000u);
-    return (hi & 0x7fffffffu) < 0x38100000u ? 0.f : __uint_as_float(f);
+    return __uint_as_float((hi & 0x7fffffffu) < 0x38100000u ? hi & 0x80000000u : f);
 }
 // float -> double on the bits (normal values; 0 becomes 2^-127)
 __device__ __forceinline__ double widen_f32(float v) {
