@@ -10,6 +10,10 @@
 //   M2M/M2L/L2L: the binomial re-expansions of Lemma 4.2.4 in zeta and eta
 //   separately; the M0 term of M2L is -(1/2k) zeta0^-k M0 (derived from
 //   log(1 - z) = -sum z^k/k).
+//   Stored in units of the box's level: Mp_n / s^n, Mm_n / s^n, Lp_n s^n, Lm_n s^n with
+//   s = 2^(we - l), W = f 2^we, 1/2 <= f < 1. The scaling is exact, every power is then
+//   one of a number of order 1, and deep boxes neither underflow nor overflow (unscaled
+//   z^40 at level 26 of a unit domain is below the smallest double).
 // 2D Helmholtz (Sec. 4.3) -- layout [c_{-P} .. c_P]: with
 //   G_n(d) = J_n(kappa r) e^{in phi}, S_n(d) = H_n^(1)(kappa r) e^{in phi}
 //   and Graf's theorem (Thm 3.2.1): for expansions about c re-centred at c',
@@ -61,11 +65,10 @@ struct Fmm2dState {
     DevBuf<int64_t> exp_off;               // per box (coefficient offset), -1 below l0
     int64_t ncoef = 0;
     int maxP = 0;
-    // Laplace: binomial table C(n, k), n, k <= NB
-    int NB = 0;
-    DevBuf<double> binom;
-    // Laplace, (maxP+1)^2 by [n][k]: C(k-1, n-1) and C(n+k-1, k)
-    DevBuf<double> cm2m, cm2l;
+    // Laplace, (maxP+1)^2 by [n][k]: C(k-1, n-1) 2^-n, C(n+k-1, k) and C(n, k) 2^-k (a
+    // child's unit is half its parent's)
+    DevBuf<double> cm2m, cm2l, cl2l;
+    int we = 0;                            // exponent of the root width: box units 2^(we - l)
     // Helmholtz translation tables
     DevBuf<cd> t_m2l;                      // per List-2 entry: S_j(c_t - c_s), j = -2P..2P
     std::vector<int64_t> m2l_base;         // per level: table base (complex units)
@@ -105,6 +108,9 @@ __device__ __forceinline__ void zeta_eta(cd d0, cd d1, cd& z, cd& e) {
 }
 
 __device__ __forceinline__ cd load_pt(const double* a, int64_t n, int axis, int64_t i) { return cd{a[axis * n + i], 0}; }
+
+// 2^k, |k| <= 1000
+__device__ __forceinline__ double pow2(int k) { return __hiloint2double((1023 + k) << 20, 0); }
 
 // tables and wavenumber constants of the quick Hankel functions (pair64.cuh)
 struct HankelArgs {
@@ -205,20 +211,23 @@ struct ExpArgs {
     const int64_t* eoff;
     int64_t ncoef;
     HankelArgs H;
+    int we;
 };
 
 // term row (Laplace) for a source at d = y - c, regular (P2M) or singular (P2L):
 //   P2M  row_k = -s eta^k/(2k) - nut t eta^{k-1}/2          (k <= P; P + k: zeta, nu)
 //   P2L  row_k = -s zeta^-k/(2k) + nu t zeta^{-k-1}/2       (P + k: eta, nut)
-// as two running products a series, 10 FP64 instructions a term
-__device__ void lap_terms(const PairTab* T, bool sing, cd zeta, cd eta, cd s, cd t, cd nu, cd nut, int P, bool slp,
-                          bool dlp, cd* row) {
-    cd x = eta, y = zeta, nx = nut, ny = nu;           // series 1..P in x, P+1..2P in y
+// as two running products a series, 10 FP64 instructions a term; iu = 1 / the box's unit
+__device__ void lap_terms(const PairTab* T, double iu, bool sing, cd zeta, cd eta, cd s, cd t, cd nu, cd nut, int P,
+                          bool slp, bool dlp, cd* row) {
+    nu = iu * nu;
+    nut = iu * nut;
+    cd x = iu * eta, y = iu * zeta, nx = nut, ny = nu;   // series 1..P in x, P+1..2P in y
     double h = -0.5;
     cd v0 = slp ? s : cd{0, 0};
     if (sing) {
-        x = crcp64(zeta);
-        y = crcp64(eta);
+        x = crcp64(iu * zeta);
+        y = crcp64(iu * eta);
         nx = nu;
         ny = nut;
         h = 0.5;
@@ -305,7 +314,7 @@ __global__ void k_point_to_exp(ExpArgs A, const int* __restrict__ boxes, const i
             cd z, e;
             if (KER == CFMM_LAPLACE) {
                 zeta_eta(y0 - cen0, y1 - cen1, z, e);   // d = y - c
-                lap_terms(A.H.T, sing != 0, z, e, s, t, nu, nut, P, A.slp, A.dlp, row);
+                lap_terms(A.H.T, pow2(A.blevel[b] - A.we), sing != 0, z, e, s, t, nu, nut, P, A.slp, A.dlp, row);
             } else {
                 if (!lrow || sing) {
                     zeta_eta(cen0 - y0, cen1 - y1, z, e);   // D = c - y
@@ -372,8 +381,7 @@ struct TransArgs {
     const int* Plev;
     const int64_t* eoff;
     int64_t ncoef;
-    const double* binom;
-    int NB;
+    int we;
     const cd* tshift;
     const int64_t* shoff;
 };
@@ -383,7 +391,8 @@ struct TransArgs {
 //   M2M  M'_k = z^k (sum_{n<=k} C(k-1,n-1) z^-n M_n - M_0/(2k))
 //   M2L  L_k  = z^-k (sum_n C(n+k-1,k) (-z)^-n M_n - M_0/(2k))
 //   L2L  L'_k = z^-k sum_{n>=k} C(n,k) z^n L_n
-// 2 FP64 instructions a term instead of 8. What bounds a level is the chain of FP64
+// with z in the parent's unit (M2M, L2L) or the level's; the factors 2^-n and 2^-k
+// between a child's and its parent's unit are in the tables. 2 FP64 instructions a term instead of 8. What bounds a level is the chain of FP64
 // instructions one warp issues (one in 64 cycles), so threads are (shift, k): a
 // group of warps takes a shift (its last warp the constant coefficient), and the
 // groups of a block work side by side.
@@ -406,6 +415,7 @@ __global__ void k_m2m_lap(TransArgs T, int lo, const cd* __restrict__ mp_in, cd*
     const int gs = lap_group(P), ng = blockDim.x / gs, g = threadIdx.x / gs, i = threadIdx.x - g * gs;
     cd *x = sm + g * nc, *red = sm + ng * nc + g * nc;
     const int c = i < 2 * P ? i + 1 : 0, k = c > P ? c - P : c;
+    const double iu = pow2(T.blevel[b] - T.we);
     cd acc = {0, 0};
     for (int c0 = T.cbeg[b]; c0 < T.cend[b]; c0 += ng) {
         const int ch = c0 + g;
@@ -421,7 +431,7 @@ __global__ void k_m2m_lap(TransArgs T, int lo, const cd* __restrict__ mp_in, cd*
                 cd z, e;
                 zeta_eta(cd{T.cre[2 * ch] - T.cre[2 * b], T.cim[2 * ch] - T.cim[2 * b]},
                          cd{T.cre[2 * ch + 1] - T.cre[2 * b + 1], T.cim[2 * ch + 1] - T.cim[2 * b + 1]}, z, e);
-                if (c <= P) z = e;
+                z = iu * (c <= P ? e : z);
                 nz = z.x != 0.0 || z.y != 0.0;
                 if (nz) pk = cpow_k(z, k);
                 x[c] = nz ? m[c] * crcp64(pk) : m[c];
@@ -435,7 +445,7 @@ __global__ void k_m2m_lap(TransArgs T, int lo, const cd* __restrict__ mp_in, cd*
                 for (int n = 1; n <= P; ++n) y = rmac(y, __ldg(cm2m + n * (P + 1) + k), xs[n]);   // 0 for n > k
                 acc = cmac(acc, pk, y);
             } else {
-                acc += xs[k];
+                acc += pow2(-k) * xs[k];
             }
         } else if (on && i == 2 * P) {
             acc += m0;
@@ -453,7 +463,7 @@ __global__ void k_m2m_lap(TransArgs T, int lo, const cd* __restrict__ mp_in, cd*
 }
 
 // L2L: child b (at level lo..) receives its parent's local expansion
-__global__ void k_l2l_lap(TransArgs T, int lo, cd* __restrict__ loc, int P) {
+__global__ void k_l2l_lap(TransArgs T, int lo, cd* __restrict__ loc, int P, const double* __restrict__ cl2l) {
     extern __shared__ cd sm[];
     const int b = lo + blockIdx.x, rhs = blockIdx.y, p = T.parent[b], i = threadIdx.x;
     const int c = i < 2 * P ? i + 1 : 0, k = c > P ? c - P : c;
@@ -466,7 +476,7 @@ __global__ void k_l2l_lap(TransArgs T, int lo, cd* __restrict__ loc, int P) {
         cd z, e;
         zeta_eta(cd{T.cre[2 * b] - T.cre[2 * p], T.cim[2 * b] - T.cim[2 * p]},
                  cd{T.cre[2 * b + 1] - T.cre[2 * p + 1], T.cim[2 * b + 1] - T.cim[2 * p + 1]}, z, e);
-        if (c > P) z = e;
+        z = pow2(T.blevel[p] - T.we) * (c > P ? e : z);
         nz = z.x != 0.0 || z.y != 0.0;
         if (nz) pk = cpow_k(z, k);
         // (a zero shift leaves the coefficients; they do not reach L_0)
@@ -478,10 +488,10 @@ __global__ void k_l2l_lap(TransArgs T, int lo, cd* __restrict__ loc, int P) {
         const cd* xs = sm + (c > P ? P : 0);
         if (nz) {
             cd y = {0, 0};
-            for (int n = 1; n <= P; ++n) y = rmac(y, __ldg(T.binom + n * (T.NB + 1) + k), xs[n]);   // 0 for n < k
+            for (int n = 1; n <= P; ++n) y = rmac(y, __ldg(cl2l + n * (P + 1) + k), xs[n]);   // 0 for n < k
             o[c] = cmac(o[c], crcp64(pk), y);
         } else {
-            o[c] += xs[k];
+            o[c] += pow2(-k) * xs[k];
         }
     } else if (i >= (int)blockDim.x - 32) {
         // the constant: the last warp sums L_0 and every scaled coefficient
@@ -568,6 +578,7 @@ struct M2LArgs {
     const cd* tab;
     const int64_t* tbase;
     const int* tq0;
+    int we;
 };
 
 // Laplace M2L (see the comment above k_m2m_lap): a block per box, groups of warps
@@ -580,6 +591,7 @@ __global__ void k_m2l_lap(M2LArgs A, int first_box, const cd* __restrict__ mp, c
     cd *x = sm + g * nc, *red = sm + ng * nc + g * nc;
     const int c = i < 2 * P ? i + 1 : 0, k = c > P ? c - P : c, q1 = A.loff[b + 1];
     const bool last = i >= gs - 32;                     // the group's last warp: the constant
+    const double iu = pow2(A.blevel[b] - A.we);
     cd acc = {0, 0};
     for (int q0 = A.loff[b]; q0 < q1; q0 += ng) {
         const bool on = q0 + g < q1;
@@ -594,7 +606,7 @@ __global__ void k_m2l_lap(M2LArgs A, int first_box, const cd* __restrict__ mp, c
                      cd{A.cre[2 * s + 1] - A.cre[2 * b + 1], A.cim[2 * s + 1] - A.cim[2 * b + 1]}, z, e);
             if (c) {
                 // L_1.. in zeta from the source's zeta series (entries P+1..), L_P+1.. in eta from 1..P
-                pk = cpow_k(crcp64(c <= P ? z : e), k);
+                pk = cpow_k(crcp64(iu * (c <= P ? z : e)), k);
                 cd v = pk * m[c <= P ? P + c : c - P];
                 x[c] = (k & 1) ? -v : v;
             }
@@ -779,7 +791,8 @@ __global__ void k_eval(ExpArgs A, const int* __restrict__ leaves, const int* __r
                          cd{A.xr[A.n + it], A.xi[A.n + it]} - cd{A.cre[2 * s + 1], A.cim[2 * s + 1]}, z, e);
                 if (KER == CFMM_LAPLACE) {
                     // Horner in 1/eta and 1/zeta
-                    cd iz = crcp64(z), ie = crcp64(e), vz = m[2 * Ps], ve = m[Ps];
+                    const double iu = pow2(A.blevel[s] - A.we);
+                    cd iz = crcp64(iu * z), ie = crcp64(iu * e), vz = m[2 * Ps], ve = m[Ps];
                     for (int nn = Ps - 1; nn >= 1; --nn) {
                         ve = cmac(m[nn], ve, ie);
                         vz = cmac(m[Ps + nn], vz, iz);
@@ -828,6 +841,9 @@ __global__ void k_eval(ExpArgs A, const int* __restrict__ leaves, const int* __r
             cd z, e;
             zeta_eta(x0 - cd{A.cre[2 * b], A.cim[2 * b]}, x1 - cd{A.cre[2 * b + 1], A.cim[2 * b + 1]}, z, e);
             if (KER == CFMM_LAPLACE) {
+                const double iu = pow2(A.blevel[b] - A.we);
+                z = iu * z;
+                e = iu * e;
                 cd vz = coef[P], ve = coef[2 * P];
                 for (int nn = P - 1; nn >= 1; --nn) {
                     vz = cmac(coef[nn], vz, z);
@@ -911,10 +927,11 @@ __global__ void k_eval_grad(ExpArgs A, const int* __restrict__ leaves, const int
             cd z, e;
             zeta_eta(x0 - cd{A.cre[2 * s], A.cim[2 * s]}, x1 - cd{A.cre[2 * s + 1], A.cim[2 * s + 1]}, z, e);
             if (KER == CFMM_LAPLACE) {
-                cd iz = cinv(z), ie = cinv(e);
-                dz += 0.5 * (coef[0] * iz);
-                de += 0.5 * (coef[0] * ie);
-                cd zp = iz * iz, ep = ie * ie;   // zeta^-n-1
+                const double iu = pow2(A.blevel[s] - A.we);
+                cd iz = cinv(iu * z), ie = cinv(iu * e);
+                dz += 0.5 * (coef[0] * (iu * iz));
+                de += 0.5 * (coef[0] * (iu * ie));
+                cd zp = iu * (iz * iz), ep = iu * (ie * ie);   // zeta^-n-1
                 for (int nn = 1; nn <= Ps; ++nn) {
                     dz -= (double)nn * (coef[Ps + nn] * zp);
                     de -= (double)nn * (coef[nn] * ep);
@@ -939,7 +956,10 @@ __global__ void k_eval_grad(ExpArgs A, const int* __restrict__ leaves, const int
         zeta_eta(x0 - cd{A.cre[2 * b], A.cim[2 * b]}, x1 - cd{A.cre[2 * b + 1], A.cim[2 * b + 1]}, z, e);
         cd lz = {0, 0}, le = {0, 0};
         if (KER == CFMM_LAPLACE) {
-            cd zp = {1, 0}, ep = {1, 0};   // zeta^n-1
+            const double iu = pow2(A.blevel[b] - A.we);
+            z = iu * z;
+            e = iu * e;
+            cd zp = {iu, 0}, ep = {iu, 0};   // zeta^n-1
             for (int nn = 1; nn <= P; ++nn) {
                 lz += (double)nn * (coef[nn] * zp);
                 le += (double)nn * (coef[P + nn] * ep);
@@ -970,7 +990,8 @@ __global__ void k_eval_grad(ExpArgs A, const int* __restrict__ leaves, const int
 // ---------------------------------------------------------------------------
 // L2P in complex64 arithmetic (mixed precision). With zeta~ = zeta/rho_b,
 // eta~ = eta/rho_b (rho_b = sqrt(2)/2 w, the leaf's radius):
-//   Laplace    u = L^_0 + sum L^_n zeta~^n + L^'_n eta~^n,  L^_n = L_n rho_b^n
+//   Laplace    u = L^_0 + sum L^_n zeta~^n + L^'_n eta~^n,  L^_n = L_n rho_b^n (rho_b in
+//              the box's unit, as L_n is)
 //   Helmholtz  u = sum_n Jh_n(k r) (L^_n zeta~^n + L^_-n eta~^n),
 //              L^_n = L_n (k rho_b/2)^n/n!,  L^_-n = (-1)^n L_-n (k rho_b/2)^n/n!
 // (G_n = J_n(k r) (zeta/r)^n, G_-n = (-1)^n J_n(k r) (eta/r)^n), where
@@ -999,7 +1020,7 @@ __global__ void __launch_bounds__(kExpThreads) k_l2p2f(ExpArgs A, const int* __r
     for (int c = threadIdx.x; c < nc; c += blockDim.x) {
         // Laplace layout [c0, zeta^1..zeta^P, eta^1..eta^P]; Helmholtz [c_-P .. c_P]
         int n = KER == CFMM_LAPLACE ? (c <= P ? c : c - P) : abs(c - P);
-        double s = 1.0, g = KER == CFMM_LAPLACE ? rb : 0.5 * A.kappa * rb;
+        double s = 1.0, g = KER == CFMM_LAPLACE ? pow2(lev - A.we) * rb : 0.5 * A.kappa * rb;
         for (int j = 1; j <= n; ++j) s *= KER == CFMM_LAPLACE ? g : g / j;
         if (KER != CFMM_LAPLACE && c < P && (n & 1)) s = -s;
         coef2[c] = to_cf(s * lc[c]);
@@ -1218,6 +1239,8 @@ void fmm2d_presetup(cfmm_plan_s* P) {
     S->ker = P->kernel;
     S->l0 = T.l0;
     S->nlev = T.nlevels;
+    std::frexp(P->W, &S->we);
+    S->we = std::min(900, std::max(-900, S->we));
     S->Plev.assign(T.nlevels, 0);
     for (int l = 0; l < T.nlevels; ++l) {
         if (P->kernel == CFMM_LAPLACE) S->Plev[l] = nterms_laplace(2, P->sep, P->eps * kPHeadroom);
@@ -1325,31 +1348,23 @@ void fmm2d_setup(cfmm_plan_s* P) {
             upload(S->d_p2l_boxes.get(), boxes.data(), sizeof(int) * boxes.size(), st);
     }
     pt.mark("setup:p2l");
-    // binomials C(n, k), n, k <= 2 maxP + 1 (exact integers up to 2^53, then rounded)
-    S->NB = 2 * maxP + 2;
-    {
-        int NB = S->NB;
-        std::vector<double> bt((size_t)(NB + 1) * (NB + 1), 0.0);
-        for (int n = 0; n <= NB; ++n) {
-            bt[(size_t)n * (NB + 1)] = 1.0;
-            for (int k = 1; k <= n; ++k)
-                bt[(size_t)n * (NB + 1) + k] = bt[(size_t)(n - 1) * (NB + 1) + k - 1] + (k <= n - 1 ? bt[(size_t)(n - 1) * (NB + 1) + k] : 0.0);
+    if (P->kernel == CFMM_LAPLACE) {
+        // binomials C(n, k), n < 2 maxP (exact integers up to 2^53, then rounded)
+        const size_t w = maxP + 1, nb = 2 * (size_t)maxP;
+        std::vector<double> bt(nb * nb, 0.0), a(w * w, 0.0), c(w * w, 0.0), d(w * w, 0.0);
+        for (size_t n = 0; n < nb; ++n) {
+            bt[n * nb] = 1.0;
+            for (size_t k = 1; k <= n; ++k) bt[n * nb + k] = bt[(n - 1) * nb + k - 1] + bt[(n - 1) * nb + k];
         }
-        S->binom.alloc(bt.size());
-        // (a copy from pageable memory returns once the source is staged)
-        upload(S->binom.get(), bt.data(), sizeof(double) * bt.size(), st);
-        if (P->kernel == CFMM_LAPLACE) {
-            size_t w = maxP + 1;
-            std::vector<double> a(w * w, 0.0), c(w * w, 0.0);
-            for (int n = 1; n <= maxP; ++n)
-                for (int k = 1; k <= maxP; ++k) {
-                    if (n <= k) a[n * w + k] = bt[(size_t)(k - 1) * (NB + 1) + n - 1];
-                    c[n * w + k] = bt[(size_t)(n + k - 1) * (NB + 1) + k];
-                }
-            S->cm2m.alloc(a.size());
-            S->cm2l.alloc(c.size());
-            upload(S->cm2m.get(), a.data(), sizeof(double) * a.size(), st);
-            upload(S->cm2l.get(), c.data(), sizeof(double) * c.size(), st);
+        for (size_t n = 1; n < w; ++n)
+            for (size_t k = 1; k < w; ++k) {
+                if (n <= k) a[n * w + k] = std::ldexp(bt[(k - 1) * nb + n - 1], -(int)n);
+                c[n * w + k] = bt[(n + k - 1) * nb + k];
+                if (n >= k) d[n * w + k] = std::ldexp(bt[n * nb + k], -(int)k);
+            }
+        for (auto t : {std::make_pair(&S->cm2m, &a), std::make_pair(&S->cm2l, &c), std::make_pair(&S->cl2l, &d)}) {
+            t.first->alloc(w * w);
+            upload(t.first->get(), t.second->data(), sizeof(double) * w * w, st);
         }
     }
     if (P->kernel == CFMM_HELMHOLTZ) {
@@ -1465,7 +1480,7 @@ static void apply_t(cfmm_plan_s* P, Fmm2dState* S, const cd* sigma, const cd* ta
     cd* lc = P->local.get();
     ExpArgs A{P->xr.get(), P->xi.get(), P->nr.get(), P->ni.get(), P->n, sigma, tau, dstride, P->slp, P->dlp,
               P->kappa, T.level.get(), source_range(P), target_range(P), T.cen_re.get(), T.cen_im.get(),
-              S->dPlev.get(), S->exp_off.get(), S->ncoef, hankel_args(P->kappa)};
+              S->dPlev.get(), S->exp_off.get(), S->ncoef, hankel_args(P->kappa), S->we};
     int maxP = S->maxP;
     // (6) P2L over List 4, added to the local expansions
     auto p2l = [&](cudaStream_t s) {
@@ -1526,7 +1541,7 @@ static void apply_t(cfmm_plan_s* P, Fmm2dState* S, const cd* sigma, const cd* ta
     rec(2);
     // (2) M2M, finest level first
     TransArgs TA{T.level.get(), T.parent.get(), T.cbeg.get(), T.cend.get(), T.cen_re.get(), T.cen_im.get(),
-                 S->dPlev.get(), S->exp_off.get(), S->ncoef, S->binom.get(), S->NB, S->t_shift.get(),
+                 S->dPlev.get(), S->exp_off.get(), S->ncoef, S->we, S->t_shift.get(),
                  S->shift_off.get()};
     // Helmholtz: parts of a coefficient's sum, threads of a block
     auto split = [](int nc) { return std::max(1, std::min(8, 512 / nc)); };
@@ -1556,7 +1571,7 @@ static void apply_t(cfmm_plan_s* P, Fmm2dState* S, const cd* sigma, const cd* ta
     // (4) M2L over List 2 (all levels >= l0)
     {
         M2LArgs MA{T.level.get(), T.cen_re.get(), T.cen_im.get(), S->dPlev.get(), S->exp_off.get(), S->ncoef,
-                   T.loff[1].get(), T.lent[1].get(), S->t_m2l.get(), S->d_m2l_base.get(), S->d_m2l_q0.get()};
+                   T.loff[1].get(), T.lent[1].get(), S->t_m2l.get(), S->d_m2l_base.get(), S->d_m2l_q0.get(), S->we};
         int first = T.level_off[S->l0], nb = T.nboxes - first;
         if (KER == CFMM_HELMHOLTZ && maxP <= 255) {
             // chunks of List-2 entries, then the per-box reduction of the chunk sums
@@ -1600,7 +1615,7 @@ static void apply_t(cfmm_plan_s* P, Fmm2dState* S, const cd* sigma, const cd* ta
         int Pp = S->Plev[l - 1], Pc = S->Plev[l];
         dim3 g(nb, nrhs);
         if (KER == CFMM_LAPLACE) {
-            k_l2l_lap<<<g, lap_group(Pc), sizeof(cd) * (4 * Pc + 1), st>>>(TA, lo, lc, Pc);
+            k_l2l_lap<<<g, lap_group(Pc), sizeof(cd) * (4 * Pc + 1), st>>>(TA, lo, lc, Pc, S->cl2l.get());
         } else {
             const int S2 = split(2 * Pc + 1);
             k_l2l_helm<<<g, threads(2 * Pc + 1, S2), sizeof(cd) * ((2 * Pp + 1) + 2 * (Pc + Pp) + 1 + S2 * (2 * Pc + 1)),
