@@ -266,6 +266,25 @@ void ensure_device_tables() {
     done[dev] = 1;
 }
 
+// once per device: the shared-memory limits of the expansions' kernels
+static void ensure_kernel_limits(int dim) {
+    static std::mutex mu;
+    static std::vector<int> done;
+    int dev = 0;
+    CFMM_CUDA(cudaGetDevice(&dev));
+    std::lock_guard<std::mutex> lk(mu);
+    if ((int)done.size() <= dev) done.resize(dev + 1, 0);
+    if (done[dev] & (1 << dim)) return;
+    if (dim == 2) {
+        init_fmm2d();
+    } else {
+        init_pairs3d();
+        init_eval3d();
+        init_helm3d();
+    }
+    done[dev] |= 1 << dim;
+}
+
 bool is_device_ptr(const void* p) {
     if (!p) return false;
     cudaPointerAttributes a;
@@ -533,6 +552,7 @@ static cfmm_plan_t plan_common(int dim, int kernel, double k, double eps, const 
         P->stream = (cudaStream_t)o.stream;
         CFMM_CUDA(cudaGetDevice(&P->device));
         ensure_device_tables();
+        ensure_kernel_limits(dim);
         for (auto& e : P->ev) CFMM_CUDA(cudaEventCreate(&e));
         for (auto& e : P->ev_p2p) CFMM_CUDA(cudaEventCreate(&e));
         CFMM_CUDA(cudaEventCreateWithFlags(&P->ev_fork, cudaEventDisableTiming));

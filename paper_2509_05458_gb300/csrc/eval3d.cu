@@ -529,12 +529,12 @@ __global__ void __launch_bounds__(kP2xThreads) k_p2x3(P2xK A) {
     }
 }
 
+// shared memory of k_eval3_items, Helmholtz
+constexpr size_t items_bytes(int maxP) { return sizeof(cd) * kEvalWarps * (size_t)(maxP + 2) * 32; }
+
 template <bool LAP, bool GRAD>
 void launch_items(EvalK A, cudaStream_t st, int nrhs, int groups) {
-    const size_t smem = LAP ? 0 : sizeof(cd) * kEvalWarps * (size_t)(A.E.maxP + 2) * 32;
-    if (smem > 48 * 1024)
-        CFMM_CUDA(cudaFuncSetAttribute((const void*)k_eval3_items<LAP, GRAD>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)smem));
+    const size_t smem = LAP ? 0 : items_bytes(A.E.maxP);
     if (A.ntask <= 0) return;
     dim3 g((unsigned)((A.ntask + kEvalWarps - 1) / kEvalWarps), groups, nrhs);
     k_eval3_items<LAP, GRAD><<<g, kEvalWarps * 32, smem, st>>>(A);
@@ -542,6 +542,13 @@ void launch_items(EvalK A, cudaStream_t st, int nrhs, int groups) {
 }
 
 }  // namespace
+
+void init_eval3d() {
+    for (auto f : {(const void*)k_eval3_items<false, false>, (const void*)k_eval3_items<false, true>})
+        CFMM_CUDA(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)items_bytes(kMaxP3Top)));
+    for (auto f : {(const void*)k_p2x3<true>, (const void*)k_p2x3<false>})
+        CFMM_CUDA(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kP2xSmem));
+}
 
 void eval3_qtable(int kind, int N, double* A, double* B, double* D) {
     double d = 1.0;
@@ -608,8 +615,6 @@ bool p2x3_apply(cfmm_plan_s* P, const Eval3Tables& T, const P2x3Args& A, const c
     fit(kP2xSmem, !dlp, 8, 1);
     if (!K.cs) return false;
     const size_t smem = bytes(K.all, K.cs, K.gs);
-    const void* f = lap ? (const void*)k_p2x3<true> : (const void*)k_p2x3<false>;
-    CFMM_CUDA(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kP2xSmem));
     dim3 g(A.cnt, nrhs);
     if (lap) k_p2x3<true><<<g, kP2xThreads, smem, P->stream>>>(K);
     else k_p2x3<false><<<g, kP2xThreads, smem, P->stream>>>(K);

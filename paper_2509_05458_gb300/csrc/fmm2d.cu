@@ -1443,6 +1443,9 @@ void fmm2d_setup(cfmm_plan_s* P) {
     }
     if (S->rows_side) near_join(P);
     pt.mark("setup:rowsjoin");
+}
+
+void init_fmm2d() {
     for (auto f : {(const void*)k_point_to_exp<CFMM_LAPLACE>, (const void*)k_point_to_exp<CFMM_HELMHOLTZ>,
                    (const void*)k_m2m_lap, (const void*)k_m2m_helm, (const void*)k_l2l_lap, (const void*)k_l2l_helm,
                    (const void*)k_m2l_lap, (const void*)k_m2l_helm,

@@ -603,10 +603,8 @@ static void launch_p2m3f(H3Tables* TB, bool helm, cfmm_plan_s* P, const int* box
     size_t smem = p2m3f_smem(PL);
     dim3 g((unsigned)cnt, nrhs);
     if (helm) {
-        if (smem > 48 * 1024) CFMM_CUDA(cudaFuncSetAttribute(k_p2m3f<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
         k_p2m3f<true><<<g, kP2m3fWarps * 32, smem, P->stream>>>(A, boxes, sigma, dstride, out);
     } else {
-        if (smem > 48 * 1024) CFMM_CUDA(cudaFuncSetAttribute(k_p2m3f<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
         k_p2m3f<false><<<g, kP2m3fWarps * 32, smem, P->stream>>>(A, boxes, sigma, dstride, out);
     }
     CFMM_LAUNCHED();
@@ -627,6 +625,11 @@ static void launch_l2p3f(H3Tables* TB, bool helm, cfmm_plan_s* P, const int* lea
 }
 
 }  // namespace
+
+void init_helm3d() {
+    for (auto f : {(const void*)k_p2m3f<true>, (const void*)k_p2m3f<false>})
+        CFMM_CUDA(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, kH3Smem));
+}
 
 // ---------------------------------------------------------------------------
 // host side

@@ -155,5 +155,13 @@ void lap3_l2p32(Lap3Tr* L, cfmm_plan_s* P, const int* leaves, int cnt, int maxP,
 
 void upload_lag_rule_p2p();
 void upload_lag_rule_fmm2d();
+// Shared-memory limits of the kernels of each file, set once per device to what their
+// largest launch takes. (The limit belongs to the function, for the whole process: set to
+// a launch's own size before each launch, a plan on another host thread lowers it between
+// the two calls and the launch is refused.)
+void init_fmm2d();
+void init_pairs3d();
+void init_eval3d();
+void init_helm3d();
 
 }  // namespace cfmm

@@ -626,7 +626,30 @@ __global__ void k_pair_sum(PairArgs A, int lo, const int* __restrict__ q_beg, co
     }
 }
 
+// shared memory of the stages
+constexpr size_t kPairRow = 32 * sizeof(cd);
+constexpr size_t rot_bytes(int Pm) { return 2 * (size_t)(2 * Pm + 1) * kPairRow; }
+constexpr size_t tri_bytes(int NR) { return 3 * (size_t)(NR + 2) * kPairRow; }
+constexpr size_t sect_bytes(int NR) { return 2 * (size_t)(NR + 2) * kPairRow; }
+constexpr size_t coax_bytes(int mode, int Pi) { return (mode == 1 ? 4 : 2) * (size_t)(Pi + 1) * kPairRow; }
+
 }  // namespace
+
+void init_pairs3d() {
+    constexpr int P = kMaxP3Top;
+    auto set = [](const void* f, size_t smem) {
+        CFMM_CUDA(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    };
+    for (auto f : {(const void*)k_pair_fwd<true>, (const void*)k_pair_fwd<false>, (const void*)k_pair_bwd<true>,
+                   (const void*)k_pair_bwd<false>})
+        set(f, rot_bytes(P));
+    set((const void*)k_pair_tri, tri_bytes(2 * P));
+    set((const void*)k_pair_sect, sect_bytes(2 * P));
+    for (auto f : {(const void*)k_pair_coax<true, 1>, (const void*)k_pair_coax<false, 1>}) set(f, coax_bytes(1, P));
+    for (auto f : {(const void*)k_pair_coax<true, 0>, (const void*)k_pair_coax<false, 0>,
+                   (const void*)k_pair_coax<true, 2>, (const void*)k_pair_coax<false, 2>})
+        set(f, coax_bytes(0, P));
+}
 
 void pair_slots_build(cfmm_plan_s* P, PairSlots* S, const std::vector<int>& l2off, int l0) {
     TreeDev& T = P->tree;
@@ -676,7 +699,7 @@ template <bool LAP, int MODE>
 void launch_stages(PairArgs& A, PairSlots* S, const cd* in, int nrhs, int nsm, cudaStream_t st) {
     const int nt = A.ntile, nv = nrhs * (MODE == 1 ? 2 : 1), NR = A.Pi + A.Po;
     if (nt <= 0) return;
-    const size_t K = (size_t)(A.Pm + 1) * (A.Pm + 1), row = 32 * sizeof(cd);
+    const size_t K = (size_t)(A.Pm + 1) * (A.Pm + 1);
     S->pw.alloc((size_t)nt * (4 * A.Pm + 2) * 32);
     S->fl.alloc((size_t)nt * (NR + 1) * 32);
     S->vec.alloc((size_t)nt * nv * K * 32);
@@ -689,15 +712,7 @@ void launch_stages(PairArgs& A, PairSlots* S, const cd* in, int nrhs, int nsm, c
     A.fl = S->fl.get();
     A.vec = S->vec.get();
     A.tri = S->tri.get();
-    const size_t rot_smem = 2 * (size_t)(2 * A.Pm + 1) * row, tri_smem = 3 * (size_t)(NR + 2) * row,
-                 cx_smem = (MODE == 1 ? 4 : 2) * (size_t)(A.Pi + 1) * row;
-    auto need = [](const void* f, size_t smem) {
-        if (smem > 48 * 1024)
-            CFMM_CUDA(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    };
-    need((const void*)k_pair_fwd<LAP>, rot_smem);
-    need((const void*)k_pair_bwd<LAP>, rot_smem);
-    need((const void*)k_pair_coax<LAP, MODE>, cx_smem);
+    const size_t rot_smem = rot_bytes(A.Pm), cx_smem = coax_bytes(MODE, A.Pi);
     // blocks of twice the warps where shared memory leaves one or two an SM
     const int wide = A.Pm > 40 ? 2 * kPairThreads : kPairThreads;
     // small launches: one thread block per order as well
@@ -707,16 +722,13 @@ void launch_stages(PairArgs& A, PairSlots* S, const cd* in, int nrhs, int nsm, c
     k_pair_pre<LAP><<<(nt + 3) / 4, 128, 0, st>>>(A);
     CFMM_LAUNCHED();
     if (!LAP) {
-        need((const void*)k_pair_tri, tri_smem);
         const bool split = nt < 4 * nsm;
         if (split) {
-            const size_t sect_smem = 2 * (size_t)(NR + 2) * row;
-            need((const void*)k_pair_sect, sect_smem);
             S->sect.alloc((size_t)nt * (A.Pn + 1) * (NR + 1) * 32);
-            k_pair_sect<<<nt, 256, sect_smem, st>>>(A, S->sect.get());
+            k_pair_sect<<<nt, 256, sect_bytes(NR), st>>>(A, S->sect.get());
             CFMM_LAUNCHED();
         }
-        k_pair_tri<<<dim3(nt, split ? A.Pn + 1 : 1), wide, tri_smem, st>>>(A, split ? S->sect.get() : nullptr);
+        k_pair_tri<<<dim3(nt, split ? A.Pn + 1 : 1), wide, tri_bytes(NR), st>>>(A, split ? S->sect.get() : nullptr);
         CFMM_LAUNCHED();
     }
     k_pair_fwd<LAP><<<dim3(nv, nt, groups(A.Pi)), wide, rot_smem, st>>>(A, in);
@@ -729,8 +741,8 @@ void launch_stages(PairArgs& A, PairSlots* S, const cd* in, int nrhs, int nsm, c
 
 // tiles of a range: T (Helmholtz) and V within the budget
 int range_tiles(bool lap, int Pm, int nv) {
-    const size_t row = 32 * sizeof(cd), K = (size_t)(Pm + 1) * (Pm + 1);
-    const size_t per = ((lap ? 0 : tri_off(Pm, Pm + 1)) + (size_t)nv * K) * row;
+    const size_t K = (size_t)(Pm + 1) * (Pm + 1);
+    const size_t per = ((lap ? 0 : tri_off(Pm, Pm + 1)) + (size_t)nv * K) * kPairRow;
     return (int)std::max<size_t>(1, std::min<size_t>(kPairBudget / per, 65535));
 }
 
