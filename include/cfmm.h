@@ -320,6 +320,9 @@ int64_t cfmm_launch_count(void);
  * workspaces, plan-construction scratch) fail with CFMM_ENOMEM, whichever
  * call makes them; 0 disarms. Returns 0, or CFMM_EINVAL for count < 0. */
 int cfmm_debug_fail_allocs(int count);
+/* cfmm_debug_fail_allocs_after: the same after `skip` more allocations that
+ * succeed, to reach the later ones of a plan or an apply. */
+int cfmm_debug_fail_allocs_after(int skip, int count);
 
 int cfmm_last_status(void);
 const char* cfmm_last_error(void);

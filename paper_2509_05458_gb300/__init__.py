@@ -86,6 +86,8 @@ def lib():
     L.cfmm_batch_destroy.argtypes = [vp]
     L.cfmm_debug_fail_allocs.restype = ci
     L.cfmm_debug_fail_allocs.argtypes = [ci]
+    L.cfmm_debug_fail_allocs_after.restype = ci
+    L.cfmm_debug_fail_allocs_after.argtypes = [ci, ci]
     L.cfmm_destroy.restype = ci
     L.cfmm_destroy.argtypes = [vp]
     L.cfmm_direct.restype = ci

@@ -26,10 +26,13 @@ std::atomic<int64_t>& launch_counter() {
     return c;
 }
 
-// failure injection (tests): the next g_fail_allocs device allocations fail
-static std::atomic<int> g_fail_allocs{0};
+// failure injection (tests): after g_fail_skip more device allocations, g_fail_allocs fail
+static std::atomic<int> g_fail_allocs{0}, g_fail_skip{0};
 static void injected_failure() {
     int n = g_fail_allocs.load();
+    if (n == 0) return;
+    for (int k = g_fail_skip.load(); k > 0;)
+        if (g_fail_skip.compare_exchange_weak(k, k - 1)) return;
     while (n > 0) {
         if (g_fail_allocs.compare_exchange_weak(n, n - 1))
             throw Error{CFMM_ENOMEM, "device allocation failed (injected)"};
@@ -372,7 +375,7 @@ void near_join(cfmm_plan_s* P) {
 }
 
 // the full apply on device buffers (densities [nrhs][ncomp][n], out [nrhs][n])
-static void apply_device(cfmm_plan_s* P, const cd* dens, int nrhs, cd* out, cd* grad = nullptr) {
+static void apply_steps(cfmm_plan_s* P, const cd* dens, int nrhs, cd* out, cd* grad) {
     cudaStream_t st = P->stream;
     int64_t n = P->n;
     int ncomp = (P->slp ? 1 : 0) + (P->dlp ? 1 : 0);
@@ -440,9 +443,25 @@ static void apply_device(cfmm_plan_s* P, const cd* dens, int nrhs, cd* out, cd* 
     }
 }
 
+// An apply that fails between the fork and the join leaves work on the side stream: the
+// plan's stream waits for it, as it does at the end of an apply that succeeds.
+static void apply_device(cfmm_plan_s* P, const cd* dens, int nrhs, cd* out, cd* grad = nullptr) {
+    try {
+        apply_steps(P, dens, nrhs, out, grad);
+    } catch (...) {
+        if (P->p2p_side) {
+            cudaEventRecord(P->ev_join, P->side);
+            cudaStreamWaitEvent(P->stream, P->ev_join, 0);
+        }
+        throw;
+    }
+}
+
 static void destroy_plan(cfmm_plan_s* P) {
     if (!P) return;
-    // queued work of this plan must finish before its buffers return to the pool
+    // queued work of this plan must finish before its buffers return to the pool (the side
+    // stream's too: a setup that failed after its fork has not joined it)
+    if (P->side) cudaStreamSynchronize(P->side);
     cudaStreamSynchronize(P->stream);
     if (P->graph_exec) cudaGraphExecDestroy(P->graph_exec);
     if (P->graph) cudaGraphDestroy(P->graph);
@@ -457,10 +476,7 @@ static void destroy_plan(cfmm_plan_s* P) {
         if (e) cudaEventDestroy(e);
     if (P->ev_fork) cudaEventDestroy(P->ev_fork);
     if (P->ev_join) cudaEventDestroy(P->ev_join);
-    if (P->side) {
-        cudaStreamSynchronize(P->side);
-        cudaStreamDestroy(P->side);
-    }
+    if (P->side) cudaStreamDestroy(P->side);
     delete P;
 }
 
@@ -499,6 +515,16 @@ int64_t cfmm_launch_count(void) { return launch_counter().load(); }
 int cfmm_debug_fail_allocs(int count) {
     return guarded([&] {
         CFMM_REQUIRE(count >= 0, CFMM_EINVAL, "count must be >= 0");
+        g_fail_skip.store(0);
+        g_fail_allocs.store(count);
+    });
+}
+
+int cfmm_debug_fail_allocs_after(int skip, int count) {
+    return guarded([&] {
+        CFMM_REQUIRE(skip >= 0 && count >= 0, CFMM_EINVAL, "skip and count must be >= 0");
+        g_fail_allocs.store(0);
+        g_fail_skip.store(skip);
         g_fail_allocs.store(count);
     });
 }

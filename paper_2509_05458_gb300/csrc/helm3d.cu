@@ -52,6 +52,7 @@
 #include <algorithm>
 #include <cmath>
 #include <map>
+#include <memory>
 #include <mutex>
 
 #include "cfmm_special.cuh"
@@ -206,7 +207,8 @@ static H3Tables* tables(int P) {
     std::lock_guard<std::mutex> lk(g_tab_mu);
     auto& sets = tab_map()[dev];
     if (!sets.empty() && sets.back()->Pmax >= P) return sets.back();
-    H3Tables* T = new H3Tables();
+    auto owned = std::make_unique<H3Tables>();
+    H3Tables* T = owned.get();
     int Pm = std::max(P, 16);
     std::vector<double> D;
     std::vector<int64_t> off;
@@ -328,7 +330,7 @@ static H3Tables* tables(int P) {
     CFMM_CUDA(cudaMemcpy(T->zA.get(), zA.data(), sizeof(double) * zA.size(), cudaMemcpyHostToDevice));
     CFMM_CUDA(cudaMemcpy(T->zB.get(), zB.data(), sizeof(double) * zB.size(), cudaMemcpyHostToDevice));
     T->Pmax = Pm;
-    sets.push_back(T);
+    sets.push_back(owned.release());
     return T;
 }
 
@@ -876,11 +878,11 @@ struct Lap3Tr {
 
 Lap3Tr* lap3_tr_create(cfmm_plan_s* P, int Pord) {
     TreeDev& T = P->tree;
-    Lap3Tr* L = new Lap3Tr();
+    auto L = std::make_unique<Lap3Tr>();
     L->tab = tables(Pord);
     L->Pord = Pord;
     pair_slots_build(P, &L->pairs, T.hloff[1], T.l0);
-    return L;
+    return L.release();
 }
 
 void lap3_p2x(Lap3Tr* L, cfmm_plan_s* P, const P2x3Args& A, const cd* sigma, const cd* tau, int64_t dstride, cd* out,
