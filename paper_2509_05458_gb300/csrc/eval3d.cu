@@ -634,14 +634,16 @@ void eval3_apply(cfmm_plan_s* P, Eval3* E, const Eval3Tables& T, const Eval3Args
     // right-hand sides whose slots fit
     const int ncomp = g ? 3 : 1;
     const int batch = (int)std::max<int64_t>(1, std::min<int64_t>(nrhs, kEvalItems / (K.nslot * ncomp)));
-    E->val.alloc((size_t)batch * ncomp * K.nslot);
+    const bool pot = u && (l2p || nl3 > 0);
+    if (pot) E->val.alloc((size_t)batch * K.nslot);
+    if (g) E->gval.alloc((size_t)batch * 3 * K.nslot);
     if (g && !lap) E->gco.alloc((size_t)6 * A.ncoef * batch);
-    K.val = E->val.get();
     for (int r = 0; r < nrhs; r += batch) {
         const int nr = std::min(batch, nrhs - r);
         K.E.mp = A.mp + (int64_t)r * A.ncoef;
         K.E.loc = A.loc + (int64_t)r * A.ncoef;
-        if (u && (l2p || nl3 > 0)) {
+        if (pot) {
+            K.val = E->val.get();
             K.l2p = l2p ? 1 : 0;
             K.nleaf_tasks = l2p ? A.nleaf : 0;
             K.ntask = K.nleaf_tasks + nl3;
@@ -651,6 +653,7 @@ void eval3_apply(cfmm_plan_s* P, Eval3* E, const Eval3Tables& T, const Eval3Args
             CFMM_LAUNCHED();
         }
         if (!g) continue;
+        K.val = E->gval.get();
         K.l2p = 1;
         K.nleaf_tasks = A.nleaf;
         K.ntask = K.nleaf_tasks + nl3;

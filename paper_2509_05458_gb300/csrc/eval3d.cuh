@@ -23,7 +23,8 @@ struct Eval3 {
     int64_t total = 0;            // items
     DevBuf<int64_t> ioff;         // first item of each leaf of the plan's list
     DevBuf<int> own;              // leaf (position in the list) of each List-3 entry
-    DevBuf<cd> val, gco;
+    DevBuf<cd> val;               // slots of the potential; an apply recorded in a graph keeps the pointer,
+    DevBuf<cd> gval, gco;         // so a gradient has slots of its own, and derived coefficients
 };
 // leaves: box index of each leaf of the plan's list; l3off, st, en: host copies of
 // the List-3 offsets and the boxes' target ranges
