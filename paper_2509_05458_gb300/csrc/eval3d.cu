@@ -36,6 +36,7 @@ __device__ __forceinline__ cd ldc(const cd* p) {
 
 constexpr int kEvalWarps = 4;
 constexpr int64_t kEvalItems = (int64_t)1 << 27;   // slots of a launch over all right-hand sides, about
+constexpr int64_t kEvalSlots = (int64_t)1 << 22;   // slots of a range of leaves (more than one only if they fit)
 
 struct EvalK {
     const double *xr, *xi;
@@ -46,7 +47,8 @@ struct EvalK {
     const double *cre, *cim;
     const int64_t* ioff;
     const int* own;
-    int64_t nslot;                // slots per right-hand side (and component): n for L2P, then the items
+    EvalRange R;                  // the leaves of this launch
+    int64_t nslot;                // its slots per right-hand side (and component): a target's L2P, then the items
     int l2p;                      // 0: List 3 only
     Eval3Tables T;
     const cd* gco;                // Helmholtz gradient: derived coefficients [3][2][ncoef] (multipole, local)
@@ -192,15 +194,16 @@ __global__ void __launch_bounds__(kEvalWarps * 32) k_eval3_items(EvalK A) {
     int b, s, li;
     int64_t slot;
     if (!sing) {
-        li = task;
+        li = A.R.leaf0 + task;
         b = s = A.E.leaves[li];
-        slot = A.trg.st[b];
+        slot = A.trg.st[b] - A.R.t0;
     } else {
         const int e = task - A.nleaf_tasks;
         li = A.own[e];
+        if (li < A.R.leaf0 || li >= A.R.leaf1) return;
         b = A.E.leaves[li];
         s = A.l3[e];
-        slot = A.n + A.ioff[li] + (int64_t)(e - A.l3off[b]) * (A.trg.en[b] - A.trg.st[b]);
+        slot = A.R.nt + (A.ioff[li] - A.ioff[A.R.leaf0]) + (int64_t)(e - A.l3off[b]) * (A.trg.en[b] - A.trg.st[b]);
     }
     const int P = A.E.Plev[A.blevel[s]], t0 = A.trg.st[b], cnt = A.trg.en[b] - t0;
     const int64_t co = (int64_t)rhs * A.E.ncoef + A.E.eoff[s];
@@ -304,13 +307,13 @@ __global__ void k_eval3_own(int nleaf, const int* __restrict__ leaves, const int
 
 // u [rhs][comp][n] += the slots of each target: L2P and its leaf's List 3 in order
 __global__ void k_eval3_sum(EvalK A, int ncomp, cd* __restrict__ u) {
-    const int li = blockIdx.x, row = blockIdx.y, b = A.E.leaves[li];
+    const int li = A.R.leaf0 + blockIdx.x, row = blockIdx.y, b = A.E.leaves[li];
     const int t0 = A.trg.st[b], cnt = A.trg.en[b] - t0, ne = A.l3off[b + 1] - A.l3off[b];
     if (!A.l2p && ne == 0) return;
     const cd* v = A.val + (int64_t)row * A.nslot;
-    const int64_t first = A.n + A.ioff[li];
+    const int64_t l0 = t0 - A.R.t0, first = A.R.nt + (A.ioff[li] - A.ioff[A.R.leaf0]);
     for (int t = threadIdx.x; t < cnt; t += blockDim.x) {
-        cd s = A.l2p ? v[t0 + t] : cd{0, 0};
+        cd s = A.l2p ? v[l0 + t] : cd{0, 0};
         for (int e = 0; e < ne; ++e) s += v[first + (int64_t)e * cnt + t];
         u[(int64_t)row * A.n + A.trg.at(t0 + t)] += s;
     }
@@ -576,7 +579,20 @@ void eval3_build(Eval3* E, const std::vector<int>& leaves, const std::vector<int
         int b = leaves[i];
         off[i + 1] = off[i] + (int64_t)(l3off[b + 1] - l3off[b]) * (en[b] - st[b]);
     }
-    E->total = off.back();
+    // leaves in Morton order: a range's targets are one interval
+    for (size_t i = 0; i < leaves.size();) {
+        EvalRange R{(int)i, (int)i, st[leaves[i]], 0, 0};
+        for (; i < leaves.size(); ++i) {
+            CFMM_REQUIRE(i == 0 || st[leaves[i]] >= en[leaves[i - 1]], CFMM_ECUDA, "leaves out of Morton order");
+            const int64_t nt = en[leaves[i]] - R.t0, slots = nt + off[i + 1] - off[R.leaf0];
+            if (slots > kEvalSlots && R.leaf1 > R.leaf0) break;
+            R.leaf1 = (int)i + 1;
+            R.nt = nt;
+            R.slots = slots;
+        }
+        E->max_slots = std::max(E->max_slots, R.slots);
+        E->ranges.push_back(R);
+    }
     E->ioff.alloc(off.size());
     upload(E->ioff.get(), off.data(), sizeof(int64_t) * off.size(), stream);
     if (l3off.back() == 0) return;
@@ -629,45 +645,51 @@ void eval3_apply(cfmm_plan_s* P, Eval3* E, const Eval3Tables& T, const Eval3Args
     const bool lap = A.kappa == 0.0;
     const int nl3 = Tr.hloff[2].back();
     EvalK K{P->xr.get(), P->xi.get(), P->n, A, target_range(P), Tr.loff[2].get(), Tr.lent[2].get(),
-            Tr.level.get(), Tr.cen_re.get(), Tr.cen_im.get(), E->ioff.get(), E->own.get(), P->n + E->total, 0, T, nullptr, nullptr, 0, 0};
+            Tr.level.get(), Tr.cen_re.get(), Tr.cen_im.get(), E->ioff.get(), E->own.get(), EvalRange{}, 0, 0, T, nullptr,
+            nullptr, 0, 0};
     const int groups = std::max(1, std::min(64, (P->leaf_size + 31) / 32));
-    // right-hand sides whose slots fit
-    const int ncomp = g ? 3 : 1;
-    const int batch = (int)std::max<int64_t>(1, std::min<int64_t>(nrhs, kEvalItems / (K.nslot * ncomp)));
     const bool pot = u && (l2p || nl3 > 0);
-    if (pot) E->val.alloc((size_t)batch * K.nslot);
-    if (g) E->gval.alloc((size_t)batch * 3 * K.nslot);
+    // right-hand sides whose slots fit (a range of one leaf may hold more on its own)
+    const int ncomp = g ? 3 : 1;
+    const int64_t per = std::max<int64_t>(1, std::max(E->max_slots * ncomp, g && !lap ? 6 * A.ncoef : 0));
+    const int batch = (int)std::max<int64_t>(1, std::min<int64_t>(nrhs, kEvalItems / per));
+    if (pot) E->val.alloc((size_t)batch * E->max_slots);
+    if (g) E->gval.alloc((size_t)batch * 3 * E->max_slots);
     if (g && !lap) E->gco.alloc((size_t)6 * A.ncoef * batch);
     for (int r = 0; r < nrhs; r += batch) {
         const int nr = std::min(batch, nrhs - r);
         K.E.mp = A.mp + (int64_t)r * A.ncoef;
         K.E.loc = A.loc + (int64_t)r * A.ncoef;
-        if (pot) {
-            K.val = E->val.get();
-            K.l2p = l2p ? 1 : 0;
-            K.nleaf_tasks = l2p ? A.nleaf : 0;
-            K.ntask = K.nleaf_tasks + nl3;
-            if (lap) launch_items<true, false>(K, st, nr, groups);
-            else launch_items<false, false>(K, st, nr, groups);
-            k_eval3_sum<<<dim3(A.nleaf, nr), 64, 0, st>>>(K, 1, u + (int64_t)r * P->n);
-            CFMM_LAUNCHED();
-        }
-        if (!g) continue;
-        K.val = E->gval.get();
-        K.l2p = 1;
-        K.nleaf_tasks = A.nleaf;
-        K.ntask = K.nleaf_tasks + nl3;
-        if (lap) {
-            launch_items<true, true>(K, st, nr, groups);
-        } else {
+        if (g && !lap) {
             const int lo = Tr.level_off[Tr.l0];
             k_grad_coef<<<dim3(Tr.nboxes - lo, nr, 2), 128, 0, st>>>(K, lo, E->gco.get());
             CFMM_LAUNCHED();
             K.gco = E->gco.get();
-            launch_items<false, true>(K, st, nr, groups);
         }
-        k_eval3_sum<<<dim3(A.nleaf, 3 * nr), 64, 0, st>>>(K, 3, g + (int64_t)r * 3 * P->n);
-        CFMM_LAUNCHED();
+        for (const EvalRange& R : E->ranges) {
+            const int nl = R.leaf1 - R.leaf0;
+            K.R = R;
+            K.nslot = R.slots;
+            if (pot) {
+                K.val = E->val.get();
+                K.l2p = l2p ? 1 : 0;
+                K.nleaf_tasks = l2p ? nl : 0;
+                K.ntask = K.nleaf_tasks + nl3;
+                if (lap) launch_items<true, false>(K, st, nr, groups);
+                else launch_items<false, false>(K, st, nr, groups);
+                k_eval3_sum<<<dim3(nl, nr), 64, 0, st>>>(K, 1, u + (int64_t)r * P->n);
+                CFMM_LAUNCHED();
+            }
+            if (!g) continue;
+            K.val = E->gval.get();
+            K.l2p = 1;
+            K.nleaf_tasks = nl;
+            K.ntask = K.nleaf_tasks + nl3;
+            if (lap) launch_items<true, true>(K, st, nr, groups);
+            else launch_items<false, true>(K, st, nr, groups);
+            k_eval3_sum<<<dim3(nl, 3 * nr), 64, 0, st>>>(K, 3, g + (int64_t)r * 3 * P->n);
+            CFMM_LAUNCHED();
+        }
     }
 }
 

@@ -18,9 +18,17 @@ struct Eval3Tables {
 // host tables of q for orders <= N (kind 0: Z, 1: U, 2: T), A and B of (N+1)^2 entries, D of N+1
 void eval3_qtable(int kind, int N, double* A, double* B, double* D);
 
-// Per plan: items (List-3 entry, target) of each leaf, and the buffers of an apply
+// Per plan: items (List-3 entry, target) of each leaf, and the buffers of an apply. An
+// apply takes ranges of leaves whose slots fit a budget (a graded cloud has far more items
+// than points).
+struct EvalRange {
+    int leaf0, leaf1;             // leaves of the list
+    int64_t t0, nt;               // their targets
+    int64_t slots;                // nt, then the items
+};
 struct Eval3 {
-    int64_t total = 0;            // items
+    std::vector<EvalRange> ranges;
+    int64_t max_slots = 0;        // of a range
     DevBuf<int64_t> ioff;         // first item of each leaf of the plan's list
     DevBuf<int> own;              // leaf (position in the list) of each List-3 entry
     DevBuf<cd> val;               // slots of the potential; an apply recorded in a graph keeps the pointer,
