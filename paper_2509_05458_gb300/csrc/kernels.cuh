@@ -76,6 +76,8 @@ void launch_p2p_grad(int dim, int ker, const KParams& K, const int* leaf_boxes, 
                      int leaf_size);
 
 // tree construction (tree.cu)
+// exclusive scan in -> out (must not alias), asynchronous; plan construction only (scratch)
+void scan_exclusive_async(const int* in, int* out, int n, cudaStream_t st);
 void build_tree(cfmm_plan_s* P, const double* re, const double* im, const double* nre, const double* nim,
                 int top_level_opt);
 // Lists 1-4 of the plan's tree (after build_tree)

@@ -77,51 +77,72 @@ __device__ int pair_shift(const double* cre, const double* cim, int a, int b, cd
     return xy && d[2].x == 0.0 && d[2].y == 0.0 ? kPairFlat : kPairGeneral;
 }
 
-// One thread per List-2 entry (a, b), a < b. Flat pairs fill their level's slots
-// from the front, the others from the back, so a tile holds one sort only and a
-// pair's arithmetic does not depend on its slot. With separate targets (src.map), a
-// pair gets a slot only where one box holds a source and the other a target; the first
-// call (box_a null) counts them. (50,007 targets of 200,000 Laplace sources, order 16:
-// M2L 39.3 -> 13.8 ms; the count is one more launch and host read of the plan.)
-__global__ void k_pair_slots(int nent, const int* __restrict__ loff, const int* __restrict__ lent, int nbox,
-                             const int* __restrict__ level, const int* __restrict__ tile0,
-                             const double* __restrict__ cre, const double* __restrict__ cim, SubRange src,
-                             SubRange trg, int* __restrict__ count, int* __restrict__ box_a, int* __restrict__ box_b, signed char* __restrict__ kind,
-                             int* __restrict__ slot) {
-    int q = blockIdx.x * blockDim.x + threadIdx.x;
-    if (q >= nent) return;
-    int lo = 0, hi = nbox - 1;                    // owner: last box with loff <= q
-    while (lo < hi) {
-        int m = (lo + hi + 1) >> 1;
-        if (loff[m] <= q) lo = m;
-        else hi = m - 1;
+// A warp per box a over its List-2 entries (a, b), a < b, in list order. Flat pairs fill
+// their level's slots from the front, the others from the back, so a tile holds one sort
+// only and a pair's arithmetic does not depend on its slot. The first call (box_a null)
+// counts a box's pairs, cnt[a] flat and cnt[nbox + a] others; the second takes the slots
+// from the counts' scan: they follow from the lists alone, so that the order in which a
+// box's terms are added is the same for every plan of a geometry. With separate targets
+// (src.map), a pair gets a slot only where one box holds a source and the other a target.
+// (50,007 targets of 200,000 Laplace sources, order 16: M2L 39.3 -> 13.8 ms.)
+__global__ void k_pair_slots(int nbox, const int* __restrict__ loff, const int* __restrict__ lent,
+                             const int* __restrict__ level, const int* __restrict__ level_off,
+                             const int* __restrict__ tile0, const double* __restrict__ cre,
+                             const double* __restrict__ cim, SubRange src, SubRange trg, int* __restrict__ cnt,
+                             const int* __restrict__ pos, int* __restrict__ box_a, int* __restrict__ box_b,
+                             signed char* __restrict__ kind, int* __restrict__ slot) {
+    const int a = (int)((blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5), lane = threadIdx.x & 31;
+    if (a >= nbox) return;
+    const int l = level[a], q1 = loff[a + 1];
+    const bool a_src = !src.map || src.st[a] < src.en[a], a_trg = !src.map || trg.st[a] < trg.en[a];
+    int nf = 0, no = 0;
+    if (box_a) {
+        nf = 32 * tile0[l] + pos[a] - pos[level_off[l]];
+        no = 32 * tile0[l + 1] - 1 - (pos[nbox + a] - pos[nbox + level_off[l]]);
     }
-    int a = lo, b = lent[q];
-    if (b <= a) return;
-    const bool use = !src.map || (src.st[a] < src.en[a] && trg.st[b] < trg.en[b]) ||
-                     (src.st[b] < src.en[b] && trg.st[a] < trg.en[a]);
-    if (!use && !box_a) return;
-    lo = loff[b];                                 // a in the list of b (sorted; List 2 is symmetric)
-    hi = loff[b + 1] - 1;
-    while (lo < hi) {
-        int m = (lo + hi) >> 1;
-        if (lent[m] < a) lo = m + 1;
-        else hi = m;
+    for (int q0 = loff[a]; q0 < q1; q0 += 32) {
+        const int q = q0 + lane, b = q < q1 ? lent[q] : -1;
+        const bool mine = b > a;
+        const bool use = mine && (!src.map || (a_src && trg.st[b] < trg.en[b]) || (a_trg && src.st[b] < src.en[b]));
+        cd d[3];
+        const int kd = use ? pair_shift(cre, cim, a, b, d) : kPairFlat;
+        const unsigned mf = __ballot_sync(0xffffffffu, use && kd == kPairFlat),
+                       mo = __ballot_sync(0xffffffffu, use && kd != kPairFlat), below = (1u << lane) - 1u;
+        if (box_a && mine) {
+            int lo = loff[b], hi = loff[b + 1] - 1;       // a in the list of b (sorted; List 2 is symmetric)
+            while (lo < hi) {
+                int m = (lo + hi) >> 1;
+                if (lent[m] < a) lo = m + 1;
+                else hi = m;
+            }
+            if (!use) {
+                slot[q] = slot[lo] = -1;
+            } else {
+                const int p = kd == kPairFlat ? nf + __popc(mf & below) : no - __popc(mo & below);
+                box_a[p] = a;
+                box_b[p] = b;
+                kind[p] = (signed char)kd;
+                slot[q] = 2 * p;
+                slot[lo] = 2 * p + 1;
+            }
+        }
+        nf += __popc(mf);
+        no += box_a ? -__popc(mo) : __popc(mo);
     }
-    if (!use) {
-        slot[q] = slot[lo] = -1;
-        return;
+    if (!box_a && lane == 0) {
+        cnt[a] = nf;
+        cnt[nbox + a] = no;
+        if (a == 0) cnt[2 * nbox] = 0;
     }
-    cd d[3];
-    int kd = pair_shift(cre, cim, a, b, d), l = level[a];
-    int i = atomicAdd(count + 2 * l + (kd == kPairFlat ? 0 : 1), 1);
-    if (!box_a) return;
-    int p = kd == kPairFlat ? 32 * tile0[l] + i : 32 * tile0[l + 1] - 1 - i;
-    box_a[p] = a;
-    box_b[p] = b;
-    kind[p] = (signed char)kd;
-    slot[q] = 2 * p;
-    slot[lo] = 2 * p + 1;
+}
+
+// pairs before each level: out[l] flat, out[nlev + 1 + l] others
+__global__ void k_pair_levels(int nlev, int nbox, const int* __restrict__ level_off, const int* __restrict__ pos,
+                              int* __restrict__ out) {
+    for (int l = threadIdx.x; l <= nlev; l += blockDim.x) {
+        out[l] = pos[level_off[l]];
+        out[nlev + 1 + l] = pos[nbox + level_off[l]];
+    }
 }
 
 // mode 0: M2M (a = parent <- b = child), 1: M2L (both directions), 2: L2L (b <- a)
@@ -152,7 +173,7 @@ struct PairArgs {
     // direction and right-hand side of vector v
     __device__ int dir(int v) const { return mode == 1 ? v & 1 : mode >> 1; }
     __device__ int rhs(int v) const { return mode == 1 ? v >> 1 : v; }
-    __device__ size_t K() const { return (size_t)(Pm + 1) * (Pm + 1); }
+    __host__ __device__ size_t K() const { return (size_t)(Pm + 1) * (Pm + 1); }
 };
 
 // e^m, e_a^m (m = -Pm..Pm) and the radial sequence, rows [..][32], one thread per
@@ -633,6 +654,9 @@ constexpr size_t tri_bytes(int NR) { return 3 * (size_t)(NR + 2) * kPairRow; }
 constexpr size_t sect_bytes(int NR) { return 2 * (size_t)(NR + 2) * kPairRow; }
 constexpr size_t coax_bytes(int mode, int Pi) { return (mode == 1 ? 4 : 2) * (size_t)(Pi + 1) * kPairRow; }
 
+// blocks of twice the warps where shared memory leaves one or two an SM
+constexpr int pair_threads(int Pm) { return Pm > 40 ? 2 * kPairThreads : kPairThreads; }
+
 }  // namespace
 
 void init_pairs3d() {
@@ -655,31 +679,40 @@ void pair_slots_build(cfmm_plan_s* P, PairSlots* S, const std::vector<int>& l2of
     TreeDev& T = P->tree;
     cudaStream_t st = P->stream;
     const int nent = l2off[T.nboxes];
-    S->tile0.assign(T.nlevels + 1, 0);
-    S->count.alloc(3 * T.nlevels + 1);
-    auto slots = [&](const int* t0, int* box_a, int* box_b, signed char* kind, int* slot) {
-        CFMM_CUDA(cudaMemsetAsync(S->count.get(), 0, sizeof(int) * 2 * T.nlevels, st));
-        k_pair_slots<<<(nent + 127) / 128, 128, 0, st>>>(nent, T.loff[1].get(), T.lent[1].get(), T.nboxes,
-                                                        T.level.get(), t0, T.cen_re.get(), T.cen_im.get(),
-                                                        source_range(P), target_range(P), S->count.get(), box_a, box_b,
-                                                        kind, slot);
+    const int nb = T.nboxes, nlev = T.nlevels;
+    S->tile0.assign(nlev + 1, 0);
+    S->d_tile0.alloc(nlev + 1);
+    int *cnt = nullptr, *pos = nullptr;
+    auto slots = [&](int* box_a, int* box_b, signed char* kind, int* slot) {
+        k_pair_slots<<<(unsigned)(((int64_t)nb * 32 + 127) / 128), 128, 0, st>>>(
+            nb, T.loff[1].get(), T.lent[1].get(), T.level.get(), T.d_level_off.get(), S->d_tile0.get(), T.cen_re.get(),
+            T.cen_im.get(), source_range(P), target_range(P), cnt, pos, box_a, box_b, kind, slot);
         CFMM_LAUNCHED();
     };
-    std::vector<int> cnt(2 * T.nlevels, 0);
-    if (P->n_trg > 0 && nent > 0) {
-        slots(nullptr, nullptr, nullptr, nullptr, nullptr);
-        CFMM_CUDA(cudaMemcpyAsync(cnt.data(), S->count.get(), sizeof(int) * 2 * T.nlevels, cudaMemcpyDeviceToHost, st));
-        CFMM_CUDA(cudaStreamSynchronize(st));
+    std::vector<int> off(2 * (nlev + 1), 0);
+    if (nent > 0) {
+        cnt = plan_scratch().take_n<int>(2 * (size_t)nb + 1);
+        pos = plan_scratch().take_n<int>(2 * (size_t)nb + 1);
+        slots(nullptr, nullptr, nullptr, nullptr);
+        scan_exclusive_async(cnt, pos, 2 * nb + 1, st);
+        if (P->n_trg > 0) {
+            int* d_off = plan_scratch().take_n<int>(off.size());
+            k_pair_levels<<<1, 64, 0, st>>>(nlev, nb, T.d_level_off.get(), pos, d_off);
+            CFMM_LAUNCHED();
+            CFMM_CUDA(cudaMemcpyAsync(off.data(), d_off, sizeof(int) * off.size(), cudaMemcpyDeviceToHost, st));
+            CFMM_CUDA(cudaStreamSynchronize(st));
+        }
     }
-    for (int l = 0; l < T.nlevels; ++l) {
-        int64_t pairs = (l2off[T.level_off[l + 1]] - l2off[T.level_off[l]]) / 2;
+    auto tiles = [](int n) { return (n + 31) / 32; };
+    for (int l = 0; l < nlev; ++l) {
+        const int pairs = (l2off[T.level_off[l + 1]] - l2off[T.level_off[l]]) / 2;
         // flat and other pairs each end with a partial tile
         S->tile0[l + 1] = S->tile0[l] + (l < l0         ? 0
-                                         : P->n_trg > 0 ? (cnt[2 * l] + 31) / 32 + (cnt[2 * l + 1] + 31) / 32
-                                         : pairs        ? (int)((pairs + 31) / 32) + 1
+                                         : P->n_trg > 0 ? tiles(off[l + 1] - off[l]) + tiles(off[nlev + 2 + l] - off[nlev + 1 + l])
+                                         : pairs        ? tiles(pairs) + 1
                                                         : 0);
     }
-    S->nslot = (int64_t)32 * S->tile0[T.nlevels];
+    S->nslot = (int64_t)32 * S->tile0[nlev];
     if (nent <= 0) return;
     S->slot.alloc(nent);
     S->box_a.alloc(std::max<int64_t>(1, S->nslot));
@@ -687,22 +720,28 @@ void pair_slots_build(cfmm_plan_s* P, PairSlots* S, const std::vector<int>& l2of
     S->kind.alloc(std::max<int64_t>(1, S->nslot));
     CFMM_CUDA(cudaMemsetAsync(S->box_a.get(), 0xff, sizeof(int) * S->nslot, st));
     CFMM_CUDA(cudaMemsetAsync(S->box_b.get(), 0xff, sizeof(int) * S->nslot, st));
-    int* t0 = S->count.get() + 2 * T.nlevels;
-    upload(t0, S->tile0.data(), sizeof(int) * (T.nlevels + 1), st);
-    slots(t0, S->box_a.get(), S->box_b.get(), S->kind.get(), S->slot.get());
+    upload(S->d_tile0.get(), S->tile0.data(), sizeof(int) * (nlev + 1), st);
+    slots(S->box_a.get(), S->box_b.get(), S->kind.get(), S->slot.get());
 }
 
 namespace {
 
-// one range of tiles of A: everything but the sum
+// right-hand sides of a range whose vectors fit beside its operators
+int range_rhs(bool lap, const PairArgs& A, int per_rhs, int nrhs) {
+    const size_t tile = (lap ? 0 : tri_off(A.Pm, A.Pm + 1)) * kPairRow, v = (size_t)per_rhs * A.K() * kPairRow;
+    const size_t nt = std::max(1, A.ntile), left = kPairBudget > nt * tile ? kPairBudget - nt * tile : 0;
+    return (int)std::max<size_t>(1, std::min<size_t>(nrhs, left / (nt * v)));
+}
+
+// one range of tiles of A: the pairs' powers, radial rows and operators
 template <bool LAP, int MODE>
-void launch_stages(PairArgs& A, PairSlots* S, const cd* in, int nrhs, int nsm, cudaStream_t st) {
-    const int nt = A.ntile, nv = nrhs * (MODE == 1 ? 2 : 1), NR = A.Pi + A.Po;
+void launch_pairs(PairArgs& A, PairSlots* S, int batch, int nsm, cudaStream_t st) {
+    const int nt = A.ntile, NR = A.Pi + A.Po;
     if (nt <= 0) return;
-    const size_t K = (size_t)(A.Pm + 1) * (A.Pm + 1);
+    const size_t K = A.K();
     S->pw.alloc((size_t)nt * (4 * A.Pm + 2) * 32);
     S->fl.alloc((size_t)nt * (NR + 1) * 32);
-    S->vec.alloc((size_t)nt * nv * K * 32);
+    S->vec.alloc((size_t)nt * batch * (MODE == 1 ? 2 : 1) * K * 32);
     if (!LAP) S->tri.alloc((size_t)nt * tri_off(A.Pm, A.Pm + 1) * 32);
     if (MODE != 1) {
         S->kind_c.alloc((size_t)nt * 32);
@@ -712,13 +751,6 @@ void launch_stages(PairArgs& A, PairSlots* S, const cd* in, int nrhs, int nsm, c
     A.fl = S->fl.get();
     A.vec = S->vec.get();
     A.tri = S->tri.get();
-    const size_t rot_smem = rot_bytes(A.Pm), cx_smem = coax_bytes(MODE, A.Pi);
-    // blocks of twice the warps where shared memory leaves one or two an SM
-    const int wide = A.Pm > 40 ? 2 * kPairThreads : kPairThreads;
-    // small launches: one thread block per order as well
-    auto groups = [&](int P) {
-        return (unsigned)std::min<int64_t>(P + 1, std::max<int64_t>(1, (int64_t)8 * nsm / ((int64_t)nt * nv)));
-    };
     k_pair_pre<LAP><<<(nt + 3) / 4, 128, 0, st>>>(A);
     CFMM_LAUNCHED();
     if (!LAP) {
@@ -728,9 +760,21 @@ void launch_stages(PairArgs& A, PairSlots* S, const cd* in, int nrhs, int nsm, c
             k_pair_sect<<<nt, 256, sect_bytes(NR), st>>>(A, S->sect.get());
             CFMM_LAUNCHED();
         }
-        k_pair_tri<<<dim3(nt, split ? A.Pn + 1 : 1), wide, tri_bytes(NR), st>>>(A, split ? S->sect.get() : nullptr);
+        k_pair_tri<<<dim3(nt, split ? A.Pn + 1 : 1), pair_threads(A.Pm), tri_bytes(NR), st>>>(A, split ? S->sect.get() : nullptr);
         CFMM_LAUNCHED();
     }
+}
+
+// the vectors of `nrhs` right-hand sides through them: everything but the sum
+template <bool LAP, int MODE>
+void launch_vectors(const PairArgs& A, const cd* in, int nrhs, int nsm, cudaStream_t st) {
+    const int nt = A.ntile, nv = nrhs * (MODE == 1 ? 2 : 1), wide = pair_threads(A.Pm);
+    if (nt <= 0) return;
+    const size_t rot_smem = rot_bytes(A.Pm), cx_smem = coax_bytes(MODE, A.Pi);
+    // small launches: one thread block per order as well
+    auto groups = [&](int P) {
+        return (unsigned)std::min<int64_t>(P + 1, std::max<int64_t>(1, (int64_t)8 * nsm / ((int64_t)nt * nv)));
+    };
     k_pair_fwd<LAP><<<dim3(nv, nt, groups(A.Pi)), wide, rot_smem, st>>>(A, in);
     CFMM_LAUNCHED();
     k_pair_coax<LAP, MODE><<<dim3(nrhs, nt, A.Pn + 1), kPairThreads, cx_smem, st>>>(A);
@@ -739,10 +783,15 @@ void launch_stages(PairArgs& A, PairSlots* S, const cd* in, int nrhs, int nsm, c
     CFMM_LAUNCHED();
 }
 
-// tiles of a range: T (Helmholtz) and V within the budget
-int range_tiles(bool lap, int Pm, int nv) {
+// Tiles of a range: T (Helmholtz) and V of kPairRhs right-hand sides within the budget.
+// The number of right-hand sides has no part in it: where a box's pairs fall into several
+// ranges, the cuts decide the order of its sum, and a right-hand side's result is the same
+// alone and among others. (4: a single one leaves half the budget unused, and T is read
+// once for every four of several.)
+constexpr int kPairRhs = 4;
+int range_tiles(bool lap, int Pm, int per_rhs) {
     const size_t K = (size_t)(Pm + 1) * (Pm + 1);
-    const size_t per = ((lap ? 0 : tri_off(Pm, Pm + 1)) + (size_t)nv * K) * kPairRow;
+    const size_t per = ((lap ? 0 : tri_off(Pm, Pm + 1)) + (size_t)(kPairRhs * per_rhs) * K) * kPairRow;
     return (int)std::max<size_t>(1, std::min<size_t>(kPairBudget / per, 65535));
 }
 
@@ -793,14 +842,19 @@ void launch_m2l(cfmm_plan_s* P, PairSlots* S, PairArgs A, int l_lo, int l_hi, co
     A.box_a = S->box_a.get();
     A.box_b = S->box_b.get();
     A.kind = S->kind.get();
-    const int cap = range_tiles(LAP, A.Pm, 2 * nrhs), end = S->tile0[l_hi];
+    const int cap = range_tiles(LAP, A.Pm, 2), end = S->tile0[l_hi];
     bool first = true;
     A.t0 = S->tile0[l_lo];
     do {                       // (also without pairs: the boxes' expansions become zero)
         A.ntile = std::min(cap, end - A.t0);
-        launch_stages<LAP, 1>(A, S, mp, nrhs, nsm, P->stream);
-        launch_sum<LAP>(A, lo, nb, Tr.loff[1].get(), Tr.loff[1].get() + 1, S->slot.get(), nullptr, first, lc, nrhs, nsm,
-                        P->stream);
+        const int batch = range_rhs(LAP, A, 2, nrhs);
+        launch_pairs<LAP, 1>(A, S, batch, nsm, P->stream);
+        for (int r = 0; r < nrhs; r += batch) {
+            const int nr = std::min(batch, nrhs - r);
+            launch_vectors<LAP, 1>(A, mp + (int64_t)r * A.ncoef, nr, nsm, P->stream);
+            launch_sum<LAP>(A, lo, nb, Tr.loff[1].get(), Tr.loff[1].get() + 1, S->slot.get(), nullptr, first,
+                            lc + (int64_t)r * A.ncoef, nr, nsm, P->stream);
+        }
         first = false;
         A.t0 += A.ntile;
     } while (A.t0 < end);
@@ -813,17 +867,24 @@ void launch_child(cfmm_plan_s* P, PairSlots* S, PairArgs A, int l, const cd* in,
     TreeDev& Tr = P->tree;
     const int c0 = Tr.level_off[l + 1], c1 = Tr.level_off[l + 2], nsm = sm_count(P);
     const int64_t need = ((int64_t)(c1 - c0) + 31) / 32;
-    const int cap = range_tiles(LAP, A.Pm, nrhs);
+    const int cap = range_tiles(LAP, A.Pm, 1);
     for (int64_t t = 0; t < need; t += cap) {
         A.ntile = (int)std::min<int64_t>(cap, need - t);
         A.lo = c0 + (int)(32 * t);
         A.hi = (int)std::min<int64_t>(c1, (int64_t)A.lo + 32 * (int64_t)A.ntile);
-        launch_stages<LAP, MODE>(A, S, in, nrhs, nsm, P->stream);
-        if (MODE == 0)
-            launch_sum<LAP>(A, Tr.level_off[l], Tr.level_off[l + 1] - Tr.level_off[l], Tr.cbeg.get(), Tr.cend.get(),
-                            nullptr, Tr.leaf.get(), true, out, nrhs, nsm, P->stream);
-        else
-            launch_sum<LAP>(A, A.lo, A.hi - A.lo, nullptr, nullptr, nullptr, nullptr, false, out, nrhs, nsm, P->stream);
+        const int batch = range_rhs(LAP, A, 1, nrhs);
+        launch_pairs<LAP, MODE>(A, S, batch, nsm, P->stream);
+        for (int r = 0; r < nrhs; r += batch) {
+            const int nr = std::min(batch, nrhs - r);
+            const int64_t at = (int64_t)r * A.ncoef;
+            launch_vectors<LAP, MODE>(A, in + at, nr, nsm, P->stream);
+            if (MODE == 0)
+                launch_sum<LAP>(A, Tr.level_off[l], Tr.level_off[l + 1] - Tr.level_off[l], Tr.cbeg.get(), Tr.cend.get(),
+                                nullptr, Tr.leaf.get(), true, out + at, nr, nsm, P->stream);
+            else
+                launch_sum<LAP>(A, A.lo, A.hi - A.lo, nullptr, nullptr, nullptr, nullptr, false, out + at, nr, nsm,
+                                P->stream);
+        }
     }
 }
 

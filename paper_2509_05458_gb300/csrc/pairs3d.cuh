@@ -27,8 +27,9 @@ struct PairSlots {
     DevBuf<int> box_a, box_b;     // the pair's boxes (a < b), -1 for an empty slot
     DevBuf<signed char> kind;     // kPairFlat, kPairGeneral, kPairIso + k
     DevBuf<int> slot;             // per List-2 entry: 2 slot + (0: owner is box_a, 1: box_b)
-    DevBuf<int> count;            // per level: slots given to flat and to other pairs
-    // workspaces of an apply
+    DevBuf<int> d_tile0;
+    // workspaces of an apply; an apply recorded in a graph keeps the pointers, and no size
+    // here grows when the right-hand sides become fewer
     DevBuf<cd> pw, fl, sect, tri, vec;
     DevBuf<signed char> kind_c;   // M2M, L2L: kind of each child's shift
 };

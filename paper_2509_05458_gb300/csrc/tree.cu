@@ -99,7 +99,7 @@ __global__ void k_scan_add(int* __restrict__ out, int n, const int* __restrict__
 }
 
 // exclusive scan in -> out (must not alias), asynchronous
-static void scan_exclusive_async(const int* in, int* out, int n, cudaStream_t st) {
+void scan_exclusive_async(const int* in, int* out, int n, cudaStream_t st) {
     if (n <= 0) return;
     int nb = (n + kScanTile - 1) / kScanTile;
     if (nb <= kScanSerial) {
