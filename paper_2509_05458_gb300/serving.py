@@ -30,6 +30,7 @@ from __future__ import annotations
 
 import concurrent.futures as cfut
 import dataclasses
+import math
 import statistics
 import threading
 import time
@@ -106,17 +107,28 @@ class Result:
 
 
 def estimate_bytes(req: Request) -> int:
-    """Conservative device-memory footprint of a request's plan and workspaces."""
+    """Conservative device-memory footprint of a request's plan and workspaces, one
+    right-hand side at a time as the server applies them."""
     n, dim = req.n, req.dim
     per_point = 8 * 4 * dim + 12 + 16 * 4          # points/normals, keys/perm, densities, results
     helm = (req.kernel & 0xF) == 1
     per_point += 2500 if helm else 400               # expansions and translation tables
     extra = 0
-    if helm and dim == 3:
-        # M2L coaxial operators built ahead for a level (about 4.4 kB per point
-        # at leaf 256, growing as the leaves shrink), capped by the library's
-        # per-launch operator budget
-        extra = min(6 << 30, int(n * 4500 * 256 / max(req.leaf_size, 1)))
+    if dim == 3:
+        extra = 64 << 20                             # evaluation slots of a range of leaves
+        budget = 6 << 30                             # of a range of List-2 pairs
+        if helm:
+            # coaxial operators and vectors of a range of pairs (4.4 kB of operators per
+            # point at leaf 256, growing as the leaves shrink, vectors and powers 0.75 of
+            # that at order 16), the powers and sectorial columns on top of the budget
+            extra += min(int(1.2 * budget), int(n * 4500 * 1.75 * 256 / max(req.leaf_size, 1)))
+        else:
+            # expansions; vectors of a range of pairs, whose budget counts four right-hand
+            # sides, and their powers. Boxes and pairs of a surface, leaves 0.3 full on average
+            P = math.ceil(math.log(0.1 * req.eps) / math.log(math.sqrt(3.0) / (2 * max(req.sep, 1) + 1)))
+            boxes = n / (0.3 * max(req.leaf_size, 1)) * 1.34
+            pairs = boxes * 1.5 * (2 * max(req.sep, 1) + 1) ** 2
+            extra += int(boxes * 32 * (P + 1) ** 2 + min(pairs * 32 * (P + 1) ** 2, budget / 4) * (1 + 3 / (P + 1)))
     return int(n * per_point + extra + (96 << 20))   # + plan-construction scratch
 
 
