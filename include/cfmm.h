@@ -305,8 +305,10 @@ int cfmm_plan_export_list(cfmm_plan_t plan, int which, int64_t* offsets, int32_t
 int cfmm_plan_timings(cfmm_plan_t plan, double* t, int nsteps);
 
 /* cfmm_plan_set_timing: 0 = off; 1 = record per-step CUDA events during apply
- * (the near field runs beside the far field on the plan's second stream, so
- * concurrent steps share the SMs); 2 = serialised: the near field runs in line
+ * (the near field runs beside the far field on the plan's second stream, in 2D
+ * P2L and a mixed plan's M2P as well; each is timed there by events of its own,
+ * so concurrent steps share the SMs and the times add up to more than the
+ * apply); 2 = serialised: the near field runs in line
  * on the plan's stream and every step's time is its kernels' alone (slower
  * apply, same result bit for bit). Returns CFMM_EINVAL for other values. */
 int cfmm_plan_set_timing(cfmm_plan_t plan, int on);

@@ -364,12 +364,11 @@ cudaStream_t near_fork(cfmm_plan_s* P) {
 }
 
 void near_launched(cfmm_plan_s* P) {
-    if (P->p2p_serial) CFMM_CUDA(cudaEventRecord(P->ev_p2p[1], P->stream));
+    if (P->timing) CFMM_CUDA(cudaEventRecord(P->ev_p2p[1], P->p2p_serial ? P->stream : P->side));
 }
 
 void near_join(cfmm_plan_s* P) {
     if (P->p2p_serial) return;
-    if (P->timing) CFMM_CUDA(cudaEventRecord(P->ev_p2p[1], P->side));
     CFMM_CUDA(cudaEventRecord(P->ev_join, P->side));
     CFMM_CUDA(cudaStreamWaitEvent(P->stream, P->ev_join, 0));
 }
@@ -396,6 +395,7 @@ static void apply_steps(cfmm_plan_s* P, const cd* dens, int nrhs, cd* out, cd* g
     cd* ta = P->dlp ? P->dens_s.get() + (P->slp ? (int64_t)n * nrhs : 0) : nullptr;
     P->p2p_side = false;
     P->p2p_serial = false;
+    P->p2l_side = P->m2p_side = false;
     record(P, 0);
     dim3 g((unsigned)((n + 255) / 256), nrhs);
     int comp = 0;
@@ -440,6 +440,13 @@ static void apply_steps(cfmm_plan_s* P, const cd* dens, int nrhs, cd* out, cd* g
             // in line it is launched inside the P2M bracket
             if (P->p2p_serial) P->step_ms[1] -= ms;
         }
+        // 2D: P2L and mixed M2P on the side stream, outside their steps' brackets
+        for (int i = 0; i < 2; ++i) {
+            if (!(i ? P->m2p_side : P->p2l_side)) continue;
+            float ms = 0.f;
+            CFMM_CUDA(cudaEventElapsedTime(&ms, P->ev_side[2 * i], P->ev_side[2 * i + 1]));
+            P->step_ms[i ? 7 : 4] += ms;
+        }
     }
 }
 
@@ -473,6 +480,8 @@ static void destroy_plan(cfmm_plan_s* P) {
     for (auto& e : P->ev_p2p)
         if (e) cudaEventDestroy(e);
     for (auto& e : P->ev_far)
+        if (e) cudaEventDestroy(e);
+    for (auto& e : P->ev_side)
         if (e) cudaEventDestroy(e);
     if (P->ev_fork) cudaEventDestroy(P->ev_fork);
     if (P->ev_join) cudaEventDestroy(P->ev_join);
@@ -583,8 +592,10 @@ static cfmm_plan_t plan_common(int dim, int kernel, double k, double eps, const 
         for (auto& e : P->ev_p2p) CFMM_CUDA(cudaEventCreate(&e));
         CFMM_CUDA(cudaEventCreateWithFlags(&P->ev_fork, cudaEventDisableTiming));
         CFMM_CUDA(cudaEventCreateWithFlags(&P->ev_join, cudaEventDisableTiming));
-        if (dim == 2)
+        if (dim == 2) {
             for (auto& e : P->ev_far) CFMM_CUDA(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
+            for (auto& e : P->ev_side) CFMM_CUDA(cudaEventCreate(&e));
+        }
         CFMM_CUDA(cudaStreamCreateWithFlags(&P->side, cudaStreamNonBlocking));
         Scratch& scr = plan_scratch();
         scr.rewind();

@@ -334,6 +334,8 @@ struct cfmm_plan_s {
     cudaStream_t side = nullptr;
     cudaEvent_t ev_fork = nullptr, ev_join = nullptr, ev_p2p[2] = {};
     cudaEvent_t ev_far[2] = {};      // far-field work on the side stream (2D): P2L done, multipoles ready
+    cudaEvent_t ev_side[4] = {};     // its timing brackets: P2L, M2P
+    bool p2l_side = false, m2p_side = false;   // which of them the last apply ran there
     bool p2p_side = false;           // the last apply ran the near field on `side`
     bool p2p_serial = false;         // the last apply ran it in line (timing mode 2)
     // captured apply

@@ -1517,9 +1517,15 @@ static void apply_t(cfmm_plan_s* P, Fmm2dState* S, const cd* sigma, const cd* ta
     cudaStream_t ns = near_fork(P);
     {
         if (p2l_first) {
+            P->p2l_side = true;
+            if (P->timing) CFMM_CUDA(cudaEventRecord(P->ev_side[0], ns));
             CFMM_CUDA(cudaMemsetAsync(lc, 0, sizeof(cd) * need, ns));
             p2l(ns);
             CFMM_CUDA(cudaEventRecord(P->ev_far[0], ns));
+            if (P->timing) {
+                CFMM_CUDA(cudaEventRecord(P->ev_side[1], ns));
+                CFMM_CUDA(cudaEventRecord(P->ev_p2p[0], ns));    // the near field begins here
+            }
         }
         launch_p2p(2, KER, K, S->d_leaves_l0.get(), (int)S->leaves_l0.size(), near_ranges(P),
                    T.loff[0].get(), T.lent[0].get(), u, nrhs, false, ns, P->precision == CFMM_MIXED, P->leaf_size);
@@ -1568,7 +1574,10 @@ static void apply_t(cfmm_plan_s* P, Fmm2dState* S, const cd* sigma, const cd* ta
     if (m2p_side) {
         CFMM_CUDA(cudaEventRecord(P->ev_far[1], st));
         CFMM_CUDA(cudaStreamWaitEvent(ns, P->ev_far[1], 0));
+        P->m2p_side = true;
+        if (P->timing) CFMM_CUDA(cudaEventRecord(P->ev_side[2], ns));
         eval(ns, 0);
+        if (P->timing) CFMM_CUDA(cudaEventRecord(P->ev_side[3], ns));
     }
     if (p2l_first) CFMM_CUDA(cudaStreamWaitEvent(st, P->ev_far[0], 0));
     // (4) M2L over List 2 (all levels >= l0)

@@ -57,7 +57,7 @@ inline NearRanges near_ranges(const cfmm_plan_s* P) {
 // near field of an apply on the plan's side stream: near_fork() makes the
 // side stream wait for what the plan's stream has queued and returns it;
 // near_join() makes the plan's stream wait for the side stream. In the
-// serialised timing mode near_fork() returns the plan's stream itself and
+// serialised timing mode near_fork() returns the plan's stream itself.
 // near_launched(), called right after the near-field launch, closes its
 // timing bracket.
 cudaStream_t near_fork(cfmm_plan_s* P);
