@@ -107,8 +107,6 @@ __device__ __forceinline__ void zeta_eta(cd d0, cd d1, cd& z, cd& e) {
     e = d0 - mul_i(d1);
 }
 
-__device__ __forceinline__ cd load_pt(const double* a, int64_t n, int axis, int64_t i) { return cd{a[axis * n + i], 0}; }
-
 // 2^k, |k| <= 1000
 __device__ __forceinline__ double pow2(int k) { return __hiloint2double((1023 + k) << 20, 0); }
 
@@ -1468,7 +1466,7 @@ static void apply_t(cfmm_plan_s* P, Fmm2dState* S, const cd* sigma, const cd* ta
     if (T.nboxes <= 1) {
         for (int i = 2; i <= 6; ++i) rec(i);
         launch_p2p(2, KER, K, T.d_leaf_boxes.get(), T.nleaves, near_ranges(P), T.loff[0].get(),
-                   T.lent[0].get(), u, nrhs, false, st, P->precision == CFMM_MIXED, P->leaf_size);
+                   T.lent[0].get(), u, nrhs, st, P->precision == CFMM_MIXED, P->leaf_size);
         if (g)
             launch_p2p_grad(2, KER, K, T.d_leaf_boxes.get(), T.nleaves, near_ranges(P), T.loff[0].get(),
                             T.lent[0].get(), g, nrhs, st, P->leaf_size);
@@ -1528,7 +1526,7 @@ static void apply_t(cfmm_plan_s* P, Fmm2dState* S, const cd* sigma, const cd* ta
             }
         }
         launch_p2p(2, KER, K, S->d_leaves_l0.get(), (int)S->leaves_l0.size(), near_ranges(P),
-                   T.loff[0].get(), T.lent[0].get(), u, nrhs, false, ns, P->precision == CFMM_MIXED, P->leaf_size);
+                   T.loff[0].get(), T.lent[0].get(), u, nrhs, ns, P->precision == CFMM_MIXED, P->leaf_size);
         if (g)
             launch_p2p_grad(2, KER, K, S->d_leaves_l0.get(), (int)S->leaves_l0.size(), near_ranges(P),
                             T.loff[0].get(), T.lent[0].get(), g, nrhs, ns, P->leaf_size);

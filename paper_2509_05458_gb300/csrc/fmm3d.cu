@@ -153,7 +153,7 @@ void fmm3d_apply(cfmm_plan_s* P, const cd* sigma, const cd* tau, int64_t dstride
     if (T.nboxes <= 1) {
         for (int i = 2; i <= 6; ++i) rec(i);
         launch_p2p(3, P->kernel, K, T.d_leaf_boxes.get(), T.nleaves, near_ranges(P), T.loff[0].get(),
-                   T.lent[0].get(), u, nrhs, false, st, mixed, P->leaf_size);
+                   T.lent[0].get(), u, nrhs, st, mixed, P->leaf_size);
         if (g)
             launch_p2p_grad(3, P->kernel, K, T.d_leaf_boxes.get(), T.nleaves, near_ranges(P), T.loff[0].get(), T.lent[0].get(), g, nrhs, st, P->leaf_size);
         rec(7);
@@ -169,7 +169,7 @@ void fmm3d_apply(cfmm_plan_s* P, const cd* sigma, const cd* tau, int64_t dstride
     // (3) P2P (writes u) on the side stream, beside the far field
     {
         cudaStream_t ns = near_fork(P);
-        launch_p2p(3, P->kernel, K, S->d_leaves_l0.get(), (int)S->leaves_l0.size(), near_ranges(P), T.loff[0].get(), T.lent[0].get(), u, nrhs, false, ns, mixed, P->leaf_size);
+        launch_p2p(3, P->kernel, K, S->d_leaves_l0.get(), (int)S->leaves_l0.size(), near_ranges(P), T.loff[0].get(), T.lent[0].get(), u, nrhs, ns, mixed, P->leaf_size);
         if (g)
             launch_p2p_grad(3, P->kernel, K, S->d_leaves_l0.get(), (int)S->leaves_l0.size(), near_ranges(P), T.loff[0].get(), T.lent[0].get(), g, nrhs, ns, P->leaf_size);
     }

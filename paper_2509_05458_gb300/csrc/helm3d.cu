@@ -78,15 +78,14 @@ struct H3Tables {
     DevBuf<double> Dh;       // D_n[m][m'] for m, m' >= 0, column-major per order
     DevBuf<double> Dg;       // the same scaled by (-1)^n/(2n+1)
     DevBuf<int64_t> Dhoff;   // [Pmax+2]
-    DevBuf<double> zA, zB;   // [(2Pmax+3)^2] by nmi(n, m), m >= 0
     DevBuf<double> al, be, ab, cg, smu, snu;   // coaxial recurrence coefficients (see Tr3Tables)
     DevBuf<double> g3, gp, gm;           // gradient coefficients c3, s+ c+, s- c- by nmi(n, m), all m
-    DevBuf<double> dg, s21;  // sqrt((2m-1)/(2m)), sqrt(2m+1), m <= Pmax+1
     DevBuf<int> knm;         // k -> n * 256 + (m + 128), k < (Pmax+1)^2
     DevBuf<double> lsm, lsd; // eps_m s_n^m and eps_m / s_n^m, s = sqrt((n-|m|)! (n+|m|)!)
     DevBuf<double> fact, ifact;  // j! and 1/j!, j <= 2 Pmax + 2
     DevBuf<double> q[3][3];  // A, B, D of Z, U, T (eval3d.cuh), orders <= Pmax + 2
-    DevBuf<float> zAf, zBf, dgf, s21f;   // FP32 copies of zA, zB, dg, s21 (mixed-precision L2P)
+    // FP32, mixed P2M and L2P: Z recurrence by nmi(n, m), m >= 0; sqrt((2m-1)/(2m)), sqrt(2m+1), m <= Pmax+1
+    DevBuf<float> zAf, zBf, dgf, s21f;
 };
 
 // Tables only grow: a larger order builds a new set and the older sets stay
@@ -282,8 +281,6 @@ static H3Tables* tables(int P) {
     up(T->g3, g3);
     up(T->gp, gp);
     up(T->gm, gm);
-    up(T->dg, dg);
-    up(T->s21, s21);
     {
         std::vector<double> f(2 * Pm + 3), fi(2 * Pm + 3), lm(knm.size()), ld(knm.size());
         f[0] = 1.0;
@@ -323,12 +320,6 @@ static H3Tables* tables(int P) {
         upf(T->dgf, dg);
         upf(T->s21f, s21);
     }
-
-    T->zA.alloc(zA.size());
-    T->zB.alloc(zB.size());
-
-    CFMM_CUDA(cudaMemcpy(T->zA.get(), zA.data(), sizeof(double) * zA.size(), cudaMemcpyHostToDevice));
-    CFMM_CUDA(cudaMemcpy(T->zB.get(), zB.data(), sizeof(double) * zB.size(), cudaMemcpyHostToDevice));
     T->Pmax = Pm;
     sets.push_back(owned.release());
     return T;
@@ -792,7 +783,7 @@ void helm3d_apply(cfmm_plan_s* P, const cd* sigma, const cd* tau, int64_t dstrid
     if (T.nboxes <= 1) {
         for (int i = 2; i <= 6; ++i) rec(i);
         launch_p2p(3, P->kernel, K, T.d_leaf_boxes.get(), T.nleaves, near_ranges(P), T.loff[0].get(),
-                   T.lent[0].get(), u, nrhs, false, st, mixed, P->leaf_size);
+                   T.lent[0].get(), u, nrhs, st, mixed, P->leaf_size);
         if (g)
             launch_p2p_grad(3, P->kernel, K, T.d_leaf_boxes.get(), T.nleaves, near_ranges(P), T.loff[0].get(), T.lent[0].get(), g, nrhs, st, P->leaf_size);
         rec(7);
@@ -809,7 +800,7 @@ void helm3d_apply(cfmm_plan_s* P, const cd* sigma, const cd* tau, int64_t dstrid
     // (3) P2P (writes u) on the side stream, beside the far field
     {
         cudaStream_t ns = near_fork(P);
-        launch_p2p(3, P->kernel, K, S->d_leaves_l0.get(), (int)S->leaves_l0.size(), near_ranges(P), T.loff[0].get(), T.lent[0].get(), u, nrhs, false, ns, mixed, P->leaf_size, T.level.get(), P->W,
+        launch_p2p(3, P->kernel, K, S->d_leaves_l0.get(), (int)S->leaves_l0.size(), near_ranges(P), T.loff[0].get(), T.lent[0].get(), u, nrhs, ns, mixed, P->leaf_size, T.level.get(), P->W,
                    P->sep);
         if (g)
             launch_p2p_grad(3, P->kernel, K, S->d_leaves_l0.get(), (int)S->leaves_l0.size(), near_ranges(P), T.loff[0].get(), T.lent[0].get(), g, nrhs, ns, P->leaf_size);

@@ -67,7 +67,7 @@ void near_join(cfmm_plan_s* P);
 // 3D Helmholtz near field sizes its coordinate grid from them; NULL = unknown);
 // leaf_size bounds the points of a leaf
 void launch_p2p(int dim, int ker, const KParams& K, const int* leaf_boxes, int nleaves, const NearRanges& R,
-                const int* l1off, const int* l1, cd* out, int nrhs, bool add, cudaStream_t st,
+                const int* l1off, const int* l1, cd* out, int nrhs, cudaStream_t st,
                 bool mixed, int leaf_size, const int* blevel = nullptr, double W = 0.0, int sep = 1);
 void launch_direct(int dim, int ker, const KParams& K, cd* out, int nrhs, cudaStream_t st, bool mixed = false);
 // near-field target gradient over List 1 in FP64: g = sorted [nrhs][dim][n], overwritten

@@ -503,14 +503,13 @@ constexpr size_t near_smem() {
 }
 
 template <int DIM, int KER>
-__device__ void finish_target(cd acc, cd* red, int tl, int split, bool tvalid, cd* out, bool add) {
+__device__ void finish_target(cd acc, cd* red, int tl, int split, bool tvalid, cd* out) {
     red[split * kP2PTargets + tl] = acc;
     __syncthreads();
     if (split == 0 && tvalid) {
         cd s = red[tl];
         for (int q = 1; q < kP2PSplit; ++q) s += red[q * kP2PTargets + tl];
-        if (add) *out += s;
-        else *out = s;
+        *out = s;
     }
     __syncthreads();
 }
@@ -818,7 +817,7 @@ __global__ void __launch_bounds__(kP2PThreads) k_p2p32(KParams K, const int* __r
                                                        const int* __restrict__ bst, const int* __restrict__ sen,
                                                        const int* __restrict__ ten,
                                                        const int* __restrict__ l1off, const int* __restrict__ l1,
-                                                       cd* __restrict__ out, int add) {
+                                                       cd* __restrict__ out) {
     __shared__ SrcTileF S;
     __shared__ cd red[kP2PThreads];
     int b = leaf_boxes[blockIdx.x];
@@ -842,7 +841,7 @@ __global__ void __launch_bounds__(kP2PThreads) k_p2p32(KParams K, const int* __r
             accumulate_sources32<DIM, KER>(S, K, rhs, bst[a], sen[a], tvalid, ref_re, ref_im, xh_r, xl_r, xh_i,
                                            xl_i, acc, split);
         }
-        finish_target<DIM, KER>(acc.value(), red, tl, split, tvalid, out + (int64_t)rhs * K.n_trg + ti, add != 0);
+        finish_target<DIM, KER>(acc.value(), red, tl, split, tvalid, out + (int64_t)rhs * K.n_trg + ti);
     }
 }
 
@@ -866,7 +865,7 @@ __global__ void __launch_bounds__(kP2PThreads) k_direct32(KParams K, cd* __restr
     Kahan acc;
     accumulate_sources32<DIM, KER>(S, K, rhs, 0, (int)K.n_src, tvalid, ref_re, ref_im, xh_r, xl_r, xh_i, xl_i,
                                    acc, split);
-    finish_target<DIM, KER>(acc.value(), red, tl, split, tvalid, out + (int64_t)rhs * K.n_trg + ti, false);
+    finish_target<DIM, KER>(acc.value(), red, tl, split, tvalid, out + (int64_t)rhs * K.n_trg + ti);
 }
 
 // ---------------------------------------------------------------------------
@@ -920,7 +919,7 @@ __global__ void __launch_bounds__(kP2PThreads) k_p2p32g_h3(KParams K, const int*
                                                            const int* __restrict__ l1off,
                                                            const int* __restrict__ l1,
                                                            const int* __restrict__ blevel, double W, int sep,
-                                                           cd* __restrict__ out, int add) {
+                                                           cd* __restrict__ out) {
     __shared__ SrcTileG S;
     __shared__ cd red[kP2PThreads];
     const int64_t n = K.n_src;
@@ -1078,8 +1077,7 @@ __global__ void __launch_bounds__(kP2PThreads) k_p2p32g_h3(KParams K, const int*
                 }
             }
         }
-        finish_target<3, CFMM_HELMHOLTZ>(acc.value(), red, tl, split, tvalid, out + (int64_t)rhs * K.n_trg + ti,
-                                        add != 0);
+        finish_target<3, CFMM_HELMHOLTZ>(acc.value(), red, tl, split, tvalid, out + (int64_t)rhs * K.n_trg + ti);
     }
 }
 
@@ -1122,12 +1120,12 @@ static void launch_near(const KParams& K, const NearLists& L, int nleaves, int l
 
 template <int DIM, int KER>
 static void launch_p2p_t(const KParams& K, const int* leaf_boxes, int nleaves, const NearRanges& R,
-                         const int* l1off, const int* l1, cd* out, int nrhs, bool add, bool mixed, cudaStream_t st,
+                         const int* l1off, const int* l1, cd* out, int nrhs, bool mixed, cudaStream_t st,
                          int leaf_size) {
     if (nleaves == 0) return;
     dim3 grid(nleaves, nrhs);
     if (mixed) {
-        k_p2p32<DIM, KER><<<grid, kP2PThreads, 0, st>>>(K, leaf_boxes, R.first, R.src.en, R.trg.en, l1off, l1, out, add ? 1 : 0);
+        k_p2p32<DIM, KER><<<grid, kP2PThreads, 0, st>>>(K, leaf_boxes, R.first, R.src.en, R.trg.en, l1off, l1, out);
         CFMM_LAUNCHED();
     } else {
         launch_near<DIM, KER, false>(K, NearLists{leaf_boxes, R.src, R.trg, l1off, l1}, nleaves, leaf_size, out, nrhs, st);
@@ -1135,20 +1133,19 @@ static void launch_p2p_t(const KParams& K, const int* leaf_boxes, int nleaves, c
 }
 
 void launch_p2p(int dim, int ker, const KParams& K0, const int* leaf_boxes, int nleaves, const NearRanges& R,
-                const int* l1off, const int* l1, cd* out, int nrhs, bool add, cudaStream_t st,
+                const int* l1off, const int* l1, cd* out, int nrhs, cudaStream_t st,
                 bool mixed, int leaf_size, const int* blevel, double W, int sep) {
     const KParams K = with_wave(K0);
     if (mixed && dim == 3 && ker == CFMM_HELMHOLTZ && blevel && nleaves > 0) {
         dim3 grid(nleaves, nrhs);
-        k_p2p32g_h3<<<grid, kP2PThreads, 0, st>>>(K, leaf_boxes, R, l1off, l1, blevel, W, sep, out,
-                                                  add ? 1 : 0);
+        k_p2p32g_h3<<<grid, kP2PThreads, 0, st>>>(K, leaf_boxes, R, l1off, l1, blevel, W, sep, out);
         CFMM_LAUNCHED();
         return;
     }
-    if (dim == 2 && ker == CFMM_LAPLACE) launch_p2p_t<2, CFMM_LAPLACE>(K, leaf_boxes, nleaves, R, l1off, l1, out, nrhs, add, mixed, st, leaf_size);
-    else if (dim == 2) launch_p2p_t<2, CFMM_HELMHOLTZ>(K, leaf_boxes, nleaves, R, l1off, l1, out, nrhs, add, mixed, st, leaf_size);
-    else if (ker == CFMM_LAPLACE) launch_p2p_t<3, CFMM_LAPLACE>(K, leaf_boxes, nleaves, R, l1off, l1, out, nrhs, add, mixed, st, leaf_size);
-    else launch_p2p_t<3, CFMM_HELMHOLTZ>(K, leaf_boxes, nleaves, R, l1off, l1, out, nrhs, add, mixed, st, leaf_size);
+    if (dim == 2 && ker == CFMM_LAPLACE) launch_p2p_t<2, CFMM_LAPLACE>(K, leaf_boxes, nleaves, R, l1off, l1, out, nrhs, mixed, st, leaf_size);
+    else if (dim == 2) launch_p2p_t<2, CFMM_HELMHOLTZ>(K, leaf_boxes, nleaves, R, l1off, l1, out, nrhs, mixed, st, leaf_size);
+    else if (ker == CFMM_LAPLACE) launch_p2p_t<3, CFMM_LAPLACE>(K, leaf_boxes, nleaves, R, l1off, l1, out, nrhs, mixed, st, leaf_size);
+    else launch_p2p_t<3, CFMM_HELMHOLTZ>(K, leaf_boxes, nleaves, R, l1off, l1, out, nrhs, mixed, st, leaf_size);
 }
 
 template <int DIM, int KER>
