@@ -342,7 +342,8 @@ __global__ void k_eval3_sum(EvalK A, int ncomp, cd* __restrict__ u) {
 // them: first the harmonics (a warp takes cs sources and 32 / cs columns m), then the
 // sums (thread = sum and (n, mu), consecutive lanes on consecutive entries of a
 // source's table). Where the sums do not fit in shared memory together (a double
-// layer at orders above 38, Laplace 48), each product is a pass of its own.
+// layer at orders above 38, Laplace 46 for P2M and 45 for P2L), each product is a pass of
+// its own.
 // ---------------------------------------------------------------------------
 constexpr int kP2xThreads = 256;
 constexpr size_t kP2xSmem = 220 * 1024;

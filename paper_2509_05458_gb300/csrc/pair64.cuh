@@ -118,7 +118,8 @@ struct Wave {
 // 31 bits, so that its product with a (b) is exact and t, v see k r unrounded.
 // Beyond |k Re r| = 8, where the rounding of r itself shows in the phase, the
 // residual r2 - r^2 corrects it (an FP32 product). sin t and cos t - 1 by their
-// Taylor series to t^5 and t^6, e^v to v^4 (|t| < 0.0123; remainders below 1e-17).
+// Taylor series to t^5 and t^6, e^v to v^4 (|t| < 0.0123, |v| < 0.00136; remainders below
+// 1e-17, that of e^v below 4e-17).
 __device__ __forceinline__ cd wave64(const PairTab* __restrict__ T, const Wave& w, cd r2, cd y, cd& r) {
     r = y * r2;
     const double kMagic = 6755399441055744.0;                            // 1.5 2^52
@@ -152,7 +153,7 @@ __device__ __forceinline__ cd wave64(const PairTab* __restrict__ T, const Wave& 
 
 // (log |z|, arg z): c = 2^-e rad_j dir_k close to 1/z with log c tabulated (the
 // products of the short table values are exact), d = z c - 1, |d| < 0.0037, and
-// log(1 + d) = d (1 - d/2 + .. - d^5/6) (remainder below 1e-18), the polynomial
+// log(1 + d) = d (1 - d/2 + .. - d^5/6) (remainder below 2e-18), the polynomial
 // with real coefficients by the two-term recurrence in 2 Re d and |d|^2.
 __device__ __forceinline__ cd clog64(const PairTab* __restrict__ T, cd z) {
     if (!seed_range(z)) return clog_general(z);
@@ -181,8 +182,10 @@ __device__ __forceinline__ cd clog64(const PairTab* __restrict__ T, cd z) {
 // H_nu(z) = e^{iz} z^{-1/2} g_nu(1/z), nu = 0, 1: g is smooth in s = 1/z away
 // from the negative imaginary z axis, so its Taylor polynomial of degree 8 about
 // the nearest grid point (step 1/64 up to |Re s|, |Im s| < 1/2, then 1/32 up to
-// 1 and 1/16 up to 2: |z| > 1/2) leaves less than 2e-17 where -pi/4 <= arg z <=
-// pi/2. Returns the cell of s and the offset from its centre, -1 outside.
+// 1 and 1/16 up to 2: |z| > 1/2) leaves at most 4.8e-16 of g where -pi/4 <= arg z <=
+// pi/2 (in 40 digits: 4.7e-16 at s = 0.0547 (1 + i), the sector's edge; 7e-17 at s =
+// (1 + i)/128, 3e-18 at s = 1/128). Returns the cell of s and the offset from its centre,
+// -1 outside.
 __device__ __forceinline__ int hankel_cell(cd s, cd& ds) {
     int hx = __double2hiint(s.x), hy = __double2hiint(s.y);
     int m = max(hx & 0x7fffffff, hy & 0x7fffffff);
