@@ -170,7 +170,10 @@ int cfmm_apply_grad(cfmm_plan_t plan, const double* densities, int nrhs, double*
  * cfmm_apply_capture: records one cfmm_apply of device buffers (densities,
  * out: device pointers, which must stay valid while the graph is used) into a
  * CUDA graph owned by the plan, replacing any earlier one. The plan must have
- * been created with a non-NULL stream. Nothing runs during capture.
+ * been created with a non-NULL stream. Nothing runs during capture. The graph
+ * keeps the plan's workspaces: between capture and replay, other calls on the
+ * plan may have fewer right-hand sides or a gradient, but not more right-hand
+ * sides than captured (that regrows them).
  * cfmm_apply_replay: launches the captured graph on the plan's stream
  * (asynchronous); the result overwrites the captured `out`.
  * Both return 0 or a negative status.
